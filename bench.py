@@ -55,7 +55,7 @@ METRIC = "point-center pairs/s (dist+argmin)"
 def _direct_kernel_name(low: str, d: int, k: int) -> str:
     """The direct-formula kernel the library launches for this shape (the
     same choice as its launcher: small d with C in shared memory, the tiled
-    FP32 kernel for 16 <= d <= 128 with d % 4 == 0, else one thread per row)."""
+    FP32 kernel for 16 <= d <= 128 with d % 4 == 0, else its general form)."""
     if low == "fp64":
         return "k_direct_assign<double>"
     if d <= 8 and k * d * 4 <= 32 * 1024:

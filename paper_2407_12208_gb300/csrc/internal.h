@@ -89,19 +89,19 @@ cudaError_t launch_predict_candidates(const float* X, int64_t n, int d, const fl
                                       const ColMax* cmx, const TestParams& tp, int nsample,
                                       unsigned long long* acc, int num_sms, cudaStream_t st);
 
-// direct-formula assignment (thread per row).  acc64: binary64 accumulation
-// (the plain FP64 path) else fp32 with certification; rows = all n, or the
-// device list row_list[0 .. *row_count).  Uncertified fp32 rows are appended
-// to amb_list / cnt->amb_count.
+// direct-formula assignment.  acc64: binary64 accumulation (the plain FP64
+// path, all n rows) else fp32 with certification; rows = all n, or the device
+// list row_list[0 .. *row_count).  Uncertified fp32 rows are appended to
+// amb_list / cnt->amb_count.
 // absmax_out (nullable, zeroed by the caller): max |x| over the rows read.
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
                                  double* min_dist, int32_t* amb_list, DevCounters* cnt, float gamma32,
                                  int num_sms, cudaStream_t st, unsigned* absmax_out = nullptr);
 // exact argmin of the rows of a device list, one block per row: fp32 direct
-// values of all centres, certified, binary64 where still open (fp32_first),
-// or binary64 for all centres.
-cudaError_t launch_rows_full(bool fp32_first, const float* X, const float* C, int k, int d, const int32_t* row_list,
+// values of all centres, certified, binary64 where still open.  count_open:
+// those rows are added to cnt->amb_rows.
+cudaError_t launch_rows_full(bool count_open, const float* X, const float* C, int k, int d, const int32_t* row_list,
                              const int* row_count, int32_t* labels, double* min_dist, DevCounters* cnt,
                              float gamma32, int num_sms, cudaStream_t st);
 

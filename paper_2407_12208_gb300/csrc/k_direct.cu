@@ -1,18 +1,18 @@
 // k_direct.cu -- direct-formula assignment kernels, Eq. (dist-direct).
 //
 //  * k_direct_assign<double>: the plain FP64 path (every pair in binary64).
-//  * k_direct_tiled (d % 4 == 0, 16 <= d <= 128), k_direct_small (d <= 8)
-//    and k_direct_assign<float> (other d): fp32 direct distances for the fp32
-//    path and for rows whose tensor-core candidate list overflowed.  Theorem
-//    4.1 bounds each value's relative error by gamma_{d+2}(2^-24); a row whose
-//    best and second-best intervals overlap is not certified and goes to
-//  * k_rows_fp64: binary64 direct distances of one row against all centres
-//    (warp per row, lanes over centres), exact argmin with the lowest index
-//    on ties.  Products and sums are rounded separately (no FMA) so the
-//    values equal the CPU oracle's bit for bit.
+//  * k_direct_tiled, its general form k_direct_assign<float> and (d <= 8, few
+//    centres) k_direct_small: fp32 direct distances for the fp32 path and for rows whose tensor-core candidate list
+//    overflowed.  Theorem 4.1 bounds each value's relative error by
+//    gamma_{d+2}(2^-24); a row whose best and second-best intervals overlap is
+//    not certified and goes to
+//  * k_rows_full: the exact argmin of one row over all centres (a block per
+//    row), lowest index on ties; binary64 values with products and sums rounded
+//    separately (no FMA), equal to the CPU oracle's bit for bit.
 #include <algorithm>
 
 #include "common.cuh"
+#include "df.cuh"
 #include "internal.h"
 
 namespace km {
@@ -21,37 +21,25 @@ constexpr int DA_ROWS = 128;  // rows (threads) per block
 constexpr int DA_TC = 32;     // centres per shared-memory tile
 
 template <typename T>
-__global__ void __launch_bounds__(DA_ROWS) k_direct_assign(const float* __restrict__ X, int64_t n,
-                                                           const float* __restrict__ C, int k, int d,
-                                                           const int32_t* __restrict__ row_list,
-                                                           const int* __restrict__ row_count,
-                                                           int32_t* __restrict__ labels,
-                                                           double* __restrict__ min_dist,
-                                                           int32_t* __restrict__ amb_list, DevCounters* cnt,
-                                                           float gamma32, unsigned* __restrict__ absmax_out) {
+__global__ void __launch_bounds__(DA_ROWS, 5) k_direct_assign(const float* __restrict__ X, int64_t n,
+                                                         const float* __restrict__ C, int k, int d,
+                                                         int32_t* __restrict__ labels, double* __restrict__ min_dist,
+                                                         unsigned* __restrict__ absmax_out) {
     extern __shared__ __align__(16) unsigned char smem[];
     float amx = 0.0f;  // largest |x| this thread stages (absmax_out)
-    // fp32 with d % 4 == 0: rows read four coordinates at a time, row stride
-    // d + 4 (16-byte aligned; consecutive rows 16 bytes apart modulo the 128
-    // banks-bytes when d % 32 == 0: conflict-free); else an odd stride
-    const bool vec4 = sizeof(T) == 4 && (d % 4) == 0;
-    const int ldx = vec4 ? d + 4 : d + 1;
+    const int ldx = d + 1;
     float* Xs = reinterpret_cast<float*>(smem);
     T* Cs = reinterpret_cast<T*>(smem + (((size_t)DA_ROWS * ldx * sizeof(float) + 15) & ~(size_t)15));
-    const int64_t nrows = row_list ? (int64_t)(*row_count) : n;
     const int tid = threadIdx.x;
-    unsigned long long local_amb = 0;
-    for (int64_t base = (int64_t)blockIdx.x * DA_ROWS; base < nrows; base += (int64_t)gridDim.x * DA_ROWS) {
-        const int rows_here = (int)min((int64_t)DA_ROWS, nrows - base);
-        // stage the rows (coalesced when rows are contiguous)
+    for (int64_t base = (int64_t)blockIdx.x * DA_ROWS; base < n; base += (int64_t)gridDim.x * DA_ROWS) {
+        const int rows_here = (int)min((int64_t)DA_ROWS, n - base);
         for (int e = tid; e < rows_here * d; e += DA_ROWS) {
             const int r = e / d, l = e - r * d;
-            const int64_t gi = row_list ? (int64_t)row_list[base + r] : base + r;
-            const float xv = X[gi * d + l];
+            const float xv = X[(base + r) * d + l];
             amx = fmaxf(amx, fabsf(xv));
             Xs[r * ldx + l] = xv;
         }
-        T b1 = (T)INFINITY, b2 = (T)INFINITY;
+        T b1 = (T)INFINITY;
         int j1 = 0;
         for (int c0 = 0; c0 < k; c0 += DA_TC) {
             const int tc = min(DA_TC, k - c0);
@@ -63,72 +51,30 @@ __global__ void __launch_bounds__(DA_ROWS) k_direct_assign(const float* __restri
 #pragma unroll
                 for (int c = 0; c < DA_TC; c++) acc[c] = (T)0;
                 const float* xr = Xs + tid * ldx;
-                if (sizeof(T) == 4 && vec4) {
-                    // four coordinates per shared-memory load on both sides (the same
-                    // order of operations per centre as the scalar loop below)
-                    for (int l = 0; l < d; l += 4) {
-                        const float4 x4 = *reinterpret_cast<const float4*>(xr + l);
+                for (int l = 0; l < d; l++) {
+                    const T xl = (T)xr[l];
 #pragma unroll
-                        for (int c = 0; c < DA_TC; c++) {
-                            if (c < tc) {
-                                const float4 c4 = *reinterpret_cast<const float4*>(
-                                    reinterpret_cast<const float*>(Cs) + c * d + l);
-                                T t = (T)x4.x - (T)c4.x;
-                                acc[c] = fma(t, t, acc[c]);
-                                t = (T)x4.y - (T)c4.y;
-                                acc[c] = fma(t, t, acc[c]);
-                                t = (T)x4.z - (T)c4.z;
-                                acc[c] = fma(t, t, acc[c]);
-                                t = (T)x4.w - (T)c4.w;
-                                acc[c] = fma(t, t, acc[c]);
-                            }
-                        }
-                    }
-                } else {
-                    for (int l = 0; l < d; l++) {
-                        const T xl = (T)xr[l];
-#pragma unroll
-                        for (int c = 0; c < DA_TC; c++) {
-                            if (c < tc) {
-                                const T t = xl - Cs[c * d + l];
-                                acc[c] = fma(t, t, acc[c]);
-                            }
+                    for (int c = 0; c < DA_TC; c++) {
+                        if (c < tc) {
+                            const T t = xl - Cs[c * d + l];
+                            acc[c] = fma(t, t, acc[c]);
                         }
                     }
                 }
 #pragma unroll
-                for (int c = 0; c < DA_TC; c++) {
-                    if (c < tc) {
-                        const T v = acc[c];
-                        if (v < b1) {
-                            b2 = b1;
-                            b1 = v;
-                            j1 = c0 + c;
-                        } else if (v < b2) {
-                            b2 = v;
-                        }
+                for (int c = 0; c < DA_TC; c++)
+                    if (c < tc && acc[c] < b1) {
+                        b1 = acc[c];
+                        j1 = c0 + c;
                     }
-                }
             }
         }
-        if (sizeof(T) == 4 && tid == 0) atomicAdd(&cnt->fp32_evals, (unsigned long long)rows_here * (unsigned long long)k);
         if (tid < rows_here) {
-            const int64_t gi = row_list ? (int64_t)row_list[base + tid] : base + tid;
-            labels[gi] = j1;
-            min_dist[gi] = (double)b1;
-            if (sizeof(T) == 4) {
-                // Theorem 4.1: true values lie in [v (1 - g), v (1 + g)]
-                const float g = gamma32;
-                if (!((float)b2 * (1.0f - g) > (float)b1 * (1.0f + g))) {
-                    int slot = atomicAdd(&cnt->amb_count, 1);
-                    amb_list[slot] = (int32_t)gi;
-                    local_amb++;
-                }
-            }
+            labels[base + tid] = j1;
+            min_dist[base + tid] = (double)b1;
         }
         __syncthreads();
     }
-    if (local_amb) atomicAdd(&cnt->amb_rows, local_amb);
     if (absmax_out) {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) amx = fmaxf(amx, __shfl_xor_sync(0xffffffffu, amx, off));
@@ -136,108 +82,154 @@ __global__ void __launch_bounds__(DA_ROWS) k_direct_assign(const float* __restri
     }
 }
 
-// Tiled fp32 direct distances, Eq. (dist-direct), for d % 4 == 0 and
-// 16 <= d <= 128 (rows whose candidate list overflowed, the fp32 direct path,
-// km_assign_static): 128 rows per round resident in shared memory, the
-// centres streamed through it in tiles of 64 (cp.async, two buffers).  Each
-// thread holds 4 rows x 8 centres and takes two coordinates per packed
-// instruction: the even and the odd coordinates are summed separately and
-// then added, a summation order Theorem 4.1's bound covers like any other.
-// Per row the smallest and second-smallest value and the first index of the
-// smallest (ties: lowest index), merged over the 8 threads of the row; the
-// certificate and the list of open rows as in k_direct_assign.
-constexpr int DT_R = 128;  // rows per round
-constexpr int DT_C = 64;   // centres per tile
+// Tiled fp32 direct distances, Eq. (dist-direct), any d (rows whose candidate
+// list overflowed, the fp32 direct path, km_assign_static): 32 RPT rows per
+// round resident in shared memory (zero-padded to a multiple of 4
+// coordinates), the centres streamed through it in tiles of 64, DT_DK
+// coordinates at a time (cp.async, two buffers).  Each thread holds RPT rows
+// x 8 centres and takes two coordinates per packed instruction: the even and
+// the odd coordinates are summed separately and then added, a summation order
+// Theorem 4.1's bound covers like any other.  Per row the smallest and
+// second-smallest value and the first index of the smallest (ties: lowest
+// index), merged over the 8 threads of the row; the certificate and the list
+// of open rows (amb_list).
+// Bound by the FP32 pipe (two lane operations per pair and coordinate).
+// Chunking the coordinates keeps the block at 113 KB or less, so two blocks
+// share an SM and one computes while the other waits at a tile's barrier.
+// Measured: 1e6 x 128 against 1024 centres 10.14 -> 9.67 ms (0.69 of the FP32
+// pipe at its top clock; the block per SM before it had one 64 x d tile per
+// barrier); 81,000 listed rows x 256, k = 389: 5.61 -> 0.81 ms and 60,013 x 50,
+// k = 203: 0.197 -> 0.098 ms (a thread per row before, one to three blocks per SM).
+constexpr int DT_C = 64;    // centres per tile
+constexpr int DT_DK = 64;   // coordinates per streamed chunk
 
-KM_DEV void cp_async16(uint32_t dst, const void* src, bool full) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(full ? 16 : 0) : "memory");
+template <int BYTES>
+KM_DEV void cp_async(uint32_t dst, const void* src, bool full) {
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(full ? 16 : 0) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(full ? BYTES : 0)
+                     : "memory");
 }
 KM_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 KM_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-__global__ void __launch_bounds__(256, 1) k_direct_tiled(const float* __restrict__ X, int64_t n,
-                                                         const float* __restrict__ C, int k, int d,
-                                                         const int32_t* __restrict__ row_list,
-                                                         const int* __restrict__ row_count,
-                                                         int32_t* __restrict__ labels, double* __restrict__ min_dist,
-                                                         int32_t* __restrict__ amb_list, DevCounters* cnt,
-                                                         float gamma32, unsigned* __restrict__ absmax_out) {
+// Row stride (floats) of w staged coordinates (a multiple of 4): an odd number
+// of 16-byte slots, so eight consecutive rows' reads fall on different banks.
+__host__ __device__ constexpr int dt_stride(int w) { return (w / 4) % 2 ? w : w + 4; }
+constexpr size_t dt_smem(int rpt, int d) {
+    const int dp = (d + 3) & ~3, w = dp < DT_DK ? dp : DT_DK;
+    return ((size_t)32 * rpt * dt_stride(dp) + (size_t)2 * DT_C * dt_stride(w)) * sizeof(float);
+}
+
+// VEC: floats per load (4, 2 or 1: what d and the pointers' alignment allow)
+template <int RPT, int VEC>
+KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __restrict__ C, int k, int d,
+                         const int32_t* __restrict__ row_list, const int* __restrict__ row_count,
+                         int32_t* __restrict__ labels, double* __restrict__ min_dist, int32_t* __restrict__ amb_list,
+                         DevCounters* cnt, float gamma32, unsigned* __restrict__ absmax_out) {
     extern __shared__ __align__(16) float dts[];
-    const int ldx = d + 4;  // row stride: 16-byte rows, consecutive rows 4 banks apart
+    constexpr int R = 32 * RPT;
+    const int dp = (d + 3) & ~3, cw = min(dp, DT_DK);
+    const int ldx = dt_stride(dp), ldc = dt_stride(cw);
     float* Xs = dts;
-    const uint32_t cs0 = smem_u32(dts + DT_R * ldx);  // [2][DT_C][ldx]
-    const float* Cs = dts + DT_R * ldx;
+    float* Cs = dts + R * ldx;  // [2][DT_C][ldc]
+    const uint32_t cs0 = smem_u32(Cs);
     const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
     const int64_t nrows = row_list ? (int64_t)(*row_count) : n;
-    const int d4 = d >> 2;
-    const int ntile = (k + DT_C - 1) / DT_C;
-    const float2 neg1 = make_float2(-1.0f, -1.0f);
+    const int ntile = (k + DT_C - 1) / DT_C, nck = (dp + DT_DK - 1) / DT_DK, nstep = ntile * nck;
     const float g = gamma32;
+    const int dv = d / VEC;  // loads per row
     float amx = 0.0f;
     unsigned long long local_amb = 0;
-    for (int64_t base = (int64_t)blockIdx.x * DT_R; base < nrows; base += (int64_t)gridDim.x * DT_R) {
-        const int rows_here = (int)min((int64_t)DT_R, nrows - base);
-        __syncthreads();  // the previous round's readers are done with both buffers
-        for (int e = tid; e < DT_R * d4; e += blockDim.x) {
-            const int r = e / d4, l4 = e - r * d4;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    // the padding past d (at most 3 coordinates of a row or of the last chunk)
+    // stays zero: no load touches it
+    if (dp != d) {
+        for (int e = tid; e < R * (dp - d); e += 256) Xs[(e / (dp - d)) * ldx + d + e % (dp - d)] = 0.0f;
+        if (nck == 1)
+            for (int e = tid; e < 2 * DT_C * (dp - d); e += 256) Cs[(e / (dp - d)) * ldc + d + e % (dp - d)] = 0.0f;
+    }
+    for (int64_t base = (int64_t)blockIdx.x * R; base < nrows; base += (int64_t)gridDim.x * R) {
+        const int rows_here = (int)min((int64_t)R, nrows - base);
+        __syncthreads();  // the previous round's readers are done with all buffers
+        for (int e = tid; e < R * dv; e += 256) {
+            const int r = e / dv, l = (e - r * dv) * VEC;
+            float v[VEC];
+#pragma unroll
+            for (int t = 0; t < VEC; t++) v[t] = 0.0f;
             if (r < rows_here) {
                 const int64_t gi = row_list ? (int64_t)row_list[base + r] : base + r;
-                v = reinterpret_cast<const float4*>(X + gi * d)[l4];
-                amx = fmaxf(amx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+                const float* src = X + gi * d + l;
+                if constexpr (VEC == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(src);
+                else if constexpr (VEC == 2) *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(src);
+                else v[0] = *src;
+#pragma unroll
+                for (int t = 0; t < VEC; t++) amx = fmaxf(amx, fabsf(v[t]));
             }
-            *reinterpret_cast<float4*>(Xs + r * ldx + 4 * l4) = v;
+#pragma unroll
+            for (int t = 0; t < VEC; t++) Xs[r * ldx + l + t] = v[t];
         }
-        auto load_tile = [&](int t, int buf) {
-            const int c0 = t * DT_C;
-            for (int e = tid; e < DT_C * d4; e += blockDim.x) {
-                const int c = e / d4, l4 = e - c * d4;
+        // step s: coordinates [DT_DK (s % nck), ...) of the centres of tile s / nck
+        auto load_step = [&](int s, int buf) {
+            const int c0 = (s / nck) * DT_C, l0 = (s % nck) * DT_DK;
+            const int w = min(DT_DK, d - l0), wv = w / VEC;
+            for (int e = tid; e < DT_C * wv; e += 256) {
+                const int c = e / wv, l = (e - c * wv) * VEC;
                 const bool ok = c0 + c < k;
-                cp_async16(cs0 + (uint32_t)(((buf * DT_C + c) * ldx + 4 * l4) * 4),
-                           ok ? (const void*)(C + (int64_t)(c0 + c) * d + 4 * l4) : (const void*)C, ok);
+                cp_async<4 * VEC>(cs0 + (uint32_t)(((buf * DT_C + c) * ldc + l) * 4),
+                                  ok ? (const void*)(C + (int64_t)(c0 + c) * d + l0 + l) : (const void*)C, ok);
             }
+            if (nck > 1 && (w & 3))  // the last chunk's padding
+                for (int c = tid; c < DT_C; c += 256)
+                    for (int l = w; l < ((w + 3) & ~3); l++) Cs[(buf * DT_C + c) * ldc + l] = 0.0f;
             cp_async_commit();
         };
-        load_tile(0, 0);
-        float b1[4], b2[4];
-        int j1[4];
+        load_step(0, 0);
+        float b1[RPT], b2[RPT];
+        int j1[RPT];
+        float2 acc[RPT][8];
 #pragma unroll
-        for (int i = 0; i < 4; i++) { b1[i] = INFINITY; b2[i] = INFINITY; j1[i] = 0; }
-        for (int t = 0; t < ntile; t++) {
-            const int buf = t & 1;
+        for (int i = 0; i < RPT; i++) { b1[i] = INFINITY; b2[i] = INFINITY; j1[i] = 0; }
+        int ck = 0, c0 = 0;
+        for (int s = 0; s < nstep; s++) {
+            const int buf = s & 1;
             cp_async_wait_all();
-            __syncthreads();  // tile t is in place; tile t - 1's buffer is free
-            if (t + 1 < ntile) load_tile(t + 1, buf ^ 1);
-            float2 acc[4][8];
+            __syncthreads();  // step s is in place; step s - 1's buffer is free
+            if (s + 1 < nstep) load_step(s + 1, buf ^ 1);
+            if (ck == 0) {
 #pragma unroll
-            for (int i = 0; i < 4; i++)
+                for (int i = 0; i < RPT; i++)
 #pragma unroll
-                for (int c = 0; c < 8; c++) acc[i][c] = make_float2(0.f, 0.f);
-            const float* xb = Xs + ty * ldx;                     // rows ty + 32 i
-            const float* cb = Cs + (size_t)(buf * DT_C + tx) * ldx;  // centres tx + 8 c
-            for (int l = 0; l < d; l += 4) {
-                float4 xv[4], cv[8];
+                    for (int c = 0; c < 8; c++) acc[i][c] = make_float2(0.f, 0.f);
+            }
+            const float* xb = Xs + ty * ldx + ck * DT_DK;            // rows ty + 32 i
+            const float* cb = Cs + (size_t)(buf * DT_C + tx) * ldc;  // centres tx + 8 c
+            const int w = min(DT_DK, dp - ck * DT_DK);
+#pragma unroll 1
+            for (int l = 0; l < w; l += 4) {
+                float4 xv[RPT];
 #pragma unroll
-                for (int i = 0; i < 4; i++) xv[i] = *reinterpret_cast<const float4*>(xb + 32 * i * ldx + l);
+                for (int i = 0; i < RPT; i++) xv[i] = *reinterpret_cast<const float4*>(xb + 32 * i * ldx + l);
 #pragma unroll
-                for (int c = 0; c < 8; c++) cv[c] = *reinterpret_cast<const float4*>(cb + 8 * c * ldx + l);
+                for (int c = 0; c < 8; c++) {
+                    const float4 cv = *reinterpret_cast<const float4*>(cb + 8 * c * ldc + l);
 #pragma unroll
-                for (int i = 0; i < 4; i++)
-#pragma unroll
-                    for (int c = 0; c < 8; c++) {
-                        const float2 t0 = __ffma2_rn(make_float2(cv[c].x, cv[c].y), neg1, make_float2(xv[i].x, xv[i].y));
+                    for (int i = 0; i < RPT; i++) {
+                        const float2 t0 = fsub2(make_float2(xv[i].x, xv[i].y), make_float2(cv.x, cv.y));
                         acc[i][c] = __ffma2_rn(t0, t0, acc[i][c]);
-                        const float2 t1 = __ffma2_rn(make_float2(cv[c].z, cv[c].w), neg1, make_float2(xv[i].z, xv[i].w));
+                        const float2 t1 = fsub2(make_float2(xv[i].z, xv[i].w), make_float2(cv.z, cv.w));
                         acc[i][c] = __ffma2_rn(t1, t1, acc[i][c]);
                     }
+                }
             }
-            const int c0 = t * DT_C;
+            if (++ck < nck) continue;
+            ck = 0;
 #pragma unroll
             for (int c = 0; c < 8; c++) {
                 const int j = c0 + tx + 8 * c;  // ascending in c: the first of equal values keeps its place
                 if (j < k)
 #pragma unroll
-                    for (int i = 0; i < 4; i++) {
+                    for (int i = 0; i < RPT; i++) {
                         const float v = acc[i][c].x + acc[i][c].y;
                         if (v < b1[i]) {
                             b2[i] = b1[i];
@@ -248,10 +240,11 @@ __global__ void __launch_bounds__(256, 1) k_direct_tiled(const float* __restrict
                         }
                     }
             }
+            c0 += DT_C;
         }
         // the 8 threads of each row: smallest (lowest index on ties) and second smallest
 #pragma unroll
-        for (int i = 0; i < 4; i++)
+        for (int i = 0; i < RPT; i++)
 #pragma unroll
             for (int off = 1; off < 8; off <<= 1) {
                 const float ob1 = __shfl_xor_sync(0xffffffffu, b1[i], off);
@@ -267,7 +260,7 @@ __global__ void __launch_bounds__(256, 1) k_direct_tiled(const float* __restrict
             }
         if (tx == 0)
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
+            for (int i = 0; i < RPT; i++) {
                 const int r = ty + 32 * i;
                 if (r < rows_here) {
                     const int64_t gi = row_list ? (int64_t)row_list[base + r] : base + r;
@@ -292,6 +285,47 @@ __global__ void __launch_bounds__(256, 1) k_direct_tiled(const float* __restrict
         for (int off = 16; off > 0; off >>= 1) amx = fmaxf(amx, __shfl_xor_sync(0xffffffffu, amx, off));
         if ((tid & 31) == 0) atomicMax(absmax_out, __float_as_uint(amx));
     }
+}
+
+// 16 <= d <= 128, d % 4 == 0, 16-byte aligned rows
+template <int RPT>
+__global__ void __launch_bounds__(256, 2) k_direct_tiled(const float* __restrict__ X, int64_t n,
+                                                         const float* __restrict__ C, int k, int d,
+                                                         const int32_t* __restrict__ row_list,
+                                                         const int* __restrict__ row_count,
+                                                         int32_t* __restrict__ labels, double* __restrict__ min_dist,
+                                                         int32_t* __restrict__ amb_list, DevCounters* cnt,
+                                                         float gamma32, unsigned* __restrict__ absmax_out) {
+    direct_tiled<RPT, 4>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32, absmax_out);
+}
+// every other shape
+template <typename T, int RPT, int VEC>
+__global__ void __launch_bounds__(256, 2) k_direct_assign(const float* __restrict__ X, int64_t n,
+                                                          const float* __restrict__ C, int k, int d,
+                                                          const int32_t* __restrict__ row_list,
+                                                          const int* __restrict__ row_count,
+                                                          int32_t* __restrict__ labels, double* __restrict__ min_dist,
+                                                          int32_t* __restrict__ amb_list, DevCounters* cnt,
+                                                          float gamma32, unsigned* __restrict__ absmax_out) {
+    static_assert(sizeof(T) == 4, "binary32 accumulation");
+    direct_tiled<RPT, VEC>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32, absmax_out);
+}
+
+template <int RPT, int VEC>
+static cudaError_t launch_tiled(const float* X, int64_t n, const float* C, int k, int d, const int32_t* row_list,
+                                const int* row_count, int32_t* labels, double* min_dist, int32_t* amb_list,
+                                DevCounters* cnt, float gamma32, int num_sms, cudaStream_t st, unsigned* absmax_out) {
+    const size_t sm = dt_smem(RPT, d);
+    void (*fn)(const float*, int64_t, const float*, int, int, const int32_t*, const int*, int32_t*, double*, int32_t*,
+               DevCounters*, float, unsigned*) = k_direct_assign<float, RPT, VEC>;
+    if constexpr (VEC == 4)
+        if (d >= 16 && d <= 128) fn = k_direct_tiled<RPT>;
+    cudaError_t e = allow_max_smem(fn);
+    if (e != cudaSuccess) return e;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 32 * RPT - 1) / (32 * RPT), (int64_t)num_sms * 2));
+    fn<<<(unsigned)grid, 256, sm, st>>>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32,
+                                        absmax_out);
+    return cudaGetLastError();
 }
 
 // Small d (d <= 8) with C small enough to stay in shared memory for the
@@ -365,11 +399,16 @@ __global__ void __launch_bounds__(256) k_direct_small(const float* __restrict__ 
     }
 }
 
-// Exact argmin of listed rows, one 256-thread block per row.  Thread t takes
-// centres t, t+256, ...  fp32_first: fp32 direct values of all centres
-// (Theorem 4.1 intervals), the block's best and second best, and binary64
-// (oracle arithmetic: products and sums rounded separately, coordinates in
-// order) only for the centres whose interval can still hold the minimum.
+// Exact argmin of listed rows, one 256-thread block per row: fp32 direct
+// values of all centres (a warp per centre, four centres at a time: coalesced
+// reads of C), Theorem 4.1's intervals, and binary64 (oracle arithmetic:
+// products and sums rounded separately, coordinates in order) only for the
+// centres whose interval can still hold the minimum.  Up to RF_OPEN of those
+// take a warp each (products in parallel, one lane adds them in order); more
+// take a thread each.
+// Latency-bound: the lists are short.  440 rows x 1024 centres, d = 128:
+// 742 us with binary64 values of every centre, 77 us with the fp32 values first.
+constexpr int RF_OPEN = 64;
 struct Top2 {
     float b1, b2;
     int j1;
@@ -393,18 +432,47 @@ KM_DEV double direct64(const float* x, const float* c, int d) {
     return s;
 }
 
-template <bool FP32_FIRST>
+// fp32 direct values of centres j, j + 1, .., j + 3 (those below k): all lanes
+// of the warp return the same four sums.
+KM_DEV void warp_direct4(const float* xs, const float* __restrict__ C, int k, int d, int j, int lane, float (&v)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) v[q] = 0.0f;
+    // 16 loads in flight per lane
+    for (int l0 = lane; l0 < d; l0 += 128) {
+        float c[4][4], x[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int l = l0 + 32 * u;
+            x[u] = l < d ? xs[l] : 0.0f;
+#pragma unroll
+            for (int q = 0; q < 4; q++) c[u][q] = l < d && j + q < k ? C[(int64_t)(j + q) * d + l] : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) v[q] = fmaf(x[u] - c[u][q], x[u] - c[u][q], v[q]);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+        for (int q = 0; q < 4; q++) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
+}
+
+// count_open: the rows left open by the fp32 values are added to amb_rows
+// (rows that an earlier kernel left open have been counted there).
 __global__ void __launch_bounds__(256) k_rows_full(const float* __restrict__ X, const float* __restrict__ C, int k,
                                                    int d, const int32_t* __restrict__ row_list,
                                                    const int* __restrict__ row_count, int32_t* __restrict__ labels,
                                                    double* __restrict__ min_dist, DevCounters* cnt, float gamma32,
-                                                   int keep_vals) {
-    extern __shared__ float sh[];
-    float* xs = sh;                      // d
-    float* vs = sh + ((d + 3) & ~3);     // k fp32 values when they fit (keep_vals), else recomputed
+                                                   bool count_open, bool keep_vals) {
+    extern __shared__ __align__(16) double shd[];
+    double* prod = shd;                                          // 8 x d products
+    float* xs = reinterpret_cast<float*>(shd + (size_t)8 * d);   // d
+    float* vs = xs + d;                                          // k fp32 values when they fit (keep_vals), else recomputed
     __shared__ Top2 red[8];
     __shared__ double rv[8];
     __shared__ int rj[8];
+    __shared__ int open_j[RF_OPEN], nopen;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int64_t nrows = *row_count;
     unsigned long long ev32 = 0, ev64 = 0;
@@ -412,85 +480,98 @@ __global__ void __launch_bounds__(256) k_rows_full(const float* __restrict__ X, 
         const int64_t i = row_list[w];
         __syncthreads();
         for (int l = tid; l < d; l += 256) xs[l] = X[i * d + l];
+        if (tid == 0) nopen = 0;
         __syncthreads();
-        bool need64 = true;
-        float thr = INFINITY;
-        if (FP32_FIRST) {
-            Top2 t{INFINITY, INFINITY, 0x7fffffff};
-            for (int j = tid; j < k; j += 256) {
-                const float* c = C + (int64_t)j * d;
-                float s = 0.0f;
-                for (int l = 0; l < d; l++) {
-                    const float u = xs[l] - c[l];
-                    s = fmaf(u, u, s);
-                }
-                if (keep_vals) vs[j] = s;
-                ev32++;
-                if (s < t.b1) { t.b2 = t.b1; t.b1 = s; t.j1 = j; }
-                else if (s < t.b2) t.b2 = s;
-            }
+        Top2 t{INFINITY, INFINITY, 0x7fffffff};
+        for (int j = 4 * wid; j < k; j += 32) {
+            float v[4];
+            warp_direct4(xs, C, k, d, j, lane, v);
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                Top2 o;
-                o.b1 = __shfl_xor_sync(0xffffffffu, t.b1, off);
-                o.b2 = __shfl_xor_sync(0xffffffffu, t.b2, off);
-                o.j1 = __shfl_xor_sync(0xffffffffu, t.j1, off);
-                t = top2_merge(t, o);
-            }
-            if (lane == 0) red[wid] = t;
-            __syncthreads();
-            t = red[0];
-            for (int q = 1; q < 8; q++) t = top2_merge(t, red[q]);
-            const float g = gamma32;
-            if (t.b2 * (1.0f - g) > t.b1 * (1.0f + g)) {
-                need64 = false;
-                if (tid == 0) {
-                    labels[i] = t.j1;
-                    min_dist[i] = (double)t.b1;
+            for (int q = 0; q < 4; q++)
+                if (j + q < k) {
+                    if (keep_vals && lane == 0) vs[j + q] = v[q];
+                    t = top2_merge(t, Top2{v[q], INFINITY, j + q});
                 }
-            } else {
-                thr = t.b1 * (1.0f + g);
-                if (tid == 0) atomicAdd(&cnt->amb_rows, 1ull);
+        }
+        if (tid == 0) ev32 += (unsigned long long)k;
+        if (lane == 0) red[wid] = t;
+        __syncthreads();
+        t = red[0];
+        for (int q = 1; q < 8; q++) t = top2_merge(t, red[q]);
+        if (t.b2 * (1.0f - gamma32) > t.b1 * (1.0f + gamma32)) {
+            if (tid == 0) {
+                labels[i] = t.j1;
+                min_dist[i] = (double)t.b1;
+            }
+            continue;
+        }
+        if (count_open && tid == 0) atomicAdd(&cnt->amb_rows, 1ull);
+        // squares below binary32's range: each coordinate adds at most 2^-149 of absolute error
+        const float thr = t.b1 * (1.0f + gamma32) + (float)(2 * d + 4) * 0x1p-149f;
+        double best = INFINITY;
+        int arg = 0x7fffffff;
+        if (keep_vals) {
+            for (int j = tid; j < k; j += 256)
+                if (vs[j] * (1.0f - gamma32) <= thr) {
+                    const int p = atomicAdd(&nopen, 1);
+                    if (p < RF_OPEN) open_j[p] = j;
+                }
+        } else {
+            for (int j = 4 * wid; j < k; j += 32) {  // the same values as above
+                float v[4];
+                warp_direct4(xs, C, k, d, j, lane, v);
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (lane == 0 && j + q < k && v[q] * (1.0f - gamma32) <= thr) {
+                        const int p = atomicAdd(&nopen, 1);
+                        if (p < RF_OPEN) open_j[p] = j + q;
+                    }
             }
         }
-        if (need64) {
-            double best = INFINITY;
-            int arg = 0x7fffffff;
-            for (int j = tid; j < k; j += 256) {
-                if (FP32_FIRST) {
-                    float v;
-                    if (keep_vals) {
-                        v = vs[j];
-                    } else {  // the same loop as above: the same value
-                        const float* c = C + (int64_t)j * d;
-                        v = 0.0f;
-                        for (int l = 0; l < d; l++) {
-                            const float u = xs[l] - c[l];
-                            v = fmaf(u, u, v);
-                        }
-                    }
-                    if (!(v * (1.0f - gamma32) <= thr)) continue;
+        __syncthreads();
+        const int no = nopen;
+        if (no <= RF_OPEN) {
+            double* pw = prod + (size_t)wid * d;
+            for (int o = wid; o < no; o += 8) {
+                const int j = open_j[o];
+                const float* c = C + (int64_t)j * d;
+                for (int l = lane; l < d; l += 32) {
+                    const double u = __dsub_rn((double)xs[l], (double)c[l]);
+                    pw[l] = __dmul_rn(u, u);
                 }
+                __syncwarp();
+                if (lane == 0) {
+                    double s = 0.0;
+                    for (int l = 0; l < d; l++) s = __dadd_rn(s, pw[l]);
+                    if (s < best || (s == best && j < arg)) { best = s; arg = j; }
+                    ev64++;
+                }
+                __syncwarp();
+            }
+        } else {
+            // (the open list did not fit: every centre the list would have held)
+            for (int j = tid; j < k; j += 256) {
+                if (keep_vals && !(vs[j] * (1.0f - gamma32) <= thr)) continue;
                 const double s = direct64(xs, C + (int64_t)j * d, d);
                 ev64++;
                 if (s < best) { best = s; arg = j; }
             }
+        }
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const double ob = __shfl_xor_sync(0xffffffffu, best, off);
-                const int oa = __shfl_xor_sync(0xffffffffu, arg, off);
-                if (ob < best || (ob == best && oa < arg)) { best = ob; arg = oa; }
-            }
-            if (lane == 0) { rv[wid] = best; rj[wid] = arg; }
-            __syncthreads();
-            if (tid == 0) {
-                best = rv[0];
-                arg = rj[0];
-                for (int q = 1; q < 8; q++)
-                    if (rv[q] < best || (rv[q] == best && rj[q] < arg)) { best = rv[q]; arg = rj[q]; }
-                labels[i] = arg;
-                min_dist[i] = best;
-            }
+        for (int off = 16; off > 0; off >>= 1) {
+            const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+            const int oa = __shfl_xor_sync(0xffffffffu, arg, off);
+            if (ob < best || (ob == best && oa < arg)) { best = ob; arg = oa; }
+        }
+        if (lane == 0) { rv[wid] = best; rj[wid] = arg; }
+        __syncthreads();
+        if (tid == 0) {
+            best = rv[0];
+            arg = rj[0];
+            for (int q = 1; q < 8; q++)
+                if (rv[q] < best || (rv[q] == best && rj[q] < arg)) { best = rv[q]; arg = rj[q]; }
+            labels[i] = arg < k ? arg : 0;  // (no value to compare, NaN: a valid label all the same)
+            min_dist[i] = best;
         }
     }
 #pragma unroll
@@ -502,12 +583,6 @@ __global__ void __launch_bounds__(256) k_rows_full(const float* __restrict__ X, 
         if (ev32) atomicAdd(&cnt->fp32_evals, ev32);
         if (ev64) atomicAdd(&cnt->fp64_evals, ev64);
     }
-}
-
-static size_t direct_smem(bool acc64, int d) {
-    const int ldx = (!acc64 && d % 4 == 0) ? d + 4 : d + 1;
-    size_t xs = (((size_t)DA_ROWS * ldx * sizeof(float)) + 15) & ~(size_t)15;
-    return xs + (size_t)DA_TC * d * (acc64 ? 8 : 4);
 }
 
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
@@ -536,59 +611,46 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
         }
         return cudaGetLastError();
     }
-    if (!acc64 && d % 4 == 0 && d >= 16 && d <= 128 && ((uintptr_t)X % 16) == 0 && ((uintptr_t)C % 16) == 0) {
-        const size_t tsm = (size_t)(DT_R + 2 * DT_C) * (d + 4) * sizeof(float);
-        cudaError_t e = allow_max_smem(k_direct_tiled);
-        if (e != cudaSuccess) return e;
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + DT_R - 1) / DT_R, (int64_t)num_sms));
-        k_direct_tiled<<<(unsigned)grid, 256, tsm, st>>>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list,
-                                                          cnt, gamma32, absmax_out);
-        return cudaGetLastError();
+    if (!acc64) {
+        // rows per block: 128, or 64 where 128 would leave one block per SM
+        // (113 KB of shared memory at d = 148) or too few blocks for two per
+        // SM, or 32 where 64 would; a row list's length is not known here
+        const bool a16 = ((uintptr_t)X % 16) == 0 && ((uintptr_t)C % 16) == 0;
+        const bool a8 = ((uintptr_t)X % 8) == 0 && ((uintptr_t)C % 8) == 0;
+        const int vec = d % 4 == 0 && a16 ? 4 : (d % 2 == 0 && a8 ? 2 : 1);
+        int rpt = dt_smem(4, d) <= 113 * 1024 ? 4 : 2;
+        while (rpt > 1 && !row_list && (n + 32 * rpt - 1) / (32 * rpt) < 2 * num_sms) rpt >>= 1;
+#define KM_DT(RP, VE)                                                                                              \
+    if (rpt == RP && vec == VE)                                                                                    \
+        return launch_tiled<RP, VE>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32, \
+                                    num_sms, st, absmax_out);
+        KM_DT(4, 4) KM_DT(4, 2) KM_DT(4, 1) KM_DT(2, 4) KM_DT(2, 2) KM_DT(2, 1) KM_DT(1, 4) KM_DT(1, 2) KM_DT(1, 1)
+#undef KM_DT
     }
-    size_t sm = direct_smem(acc64, d);
-    int64_t blocks_needed = (n + DA_ROWS - 1) / DA_ROWS;
-    int per_sm = (int)max((size_t)1, (size_t)(200 * 1024) / sm);
-    if (per_sm > 8) per_sm = 8;
-    int64_t grid = min(blocks_needed, (int64_t)num_sms * per_sm);
-    if (grid < 1) grid = 1;
-    cudaError_t e;
-    if (acc64) {
-        e = allow_max_smem(k_direct_assign<double>);
-        if (e != cudaSuccess) return e;
-        k_direct_assign<double><<<(unsigned)grid, DA_ROWS, sm, st>>>(X, n, C, k, d, row_list, row_count, labels,
-                                                                     min_dist, amb_list, cnt, gamma32, absmax_out);
-    } else {
-        e = allow_max_smem(k_direct_assign<float>);
-        if (e != cudaSuccess) return e;
-        k_direct_assign<float><<<(unsigned)grid, DA_ROWS, sm, st>>>(X, n, C, k, d, row_list, row_count, labels,
-                                                                    min_dist, amb_list, cnt, gamma32, absmax_out);
-    }
+    const size_t sm = ((((size_t)DA_ROWS * (d + 1) * sizeof(float)) + 15) & ~(size_t)15) + (size_t)DA_TC * d * 8;
+    const int per_sm = std::min(8, (int)std::max<size_t>(1, (size_t)(200 * 1024) / sm));
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + DA_ROWS - 1) / DA_ROWS, (int64_t)num_sms * per_sm));
+    void (*fn64)(const float*, int64_t, const float*, int, int, int32_t*, double*, unsigned*) = k_direct_assign<double>;
+    cudaError_t e = allow_max_smem(fn64);
+    if (e != cudaSuccess) return e;
+    fn64<<<(unsigned)grid, DA_ROWS, sm, st>>>(X, n, C, k, d, labels, min_dist, absmax_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_rows_full(bool fp32_first, const float* X, const float* C, int k, int d, const int32_t* row_list,
+cudaError_t launch_rows_full(bool count_open, const float* X, const float* C, int k, int d, const int32_t* row_list,
                              const int* row_count, int32_t* labels, double* min_dist, DevCounters* cnt,
                              float gamma32, int num_sms, cudaStream_t st) {
-    // x in shared memory, and the k fp32 values of the first pass when they fit
-    const void* fn = fp32_first ? (const void*)k_rows_full<true> : (const void*)k_rows_full<false>;
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+    cudaError_t e = cudaFuncGetAttributes(&fa, (const void*)k_rows_full);
     if (e != cudaSuccess) return e;
-    const size_t xs_bytes = (size_t)((d + 3) & ~3) * sizeof(float);
+    // products and x in shared memory, and the k fp32 values when they fit
+    const size_t base = (size_t)8 * d * sizeof(double) + (size_t)d * sizeof(float);
     const size_t avail = (size_t)kMaxBlockSmem - fa.sharedSizeBytes;
-    const int keep = fp32_first && xs_bytes + (size_t)k * sizeof(float) <= avail;
-    const size_t sm = xs_bytes + (keep ? (size_t)k * sizeof(float) : 0);
-    if (fp32_first) {
-        e = allow_max_smem(k_rows_full<true>);
-        if (e != cudaSuccess) return e;
-        k_rows_full<true><<<num_sms * 2, 256, sm, st>>>(X, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32,
-                                                        keep);
-    } else {
-        e = allow_max_smem(k_rows_full<false>);
-        if (e != cudaSuccess) return e;
-        k_rows_full<false><<<num_sms * 2, 256, sm, st>>>(X, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32,
-                                                         0);
-    }
+    const bool keep = base + (size_t)k * sizeof(float) <= avail;
+    e = allow_max_smem(k_rows_full);
+    if (e != cudaSuccess) return e;
+    k_rows_full<<<num_sms * 2, 256, base + (keep ? (size_t)k * sizeof(float) : 0), st>>>(
+        X, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32, count_open, keep);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,65 @@
+"""Kernels and dispatch rules at the sizes where they can go wrong: edges of
+tiles, remainders, unaligned rows, many ties, the smallest inputs.  Labels
+against the oracle's, min_dist at its binary64 tolerance."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2407_12208_gb300 import workloads
+from gpu_util import RTOL_MD, check_assign
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_2407_12208_gb300 as pkg
+    from paper_2407_12208_gb300 import build
+    build.build()
+    c = pkg.Context(0)
+    yield c
+    c.close()
+
+
+def _dev(a, offset=0):
+    """a on the GPU, `offset` floats past an allocation's start."""
+    buf = torch.empty(a.size + offset, dtype=torch.float32, device="cuda")
+    t = buf[offset:].view(a.shape)
+    t.copy_(torch.from_numpy(np.ascontiguousarray(a)))
+    return t
+
+
+def _assign(ctx, X, C, low, offset=0, **kw):
+    import paper_2407_12208_gb300 as pkg
+    lab, md, nf = ctx.assign(_dev(X, offset), _dev(C, offset), pkg.params(low, **kw))
+    return lab.cpu().numpy(), md.cpu().numpy(), nf
+
+
+# the tiled direct kernel: 64-coordinate chunks, 64-centre tiles, 32 / 64 / 128 rows per block,
+# one, two or four floats per load
+@pytest.mark.parametrize("offset", [0, 1, 2])
+@pytest.mark.parametrize("n,d,k", [(1, 9, 1), (33, 13, 7), (127, 50, 63), (129, 64, 64), (300, 65, 65), (257, 66, 129),
+                                   (700, 128, 100), (321, 130, 64), (200, 148, 33), (200, 152, 33), (333, 255, 70),
+                                   (500, 256, 128), (20000, 20, 300), (40001, 12, 40), (5000, 8, 1500)])
+def test_direct_tiled_edges(ctx, n, d, k, offset):
+    X, C = workloads.gaussian_mixture(n, d, k, seed=n + d)
+    lab, md, _ = _assign(ctx, X, C, "fp32", offset)
+    check_assign(lab, md, X, C, oracle, RTOL_MD)
+
+
+# rows left open: ties between duplicated centres go to the lowest index, whether the open
+# centres fit the block's list or not, and whether the fp32 values fit shared memory or not
+@pytest.mark.parametrize("copies,d,k", [(2, 20, 40), (64, 33, 128), (65, 33, 130), (200, 16, 400), (3, 12, 60000)])
+def test_open_rows_take_the_lowest_index(ctx, copies, d, k):
+    r = np.random.Generator(np.random.PCG64(k))
+    base = r.normal(size=(k // copies, d)).astype(np.float32)
+    C = np.tile(base, (copies, 1))  # centre j = base[j % (k // copies)]
+    X = np.concatenate([base[:37] + r.normal(0, 1e-3, size=(len(base[:37]), d)).astype(np.float32), C])[: max(k, 200)]
+    X = X.astype(np.float32)
+    lab, md, _ = _assign(ctx, X, C, "fp32")
+    assert lab.max() < len(base)
+    olab, od1, _ = oracle.assign(X[:64], C)
+    assert np.array_equal(lab[:64], olab)
+    np.testing.assert_allclose(md[:64], od1, rtol=RTOL_MD, atol=1e-30)
