@@ -225,6 +225,33 @@ AssignWs carve_assign(Carve& cv, int64_t n, int d, int k, int low, bool distance
     return w;
 }
 
+// The centred screen (k_refine.cu) pays where the full-row kernel would be
+// expensive: at 2^30 pair-coordinates that takes about 80 us when every row
+// overflows, and its two launches, empty in most calls, about 4 us.
+bool centred_applies(int64_t n, int d, int k, int low) {
+    return is_tc(low) && d <= 256 && (double)n * k * d >= (double)(1 << 30) && tc_smem_bytes(1, d, 1) != 0;
+}
+// Its buffers come last in every workspace: a workspace without room for them
+// does without (the rows then go to the full-row kernel).
+Centred carve_centred(Carve& cv, int64_t n, int d, int k, int low) {
+    Centred c{};
+    if (!centred_applies(n, d, k, low)) return c;
+    c.ldq = ldq_of(1, d);
+    c.Xq = cv.take<char>((size_t)n * c.ldq * 2);
+    c.xstat = cv.take<float4>((size_t)n);
+    c.Cq = cv.take<char>((size_t)k * c.ldq * 2);
+    c.cstat = cv.take<float4>((size_t)k);
+    c.colmax = cv.take<ColMax>(1);
+    c.qpad = cv.take<float>((size_t)kpad_of(k));
+    return c;
+}
+// cv stands at the end of what the call needs
+Centred take_centred(const Carve& cv, size_t ws_bytes, int64_t n, int d, int k, int low) {
+    Carve t = cv;
+    const Centred c = carve_centred(t, n, d, k, low);
+    return t.off <= ws_bytes ? c : Centred{};
+}
+
 struct UpdateWs {
     long long* sums;
     long long* counts;
@@ -277,6 +304,7 @@ struct LloydWs {
     int64_t* counts;
     double* sse_slot;  // a replayed iteration's SSE, appended to sse_hist on the device
     int* hist_len;     // entries of sse_hist / flag_hist written by replayed iterations
+    Centred cen;
 };
 LloydWs carve_lloyd(Carve& cv, int64_t n, int d, int k, int low, int max_iter) {
     LloydWs L{};
@@ -378,19 +406,20 @@ int screen_variant(km_ctx* ctx, int fmt, int kchunks, int k, int64_t n) {
     return kchunks == 2 ? TC_SV_HALF : TC_SV_FULL;
 }
 
+// The caller has zeroed the counters of one assignment (zero_counters, or all).
 // c_prepared: the workspace already holds C's low-precision copy, statistics
 // and column maxima for this C and format (later row chunks of one call).
 km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int k, int d, const km_params* p,
-                     int32_t* labels, double* min_dist, const AssignWs& w, bool x_prepared, cudaStream_t st,
-                     unsigned* x_absmax = nullptr, bool c_prepared = false) {
+                     int32_t* labels, double* min_dist, const AssignWs& w, const Centred& cen, bool x_prepared,
+                     cudaStream_t st, unsigned* x_absmax = nullptr, bool c_prepared = false) {
     const TestParams tp = make_tp(p, d);
     km_status s = KM_OK;
     if (p->low == KM_FP64_DIRECT || p->low == KM_FP32_DIRECT) {
         const bool acc64 = p->low == KM_FP64_DIRECT;
         {
             PhaseScope ps(ctx, KM_PHASE_DIRECT, st);
-            KL(1, launch_direct_assign(acc64, X, n, C, k, d, nullptr, nullptr, labels, min_dist, w.amb_list, w.cnt,
-                                       tp.gamma32, ctx->num_sms, st, x_absmax));
+            KL(1, launch_direct_assign(acc64, X, n, C, k, d, nullptr, nullptr, labels, min_dist, w.amb_list,
+                                       &w.cnt->amb_count, w.cnt, tp.gamma32, ctx->num_sms, st, x_absmax));
         }
         if (!acc64) {
             PhaseScope ps(ctx, KM_PHASE_FULLROW, st);
@@ -423,29 +452,54 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
     }
     {
         PhaseScope ps(ctx, KM_PHASE_REFINE, st);
-        CK(cudaMemsetAsync(&w.cnt->npairs, 0, sizeof(unsigned long long), st));
         int nl = 0;
-        CK(launch_refine(X, C, a, labels, min_dist, w.ovf_list, w.amb_list, ctx->num_sms, st, &nl));
+        CK(launch_refine(X, C, a, labels, min_dist, w.ovf_list, w.amb_list, cen, ctx->num_sms, st, &nl));
         ctx->launches += (uint64_t)nl;
     }
     {
         // rows whose candidate list overflowed (all of them when every pair fails
-        // the reliability test): fp32 direct distances to every centre with
-        // Theorem 4.1's certificate, then binary64 for the rows left open.  The
-        // near-tie list was consumed by the refinement and now takes those rows.
+        // the reliability test): the centred screen where it applies, then, for
+        // what is left, fp32 direct distances to every centre with Theorem 4.1's
+        // certificate, then binary64 for the rows left open.  The near-tie list was
+        // consumed by the refinement and now takes those rows; the rows' pair
+        // ranges, consumed as well, hold the list of what the centred screen left.
         PhaseScope ps(ctx, KM_PHASE_FULLROW, st);
+        const int32_t* list = w.ovf_list;
+        const int* list_n = &w.cnt->ovf_count;
+        if (cen.Xq) {
+            TcArgs b = a;
+            b.fmt = 1;
+            b.kchunks = (cen.ldq * 2 + 127) / 128;
+            b.nrows = list_n;
+            b.xstat = cen.xstat; b.cstat = cen.cstat; b.qpad = cen.qpad; b.colmax = cen.colmax;
+            // no reliability test here; k_n also covers the rounding of x - mu and c - mu
+            km_params q = *p;
+            q.low = KM_BF16;
+            q.test = KM_TEST_OFF;
+            b.tp = make_tp(&q, d);
+            b.tp.kn = (float)(10.0 * std::ldexp(1.0, -24));
+            b.variant = screen_variant(ctx, 1, b.kchunks, k, n);
+            KL(1, launch_tc(cen.Xq, cen.Cq, cen.ldq, b, ctx->num_sms, st));
+            int32_t* list2 = reinterpret_cast<int32_t*>(w.rowpair);
+            KL(1, launch_refine_centred(X, C, b, list, labels, list2, ctx->num_sms, st));
+            list = list2;
+            list_n = &w.cnt->ovf2_count;
+        }
         if (d <= 256) {  // the direct kernel's row tile fits in shared memory
-            CK(cudaMemsetAsync(&w.cnt->amb_count, 0, sizeof(int), st));
-            KL(1, launch_direct_assign(false, X, n, C, k, d, w.ovf_list, &w.cnt->ovf_count, labels, min_dist,
-                                       w.amb_list, w.cnt, tp.gamma32, ctx->num_sms, st));
-            KL(1, launch_rows_full(false, X, C, k, d, w.amb_list, &w.cnt->amb_count, labels, min_dist, w.cnt,
+            KL(1, launch_direct_assign(false, X, n, C, k, d, list, list_n, labels, min_dist, w.amb_list,
+                                       &w.cnt->open_count, w.cnt, tp.gamma32, ctx->num_sms, st));
+            KL(1, launch_rows_full(false, X, C, k, d, w.amb_list, &w.cnt->open_count, labels, min_dist, w.cnt,
                                    tp.gamma32, ctx->num_sms, st));
         } else {  // one block per row
-            KL(1, launch_rows_full(true, X, C, k, d, w.ovf_list, &w.cnt->ovf_count, labels, min_dist, w.cnt,
-                                   tp.gamma32, ctx->num_sms, st));
+            KL(1, launch_rows_full(true, X, C, k, d, list, list_n, labels, min_dist, w.cnt, tp.gamma32, ctx->num_sms, st));
         }
     }
     (void)esz;
+    return KM_OK;
+}
+
+km_status zero_counters(km_ctx* ctx, DevCounters* cnt, cudaStream_t st) {
+    CK(cudaMemsetAsync(&cnt->amb_count, 0, kAssignCounterBytes, st));
     return KM_OK;
 }
 
@@ -551,6 +605,7 @@ km_status km_workspace_size(const km_ctx* cctx, int64_t n, int d, int k, const k
     if (n < 1 || d < 1 || k < 1) return fail(ctx, KM_EINVAL, "need n, d, k >= 1");
     Carve a{nullptr};
     carve_lloyd(a, n, d, k, p->low, std::max(0, (int)p->max_iter));
+    carve_centred(a, n, d, k, p->low);
     Carve b{nullptr};
     carve_assign(b, n, d, k, p->low, true);
     *bytes = std::max(a.off, b.off) + 256;
@@ -643,11 +698,13 @@ km_status km_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int 
         md = c2.take<double>((size_t)n);
         need = c2.off;
     }
+    cv.off = need;
+    const Centred cen = take_centred(cv, ws_bytes, n, d, k, p->low);
     if (ws_bytes < need) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, need);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     CK(cudaMemsetAsync(w.cnt, 0, sizeof(DevCounters), st));
-    s = run_assign(ctx, X, n, C, k, d, p, labels, md, w, false, st);
+    s = run_assign(ctx, X, n, C, k, d, p, labels, md, w, cen, false, st);
     if (s != KM_OK) return s;
     if ((s = refine_winners(ctx, X, n, d, C, p, labels, md, st)) != KM_OK) return s;
     KL(2, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, st));
@@ -943,6 +1000,7 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
     AssignWs w = carve_assign(cv, n, d, k, p->low, false);
     UpdateWs u = carve_update(cv, n, d, k);
     double* md = min_dist ? min_dist : cv.take<double>((size_t)n);
+    const Centred cen = take_centred(cv, ws_bytes, n, d, k, p->low);
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
@@ -950,7 +1008,7 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
     // assignment (Alg. 3 step 1); its pass over X (quantisation, or the direct
     // distances) also yields max |x|
     CK(cudaMemsetAsync(u.absmax, 0, sizeof(unsigned), st));
-    s = run_assign(ctx, X, n, C_old, k, d, p, labels, md, w, false, st, u.absmax);
+    s = run_assign(ctx, X, n, C_old, k, d, p, labels, md, w, cen, false, st, u.absmax);
     if (s != KM_OK) return s;
     // centre update (Eq. (center)) on the labels just computed; its pass over
     // X also refines the winners' distances (min_dist, binary64 accuracy)
@@ -981,6 +1039,7 @@ km_status km_host_workspace_size(const km_ctx* cctx, int64_t n, int d, int k, co
     carve_host(a, n, d, k);
     carve_assign(a, n, d, k, p->low, false);
     carve_update(a, n, d, k);
+    carve_centred(a, n, d, k, p->low);
     *bytes = a.off + 256;
     return KM_OK;
 }
@@ -998,6 +1057,7 @@ km_status km_lloyd_step_host(km_ctx* ctx, const float* X_host, int64_t n, int d,
     HostWs h = carve_host(cv, n, d, k);
     AssignWs w = carve_assign(cv, n, d, k, p->low, false);
     UpdateWs u = carve_update(cv, n, d, k);
+    const Centred cen = take_centred(cv, ws_bytes, n, d, k, p->low);
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
@@ -1059,10 +1119,10 @@ km_status km_lloyd_step_host(km_ctx* ctx, const float* X_host, int64_t n, int d,
             const int64_t r0 = chunk_r0(c), rows = cend[c] - r0;
             cudaStream_t cs = ctx->copy_st[1];
             CK(cudaStreamWaitEvent(st, ev_in[c], 0));
-            CK(cudaMemsetAsync(&w.cnt->amb_count, 0, 2 * sizeof(int), st));
+            if ((s = zero_counters(ctx, w.cnt, st)) != KM_OK) return s;
             // the centres are prepared once, with the first chunk
-            s = run_assign(ctx, h.X + r0 * d, rows, h.C, k, d, p, h.labels + r0, h.min_dist + r0, w, false, st, u.absmax,
-                           c > 0);
+            s = run_assign(ctx, h.X + r0 * d, rows, h.C, k, d, p, h.labels + r0, h.min_dist + r0, w, cen, false, st,
+                           u.absmax, c > 0);
             if (s != KM_OK) return s;
             // the chunk's winner distances (binary64 accuracy) while the next
             // chunk is still on its way: the update's pass then only sums
@@ -1177,8 +1237,9 @@ __global__ void k_record_iteration(const double* __restrict__ sse_slot, const De
 static km_status lloyd_iteration(km_ctx* ctx, const float* X, int64_t n, int d, int k, const km_params* p,
                                  int32_t* labels, const LloydWs& L, const float* cur, float* nxt, double* sse_out,
                                  unsigned long long* flag_out, bool graph, int cap, cudaStream_t st) {
-    CK(cudaMemsetAsync(&L.a.cnt->amb_count, 0, 2 * sizeof(int), st));
-    km_status s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, true, st);
+    km_status s = zero_counters(ctx, L.a.cnt, st);
+    if (s != KM_OK) return s;
+    s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, true, st);
     if (s != KM_OK) return s;
     if (!graph) CK(cudaMemcpyAsync(flag_out, &L.a.cnt->flagged, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
     PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
@@ -1237,6 +1298,7 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
     if (!aligned256(ws)) return fail(ctx, KM_EINVAL, "workspace must be 256-byte aligned");
     Carve cv{(char*)ws};
     LloydWs L = carve_lloyd(cv, n, d, k, p->low, p->max_iter);
+    L.cen = take_centred(cv, ws_bytes, n, d, k, p->low);
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
@@ -1319,8 +1381,8 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
         CK(cudaEventRecord(ctx->graph_ev[1], gs));
         CK(cudaStreamWaitEvent(st, ctx->graph_ev[1], 0));
     }
-    CK(cudaMemsetAsync(&L.a.cnt->amb_count, 0, 2 * sizeof(int), st));
-    s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, true, st);
+    if ((s = zero_counters(ctx, L.a.cnt, st)) != KM_OK) return s;
+    s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, true, st);
     if (s != KM_OK) return s;
     if ((s = refine_winners(ctx, X, n, d, cur, p, labels, L.min_dist, st)) != KM_OK) return s;
     KL(2, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.sse_hist + t, st));
@@ -1437,9 +1499,11 @@ km_status km_cancel(km_ctx* ctx, uint64_t job_id) {
 size_t km_internal_ws_bytes(int64_t n, int d, int k, const km_params* p) {
     Carve a{nullptr};
     carve_lloyd(a, n, d, k, p->low, std::max(0, (int)p->max_iter));
+    carve_centred(a, n, d, k, p->low);
     Carve b{nullptr};
     carve_assign(b, n, d, k, p->low, false);
     b.take<double>((size_t)n);
+    carve_centred(b, n, d, k, p->low);
     return std::max(a.off, b.off) + 256;
 }
 
@@ -1622,8 +1686,8 @@ extern "C" km_status km_assign_static(km_ctx* ctx, const float* X, int64_t n, co
     // the counters (amb_count above all) must start at zero; the row list is
     // written before it is read
     CK(cudaMemsetAsync(cnt, 0, sizeof(DevCounters), st));
-    KL(1, launch_direct_assign(false, X, n, C, k, d, nullptr, nullptr, labels, min_dist, amb_list, cnt, tp.gamma32,
-                               ctx->num_sms, st));
+    KL(1, launch_direct_assign(false, X, n, C, k, d, nullptr, nullptr, labels, min_dist, amb_list, &cnt->amb_count, cnt,
+                               tp.gamma32, ctx->num_sms, st));
     KL(1, launch_rows_full(false, X, C, k, d, amb_list, &cnt->amb_count, labels, min_dist, cnt, tp.gamma32,
                            ctx->num_sms, st));
     // the winners' distances to binary64 accuracy, as km_assign (no scratch)

@@ -2,6 +2,7 @@
 // translation units of libmpkm.  Not part of the public ABI.
 #pragma once
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 namespace km {
@@ -24,11 +25,17 @@ struct DevCounters {
     unsigned long long amb_rows;
     unsigned long long ovf_rows;
     unsigned status;     // KM_DEVERR_* bits
-    int amb_count;       // length of the ambiguous-row list
-    int ovf_count;       // length of the overflow-row list
-    int pad;
+    unsigned pad;
+    // zeroed before every assignment (from amb_count on)
+    int amb_count;       // rows whose fp32 argmin is open (refinement; the fp32 direct path)
+    int ovf_count;       // rows whose candidate list overflowed
+    int ovf2_count;      // of those, rows that the centred screen left for the full-row kernel
+    int open_count;      // of those, rows whose fp32 argmin is open
+    unsigned ticket;     // blocks of k_amb_fp64 that have written their centred rows
+    unsigned pad2;
     unsigned long long npairs;  // candidate pairs written by the screening kernel
 };
+constexpr size_t kAssignCounterBytes = sizeof(DevCounters) - offsetof(DevCounters, amb_count);
 
 // Column-side constants of the reliability bound: maxima over centres.
 struct ColMax {
@@ -41,6 +48,18 @@ struct ColMax {
     // minima of the same statistics: a lower bound of every pair's threshold
     float nc_min, nrc_min, ncq_min, q_min, ncq2_min;
     float pad2[3];
+};
+
+// Inputs of the centred screen: bf16 copies of x - mu of the listed rows and of
+// c - mu of all centres, with their statistics (k_prep.cu).  Null Xq: not used.
+struct Centred {
+    void* Xq;
+    float4* xstat;
+    void* Cq;
+    float4* cstat;
+    ColMax* colmax;
+    float* qpad;
+    int ldq;
 };
 
 // Parameters of the reliability test / candidate window, host-computed.
@@ -92,11 +111,11 @@ cudaError_t launch_predict_candidates(const float* X, int64_t n, int d, const fl
 // direct-formula assignment.  acc64: binary64 accumulation (the plain FP64
 // path, all n rows) else fp32 with certification; rows = all n, or the device
 // list row_list[0 .. *row_count).  Uncertified fp32 rows are appended to
-// amb_list / cnt->amb_count.
+// open_list / *open_count.
 // absmax_out (nullable, zeroed by the caller): max |x| over the rows read.
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
-                                 double* min_dist, int32_t* amb_list, DevCounters* cnt, float gamma32,
+                                 double* min_dist, int32_t* open_list, int* open_count, DevCounters* cnt, float gamma32,
                                  int num_sms, cudaStream_t st, unsigned* absmax_out = nullptr);
 // exact argmin of the rows of a device list, one block per row: fp32 direct
 // values of all centres, certified, binary64 where still open.  count_open:
@@ -112,7 +131,8 @@ cudaError_t launch_rows_full(bool count_open, const float* X, const float* C, in
 // second A stage), or 32-column steps (C32).  Wider K: REG only.
 constexpr int TC_SV_FULL = 0, TC_SV_HALF = 1, TC_SV_C32 = 2, TC_SV_REG = 3;
 struct TcArgs {
-    int64_t n;
+    int64_t n;                // rows (capacity when nrows is given)
+    const int* nrows;         // nullable: the row count on the device (at most n)
     int k, d, fmt, kchunks;   // kchunks = number of 128-byte K atoms
     const float4* xstat;
     const float* xscale;
@@ -143,10 +163,16 @@ size_t tc_smem_bytes(int fmt, int d, int k);
 
 // candidate refinement: fp32 direct values of the pairs, then certified
 // argmin + min_dist per row; rows left open are appended to full_list
-// (cnt->ovf_count) for the full-row kernel
+// (cnt->ovf_count) for the full-row kernel; cen (Xq null: not used) receives
+// the centred bf16 copies of those rows and of the centres when there are any
 cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, int32_t* labels,
-                          double* min_dist, int32_t* full_list, int32_t* amb_list, int num_sms, cudaStream_t st,
-                          int* nlaunch);
+                          double* min_dist, int32_t* full_list, int32_t* amb_list, const Centred& cen, int num_sms,
+                          cudaStream_t st, int* nlaunch);
+// the centred screen's candidates (a.cand, a.rowinfo; its row r is row
+// list[r] of X): fp32 direct values, certified, binary64 where still open;
+// rows with too many candidates go to list2 / cnt->ovf2_count
+cudaError_t launch_refine_centred(const float* X, const float* C, const TcArgs& a, const int32_t* list, int32_t* labels,
+                                  int32_t* list2, int num_sms, cudaStream_t st);
 // the fallback's direct values for the flagged pairs of the distance matrix
 // (marked -1 in D): fb 0 binary64, 1 binary32, 2 the low format fmt (0
 // fp16, 1 bf16) itself; from the queue, or by a scan of D when it overflowed

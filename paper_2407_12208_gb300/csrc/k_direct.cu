@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(DA_ROWS, 5) k_direct_assign(const float* __res
 // Theorem 4.1's bound covers like any other.  Per row the smallest and
 // second-smallest value and the first index of the smallest (ties: lowest
 // index), merged over the 8 threads of the row; the certificate and the list
-// of open rows (amb_list).
+// of open rows (open_list).
 // Bound by the FP32 pipe (two lane operations per pair and coordinate).
 // Chunking the coordinates keeps the block at 113 KB or less, so two blocks
 // share an SM and one computes while the other waits at a tile's barrier.
@@ -126,8 +126,8 @@ constexpr size_t dt_smem(int rpt, int d) {
 template <int RPT, int VEC>
 KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __restrict__ C, int k, int d,
                          const int32_t* __restrict__ row_list, const int* __restrict__ row_count,
-                         int32_t* __restrict__ labels, double* __restrict__ min_dist, int32_t* __restrict__ amb_list,
-                         DevCounters* cnt, float gamma32, unsigned* __restrict__ absmax_out) {
+                         int32_t* __restrict__ labels, double* __restrict__ min_dist, int32_t* __restrict__ open_list,
+                         int* open_count, DevCounters* cnt, float gamma32, unsigned* __restrict__ absmax_out) {
     extern __shared__ __align__(16) float dts[];
     constexpr int R = 32 * RPT;
     const int dp = (d + 3) & ~3, cw = min(dp, DT_DK);
@@ -268,8 +268,8 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
                     min_dist[gi] = (double)b1[i];
                     // Theorem 4.1: true values lie in [v (1 - g), v (1 + g)]
                     if (!(b2[i] * (1.0f - g) > b1[i] * (1.0f + g))) {
-                        const int slot = atomicAdd(&cnt->amb_count, 1);
-                        amb_list[slot] = (int32_t)gi;
+                        const int slot = atomicAdd(open_count, 1);
+                        open_list[slot] = (int32_t)gi;
                         local_amb++;
                     }
                 }
@@ -294,9 +294,9 @@ __global__ void __launch_bounds__(256, 2) k_direct_tiled(const float* __restrict
                                                          const int32_t* __restrict__ row_list,
                                                          const int* __restrict__ row_count,
                                                          int32_t* __restrict__ labels, double* __restrict__ min_dist,
-                                                         int32_t* __restrict__ amb_list, DevCounters* cnt,
+                                                         int32_t* __restrict__ open_list, int* open_count, DevCounters* cnt,
                                                          float gamma32, unsigned* __restrict__ absmax_out) {
-    direct_tiled<RPT, 4>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32, absmax_out);
+    direct_tiled<RPT, 4>(X, n, C, k, d, row_list, row_count, labels, min_dist, open_list, open_count, cnt, gamma32, absmax_out);
 }
 // every other shape
 template <typename T, int RPT, int VEC>
@@ -305,25 +305,25 @@ __global__ void __launch_bounds__(256, 2) k_direct_assign(const float* __restric
                                                           const int32_t* __restrict__ row_list,
                                                           const int* __restrict__ row_count,
                                                           int32_t* __restrict__ labels, double* __restrict__ min_dist,
-                                                          int32_t* __restrict__ amb_list, DevCounters* cnt,
+                                                          int32_t* __restrict__ open_list, int* open_count, DevCounters* cnt,
                                                           float gamma32, unsigned* __restrict__ absmax_out) {
     static_assert(sizeof(T) == 4, "binary32 accumulation");
-    direct_tiled<RPT, VEC>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32, absmax_out);
+    direct_tiled<RPT, VEC>(X, n, C, k, d, row_list, row_count, labels, min_dist, open_list, open_count, cnt, gamma32, absmax_out);
 }
 
 template <int RPT, int VEC>
 static cudaError_t launch_tiled(const float* X, int64_t n, const float* C, int k, int d, const int32_t* row_list,
-                                const int* row_count, int32_t* labels, double* min_dist, int32_t* amb_list,
-                                DevCounters* cnt, float gamma32, int num_sms, cudaStream_t st, unsigned* absmax_out) {
+                                const int* row_count, int32_t* labels, double* min_dist, int32_t* open_list,
+                                int* open_count, DevCounters* cnt, float gamma32, int num_sms, cudaStream_t st, unsigned* absmax_out) {
     const size_t sm = dt_smem(RPT, d);
-    void (*fn)(const float*, int64_t, const float*, int, int, const int32_t*, const int*, int32_t*, double*, int32_t*,
+    void (*fn)(const float*, int64_t, const float*, int, int, const int32_t*, const int*, int32_t*, double*, int32_t*, int*,
                DevCounters*, float, unsigned*) = k_direct_assign<float, RPT, VEC>;
     if constexpr (VEC == 4)
         if (d >= 16 && d <= 128) fn = k_direct_tiled<RPT>;
     cudaError_t e = allow_max_smem(fn);
     if (e != cudaSuccess) return e;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 32 * RPT - 1) / (32 * RPT), (int64_t)num_sms * 2));
-    fn<<<(unsigned)grid, 256, sm, st>>>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32,
+    fn<<<(unsigned)grid, 256, sm, st>>>(X, n, C, k, d, row_list, row_count, labels, min_dist, open_list, open_count, cnt, gamma32,
                                         absmax_out);
     return cudaGetLastError();
 }
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(256) k_direct_small(const float* __restrict__ 
                                                       const int32_t* __restrict__ row_list,
                                                       const int* __restrict__ row_count,
                                                       int32_t* __restrict__ labels, double* __restrict__ min_dist,
-                                                      int32_t* __restrict__ amb_list, DevCounters* cnt,
+                                                      int32_t* __restrict__ open_list, int* open_count, DevCounters* cnt,
                                                       float gamma32, unsigned* __restrict__ absmax_out) {
     extern __shared__ __align__(16) float Csm[];
     float amx = 0.0f;  // largest |x| of this thread's rows (absmax_out)
@@ -378,8 +378,8 @@ __global__ void __launch_bounds__(256) k_direct_small(const float* __restrict__ 
         rows_done++;
         // Theorem 4.1: true values lie in [v (1 - g), v (1 + g)]
         if (!(b2 * (1.0f - g) > b1 * (1.0f + g))) {
-            const int slot = atomicAdd(&cnt->amb_count, 1);
-            amb_list[slot] = (int32_t)gi;
+            const int slot = atomicAdd(open_count, 1);
+            open_list[slot] = (int32_t)gi;
             local_amb++;
         }
     }
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(256) k_rows_full(const float* __restrict__ X, 
 
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
-                                 double* min_dist, int32_t* amb_list, DevCounters* cnt, float gamma32,
+                                 double* min_dist, int32_t* open_list, int* open_count, DevCounters* cnt, float gamma32,
                                  int num_sms, cudaStream_t st, unsigned* absmax_out) {
     if (!acc64 && d <= 8 && (size_t)k * d * sizeof(float) <= 32 * 1024) {
         // small d: C resident in shared memory, one thread per row, persistent grid
@@ -604,7 +604,7 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
 #define KM_SMALL(DD)                                                                                                  \
     case DD:                                                                                                          \
         k_direct_small<DD><<<(unsigned)grid, 256, csm, st>>>(X, n, C, k, row_list, row_count, labels, min_dist,      \
-                                                              amb_list, cnt, gamma32, absmax_out);                                \
+                                                              open_list, open_count, cnt, gamma32, absmax_out);                                \
         break;
             KM_SMALL(1) KM_SMALL(2) KM_SMALL(3) KM_SMALL(4) KM_SMALL(5) KM_SMALL(6) KM_SMALL(7) KM_SMALL(8)
 #undef KM_SMALL
@@ -622,7 +622,7 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
         while (rpt > 1 && !row_list && (n + 32 * rpt - 1) / (32 * rpt) < 2 * num_sms) rpt >>= 1;
 #define KM_DT(RP, VE)                                                                                              \
     if (rpt == RP && vec == VE)                                                                                    \
-        return launch_tiled<RP, VE>(X, n, C, k, d, row_list, row_count, labels, min_dist, amb_list, cnt, gamma32, \
+        return launch_tiled<RP, VE>(X, n, C, k, d, row_list, row_count, labels, min_dist, open_list, open_count, cnt, gamma32, \
                                     num_sms, st, absmax_out);
         KM_DT(4, 4) KM_DT(4, 2) KM_DT(4, 1) KM_DT(2, 4) KM_DT(2, 2) KM_DT(2, 1) KM_DT(1, 4) KM_DT(1, 2) KM_DT(1, 1)
 #undef KM_DT

@@ -21,11 +21,9 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "rowstat.cuh"
 
 namespace km {
-
-constexpr float kNormInflate = 1.0f + 1.0f / 4096.0f;
-constexpr float kTinyNorm2 = 0x1p-100f;  // below this ||x||^2 the fp32 statistics are not trusted
 
 KM_DEV float quant_val(float v, int fmt) {
     if (fmt == 0) return __half2float(__float2half_rn(v));
@@ -137,23 +135,6 @@ __global__ void k_quantize(const float* __restrict__ A, int64_t m, int d, int fm
 // Group path (d % 4 == 0, padded width <= 256): 8 lanes per row, 4 rows per
 // warp, so the row reductions take 3 shuffle levels and serve 4 rows at once.
 // Lane l of a row's 8 holds float4 l, l + 8, ... (NV of them).
-// Two coordinates (scale 1, 16-bit formats) into the row's running sums, two
-// per packed instruction: ||x||^2 as a pair of double-floats (exact product,
-// two-sum), ||x~||^2 and ||x~ - x||^2 in fp32.
-KM_DEV float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-KM_DEV void row_sums2(float2 x, float2 q, float2& hi, float2& lo, float2& qq, float2& rr) {
-    const float2 p = __fmul2_rn(x, x);
-    const float2 pe = __ffma2_rn(x, x, neg2(p));
-    const float2 s = __fadd2_rn(hi, p);
-    const float2 bb = __fadd2_rn(s, neg2(hi));
-    const float2 e = __fadd2_rn(__fadd2_rn(hi, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
-    hi = s;
-    lo = __fadd2_rn(lo, __fadd2_rn(e, pe));
-    qq = __ffma2_rn(q, q, qq);
-    const float2 r = __fadd2_rn(q, neg2(x));  // exact (Sterbenz)
-    rr = __ffma2_rn(r, r, rr);
-}
-
 template <int NV>
 __global__ void k_quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
                               float4* __restrict__ stat, float* __restrict__ rscale, unsigned* __restrict__ absmax_out) {
@@ -390,63 +371,17 @@ __global__ void k_quantize_vec(const float* __restrict__ A, int64_t m, int d, in
     if (absmax_out) block_absmax(amx, absmax_out);
 }
 
-__global__ void k_colmax(const float4* __restrict__ cstat, int k, const float* __restrict__ cscale, ColMax* out,
-                         float* __restrict__ qpad, float* __restrict__ spad, int kpad) {
-    // q_j for the screening kernel, +inf on the padding so padded columns never
-    // win; the centres' E4M3 scales (cscale, nullable: 1), 1 on the padding
+// q_j for the screening kernel, +inf on the padding so padded columns never
+// win; the centres' E4M3 scales (cscale, nullable: 1), 1 on the padding; the
+// column maxima.
+__global__ void __launch_bounds__(1024) k_colmax(const float4* __restrict__ cstat, int k,
+                                                 const float* __restrict__ cscale, ColMax* out,
+                                                 float* __restrict__ qpad, float* __restrict__ spad, int kpad) {
     for (int j = threadIdx.x; j < kpad; j += blockDim.x) {
         qpad[j] = (j < k) ? cstat[j].x : INFINITY;
         spad[j] = (j < k && cscale) ? cscale[j] : 1.0f;
     }
-    __shared__ float red[10][32];
-    float a = 0, b = 0, c = 0, q = 0, c2 = 0;
-    float an = INFINITY, bn = INFINITY, cn = INFINITY, qn = INFINITY, c2n = INFINITY;
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
-        float4 s = cstat[j];
-        a = fmaxf(a, s.y);
-        b = fmaxf(b, s.w);
-        c = fmaxf(c, s.z);
-        q = fmaxf(q, s.x);
-        c2 = fmaxf(c2, s.z * s.z);
-        an = fminf(an, s.y);
-        bn = fminf(bn, s.w);
-        cn = fminf(cn, s.z);
-        qn = fminf(qn, s.x);
-        c2n = fminf(c2n, s.z * s.z);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, off));
-        b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, off));
-        c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, off));
-        q = fmaxf(q, __shfl_xor_sync(0xffffffffu, q, off));
-        c2 = fmaxf(c2, __shfl_xor_sync(0xffffffffu, c2, off));
-        an = fminf(an, __shfl_xor_sync(0xffffffffu, an, off));
-        bn = fminf(bn, __shfl_xor_sync(0xffffffffu, bn, off));
-        cn = fminf(cn, __shfl_xor_sync(0xffffffffu, cn, off));
-        qn = fminf(qn, __shfl_xor_sync(0xffffffffu, qn, off));
-        c2n = fminf(c2n, __shfl_xor_sync(0xffffffffu, c2n, off));
-    }
-    const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
-    if (ln == 0) {
-        red[0][w] = a; red[1][w] = b; red[2][w] = c; red[3][w] = q; red[4][w] = c2;
-        red[5][w] = an; red[6][w] = bn; red[7][w] = cn; red[8][w] = qn; red[9][w] = c2n;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < (int)(blockDim.x / 32); i++) {
-            a = fmaxf(a, red[0][i]); b = fmaxf(b, red[1][i]); c = fmaxf(c, red[2][i]);
-            q = fmaxf(q, red[3][i]); c2 = fmaxf(c2, red[4][i]);
-            an = fminf(an, red[5][i]); bn = fminf(bn, red[6][i]); cn = fminf(cn, red[7][i]);
-            qn = fminf(qn, red[8][i]); c2n = fminf(c2n, red[9][i]);
-        }
-        ColMax o;
-        o.nc = a; o.nrc = b; o.ncq = c; o.q = q; o.ncq2 = c2;
-        o.pad[0] = o.pad[1] = o.pad[2] = 0.0f;
-        o.nc_min = an; o.nrc_min = bn; o.ncq_min = cn; o.q_min = qn; o.ncq2_min = c2n;
-        o.pad2[0] = o.pad2[1] = o.pad2[2] = 0.0f;
-        *out = o;
-    }
+    colmax_block(cstat, k, out);
 }
 
 cudaError_t launch_quantize(const float* A, int64_t m, int d, int fmt, int ldq, void* Aq, float4* stat,

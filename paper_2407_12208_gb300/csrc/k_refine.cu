@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "rowstat.cuh"
 
 namespace km {
 
@@ -127,6 +128,8 @@ __global__ void __launch_bounds__(256) k_cand_select(const int4* __restrict__ ro
                 W = __int_as_float(ig.z);
             }
             lim = dmin + W;
+            // an infinite window (or nothing comparable) takes in the columns' padding too: the whole row
+            full |= !(lim < INFINITY);
         }
         // the first SPEC slots of every list in one round of loads, the rest (rare) after
         constexpr int SPEC = (16 / TC_GROUPS < TC_LIST) ? 16 / TC_GROUPS : TC_LIST;
@@ -277,8 +280,9 @@ constexpr int AMB_B = 4;
 __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ amb_list, const int* __restrict__ amb_count,
                                                   const int2* __restrict__ rowpair, const int2* __restrict__ pairs,
                                                   const float* __restrict__ v32, const float* __restrict__ X,
-                                                  const float* __restrict__ C, int d, float gamma32,
+                                                  const float* __restrict__ C, int k, int d, float gamma32,
                                                   int32_t* __restrict__ labels, double* __restrict__ min_dist,
+                                                  const int32_t* __restrict__ full_list, const Centred cen,
                                                   DevCounters* cnt) {
     extern __shared__ double amb_sm[];  // per warp: AMB_B x d products
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -338,7 +342,7 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
             if (ob < best || (ob == best && oj < bj)) { best = ob; bj = oj; }
         }
         if (lane == 0) {
-            labels[row] = bj;
+            labels[row] = bj != 0x7fffffff ? bj : pairs[rp.x].y;  // (not a number: a valid label all the same)
             min_dist[row] = best;
         }
         __syncwarp();
@@ -346,10 +350,280 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ev64 += __shfl_xor_sync(0xffffffffu, ev64, off);
     if (lane == 0 && ev64) atomicAdd(&cnt->fp64_evals, ev64);
+    // the centres and the rows whose list overflowed, centred, for the second
+    // screen; the last block to finish forms the column maxima and q_j
+    const int nf = cen.Xq ? cnt->ovf_count : 0;
+    if (nf == 0) return;
+    __shared__ __align__(16) float mu[256];
+    __shared__ bool last;
+    centre_mean(C, k, d, cen.ldq, mu);
+    const int sl = lane & 7;
+    const unsigned gmask = 0xFFu << (lane & ~7);
+    const bool vec = d % 4 == 0 && (((uintptr_t)X | (uintptr_t)C) & 15) == 0;
+    for (int64_t r = 4 * w0 + (lane >> 3); r < (int64_t)k + nf; r += 4 * nw) {
+        const bool isc = r < k;
+        const float* x = isc ? C + r * d : X + (int64_t)full_list[r - k] * d;
+        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(isc ? cen.Cq : cen.Xq) + (isc ? r : r - k) * cen.ldq;
+        float4* stat = isc ? cen.cstat + r : cen.xstat + (r - k);
+        if (vec) centred_row<true>(x, mu, d, cen.ldq, dst, stat, sl, gmask);
+        else centred_row<false>(x, mu, d, cen.ldq, dst, stat, sl, gmask);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&cnt->ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int kpad = (k + 255) / 256 * 256;
+    for (int j = threadIdx.x; j < kpad; j += blockDim.x) cen.qpad[j] = j < k ? __ldcg(cen.cstat + j).x : INFINITY;
+    colmax_block(cen.cstat, k, cen.colmax);
+}
+
+// The centred screen's candidates, 32 listed rows per warp.  A lane per row
+// finds the candidates inside the window of the row's final d^ minimum; a row
+// with one is decided there.  Rows with a few take eight lanes each for their
+// fp32 direct values and Theorem 4.1's intervals; rows with many, and those
+// whose intervals overlap, the whole warp, which ends in binary64 in the
+// oracle's order.  Labels only: every caller refines the winner's distance
+// afterwards.  Few rows come here in most calls; when all do
+// it is bound by the latency of a row's chain of loads.
+// 1e6 x 128, k = 1024, all rows: 151 us (one row per warp at a time: 558 us).
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__ rowinfo,
+                                                        const uint32_t* __restrict__ cand, int64_t n, int ebits,
+                                                        const int32_t* __restrict__ list, const float* __restrict__ X,
+                                                        const float* __restrict__ C, int d, float gamma32,
+                                                        int32_t* __restrict__ labels, int32_t* __restrict__ list2,
+                                                        DevCounters* cnt) {
+    constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
+    static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
+    extern __shared__ double rc_sm[];  // per warp: d products
+    constexpr int JC = 12;
+    __shared__ int js_sh[8][4 * NE];
+    __shared__ float vs_sh[8][4 * NE];
+    __shared__ int jl_sh[8][JC * 32], ord_sh[8][32];
+    const int nrows = cnt->ovf_count;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, sl = lane & 7;
+    double* prod = rc_sm + (size_t)wib * d;
+    int* js = js_sh[wib];
+    float* vs = vs_sh[wib];
+    int *jl = jl_sh[wib], *ord = ord_sh[wib];
+    const uint32_t emask = (1u << ebits) - 1u;
+    const float lscale = __uint_as_float((uint32_t)(127 + ebits - 23) << 23);  // 2^(ebits - 23)
+    const float g = gamma32;
+    unsigned long long ev32 = 0, ev64 = 0, amb = 0;
+    for (int64_t r0 = ((int64_t)blockIdx.x * 8 + wib) * 32; r0 < nrows; r0 += (int64_t)gridDim.x * 256) {
+        const int64_t r = r0 + lane;
+        const bool valid = r < nrows;
+        const int myrow = valid ? list[r] : 0;
+        bool full = false;
+        int cnt_g[TC_GROUPS];
+        float lim = INFINITY, W = 0.0f;
+#pragma unroll
+        for (int q = 0; q < TC_GROUPS; q++) {
+            const int4 ig = valid ? rowinfo[r * TC_GROUPS + q] : make_int4(0, 0, 0, __float_as_int(INFINITY));
+            full |= ig.y != 0;
+            cnt_g[q] = ig.x;
+            lim = fminf(lim, __int_as_float(ig.w));
+            W = __int_as_float(ig.z);
+        }
+        lim += W;
+        // an overflowed list or an infinite window (which takes in the padding): every centre
+        full = valid && (full || !(lim < INFINITY));
+        if (full) list2[atomicAdd(&cnt->ovf2_count, 1)] = myrow;
+        int c = 0;
+#pragma unroll
+        for (int q = 0; q < TC_GROUPS; q++) {
+            const int ng = valid && !full ? cnt_g[q] : 0;
+            const uint32_t* cg = cand + (size_t)q * TC_LIST * n + r;
+            for (int s0 = 0; __any_sync(0xffffffffu, s0 < ng); s0 += 4) {
+                uint32_t e[4];
+#pragma unroll
+                for (int s = 0; s < 4; s++) e[s] = s0 + s < ng ? cg[(size_t)(s0 + s) * n] : 0u;
+#pragma unroll
+                for (int s = 0; s < 4; s++)
+                    if (s0 + s < ng && cand_lower(e[s], emask, lscale) <= lim)
+                        for (unsigned bb = entry_mask(e[s]); bb; bb &= bb - 1, c++)
+                            if (c < JC) jl[c * 32 + lane] = 4 * entry_quad(e[s], emask) + __ffs(bb) - 1;
+            }
+        }
+        if (c == 1) labels[myrow] = jl[lane];
+        // rows of two to JC candidates, eight lanes each
+        const bool few = c > 1 && c <= JC;
+        const unsigned fm = __ballot_sync(0xffffffffu, few);
+        if (few) ord[__popc(fm & ((1u << lane) - 1u))] = lane;
+        __syncwarp();
+        unsigned slow = __ballot_sync(0xffffffffu, c > JC);
+        const int nfew = __popc(fm);
+        for (int i0 = 0; i0 < nfew; i0 += 4) {
+            const int i = i0 + (lane >> 3);
+            const int b = ord[min(i, nfew - 1)];
+            const int cb = __shfl_sync(0xffffffffu, c, b), cc = i < nfew ? cb : 0;
+            const int64_t row = __shfl_sync(0xffffffffu, myrow, b);
+            const int most = __reduce_max_sync(0xffffffffu, cc);
+            const float* x = X + row * d;
+            float b1 = INFINITY, b2 = INFINITY;
+            int j1 = 0;
+            for (int t = 0; t < most; t++) {
+                const bool on = t < cc;
+                const int j = jl[(on ? t : 0) * 32 + b];
+                const float* cj = C + (int64_t)j * d;
+                float acc = 0.0f;
+                if (VEC) {
+#pragma unroll 4
+                    for (int q = sl; q < (d >> 2); q += 8) {
+                        const float4 xv = reinterpret_cast<const float4*>(x)[q], cv = reinterpret_cast<const float4*>(cj)[q];
+                        const float u0 = xv.x - cv.x, u1 = xv.y - cv.y, u2 = xv.z - cv.z, u3 = xv.w - cv.w;
+                        acc = fmaf(u0, u0, acc);
+                        acc = fmaf(u1, u1, acc);
+                        acc = fmaf(u2, u2, acc);
+                        acc = fmaf(u3, u3, acc);
+                    }
+                } else {
+#pragma unroll 4
+                    for (int l = sl; l < d; l += 8) {
+                        const float u = x[l] - cj[l];
+                        acc = fmaf(u, u, acc);
+                    }
+                }
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                if (on) {
+                    if (acc < b1) { b2 = b1; b1 = acc; j1 = j; }
+                    else b2 = fminf(b2, acc);
+                }
+            }
+            const bool sure = b2 * (1.0f - g) > b1 * (1.0f + g);  // false where nothing is comparable
+            if (sl == 0 && cc) {
+                ev32 += (unsigned long long)cc;
+                if (sure) labels[row] = j1;
+            }
+            slow |= __reduce_or_sync(0xffffffffu, cc && !sure ? 1u << b : 0u);
+        }
+        // the others (many candidates, near-ties), the warp on one row at a time
+        for (unsigned todo = slow; todo; todo &= todo - 1) {
+            const int b = __ffs(todo) - 1;
+            const int64_t row = __shfl_sync(0xffffffffu, myrow, b);
+            const float rlim = __shfl_sync(0xffffffffu, lim, b);
+            const int total = __shfl_sync(0xffffffffu, c, b);
+            const int n0 = __shfl_sync(0xffffffffu, cnt_g[0], b), n1 = __shfl_sync(0xffffffffu, cnt_g[1], b);
+            const int n2 = __shfl_sync(0xffffffffu, cnt_g[2], b);
+            uint32_t e[2];
+            unsigned m[2];
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int t = lane + 32 * h, gr = t / TC_LIST, slot = t % TC_LIST;
+                const bool have = t < NE && slot < (gr == 0 ? n0 : (gr == 1 ? n1 : n2));
+                e[h] = have ? cand[(size_t)t * n + r0 + b] : 0u;
+                m[h] = have && cand_lower(e[h], emask, lscale) <= rlim ? entry_mask(e[h]) : 0u;
+            }
+            const int mine = __popc(m[0]) + __popc(m[1]);
+            int incl = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += o;
+            }
+            __syncwarp();
+            int w = incl - mine;
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+                for (unsigned bb = m[h]; bb; bb &= bb - 1) js[w++] = 4 * entry_quad(e[h], emask) + __ffs(bb) - 1;
+            __syncwarp();
+            const float* x = X + row * d;
+            for (int t0 = 0; t0 < total; t0 += 4) {
+                const int t = t0 + (lane >> 3);
+                float acc = 0.0f;
+                if (t < total) {
+                    const float* cj = C + (int64_t)js[t] * d;
+                    if (VEC) {
+#pragma unroll 4
+                        for (int q = sl; q < (d >> 2); q += 8) {
+                            const float4 xv = reinterpret_cast<const float4*>(x)[q], cv = reinterpret_cast<const float4*>(cj)[q];
+                            const float u0 = xv.x - cv.x, u1 = xv.y - cv.y, u2 = xv.z - cv.z, u3 = xv.w - cv.w;
+                            acc = fmaf(u0, u0, acc);
+                            acc = fmaf(u1, u1, acc);
+                            acc = fmaf(u2, u2, acc);
+                            acc = fmaf(u3, u3, acc);
+                        }
+                    } else {
+#pragma unroll 4
+                        for (int l = sl; l < d; l += 8) {
+                            const float u = x[l] - cj[l];
+                            acc = fmaf(u, u, acc);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                if (sl == 0 && t < total) vs[t] = acc;
+            }
+            __syncwarp();
+            if (lane == 0 && total > JC) ev32 += (unsigned long long)total;
+            float up = INFINITY;
+            for (int t = lane; t < total; t += 32) up = fminf(up, vs[t] * (1.0f + g));
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) up = fminf(up, __shfl_xor_sync(0xffffffffu, up, off));
+            int open = 0, bj = 0x7fffffff;
+            for (int t = lane; t < total; t += 32)
+                if (vs[t] * (1.0f - g) <= up) {
+                    open++;
+                    bj = js[t];  // (the only one, when open is 1 over the warp)
+                }
+            const unsigned who = __ballot_sync(0xffffffffu, open != 0);
+            open = __reduce_add_sync(0xffffffffu, open);
+            if (open == 1) {
+                const int src = __ffs(who) - 1;
+                if (lane == src) labels[row] = bj;
+                continue;
+            }
+            if (lane == 0) amb++;
+            double best = INFINITY;
+            bj = 0x7fffffff;
+            for (int t = 0; t < total; t++) {
+                if (!(vs[t] * (1.0f - g) <= up)) continue;
+                const int j = js[t];
+                const float* cj = C + (int64_t)j * d;
+                for (int l = lane; l < d; l += 32) {
+                    const double u = __dsub_rn((double)x[l], (double)cj[l]);
+                    prod[l] = __dmul_rn(u, u);
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    double s = 0.0;
+                    for (int l = 0; l < d; l++) s = __dadd_rn(s, prod[l]);
+                    ev64++;
+                    if (s < best || (s == best && j < bj)) { best = s; bj = j; }
+                }
+                __syncwarp();
+            }
+            if (lane == 0) labels[row] = bj != 0x7fffffff ? bj : js[0];
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) ev32 += __shfl_xor_sync(0xffffffffu, ev32, off);
+    if (lane == 0) {
+        if (ev32) atomicAdd(&cnt->fp32_evals, ev32);
+        if (ev64) atomicAdd(&cnt->fp64_evals, ev64);
+        if (amb) atomicAdd(&cnt->amb_rows, amb);
+    }
+}
+
+cudaError_t launch_refine_centred(const float* X, const float* C, const TcArgs& a, const int32_t* list, int32_t* labels,
+                                  int32_t* list2, int num_sms, cudaStream_t st) {
+    const bool vec = a.d % 4 == 0 && ((uintptr_t)X % 16 == 0) && ((uintptr_t)C % 16 == 0);
+    auto fn = vec ? k_refine_centred<true> : k_refine_centred<false>;
+    const size_t sm = (size_t)8 * a.d * sizeof(double);
+    const unsigned blocks = (unsigned)std::min<int64_t>((a.n + 255) / 256, (int64_t)num_sms * 6);
+    fn<<<blocks, 256, sm, st>>>(a.rowinfo, a.cand, a.n, a.ebits, list, X, C, a.d, a.tp.gamma32, labels, list2,
+                                a.cnt);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, int32_t* labels, double* min_dist,
-                          int32_t* full_list, int32_t* amb_list, int num_sms, cudaStream_t st, int* nlaunch) {
+                          int32_t* full_list, int32_t* amb_list, const Centred& cen, int num_sms, cudaStream_t st,
+                          int* nlaunch) {
     // persistent grids: the resident blocks only
     int sel_per_sm = 1, cert_per_sm = 1;
     cudaError_t e0 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sel_per_sm, k_cand_select, 256, 0);
@@ -387,8 +661,10 @@ cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, int32
     const size_t amb_smem = (size_t)8 * AMB_B * a.d * sizeof(double);  // 8 warps per block
     e = allow_max_smem(k_amb_fp64);
     if (e != cudaSuccess) return e;
-    k_amb_fp64<<<(unsigned)num_sms, 256, amb_smem, st>>>(amb_list, &a.cnt->amb_count, a.rowpair, a.pairs, a.v32, X, C,
-                                                          a.d, a.tp.gamma32, labels, min_dist, a.cnt);
+    // (three blocks per SM quantise overflowed rows faster than one: they are bound by loads)
+    k_amb_fp64<<<(unsigned)num_sms * (cen.Xq ? 3 : 1), 256, amb_smem, st>>>(
+        amb_list, &a.cnt->amb_count, a.rowpair, a.pairs, a.v32, X, C, a.k, a.d, a.tp.gamma32, labels, min_dist, full_list,
+        cen, a.cnt);
     return cudaGetLastError();
 }
 

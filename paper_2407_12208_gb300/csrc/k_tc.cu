@@ -164,6 +164,8 @@ template <int FMT, int BN, int MODE, int SV>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmC, const TcArgs a) {
     extern __shared__ unsigned char smem_raw[];
+    const int64_t nrows = a.nrows ? min((int64_t)*a.nrows, a.n) : a.n;
+    if (nrows == 0) return;
     // 1024-byte aligned base, derived from the shared array by an offset so that
     // every pointer below stays in the shared state space (LDS/STS, not generic)
     const uint32_t sraw = smem_u32(smem_raw);
@@ -195,7 +197,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     constexpr int NBUF = 512 / BN;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t nrb = (a.n + TC_BM - 1) / TC_BM;
+    const int64_t nrb = (nrows + TC_BM - 1) / TC_BM;
     const int NT = (a.k + BN - 1) / BN;
     constexpr uint32_t ESIZE = (FMT == 2) ? 1 : 2;
     constexpr int ATOM_ELEMS = 128 / ESIZE;
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         int iter = 0;
         for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, iter++) {
             const int64_t row = rb * TC_BM + r_in;
-            const bool valid = row < a.n;
+            const bool valid = row < nrows;
             float4 xs = make_float4(0.f, 0.f, 0.f, 0.f);
             float rs = 1.0f;
             if (valid) {

@@ -63,3 +63,49 @@ def test_open_rows_take_the_lowest_index(ctx, copies, d, k):
     olab, od1, _ = oracle.assign(X[:64], C)
     assert np.array_equal(lab[:64], olab)
     np.testing.assert_allclose(md[:64], od1, rtol=RTOL_MD, atol=1e-30)
+
+
+# rows that the plain screen cannot decide go through the centred screen (from 2^30
+# pair-coordinates on): far from the origin, past fp16's range, 8 bits on close distances
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("low,kind,n,d,k", [("bf16", "cancellation", 20011, 53, 1024), ("bf16", "cancellation", 16500, 128, 513),
+                                            ("fp16", "cancellation", 17000, 256, 250), ("fp16", "huge", 17001, 64, 1000),
+                                            ("e4m3", "uniform", 17000, 64, 1024), ("e4m3", "uniform", 16999, 250, 255),
+                                            ("bf16", "copies3", 17001, 128, 510), ("bf16", "copies20", 17001, 128, 500),
+                                            ("bf16", "copies64", 17001, 128, 512), ("bf16", "copies3", 60001, 9, 2001)])
+def test_centred_screen(ctx, low, kind, n, d, k, offset):
+    if kind == "uniform":
+        X, C = workloads.uniform_pairs(n, d, k, seed=5)
+    elif kind == "huge":
+        X, C = workloads.gaussian_mixture(n, d, k, seed=5)
+        X, C = X * np.float32(1e5), C * np.float32(1e5)
+    else:
+        X, C = workloads.cancellation(n, d, k, seed=5)
+        if kind.startswith("copies"):  # ties: two candidates to more than a list holds
+            c = int(kind[6:])
+            C = np.tile(C[: k // c], (c, 1))
+    lab, md, _ = _assign(ctx, X, C, low, offset)
+    assert ctx.stats()["overflow_rows"] > n // 2
+    check_assign(lab, md, X, C, oracle, RTOL_MD)
+    if kind.startswith("copies"):
+        assert lab.max() < len(C) // int(kind[6:])
+
+
+def test_smallest_accepted_workspace(ctx):
+    """A workspace without room for the centred screen is still accepted."""
+    import paper_2407_12208_gb300 as pkg
+    X, C = workloads.cancellation(17000, 64, 1000, seed=6)
+    Xd, Cd, p = _dev(X), _dev(C), pkg.params("bf16")
+    ws = ctx.workspace(17000, 64, 1000, p)
+    lo, hi = 0, ws.numel()  # refused at lo, accepted at hi
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        try:
+            ctx.assign(Xd, Cd, p, ws=ws[:mid])
+            hi = mid
+        except pkg.KmError:
+            lo = mid
+    full = ctx.assign(Xd, Cd, p)
+    small = ctx.assign(Xd, Cd, p, ws=ws[:hi])
+    assert hi < ws.numel() - 17000 * 64 * 2
+    assert torch.equal(full[0], small[0]) and torch.equal(full[1], small[1]) and full[2] == small[2]
