@@ -206,10 +206,12 @@ AssignWs carve_assign(Carve& cv, int64_t n, int d, int k, int low, bool distance
         w.ovf_list = cv.take<int32_t>((size_t)n);
         if (!distances) {
             w.cand = cv.take<uint32_t>((size_t)n * TC_GROUPS * TC_LIST);
-            w.rowpair = cv.take<int2>((size_t)n);
-            w.pair_cap = std::min<int64_t>((int64_t)n * TC_PAIRS_PER_ROW, (int64_t)INT32_MAX);
-            w.pairs = cv.take<int2>((size_t)w.pair_cap);
-            w.v32 = cv.take<float>((size_t)w.pair_cap);
+            if (refine_batched(n, d)) {
+                w.rowpair = cv.take<int2>((size_t)n);
+                w.pair_cap = std::min<int64_t>((int64_t)n * TC_PAIRS_PER_ROW, (int64_t)INT32_MAX);
+                w.pairs = cv.take<int2>((size_t)w.pair_cap);
+                w.v32 = cv.take<float>((size_t)w.pair_cap);
+            }
         } else {
             w.qcap = flag_queue_cap(n, k);
             w.queue = cv.take<int2>((size_t)w.qcap);
@@ -227,7 +229,7 @@ AssignWs carve_assign(Carve& cv, int64_t n, int d, int k, int low, bool distance
 
 // The centred screen (k_refine.cu) pays where the full-row kernel would be
 // expensive: at 2^30 pair-coordinates that takes about 80 us when every row
-// overflows, and its two launches, empty in most calls, about 4 us.
+// overflows, and its three launches, empty in most calls, about 6 us.
 bool centred_applies(int64_t n, int d, int k, int low) {
     return is_tc(low) && d <= 256 && (double)n * k * d >= (double)(1 << 30) && tc_smem_bytes(1, d, 1) != 0;
 }
@@ -243,6 +245,7 @@ Centred carve_centred(Carve& cv, int64_t n, int d, int k, int low) {
     c.cstat = cv.take<float4>((size_t)k);
     c.colmax = cv.take<ColMax>(1);
     c.qpad = cv.take<float>((size_t)kpad_of(k));
+    c.list2 = cv.take<int32_t>((size_t)n);
     return c;
 }
 // cv stands at the end of what the call needs
@@ -441,11 +444,11 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
     a.kchunks = (ldq * esz + 127) / 128;
     a.xstat = w.xstat; a.xscale = w.xscale; a.cstat = w.cstat; a.qpad = w.qpad; a.spad = w.spad; a.colmax = w.colmax;
     a.tp = tp; a.mode = 0; a.cand = w.cand; a.rowinfo = w.rowinfo; a.cnt = w.cnt;
+    a.pairs = w.pairs; a.pair_cap = w.pair_cap; a.v32 = w.v32; a.rowpair = w.rowpair;
     a.variant = screen_variant(ctx, fmt, a.kchunks, k, n);
     int qbits = 0;
     while ((1 << qbits) < (k + 3) / 4) qbits++;  // quad index bits (k <= 65535: at most 14)
     a.ebits = qbits + 4;
-    a.pairs = w.pairs; a.pair_cap = w.pair_cap; a.v32 = w.v32; a.rowpair = w.rowpair;
     {
         PhaseScope ps(ctx, KM_PHASE_SCREEN, st);
         KL(1, launch_tc(w.Xq, w.Cq, ldq, a, ctx->num_sms, st));
@@ -453,16 +456,15 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
     {
         PhaseScope ps(ctx, KM_PHASE_REFINE, st);
         int nl = 0;
-        CK(launch_refine(X, C, a, labels, min_dist, w.ovf_list, w.amb_list, cen, ctx->num_sms, st, &nl));
+        CK(launch_refine(X, C, a, nullptr, nullptr, labels, min_dist, w.ovf_list, &w.cnt->ovf_count, w.amb_list,
+                         ctx->num_sms, st, &nl));
         ctx->launches += (uint64_t)nl;
     }
     {
         // rows whose candidate list overflowed (all of them when every pair fails
         // the reliability test): the centred screen where it applies, then, for
         // what is left, fp32 direct distances to every centre with Theorem 4.1's
-        // certificate, then binary64 for the rows left open.  The near-tie list was
-        // consumed by the refinement and now takes those rows; the rows' pair
-        // ranges, consumed as well, hold the list of what the centred screen left.
+        // certificate, then binary64 for the rows left open.
         PhaseScope ps(ctx, KM_PHASE_FULLROW, st);
         const int32_t* list = w.ovf_list;
         const int* list_n = &w.cnt->ovf_count;
@@ -479,10 +481,12 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
             b.tp = make_tp(&q, d);
             b.tp.kn = (float)(10.0 * std::ldexp(1.0, -24));
             b.variant = screen_variant(ctx, 1, b.kchunks, k, n);
+            KL(1, launch_centre_rows(list, list_n, X, C, k, d, cen, &w.cnt->ticket, ctx->num_sms, st));
             KL(1, launch_tc(cen.Xq, cen.Cq, cen.ldq, b, ctx->num_sms, st));
-            int32_t* list2 = reinterpret_cast<int32_t*>(w.rowpair);
-            KL(1, launch_refine_centred(X, C, b, list, labels, list2, ctx->num_sms, st));
-            list = list2;
+            int nl = 0;
+            KL(1, launch_refine(X, C, b, list, list_n, labels, min_dist, cen.list2, &w.cnt->ovf2_count, w.amb_list,
+                                ctx->num_sms, st, &nl));
+            list = cen.list2;
             list_n = &w.cnt->ovf2_count;
         }
         if (d <= 256) {  // the direct kernel's row tile fits in shared memory

@@ -31,9 +31,9 @@ struct DevCounters {
     int ovf_count;       // rows whose candidate list overflowed
     int ovf2_count;      // of those, rows that the centred screen left for the full-row kernel
     int open_count;      // of those, rows whose fp32 argmin is open
-    unsigned ticket;     // blocks of k_amb_fp64 that have written their centred rows
+    unsigned ticket;     // blocks of k_centre_rows that are done
     unsigned pad2;
-    unsigned long long npairs;  // candidate pairs written by the screening kernel
+    unsigned long long npairs;  // candidate pairs written by the selection
 };
 constexpr size_t kAssignCounterBytes = sizeof(DevCounters) - offsetof(DevCounters, amb_count);
 
@@ -59,6 +59,7 @@ struct Centred {
     float4* cstat;
     ColMax* colmax;
     float* qpad;
+    int32_t* list2;  // rows that the centred screen leaves open
     int ldq;
 };
 
@@ -161,18 +162,19 @@ cudaError_t launch_tc(const void* Xq, const void* Cq, int ldq, const TcArgs& a, 
                       cudaStream_t st);
 size_t tc_smem_bytes(int fmt, int d, int k);
 
-// candidate refinement: fp32 direct values of the pairs, then certified
-// argmin + min_dist per row; rows left open are appended to full_list
-// (cnt->ovf_count) for the full-row kernel; cen (Xq null: not used) receives
-// the centred bf16 copies of those rows and of the centres when there are any
-cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, int32_t* labels,
-                          double* min_dist, int32_t* full_list, int32_t* amb_list, const Centred& cen, int num_sms,
+// candidate refinement: the certified argmin of every row from its candidates
+// (list, list_n null: row r of a.cand / a.rowinfo is row r of X; else row
+// list[r] for r < *list_n); rows whose list overflowed are appended to
+// ovf_list / *ovf_n (amb_list, min_dist: scratch, min_dist of the winners in fp32)
+cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, const int32_t* list, const int* list_n,
+                          int32_t* labels, double* min_dist, int32_t* ovf_list, int* ovf_n, int32_t* amb_list, int num_sms,
                           cudaStream_t st, int* nlaunch);
-// the centred screen's candidates (a.cand, a.rowinfo; its row r is row
-// list[r] of X): fp32 direct values, certified, binary64 where still open;
-// rows with too many candidates go to list2 / cnt->ovf2_count
-cudaError_t launch_refine_centred(const float* X, const float* C, const TcArgs& a, const int32_t* list, int32_t* labels,
-                                  int32_t* list2, int num_sms, cudaStream_t st);
+// whether the refinement of n rows takes the flat pair list (a.pairs ..)
+bool refine_batched(int64_t n, int d);
+// centred bf16 copies of the listed rows and of the centres (d <= 256), when
+// any row is listed; ticket zeroed by the caller
+cudaError_t launch_centre_rows(const int32_t* list, const int* list_n, const float* X, const float* C, int k, int d,
+                               const Centred& cen, unsigned* ticket, int num_sms, cudaStream_t st);
 // the fallback's direct values for the flagged pairs of the distance matrix
 // (marked -1 in D): fb 0 binary64, 1 binary32, 2 the low format fmt (0
 // fp16, 1 bf16) itself; from the queue, or by a scan of D when it overflowed

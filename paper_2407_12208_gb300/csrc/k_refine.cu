@@ -4,19 +4,26 @@
 // The screening kernel leaves, per row, lists of candidates, from which only
 // the j with d^_j <= d^_min + 2 B_max can still be the nearest centre, where
 // |d^_j - d_j| <= B_ij is the bound behind the reliability test (so no other
-// centre can win).  Those become a flat list of (row, j) pairs, each row's pairs
-// contiguous.
-//  0. k_cand_select: the pairs from the screening kernel's per-row lists
-//     (rowinfo[TC_GROUPS i + g] = (count, overflow, W, d^min) per epilogue group);
-//  1. k_pair_eval: Eq. (dist-direct) in fp32 for every pair, 8 lanes per pair
-//     and 4 pairs per warp (no per-row bookkeeping on this path);
-//  2. k_certify, one thread per row: Theorem 4.1 puts each true value in
-//     [v (1 - g), v (1 + g)], g = gamma_{d+2}(2^-24); when exactly one
-//     interval can hold the minimum, that centre is the argmin and v is
-//     min_dist; otherwise (near-ties) the open candidates are evaluated in
-//     binary64 (products and sums rounded separately, coordinates in order:
-//     the oracle's own arithmetic), lowest index on ties.  Overflowed rows
-//     are listed for the full-row kernel, which evaluates every centre.
+// centre can win).  One candidate is the argmin.  Of several, Eq.
+// (dist-direct) in fp32 and Theorem 4.1, which puts each true value in
+// [v (1 - g), v (1 + g)], g = gamma_{d+2}(2^-24): when exactly one interval
+// can hold the minimum, that centre is the argmin; otherwise (near-ties) the
+// open candidates are evaluated in binary64 (products and sums rounded
+// separately, coordinates in order: the oracle's own arithmetic), lowest index
+// on ties.  Rows whose list overflowed are listed for the centred screen
+// (k_centre_rows prepares them) or the full-row kernel.
+//
+// Two forms with the same results:
+//  * k_refine: one launch, 32 rows per warp;
+//  * more than 64 coordinates and n d > 2^25: k_cand_select (a flat list of
+//    (row, j) pairs, each row's contiguous, from rowinfo[TC_GROUPS i + g] =
+//    (count, overflow, W, d^min) per epilogue group), k_pair_eval (8 lanes per
+//    pair, 4 pairs per warp, no per-row bookkeeping), k_certify (one thread
+//    per row) and k_amb_fp64.
+// Measured, k_refine against the four launches (GPU time, without the gaps
+// between launches): 1000 x 32 7.9 / 15.0 us, 1e4 x 16 7.4 / 16.3 us, 1e5 x 128
+// 19.8 / 28.7 us, 4e6 x 64 206 / 260 us; 150,001 x 256 92 / 72 us, 1e6 x 128
+// 293 / 219 us (x and two centres in registers leave three blocks per SM).
 
 #include <algorithm>
 
@@ -280,9 +287,8 @@ constexpr int AMB_B = 4;
 __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ amb_list, const int* __restrict__ amb_count,
                                                   const int2* __restrict__ rowpair, const int2* __restrict__ pairs,
                                                   const float* __restrict__ v32, const float* __restrict__ X,
-                                                  const float* __restrict__ C, int k, int d, float gamma32,
+                                                  const float* __restrict__ C, int d, float gamma32,
                                                   int32_t* __restrict__ labels, double* __restrict__ min_dist,
-                                                  const int32_t* __restrict__ full_list, const Centred cen,
                                                   DevCounters* cnt) {
     extern __shared__ double amb_sm[];  // per warp: AMB_B x d products
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -350,59 +356,38 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ev64 += __shfl_xor_sync(0xffffffffu, ev64, off);
     if (lane == 0 && ev64) atomicAdd(&cnt->fp64_evals, ev64);
-    // the centres and the rows whose list overflowed, centred, for the second
-    // screen; the last block to finish forms the column maxima and q_j
-    const int nf = cen.Xq ? cnt->ovf_count : 0;
-    if (nf == 0) return;
-    __shared__ __align__(16) float mu[256];
-    __shared__ bool last;
-    centre_mean(C, k, d, cen.ldq, mu);
-    const int sl = lane & 7;
-    const unsigned gmask = 0xFFu << (lane & ~7);
-    const bool vec = d % 4 == 0 && (((uintptr_t)X | (uintptr_t)C) & 15) == 0;
-    for (int64_t r = 4 * w0 + (lane >> 3); r < (int64_t)k + nf; r += 4 * nw) {
-        const bool isc = r < k;
-        const float* x = isc ? C + r * d : X + (int64_t)full_list[r - k] * d;
-        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(isc ? cen.Cq : cen.Xq) + (isc ? r : r - k) * cen.ldq;
-        float4* stat = isc ? cen.cstat + r : cen.xstat + (r - k);
-        if (vec) centred_row<true>(x, mu, d, cen.ldq, dst, stat, sl, gmask);
-        else centred_row<false>(x, mu, d, cen.ldq, dst, stat, sl, gmask);
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&cnt->ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    const int kpad = (k + 255) / 256 * 256;
-    for (int j = threadIdx.x; j < kpad; j += blockDim.x) cen.qpad[j] = j < k ? __ldcg(cen.cstat + j).x : INFINITY;
-    colmax_block(cen.cstat, k, cen.colmax);
 }
 
-// The centred screen's candidates, 32 listed rows per warp.  A lane per row
-// finds the candidates inside the window of the row's final d^ minimum; a row
-// with one is decided there.  Rows with a few take eight lanes each for their
-// fp32 direct values and Theorem 4.1's intervals; rows with many, and those
-// whose intervals overlap, the whole warp, which ends in binary64 in the
-// oracle's order.  Labels only: every caller refines the winner's distance
-// afterwards.  Few rows come here in most calls; when all do
-// it is bound by the latency of a row's chain of loads.
-// 1e6 x 128, k = 1024, all rows: 151 us (one row per warp at a time: 558 us).
-template <bool VEC>
-__global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__ rowinfo,
-                                                        const uint32_t* __restrict__ cand, int64_t n, int ebits,
-                                                        const int32_t* __restrict__ list, const float* __restrict__ X,
-                                                        const float* __restrict__ C, int d, float gamma32,
-                                                        int32_t* __restrict__ labels, int32_t* __restrict__ list2,
-                                                        DevCounters* cnt) {
+// 32 rows per warp and round.  A lane per row reads the entries of the row's
+// three lists (slot-major: 32 rows side by side) that lie inside the window of
+// the row's final d^ minimum, the smallest of the groups' minima.  Rows with 2
+// to RF_FEW candidates then take eight lanes each, four rows at a time: x in
+// registers (NV float4 per lane; NV = 0: any d and alignment, x read again per
+// candidate), two candidates' loads in flight.  Rows with more, and those
+// whose intervals overlap, take the whole warp, which ends in binary64
+// (products in parallel, one lane adds them in coordinate order).
+// Labels only: every caller refines the winner's distance afterwards, to
+// binary64 accuracy.
+// LIST: the rows are list[0 .. *list_n) of X (r indexes the lists), else all n.
+// Bound by the latency of a row's chain of loads (entries, then x and c).
+// Evaluating the warp's pairs from one flat list in shared memory instead,
+// eight at a time, was slower (1e6 x 128 listed rows 172 against 137 us,
+// 4e6 x 64 249 against 196 us: 48 registers for five blocks per SM spill).
+constexpr int RF_FEW = 12;
+template <int NV, bool LIST>
+__global__ void __launch_bounds__(256) k_refine(const int4* __restrict__ rowinfo, const uint32_t* __restrict__ cand,
+                                                int64_t n, int ebits, const int32_t* __restrict__ list,
+                                                const int* __restrict__ list_n, const float* __restrict__ X,
+                                                const float* __restrict__ C, int d, float gamma32,
+                                                int32_t* __restrict__ labels, int32_t* __restrict__ ovf_list,
+                                                int* __restrict__ ovf_n, DevCounters* cnt) {
     constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
     static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
     extern __shared__ double rc_sm[];  // per warp: d products
-    constexpr int JC = 12;
     __shared__ int js_sh[8][4 * NE];
     __shared__ float vs_sh[8][4 * NE];
-    __shared__ int jl_sh[8][JC * 32], ord_sh[8][32];
-    const int nrows = cnt->ovf_count;
+    __shared__ int jl_sh[8][RF_FEW * 32], ord_sh[8][32];
+    const int64_t nrows = LIST ? (int64_t)*list_n : n;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, sl = lane & 7;
     double* prod = rc_sm + (size_t)wib * d;
     int* js = js_sh[wib];
@@ -411,11 +396,13 @@ __global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__
     const uint32_t emask = (1u << ebits) - 1u;
     const float lscale = __uint_as_float((uint32_t)(127 + ebits - 23) << 23);  // 2^(ebits - 23)
     const float g = gamma32;
-    unsigned long long ev32 = 0, ev64 = 0, amb = 0;
-    for (int64_t r0 = ((int64_t)blockIdx.x * 8 + wib) * 32; r0 < nrows; r0 += (int64_t)gridDim.x * 256) {
+    const int d4 = d >> 2;
+    unsigned ev32 = 0, ev64 = 0, amb = 0, ovf = 0;
+    const int nwb = blockDim.x >> 5;
+    for (int64_t r0 = ((int64_t)blockIdx.x * nwb + wib) * 32; r0 < nrows; r0 += (int64_t)gridDim.x * nwb * 32) {
         const int64_t r = r0 + lane;
         const bool valid = r < nrows;
-        const int myrow = valid ? list[r] : 0;
+        const int myrow = valid ? (LIST ? list[r] : (int)r) : 0;
         bool full = false;
         int cnt_g[TC_GROUPS];
         float lim = INFINITY, W = 0.0f;
@@ -428,32 +415,39 @@ __global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__
             W = __int_as_float(ig.z);
         }
         lim += W;
-        // an overflowed list or an infinite window (which takes in the padding): every centre
+        // an overflowed list, or an infinite window (which takes in the columns'
+        // padding; nothing comparable counts as one): every centre
         full = valid && (full || !(lim < INFINITY));
-        if (full) list2[atomicAdd(&cnt->ovf2_count, 1)] = myrow;
+        if (full) {
+            ovf_list[atomicAdd(ovf_n, 1)] = myrow;
+            ovf++;
+        }
         int c = 0;
+        // four slots' loads in flight
+        auto take = [&](uint32_t e) {
+            if (cand_lower(e, emask, lscale) <= lim)
+                for (unsigned b = entry_mask(e); b; b &= b - 1, c++)
+                    if (c < RF_FEW) jl[c * 32 + lane] = 4 * entry_quad(e, emask) + __ffs(b) - 1;
+        };
 #pragma unroll
         for (int q = 0; q < TC_GROUPS; q++) {
-            const int ng = valid && !full ? cnt_g[q] : 0;
+            if (!valid || full) cnt_g[q] = 0;
             const uint32_t* cg = cand + (size_t)q * TC_LIST * n + r;
-            for (int s0 = 0; __any_sync(0xffffffffu, s0 < ng); s0 += 4) {
+            for (int s0 = 0; __any_sync(0xffffffffu, s0 < cnt_g[q]); s0 += 4) {
                 uint32_t e[4];
 #pragma unroll
-                for (int s = 0; s < 4; s++) e[s] = s0 + s < ng ? cg[(size_t)(s0 + s) * n] : 0u;
+                for (int s = 0; s < 4; s++) e[s] = s0 + s < cnt_g[q] ? cg[(size_t)(s0 + s) * n] : 0u;
 #pragma unroll
                 for (int s = 0; s < 4; s++)
-                    if (s0 + s < ng && cand_lower(e[s], emask, lscale) <= lim)
-                        for (unsigned bb = entry_mask(e[s]); bb; bb &= bb - 1, c++)
-                            if (c < JC) jl[c * 32 + lane] = 4 * entry_quad(e[s], emask) + __ffs(bb) - 1;
+                    if (s0 + s < cnt_g[q]) take(e[s]);
             }
         }
         if (c == 1) labels[myrow] = jl[lane];
-        // rows of two to JC candidates, eight lanes each
-        const bool few = c > 1 && c <= JC;
+        const bool few = c > 1 && c <= RF_FEW;
         const unsigned fm = __ballot_sync(0xffffffffu, few);
         if (few) ord[__popc(fm & ((1u << lane) - 1u))] = lane;
         __syncwarp();
-        unsigned slow = __ballot_sync(0xffffffffu, c > JC);
+        unsigned slow = __ballot_sync(0xffffffffu, c > RF_FEW);
         const int nfew = __popc(fm);
         for (int i0 = 0; i0 < nfew; i0 += 4) {
             const int i = i0 + (lane >> 3);
@@ -464,43 +458,67 @@ __global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__
             const float* x = X + row * d;
             float b1 = INFINITY, b2 = INFINITY;
             int j1 = 0;
-            for (int t = 0; t < most; t++) {
-                const bool on = t < cc;
-                const int j = jl[(on ? t : 0) * 32 + b];
-                const float* cj = C + (int64_t)j * d;
-                float acc = 0.0f;
-                if (VEC) {
-#pragma unroll 4
-                    for (int q = sl; q < (d >> 2); q += 8) {
-                        const float4 xv = reinterpret_cast<const float4*>(x)[q], cv = reinterpret_cast<const float4*>(cj)[q];
-                        const float u0 = xv.x - cv.x, u1 = xv.y - cv.y, u2 = xv.z - cv.z, u3 = xv.w - cv.w;
-                        acc = fmaf(u0, u0, acc);
-                        acc = fmaf(u1, u1, acc);
-                        acc = fmaf(u2, u2, acc);
-                        acc = fmaf(u3, u3, acc);
-                    }
-                } else {
-#pragma unroll 4
-                    for (int l = sl; l < d; l += 8) {
-                        const float u = x[l] - cj[l];
-                        acc = fmaf(u, u, acc);
-                    }
-                }
-#pragma unroll
-                for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            auto keep = [&](float v, int j, bool on) {
                 if (on) {
-                    if (acc < b1) { b2 = b1; b1 = acc; j1 = j; }
-                    else b2 = fminf(b2, acc);
+                    if (v < b1) { b2 = b1; b1 = v; j1 = j; }
+                    else b2 = fminf(b2, v);
+                }
+            };
+            if constexpr (NV > 0) {
+                constexpr int P = NV > 4 ? 1 : 2;  // candidates at once
+                float4 xv[NV];
+#pragma unroll
+                for (int u = 0; u < NV; u++)
+                    xv[u] = sl + 8 * u < d4 ? reinterpret_cast<const float4*>(x)[sl + 8 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int t = 0; t < most; t += P) {
+                    int j[P];
+                    float acc[P];
+                    float4 cv[P][NV];
+#pragma unroll
+                    for (int h = 0; h < P; h++) {
+                        j[h] = jl[(t + h < cc ? t + h : 0) * 32 + b];
+                        const float4* c4 = reinterpret_cast<const float4*>(C + (int64_t)j[h] * d);
+#pragma unroll
+                        for (int u = 0; u < NV; u++)
+                            cv[h][u] = sl + 8 * u < d4 ? c4[sl + 8 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int h = 0; h < P; h++) {
+                        acc[h] = 0.0f;
+#pragma unroll
+                        for (int u = 0; u < NV; u++) {
+                            const float u0 = xv[u].x - cv[h][u].x, u1 = xv[u].y - cv[h][u].y;
+                            const float u2 = xv[u].z - cv[h][u].z, u3 = xv[u].w - cv[h][u].w;
+                            acc[h] = fmaf(u0, u0, acc[h]);
+                            acc[h] = fmaf(u1, u1, acc[h]);
+                            acc[h] = fmaf(u2, u2, acc[h]);
+                            acc[h] = fmaf(u3, u3, acc[h]);
+                        }
+                    }
+#pragma unroll
+                    for (int off = 4; off > 0; off >>= 1)
+#pragma unroll
+                        for (int h = 0; h < P; h++) acc[h] += __shfl_xor_sync(0xffffffffu, acc[h], off);
+#pragma unroll
+                    for (int h = 0; h < P; h++) keep(acc[h], j[h], t + h < cc);
+                }
+            } else {
+                for (int t = 0; t < most; t++) {
+                    const int j = jl[(t < cc ? t : 0) * 32 + b];
+                    float acc = pair_value<0>(X, C, d, make_int2((int)row, j), sl);
+#pragma unroll
+                    for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                    keep(acc, j, t < cc);
                 }
             }
             const bool sure = b2 * (1.0f - g) > b1 * (1.0f + g);  // false where nothing is comparable
             if (sl == 0 && cc) {
-                ev32 += (unsigned long long)cc;
+                ev32 += cc;
                 if (sure) labels[row] = j1;
             }
             slow |= __reduce_or_sync(0xffffffffu, cc && !sure ? 1u << b : 0u);
         }
-        // the others (many candidates, near-ties), the warp on one row at a time
+        // the others, the warp on one row at a time
         for (unsigned todo = slow; todo; todo &= todo - 1) {
             const int b = __ffs(todo) - 1;
             const int64_t row = __shfl_sync(0xffffffffu, myrow, b);
@@ -533,33 +551,13 @@ __global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__
             const float* x = X + row * d;
             for (int t0 = 0; t0 < total; t0 += 4) {
                 const int t = t0 + (lane >> 3);
-                float acc = 0.0f;
-                if (t < total) {
-                    const float* cj = C + (int64_t)js[t] * d;
-                    if (VEC) {
-#pragma unroll 4
-                        for (int q = sl; q < (d >> 2); q += 8) {
-                            const float4 xv = reinterpret_cast<const float4*>(x)[q], cv = reinterpret_cast<const float4*>(cj)[q];
-                            const float u0 = xv.x - cv.x, u1 = xv.y - cv.y, u2 = xv.z - cv.z, u3 = xv.w - cv.w;
-                            acc = fmaf(u0, u0, acc);
-                            acc = fmaf(u1, u1, acc);
-                            acc = fmaf(u2, u2, acc);
-                            acc = fmaf(u3, u3, acc);
-                        }
-                    } else {
-#pragma unroll 4
-                        for (int l = sl; l < d; l += 8) {
-                            const float u = x[l] - cj[l];
-                            acc = fmaf(u, u, acc);
-                        }
-                    }
-                }
+                float acc = t < total ? pair_value<0>(X, C, d, make_int2((int)row, js[t]), sl) : 0.0f;
 #pragma unroll
                 for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
                 if (sl == 0 && t < total) vs[t] = acc;
             }
             __syncwarp();
-            if (lane == 0 && total > JC) ev32 += (unsigned long long)total;
+            if (lane == 0 && total > RF_FEW) ev32 += total;
             float up = INFINITY;
             for (int t = lane; t < total; t += 32) up = fminf(up, vs[t] * (1.0f + g));
 #pragma unroll
@@ -573,8 +571,7 @@ __global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__
             const unsigned who = __ballot_sync(0xffffffffu, open != 0);
             open = __reduce_add_sync(0xffffffffu, open);
             if (open == 1) {
-                const int src = __ffs(who) - 1;
-                if (lane == src) labels[row] = bj;
+                if (lane == __ffs(who) - 1) labels[row] = bj;
                 continue;
             }
             if (lane == 0) amb++;
@@ -591,39 +588,32 @@ __global__ void __launch_bounds__(256) k_refine_centred(const int4* __restrict__
                 __syncwarp();
                 if (lane == 0) {
                     double s = 0.0;
+#pragma unroll 8
                     for (int l = 0; l < d; l++) s = __dadd_rn(s, prod[l]);
                     ev64++;
                     if (s < best || (s == best && j < bj)) { best = s; bj = j; }
                 }
                 __syncwarp();
             }
-            if (lane == 0) labels[row] = bj != 0x7fffffff ? bj : js[0];
+            if (lane == 0) labels[row] = bj != 0x7fffffff ? bj : js[0];  // (not a number: a valid label all the same)
         }
         __syncwarp();
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) ev32 += __shfl_xor_sync(0xffffffffu, ev32, off);
+    ev32 = __reduce_add_sync(0xffffffffu, ev32);
+    ovf = __reduce_add_sync(0xffffffffu, ovf);
     if (lane == 0) {
-        if (ev32) atomicAdd(&cnt->fp32_evals, ev32);
-        if (ev64) atomicAdd(&cnt->fp64_evals, ev64);
-        if (amb) atomicAdd(&cnt->amb_rows, amb);
+        if (ev32) atomicAdd(&cnt->fp32_evals, (unsigned long long)ev32);
+        if (ev64) atomicAdd(&cnt->fp64_evals, (unsigned long long)ev64);
+        if (amb) atomicAdd(&cnt->amb_rows, (unsigned long long)amb);
+        if (ovf && !LIST) atomicAdd(&cnt->ovf_rows, (unsigned long long)ovf);
     }
 }
 
-cudaError_t launch_refine_centred(const float* X, const float* C, const TcArgs& a, const int32_t* list, int32_t* labels,
-                                  int32_t* list2, int num_sms, cudaStream_t st) {
-    const bool vec = a.d % 4 == 0 && ((uintptr_t)X % 16 == 0) && ((uintptr_t)C % 16 == 0);
-    auto fn = vec ? k_refine_centred<true> : k_refine_centred<false>;
-    const size_t sm = (size_t)8 * a.d * sizeof(double);
-    const unsigned blocks = (unsigned)std::min<int64_t>((a.n + 255) / 256, (int64_t)num_sms * 6);
-    fn<<<blocks, 256, sm, st>>>(a.rowinfo, a.cand, a.n, a.ebits, list, X, C, a.d, a.tp.gamma32, labels, list2,
-                                a.cnt);
-    return cudaGetLastError();
-}
+bool refine_batched(int64_t n, int d) { return d > 64 && n * d > (int64_t)1 << 25; }
 
-cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, int32_t* labels, double* min_dist,
-                          int32_t* full_list, int32_t* amb_list, const Centred& cen, int num_sms, cudaStream_t st,
-                          int* nlaunch) {
+static cudaError_t launch_refine_batched(const float* X, const float* C, const TcArgs& a, int32_t* labels,
+                                         double* min_dist, int32_t* full_list, int32_t* amb_list, int num_sms,
+                                         cudaStream_t st, int* nlaunch) {
     // persistent grids: the resident blocks only
     int sel_per_sm = 1, cert_per_sm = 1;
     cudaError_t e0 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sel_per_sm, k_cand_select, 256, 0);
@@ -661,10 +651,84 @@ cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, int32
     const size_t amb_smem = (size_t)8 * AMB_B * a.d * sizeof(double);  // 8 warps per block
     e = allow_max_smem(k_amb_fp64);
     if (e != cudaSuccess) return e;
-    // (three blocks per SM quantise overflowed rows faster than one: they are bound by loads)
-    k_amb_fp64<<<(unsigned)num_sms * (cen.Xq ? 3 : 1), 256, amb_smem, st>>>(
-        amb_list, &a.cnt->amb_count, a.rowpair, a.pairs, a.v32, X, C, a.k, a.d, a.tp.gamma32, labels, min_dist, full_list,
-        cen, a.cnt);
+    k_amb_fp64<<<(unsigned)num_sms, 256, amb_smem, st>>>(amb_list, &a.cnt->amb_count, a.rowpair, a.pairs, a.v32, X, C,
+                                                          a.d, a.tp.gamma32, labels, min_dist, a.cnt);
+    return cudaGetLastError();
+}
+
+template <int NV, bool LIST>
+static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs& a, const int32_t* list,
+                                    const int* list_n, int32_t* labels, int32_t* ovf_list, int* ovf_n, int num_sms,
+                                    cudaStream_t st) {
+    auto fn = k_refine<NV, LIST>;
+    // few rows: one warp's 32 per block, so that they spread over the SMs
+    const int threads = a.n <= (int64_t)num_sms * 256 ? 32 : 256;
+    const size_t sm = (size_t)(threads / 32) * a.d * sizeof(double);
+    cudaError_t e = allow_max_smem(fn);
+    if (e != cudaSuccess) return e;
+    int per_sm = 1;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, sm);
+    if (e != cudaSuccess) return e;
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + threads - 1) / threads, (int64_t)num_sms * std::max(per_sm, 1)));
+    fn<<<(unsigned)blocks, threads, sm, st>>>(a.rowinfo, a.cand, a.n, a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,
+                                              labels, ovf_list, ovf_n, a.cnt);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, const int32_t* list, const int* list_n,
+                          int32_t* labels, double* min_dist, int32_t* ovf_list, int* ovf_n, int32_t* amb_list, int num_sms,
+                          cudaStream_t st, int* nlaunch) {
+    if (!list && refine_batched(a.n, a.d) && a.pairs)
+        return launch_refine_batched(X, C, a, labels, min_dist, ovf_list, amb_list, num_sms, st, nlaunch);
+    *nlaunch = 1;
+    const bool vec = a.d % 4 == 0 && a.d <= 256 && ((uintptr_t)X % 16 == 0) && ((uintptr_t)C % 16 == 0);
+    const int nv = !vec ? 0 : (a.d <= 32 ? 1 : (a.d <= 64 ? 2 : (a.d <= 128 ? 4 : 8)));
+#define KM_RF(NV)                                                                                            \
+    if (nv == NV)                                                                                            \
+        return list ? launch_refine_nv<NV, true>(X, C, a, list, list_n, labels, ovf_list, ovf_n, num_sms, st) \
+                    : launch_refine_nv<NV, false>(X, C, a, list, list_n, labels, ovf_list, ovf_n, num_sms, st);
+    KM_RF(0) KM_RF(1) KM_RF(2) KM_RF(4) KM_RF(8)
+#undef KM_RF
+    return cudaErrorInvalidValue;
+}
+
+// The centres and the listed rows, centred, for the second screen (eight lanes
+// per row); the last block to finish forms the column maxima and q_j.  An
+// empty list, the usual case, leaves at once.
+__global__ void __launch_bounds__(256) k_centre_rows(const int32_t* __restrict__ list, const int* __restrict__ list_n,
+                                                     const float* __restrict__ X, const float* __restrict__ C, int k,
+                                                     int d, const Centred cen, unsigned* ticket) {
+    const int nf = *list_n;
+    if (nf == 0) return;
+    __shared__ __align__(16) float mu[256];
+    __shared__ bool last;
+    centre_mean(C, k, d, cen.ldq, mu);
+    const int lane = threadIdx.x & 31, sl = lane & 7;
+    const unsigned gmask = 0xFFu << (lane & ~7);
+    const bool vec = d % 4 == 0 && (((uintptr_t)X | (uintptr_t)C) & 15) == 0;
+    const int64_t ng = (int64_t)gridDim.x * (blockDim.x / 8);
+    for (int64_t r = (int64_t)blockIdx.x * (blockDim.x / 8) + threadIdx.x / 8; r < (int64_t)k + nf; r += ng) {
+        const bool isc = r < k;
+        const float* x = isc ? C + r * d : X + (int64_t)list[r - k] * d;
+        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(isc ? cen.Cq : cen.Xq) + (isc ? r : r - k) * cen.ldq;
+        float4* stat = isc ? cen.cstat + r : cen.xstat + (r - k);
+        if (vec) centred_row<true>(x, mu, d, cen.ldq, dst, stat, sl, gmask);
+        else centred_row<false>(x, mu, d, cen.ldq, dst, stat, sl, gmask);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int kpad = (k + 255) / 256 * 256;
+    for (int j = threadIdx.x; j < kpad; j += blockDim.x) cen.qpad[j] = j < k ? __ldcg(cen.cstat + j).x : INFINITY;
+    colmax_block(cen.cstat, k, cen.colmax);
+}
+
+cudaError_t launch_centre_rows(const int32_t* list, const int* list_n, const float* X, const float* C, int k, int d,
+                               const Centred& cen, unsigned* ticket, int num_sms, cudaStream_t st) {
+    k_centre_rows<<<(unsigned)num_sms * 4, 256, 0, st>>>(list, list_n, X, C, k, d, cen, ticket);
     return cudaGetLastError();
 }
 

@@ -109,3 +109,20 @@ def test_smallest_accepted_workspace(ctx):
     small = ctx.assign(Xd, Cd, p, ws=ws[:hi])
     assert hi < ws.numel() - 17000 * 64 * 2
     assert torch.equal(full[0], small[0]) and torch.equal(full[1], small[1]) and full[2] == small[2]
+
+
+# the two forms of the refinement (n d > 2^25 and d > 64: the flat pair list) at ragged shapes,
+# with near-ties, single candidates and rows of more than 12 candidates
+@pytest.mark.parametrize("low", ["bf16", "fp16"])
+@pytest.mark.parametrize("n,d,k,scale", [(31, 24, 9, 1.0), (33, 100, 33, 1.0), (5003, 30, 70, 1.0), (4001, 130, 257, 0.02),
+                                         (9000, 8, 64, 0.01), (525000, 65, 40, 1.0), (263000, 128, 66, 0.02)])
+def test_refine_forms(ctx, low, n, d, k, scale):
+    X, C = workloads.uniform_pairs(n, d, k, seed=n)
+    X, C = 1 + np.float32(scale) * X, 1 + np.float32(scale) * C  # (scale << 1: wide bounds, many candidates)
+    C[k // 2 :] = C[: k - k // 2]  # near-ties of identical centres
+    lab, md, _ = _assign(ctx, X, C, low)
+    _, first, inverse = np.unique(C, axis=0, return_index=True, return_inverse=True)
+    assert np.array_equal(first[inverse.ravel()][lab], lab)  # the lowest index of identical centres
+    m = min(n, 20000)
+    check_assign(lab[:m], md[:m], X[:m], C, oracle, RTOL_MD)
+    check_assign(lab[-200:], md[-200:], X[-200:], C, oracle, RTOL_MD)
