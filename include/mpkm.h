@@ -410,9 +410,8 @@ km_status km_get_launch_count(const km_ctx* ctx, uint64_t* launches);
  * device memory is all held by a caching pool or by another framework,
  * where a cudaMalloc would fail, and latency-bound loops
  * that must not call cudaMalloc/cudaFree (cudaFree can synchronise the whole
- * device).  It takes no workspace.  Its scratch (the device counters and the
- * list of rows left open, one int32 per row) is a file-scope device array of
- * the library sized for KM_STATIC_MAX_ROWS rows: 4 MiB + 256 B per device.
+ * device).  It takes no workspace.  Its scratch (the device counters) is a
+ * file-scope device array of the library, 256 B per device.
  *  - n > KM_STATIC_MAX_ROWS returns KM_ENOMEM before any launch; the other
  *    argument errors are km_assign's (d <= 256 as on every direct path).
  *  - labels (n int32) and min_dist (n doubles) are required device outputs.

@@ -383,12 +383,15 @@ TestParams make_tp(const km_params* p, int d) {
 
 bool aligned256(const void* p) { return ((uintptr_t)p & 255) == 0; }
 
-// The centres in the low format with their statistics (per-row power-of-two
-// scales for E4M3), the column maxima of the bound, q_j and the scales padded
-// to the tile width.
-km_status prepare_centres(km_ctx* ctx, const float* C, int k, int d, int fmt, const AssignWs& w, cudaStream_t st) {
-    KL(1, launch_quantize(C, k, d, fmt, ldq_of(fmt, d), w.Cq, w.cstat, w.cscale, st));
-    KL(1, launch_colmax(w.cstat, k, fmt == 2 ? w.cscale : nullptr, w.colmax, w.qpad, w.spad, kpad_of(k), st));
+// X (null: prepared already) and the centres in the low format with their
+// statistics (per-row power-of-two scales for E4M3), the column maxima of the
+// bound, q_j and the scales padded to the tile width.
+km_status prepare(km_ctx* ctx, const float* X, int64_t n, const float* C, int k, int d, int fmt, const AssignWs& w,
+                  unsigned* x_absmax, cudaStream_t st) {
+    int nl = 0;
+    CK(launch_prepare(X, n, w.Xq, w.xstat, w.xscale, x_absmax, C, k, w.Cq, w.cstat, w.cscale, w.colmax, w.qpad, w.spad,
+                      kpad_of(k), &w.cnt->prep_ticket, d, fmt, ldq_of(fmt, d), st, &nl));
+    ctx->launches += (uint64_t)nl;
     return KM_OK;
 }
 
@@ -421,13 +424,8 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
         const bool acc64 = p->low == KM_FP64_DIRECT;
         {
             PhaseScope ps(ctx, KM_PHASE_DIRECT, st);
-            KL(1, launch_direct_assign(acc64, X, n, C, k, d, nullptr, nullptr, labels, min_dist, w.amb_list,
-                                       &w.cnt->amb_count, w.cnt, tp.gamma32, ctx->num_sms, st, x_absmax));
-        }
-        if (!acc64) {
-            PhaseScope ps(ctx, KM_PHASE_FULLROW, st);
-            KL(1, launch_rows_full(false, X, C, k, d, w.amb_list, &w.cnt->amb_count, labels, min_dist, w.cnt,
-                                   tp.gamma32, ctx->num_sms, st));
+            KL(1, launch_direct_assign(acc64, X, n, C, k, d, nullptr, nullptr, labels, min_dist, w.cnt, tp.gamma32,
+                                       ctx->num_sms, st, x_absmax));
         }
         return KM_OK;
     }
@@ -436,8 +434,11 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
     const int esz = fmt == 2 ? 1 : 2;
     {
         PhaseScope ps(ctx, KM_PHASE_QUANTISE, st);
-        if (!x_prepared) KL(1, launch_quantize(X, n, d, fmt, ldq, w.Xq, w.xstat, w.xscale, st, x_absmax));
-        if (!c_prepared && (s = prepare_centres(ctx, C, k, d, fmt, w, st)) != KM_OK) return s;
+        if (!c_prepared) {
+            if ((s = prepare(ctx, x_prepared ? nullptr : X, n, C, k, d, fmt, w, x_absmax, st)) != KM_OK) return s;
+        } else if (!x_prepared) {
+            KL(1, launch_quantize(X, n, d, fmt, ldq, w.Xq, w.xstat, w.xscale, st, x_absmax));
+        }
     }
     TcArgs a{};
     a.n = n; a.k = k; a.d = d; a.fmt = fmt;
@@ -490,12 +491,10 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
             list_n = &w.cnt->ovf2_count;
         }
         if (d <= 256) {  // the direct kernel's row tile fits in shared memory
-            KL(1, launch_direct_assign(false, X, n, C, k, d, list, list_n, labels, min_dist, w.amb_list,
-                                       &w.cnt->open_count, w.cnt, tp.gamma32, ctx->num_sms, st));
-            KL(1, launch_rows_full(false, X, C, k, d, w.amb_list, &w.cnt->open_count, labels, min_dist, w.cnt,
-                                   tp.gamma32, ctx->num_sms, st));
+            KL(1, launch_direct_assign(false, X, n, C, k, d, list, list_n, labels, min_dist, w.cnt, tp.gamma32,
+                                       ctx->num_sms, st));
         } else {  // one block per row
-            KL(1, launch_rows_full(true, X, C, k, d, list, list_n, labels, min_dist, w.cnt, tp.gamma32, ctx->num_sms, st));
+            KL(1, launch_rows_full(X, C, k, d, list, list_n, labels, min_dist, w.cnt, tp.gamma32, ctx->num_sms, st));
         }
     }
     (void)esz;
@@ -644,7 +643,8 @@ km_status km_choose_low(km_ctx* ctx, const float* X, int64_t n, const float* C, 
         return fail(ctx, KM_EUNSUPPORTED, "no tensor-core path for d=%d, k=%d", d, k);
     constexpr int kSample = 2048;
     Carve cv{(char*)ws};
-    unsigned long long* acc = cv.take<unsigned long long>(4);
+    unsigned long long* acc = cv.take<unsigned long long>(5);
+    unsigned* ticket = reinterpret_cast<unsigned*>(acc + 4);
     ColMax* colmax = cv.take<ColMax>(1);
     void* Cq = cv.take<char>((size_t)k * ldq_of(1, d) * 2);
     float4* cstat = cv.take<float4>((size_t)k);
@@ -654,7 +654,7 @@ km_status km_choose_low(km_ctx* ctx, const float* X, int64_t n, const float* C, 
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
-    CK(cudaMemsetAsync(acc, 0, 4 * sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(acc, 0, 5 * sizeof(unsigned long long), st));
     const int fmts[2] = {1, 2};  // bf16, E4M3
     for (int f = 0; f < 2; f++) {
         const int fmt = fmts[f];
@@ -662,8 +662,10 @@ km_status km_choose_low(km_ctx* ctx, const float* X, int64_t n, const float* C, 
         km_params q;
         km_default_params(&q);
         q.low = fmt == 2 ? KM_E4M3 : KM_BF16;
-        KL(1, launch_quantize(C, k, d, fmt, ldq_of(fmt, d), Cq, cstat, cscale, st));
-        KL(1, launch_colmax(cstat, k, fmt == 2 ? cscale : nullptr, colmax, qpad, spad, kpad_of(k), st));
+        int nl = 0;
+        CK(launch_prepare(nullptr, 0, nullptr, nullptr, nullptr, nullptr, C, k, Cq, cstat, cscale, colmax, qpad, spad,
+                          kpad_of(k), ticket, d, fmt, ldq_of(fmt, d), st, &nl));
+        ctx->launches += (uint64_t)nl;
         KL(1, launch_predict_candidates(X, n, d, C, k, fmt, colmax, make_tp(&q, d), kSample, acc + 2 * f,
                                         ctx->num_sms, st));
     }
@@ -711,7 +713,7 @@ km_status km_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int 
     s = run_assign(ctx, X, n, C, k, d, p, labels, md, w, cen, false, st);
     if (s != KM_OK) return s;
     if ((s = refine_winners(ctx, X, n, d, C, p, labels, md, st)) != KM_OK) return s;
-    KL(2, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, st));
+    KL(1, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, &w.cnt->sum_ticket, st));
     ctx->last_cnt = w.cnt;
     ctx->last_sse = w.sse;
     ctx->last_stream = st;
@@ -844,8 +846,7 @@ km_status km_distances(km_ctx* ctx, const float* X, int64_t n, const float* C, i
         const int fmt = fmt_of(p->low);
         const int ldq = ldq_of(fmt, d);
         const int esz = fmt == 2 ? 1 : 2;
-        KL(1, launch_quantize(X, n, d, fmt, ldq, w.Xq, w.xstat, w.xscale, st));
-        if ((s = prepare_centres(ctx, C, k, d, fmt, w, st)) != KM_OK) return s;
+        if ((s = prepare(ctx, X, n, C, k, d, fmt, w, nullptr, st)) != KM_OK) return s;
         TcArgs a{};
         a.n = n; a.k = k; a.d = d; a.fmt = fmt;
         a.kchunks = (ldq * esz + 127) / 128;
@@ -1020,7 +1021,7 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
         PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
         s = accumulate(ctx, X, n, d, labels, k, u, C_old, p->low == KM_FP64_DIRECT ? nullptr : md, st);
         if (s != KM_OK) return s;
-        KL(2, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, st));
+        KL(1, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, &w.cnt->sum_ticket, st));
         if ((s = finalize(ctx, u, n, k, d, C_old, p, X, md, C_new, counts, w.cnt, st, shift_host != nullptr)) != KM_OK)
             return s;
     }
@@ -1145,7 +1146,7 @@ km_status km_lloyd_step_host(km_ctx* ctx, const float* X_host, int64_t n, int d,
             PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
             s = accumulate(ctx, h.X, n, d, h.labels, k, u, h.C, nullptr, st);
             if (s != KM_OK) return s;
-            KL(2, launch_sum_f64(h.min_dist, n, w.partials, kSumParts, w.sse, st));
+            KL(1, launch_sum_f64(h.min_dist, n, w.partials, kSumParts, w.sse, &w.cnt->sum_ticket, st));
             if ((s = finalize(ctx, u, n, k, d, h.C, p, h.X, h.min_dist, h.C_new, h.counts, w.cnt, st,
                               shift_host != nullptr)) != KM_OK)
                 return s;
@@ -1249,7 +1250,7 @@ static km_status lloyd_iteration(km_ctx* ctx, const float* X, int64_t n, int d, 
     PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
     s = accumulate(ctx, X, n, d, labels, k, L.u, cur, p->low == KM_FP64_DIRECT ? nullptr : L.min_dist, st);
     if (s != KM_OK) return s;
-    KL(2, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, graph ? L.sse_slot : sse_out, st));
+    KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, graph ? L.sse_slot : sse_out, &L.a.cnt->sum_ticket, st));
     if ((s = finalize(ctx, L.u, n, k, d, cur, p, X, L.min_dist, nxt, L.counts, L.a.cnt, st, true)) != KM_OK) return s;
     if (graph) {
         k_record_iteration<<<1, 1, 0, st>>>(L.sse_slot, L.a.cnt, L.sse_hist, L.flag_hist, L.hist_len, cap);
@@ -1389,9 +1390,9 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
     s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, true, st);
     if (s != KM_OK) return s;
     if ((s = refine_winners(ctx, X, n, d, cur, p, labels, L.min_dist, st)) != KM_OK) return s;
-    KL(2, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.sse_hist + t, st));
+    KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.sse_hist + t, &L.a.cnt->sum_ticket, st));
     CK(cudaMemcpyAsync(L.flag_hist + t, &L.a.cnt->flagged, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
-    KL(2, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.a.sse, st));
+    KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.a.sse, &L.a.cnt->sum_ticket, st));
     CK(cudaMemcpyAsync(C_out, cur, sizeof(float) * (size_t)k * d, cudaMemcpyDeviceToDevice, st));
     ctx->last_cnt = L.a.cnt;
     ctx->last_sse = L.a.sse;
@@ -1582,8 +1583,7 @@ km_status km_internal_run_job(km_ctx_view* v, const float* X, int64_t n, int d, 
 // For callers that cannot allocate device memory at assignment time (device
 // memory held by another pool, where cudaMalloc fails; loops that must not
 // pay for cudaMalloc/cudaFree, which can synchronise the device).  The
-// scratch is a file-scope device array: the counters in the first 256 bytes,
-// then the list of rows whose fp32 argmin stayed open.  There is one copy per
+// scratch is a file-scope device array of the counters.  There is one copy per
 // device, so calls that overlap in time on one device race on it.
 namespace {
 constexpr size_t kStaticCntBytes = 256;
@@ -1593,7 +1593,7 @@ std::mutex g_static_mu;
 void* g_static_addr[kStaticMaxDevices];  // resolved scratch address per device, null until first use
 }  // namespace
 
-static __device__ __align__(256) unsigned char g_static_scratch[kStaticCntBytes + (size_t)KM_STATIC_MAX_ROWS * sizeof(int32_t)];
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticCntBytes];
 
 namespace {
 // Failure-path check: one warp waits on an mbarrier that no thread arrives at.
@@ -1684,16 +1684,10 @@ extern "C" km_status km_assign_static(km_ctx* ctx, const float* X, int64_t n, co
         base = g_static_addr[ctx->device];
     }
     DevCounters* cnt = reinterpret_cast<DevCounters*>(base);
-    int32_t* amb_list = reinterpret_cast<int32_t*>(static_cast<char*>(base) + kStaticCntBytes);
     cudaStream_t st = (cudaStream_t)stream;
     const TestParams tp = make_tp(&p, d);
-    // the counters (amb_count above all) must start at zero; the row list is
-    // written before it is read
     CK(cudaMemsetAsync(cnt, 0, sizeof(DevCounters), st));
-    KL(1, launch_direct_assign(false, X, n, C, k, d, nullptr, nullptr, labels, min_dist, amb_list, &cnt->amb_count, cnt,
-                               tp.gamma32, ctx->num_sms, st));
-    KL(1, launch_rows_full(false, X, C, k, d, amb_list, &cnt->amb_count, labels, min_dist, cnt, tp.gamma32,
-                           ctx->num_sms, st));
+    KL(1, launch_direct_assign(false, X, n, C, k, d, nullptr, nullptr, labels, min_dist, cnt, tp.gamma32, ctx->num_sms, st));
     // the winners' distances to binary64 accuracy, as km_assign (no scratch)
     KL(1, launch_winner_dist(X, n, d, C, labels, min_dist, ctx->num_sms, st));
     return KM_OK;

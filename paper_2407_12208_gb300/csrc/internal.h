@@ -25,14 +25,14 @@ struct DevCounters {
     unsigned long long amb_rows;
     unsigned long long ovf_rows;
     unsigned status;     // KM_DEVERR_* bits
+    unsigned sum_ticket;   // blocks of the deterministic sum that are done
+    unsigned prep_ticket;  // blocks of the centre preparation that are done
     unsigned pad;
     // zeroed before every assignment (from amb_count on)
-    int amb_count;       // rows whose fp32 argmin is open (refinement; the fp32 direct path)
+    int amb_count;       // rows whose fp32 argmin the refinement left open
     int ovf_count;       // rows whose candidate list overflowed
     int ovf2_count;      // of those, rows that the centred screen left for the full-row kernel
-    int open_count;      // of those, rows whose fp32 argmin is open
     unsigned ticket;     // blocks of k_centre_rows that are done
-    unsigned pad2;
     unsigned long long npairs;  // candidate pairs written by the selection
 };
 constexpr size_t kAssignCounterBytes = sizeof(DevCounters) - offsetof(DevCounters, amb_count);
@@ -97,10 +97,14 @@ inline cudaError_t allow_max_smem(F* func) {
 // (the caller zeroes it first).
 cudaError_t launch_quantize(const float* A, int64_t m, int d, int fmt, int ldq, void* Aq, float4* stat,
                             float* rscale, cudaStream_t st, unsigned* absmax_out = nullptr);
-// column maxima of the centre statistics, q_j padded with +inf to kpad
-// entries and the centres' scales (cscale, nullable: all 1) padded with 1
-cudaError_t launch_colmax(const float4* cstat, int k, const float* cscale, ColMax* out, float* qpad, float* spad,
-                          int kpad, cudaStream_t st);
+// the points (X null: they are prepared already) and the centres quantised in
+// one launch where their rows take the same form (else two: *nlaunch), and the
+// centres' column data: maxima of the bound terms, q_j padded with +inf to
+// kpad entries, the E4M3 scales padded with 1; ticket: 0 before and after
+cudaError_t launch_prepare(const float* X, int64_t n, void* Xq, float4* xstat, float* xscale, unsigned* absmax_out,
+                           const float* C, int k, void* Cq, float4* cstat, float* cscale, ColMax* colmax, float* qpad,
+                           float* spad, int kpad, unsigned* ticket, int d, int fmt, int ldq, cudaStream_t st,
+                           int* nlaunch);
 
 // candidates per sampled row under the format's certification window (the
 // choice of the low format): acc[0] += candidates, acc[1] += rows above one
@@ -110,18 +114,18 @@ cudaError_t launch_predict_candidates(const float* X, int64_t n, int d, const fl
                                       unsigned long long* acc, int num_sms, cudaStream_t st);
 
 // direct-formula assignment.  acc64: binary64 accumulation (the plain FP64
-// path, all n rows) else fp32 with certification; rows = all n, or the device
-// list row_list[0 .. *row_count).  Uncertified fp32 rows are appended to
-// open_list / *open_count.
+// path, all n rows) else fp32 with certification, rows left open decided in
+// binary64 (counted in cnt->amb_rows); rows = all n, or the device list
+// row_list[0 .. *row_count).
 // absmax_out (nullable, zeroed by the caller): max |x| over the rows read.
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
-                                 double* min_dist, int32_t* open_list, int* open_count, DevCounters* cnt, float gamma32,
+                                 double* min_dist, DevCounters* cnt, float gamma32,
                                  int num_sms, cudaStream_t st, unsigned* absmax_out = nullptr);
 // exact argmin of the rows of a device list, one block per row: fp32 direct
-// values of all centres, certified, binary64 where still open.  count_open:
-// those rows are added to cnt->amb_rows.
-cudaError_t launch_rows_full(bool count_open, const float* X, const float* C, int k, int d, const int32_t* row_list,
+// values of all centres, certified, binary64 where still open (counted in
+// cnt->amb_rows).
+cudaError_t launch_rows_full(const float* X, const float* C, int k, int d, const int32_t* row_list,
                              const int* row_count, int32_t* labels, double* min_dist, DevCounters* cnt,
                              float gamma32, int num_sms, cudaStream_t st);
 
@@ -224,8 +228,8 @@ cudaError_t launch_finalize(const long long* sums, const long long* counts, cons
 // rows_out / vals_out; esel: empty_select_bytes(e) bytes
 cudaError_t launch_farthest_rows(const double* min_dist, int64_t n, int e, long long* rows_out, double* vals_out,
                                  void* esel, unsigned* status, int num_sms, cudaStream_t st);
-// deterministic sum of n doubles (fixed two-level order)
-cudaError_t launch_sum_f64(const double* v, int64_t n, double* partials, int nparts, double* out,
+// deterministic sum of n doubles (fixed two-level order); ticket: 0 before and after
+cudaError_t launch_sum_f64(const double* v, int64_t n, double* partials, int nparts, double* out, unsigned* ticket,
                            cudaStream_t st);
 
 }  // namespace km

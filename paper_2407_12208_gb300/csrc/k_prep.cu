@@ -64,12 +64,13 @@ KM_DEV void block_absmax(float v, unsigned* out) {
     }
 }
 
-__global__ void k_quantize(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
-                           float4* __restrict__ stat, float* __restrict__ rscale, unsigned* __restrict__ absmax_out) {
-    float amx = 0.0f;  // largest |a| of this thread's elements (absmax_out)
+// Any d and alignment: one warp per row.
+KM_DEV void quantize_warp(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
+                          float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
+                          unsigned nblocks) {
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t warp = ((int64_t)block * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)nblocks * blockDim.x) >> 5;
     for (int64_t i = warp; i < m; i += nw) {
         const float* a = A + i * d;
         float s = 1.0f;
@@ -128,7 +129,6 @@ __global__ void k_quantize(const float* __restrict__ A, int64_t m, int d, int fm
             if (rscale) rscale[i] = s;
         }
     }
-    if (absmax_out) block_absmax(amx, absmax_out);
 }
 
 
@@ -136,13 +136,13 @@ __global__ void k_quantize(const float* __restrict__ A, int64_t m, int d, int fm
 // warp, so the row reductions take 3 shuffle levels and serve 4 rows at once.
 // Lane l of a row's 8 holds float4 l, l + 8, ... (NV of them).
 template <int NV>
-__global__ void k_quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
-                              float4* __restrict__ stat, float* __restrict__ rscale, unsigned* __restrict__ absmax_out) {
-    float amx = 0.0f;  // largest |a| of this thread's elements (absmax_out)
+KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
+                        float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
+                        unsigned nblocks) {
     const int lane = threadIdx.x & 31, sl = lane & 7;
     const unsigned gmask = 0xFFu << (lane & ~7);
-    const int64_t gid = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4 + (lane >> 3);
-    const int64_t ngroups = (((int64_t)gridDim.x * blockDim.x) >> 5) * 4;
+    const int64_t gid = (((int64_t)block * blockDim.x + threadIdx.x) >> 5) * 4 + (lane >> 3);
+    const int64_t ngroups = (((int64_t)nblocks * blockDim.x) >> 5) * 4;
     const int d4 = d >> 2, ldq4 = ldq >> 2;
     // R rows per group and round, all their loads issued first: at least four
     // 16-byte loads in flight per lane
@@ -276,18 +276,17 @@ __global__ void k_quantize_g8(const float* __restrict__ A, int64_t m, int d, int
         }
         }
     }
-    if (absmax_out) block_absmax(amx, absmax_out);
 }
 
 // Vector path (d % 4 == 0, d <= 512): one warp per row, each lane holds up to
 // four float4 of the row in registers (coalesced 16-byte loads).
 template <int NV>
-__global__ void k_quantize_vec(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
-                               float4* __restrict__ stat, float* __restrict__ rscale, unsigned* __restrict__ absmax_out) {
-    float amx = 0.0f;  // largest |a| of this thread's elements (absmax_out)
+KM_DEV void quantize_vec(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
+                         float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
+                         unsigned nblocks) {
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t warp = ((int64_t)block * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)nblocks * blockDim.x) >> 5;
     const int d4 = d >> 2, ldq4 = ldq >> 2;
     for (int64_t i = warp; i < m; i += nw) {
         const float4* a4 = reinterpret_cast<const float4*>(A + i * d);
@@ -368,52 +367,187 @@ __global__ void k_quantize_vec(const float* __restrict__ A, int64_t m, int d, in
             if (rscale) rscale[i] = s;
         }
     }
-    if (absmax_out) block_absmax(amx, absmax_out);
 }
 
-// q_j for the screening kernel, +inf on the padding so padded columns never
-// win; the centres' E4M3 scales (cscale, nullable: 1), 1 on the padding; the
-// column maxima.
-__global__ void __launch_bounds__(1024) k_colmax(const float4* __restrict__ cstat, int k,
-                                                 const float* __restrict__ cscale, ColMax* out,
-                                                 float* __restrict__ qpad, float* __restrict__ spad, int kpad) {
-    for (int j = threadIdx.x; j < kpad; j += blockDim.x) {
-        qpad[j] = (j < k) ? cstat[j].x : INFINITY;
-        spad[j] = (j < k && cscale) ? cscale[j] : 1.0f;
+// Any alignment, short rows (d <= 64): eight lanes per row, each standing for
+// four lanes of quantize_warp (lane l = sl + 8 i of 32: the same sums in the
+// same tree, so the same statistics bit for bit), four rows per warp.  A warp
+// per row spent its time on reductions of mostly idle lanes: 1e5 x 10 took 27 us
+// (now 16 with the centres in the same launch).
+KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
+                           float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
+                           unsigned nblocks) {
+    const int lane = threadIdx.x & 31, sl = lane & 7;
+    const unsigned gmask = 0xFFu << (lane & ~7);
+    const int64_t ng = (int64_t)nblocks * (blockDim.x / 8);
+    for (int64_t i = (int64_t)block * (blockDim.x / 8) + threadIdx.x / 8; i < m; i += ng) {
+        const float* a = A + i * d;
+        float v[8];  // coordinate sl + 8 t
+#pragma unroll
+        for (int t = 0; t < 8; t++) {
+            v[t] = sl + 8 * t < d ? a[sl + 8 * t] : 0.0f;
+            amx = fmaxf(amx, fabsf(v[t]));
+        }
+        float s = 1.0f;
+        if (fmt == 2) {
+            float amax = 0.0f;
+#pragma unroll
+            for (int t = 0; t < 8; t++) amax = fmaxf(amax, fabsf(v[t]));
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(gmask, amax, off));
+            s = e4m3_row_scale(amax);
+        }
+        const float inv = 1.0f / s;  // exact: s is a power of two
+        float ph[4], pl[4], q2[4], r2[4];
+        bool nz = false;
+#pragma unroll
+        for (int l = 0; l < 4; l++) ph[l] = pl[l] = q2[l] = r2[l] = 0.0f;
+#pragma unroll
+        for (int t = 0; t < 8; t++) {
+            const int c = sl + 8 * t, l = t & 3;
+            if (c < ldq) {
+                const float qv = quant_val(v[t] * inv, fmt);
+                nz |= v[t] != 0.0f;
+                if (c < d) {
+                    df_add_sq(v[t], ph[l], pl[l]);
+                    const float qs = qv * s;
+                    q2[l] = fmaf(qs, qs, q2[l]);
+                    const float rr = qs - v[t];
+                    r2[l] = fmaf(rr, rr, r2[l]);
+                }
+                if (fmt == 0) reinterpret_cast<__half*>(Aq)[i * ldq + c] = __float2half_rn(qv);
+                else if (fmt == 1) reinterpret_cast<__nv_bfloat16*>(Aq)[i * ldq + c] = __float2bfloat16_rn(qv);
+                else
+                    reinterpret_cast<__nv_fp8_storage_t*>(Aq)[i * ldq + c] =
+                        __nv_cvt_float_to_fp8(v[t] * inv, __NV_SATFINITE, __NV_E4M3);
+            }
+        }
+        // levels 16 and 8 of the tree lie inside the lane
+#pragma unroll
+        for (int h = 2; h > 0; h >>= 1)
+#pragma unroll
+            for (int l = 0; l < h; l++) {
+                df_add(ph[l], pl[l], ph[l + h], pl[l + h]);
+                q2[l] += q2[l + h];
+                r2[l] += r2[l + h];
+            }
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) {
+            const float oh = __shfl_xor_sync(gmask, ph[0], off);
+            const float ol = __shfl_xor_sync(gmask, pl[0], off);
+            df_add(ph[0], pl[0], oh, ol);
+            q2[0] += __shfl_xor_sync(gmask, q2[0], off);
+            r2[0] += __shfl_xor_sync(gmask, r2[0], off);
+        }
+        const bool nzr = (__ballot_sync(gmask, nz) & gmask) != 0u;
+        if (sl == 0) {
+            const float p = ph[0] + pl[0];
+            float4 o = make_float4(p, sqrtf(p) * kNormInflate, sqrtf(q2[0]) * kNormInflate, sqrtf(r2[0]) * kNormInflate);
+            if (!isfinite(o.z) || (nzr && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
+            stat[i] = o;
+            if (rscale) rscale[i] = s;
+        }
     }
-    colmax_block(cstat, k, out);
+}
+
+// The rows of a matrix, quantised (one side of a launch).
+struct QuantSide {
+    const float* A;
+    int64_t m;
+    void* Aq;
+    float4* stat;
+    float* rscale;
+    unsigned* absmax;  // nullable: max |a| folded in
+};
+// What the screen needs of the centres beside their rows.
+struct ColSide {
+    ColMax* out;
+    float* qpad;
+    float* spad;
+    int kpad;
+    unsigned* ticket;
+};
+
+// KIND: NV of quantize_g8 (1, 2, 4, 8), 16 + NV of quantize_vec, 0
+// quantize_warp, -1 quantize_short.  The first cblocks blocks take the centres
+// and the last of them to finish forms their column data (q_j, +inf on the
+// padding so padded columns never win; the E4M3 scales, 1 on the padding; the
+// column maxima); the rest take the points.  One launch instead of three: the
+// centres' part, 5 to 9 us of latency by itself, hides behind the points'.
+constexpr int quant_blocks(int kind) { return kind == 0 ? 6 : (kind == 8 ? 3 : (kind == 17 || kind == 18 ? 5 : 4)); }  // per SM
+template <int KIND>
+__global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const QuantSide x, const QuantSide c, const ColSide col, int d, int fmt,
+                                                  int ldq, int cblocks) {
+    __shared__ bool last;
+    const bool cs = (int)blockIdx.x < cblocks;
+    const QuantSide& q = cs ? c : x;
+    const unsigned block = cs ? blockIdx.x : blockIdx.x - cblocks, nblocks = cs ? cblocks : gridDim.x - cblocks;
+    float amx = 0.0f;  // largest |a| of this thread's elements
+    if constexpr (KIND == -1) quantize_short(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
+    else if constexpr (KIND == 0) quantize_warp(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
+    else if constexpr (KIND < 16) quantize_g8<KIND>(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
+    else quantize_vec<KIND - 16>(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
+    if (q.absmax) block_absmax(amx, q.absmax);
+    if (!cs || !col.out) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(col.ticket, cblocks - 1) == (unsigned)cblocks - 1;  // back to 0 for the next call
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int k = (int)c.m;
+    for (int j = threadIdx.x; j < col.kpad; j += blockDim.x) {
+        col.qpad[j] = (j < k) ? __ldcg(c.stat + j).x : INFINITY;
+        col.spad[j] = (j < k && fmt == 2) ? __ldcg(c.rscale + j) : 1.0f;
+    }
+    colmax_block(c.stat, k, col.out);
+}
+
+// The kernel form for rows at A: -1, 0, NV or 16 + NV (k_quantize).
+static int quant_kind(const float* A, const void* Aq, int d, int ldq) {
+    const bool vec = (d % 4 == 0) && (ldq % 4 == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)Aq % 16 == 0);
+    const int nv = (ldq / 4 + 31) / 32, nv8 = (ldq / 4 + 7) / 8;
+    if (vec && nv8 <= 8) return nv8 <= 1 ? 1 : (nv8 <= 2 ? 2 : (nv8 <= 4 ? 4 : 8));
+    if (vec && nv <= 4) return 16 + (nv == 1 ? 1 : (nv == 2 ? 2 : 4));
+    return ldq <= 64 ? -1 : 0;
+}
+
+static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c, const ColSide& col, int d, int fmt,
+                                int ldq, cudaStream_t st) {
+    // 8 lanes or a warp per row, enough warps in flight to cover the memory latency
+    const int rows = kind == 0 || kind >= 16 ? 8 : 32;  // per block and round
+    const int64_t most = kind == 0 || kind >= 16 ? 152 * 64 : 152 * 16;
+    const int64_t xb = x.m ? std::min<int64_t>((x.m + rows - 1) / rows, most) : 0;
+    const int64_t cb = c.m ? std::min<int64_t>((c.m + rows - 1) / rows, 152) : 0;
+    switch (kind) {
+#define KM_Q(K)                                                                                       \
+    case K: k_quantize<K><<<(unsigned)(xb + cb), 256, 0, st>>>(x, c, col, d, fmt, ldq, (int)cb); break;
+        KM_Q(-1) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(17) KM_Q(18) KM_Q(20)
+#undef KM_Q
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_quantize(const float* A, int64_t m, int d, int fmt, int ldq, void* Aq, float4* stat,
                             float* rscale, cudaStream_t st, unsigned* absmax_out) {
-    // one warp per row, enough warps in flight to cover the memory latency
-    int64_t blocks = (m * 32 + 255) / 256;
-    if (blocks > 152 * 64) blocks = 152 * 64;
-    if (blocks < 1) blocks = 1;
-    const bool vec = (d % 4 == 0) && (ldq % 4 == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)Aq % 16 == 0);
-    const int nv = (ldq / 4 + 31) / 32;
-    const int nv8 = (ldq / 4 + 7) / 8;
-    if (vec && nv8 <= 8) {
-        blocks = std::min<int64_t>(std::max<int64_t>(1, (m * 8 + 255) / 256), (int64_t)152 * 16);
-        if (nv8 <= 1)
-            k_quantize_g8<1><<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-        else if (nv8 <= 2)
-            k_quantize_g8<2><<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-        else if (nv8 <= 4)
-            k_quantize_g8<4><<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-        else
-            k_quantize_g8<8><<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-    } else if (vec && nv <= 4) {
-        if (nv == 1)
-            k_quantize_vec<1><<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-        else if (nv == 2)
-            k_quantize_vec<2><<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-        else
-            k_quantize_vec<4><<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-    } else {
-        k_quantize<<<(unsigned)blocks, 256, 0, st>>>(A, m, d, fmt, ldq, Aq, stat, rscale, absmax_out);
-    }
-    return cudaGetLastError();
+    return launch_quant(quant_kind(A, Aq, d, ldq), QuantSide{A, m, Aq, stat, rscale, absmax_out}, QuantSide{}, ColSide{}, d,
+                        fmt, ldq, st);
+}
+
+cudaError_t launch_prepare(const float* X, int64_t n, void* Xq, float4* xstat, float* xscale, unsigned* absmax_out,
+                           const float* C, int k, void* Cq, float4* cstat, float* cscale, ColMax* colmax, float* qpad,
+                           float* spad, int kpad, unsigned* ticket, int d, int fmt, int ldq, cudaStream_t st,
+                           int* nlaunch) {
+    const QuantSide x{X, X ? n : 0, Xq, xstat, xscale, absmax_out}, c{C, k, Cq, cstat, cscale, nullptr};
+    const ColSide col{colmax, qpad, spad, kpad, ticket};
+    const int kc = quant_kind(C, Cq, d, ldq), kx = X ? quant_kind(X, Xq, d, ldq) : kc;
+    *nlaunch = 1;
+    if (kx == kc) return launch_quant(kc, x, c, col, d, fmt, ldq, st);
+    // points and centres aligned differently: each in its own form
+    *nlaunch = 2;
+    const cudaError_t e = launch_quant(kx, x, QuantSide{}, col, d, fmt, ldq, st);
+    return e != cudaSuccess ? e : launch_quant(kc, QuantSide{}, c, col, d, fmt, ldq, st);
 }
 
 // ---- candidate-count prediction (the choice of the low format) ----------
@@ -519,12 +653,6 @@ cudaError_t launch_predict_candidates(const float* X, int64_t n, int d, const fl
     if (e != cudaSuccess) return e;
     k_predict_candidates<<<(unsigned)std::max(1, std::min(ns, num_sms * 4)), 256, sm, st>>>(X, n, d, C, k, fmt, cmx, tp,
                                                                                            stride, ns, acc);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_colmax(const float4* cstat, int k, const float* cscale, ColMax* out, float* qpad, float* spad,
-                          int kpad, cudaStream_t st) {
-    k_colmax<<<1, 1024, 0, st>>>(cstat, k, cscale, out, qpad, spad, kpad);
     return cudaGetLastError();
 }
 

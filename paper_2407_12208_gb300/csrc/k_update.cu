@@ -545,14 +545,18 @@ __global__ void k_means(const long long* __restrict__ sums, const long long* __r
 // One cooperative launch over the resident blocks:
 //   1. block 0 lists the empty clusters (E of them, ascending) and clears the
 //      histograms; every block returns at once when E == 0;
-//   2. radix select (eight passes of 8 bits, most significant first) of T,
-//      the E-th largest min_dist bit pattern (non-negative doubles order like
-//      their bits), and A, the number of rows above it;
-//   3. among the rows equal to T, radix select (four passes) of the
+//   2. radix select (up to eight passes of 8 bits, most significant first) of
+//      T, the E-th largest min_dist bit pattern (non-negative doubles order
+//      like their bits), and A, the number of rows above it; as soon as every
+//      row of the digit picked is wanted, T is the digit's lowest pattern and
+//      all rows from T on are the ones;
+//   3. else, among the rows equal to T, radix select (four passes) of the
 //      (E - A)-th smallest row index I;
 //   4. the E rows {md > T} + {md == T, index <= I} are collected, ranked by
 //      (md desc, index asc) and copied into the clusters in order.
-// Work is O(n) per pass whatever E is.  The blocks meet at a grid barrier
+// Work is O(n) per pass whatever E is; bound by the grid barriers, about 2 us
+// each.  1e5 rows, a few empty clusters: 80 -> 10 us (the digits walked one L2
+// read after another, and all twelve passes, before).  The blocks meet at a grid barrier
 // whose every wait is bounded: on timeout the status word's timeout bit is
 // set and the kernel winds down.
 struct EmptySel {
@@ -596,21 +600,34 @@ KM_DEV bool grid_barrier(EmptySel* es, unsigned nblocks, unsigned* status) {
 
 // From a pass's histogram: the digit holding the rank-th key (1-based) in the
 // given direction (descending: from 255 down), the keys before that digit and
-// the rank left within it.  Every thread computes the same answer.
-KM_DEV void radix_pick(const unsigned* hist, bool descending, unsigned rank, unsigned& digit, unsigned& before) {
-    unsigned acc = 0;
-    digit = 0;
-    before = 0;
-    for (int t = 0; t < 256; t++) {
-        const int dgt = descending ? 255 - t : t;
-        const unsigned c = __ldcg(hist + dgt);  // written by other blocks' atomics
-        if (acc + c >= rank) {
-            digit = (unsigned)dgt;
-            before = acc;
-            return;
-        }
-        acc += c;
+// in it.  All 256 threads take part: thread t holds the t-th digit in that
+// direction, prefix sums over the warps, and the one that covers the rank
+// tells the others (walked digit by digit, the L2 reads alone took 6 us a pass).
+KM_DEV void radix_pick(const unsigned* hist, bool descending, unsigned rank, unsigned& digit, unsigned& before,
+                       unsigned& in) {
+    __shared__ unsigned wtot[8], pick[3];
+    const int t = threadIdx.x, lane = t & 31;
+    const unsigned dgt = descending ? 255u - t : (unsigned)t;
+    const unsigned c = __ldcg(hist + dgt);  // written by other blocks' atomics
+    unsigned incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
     }
+    __syncthreads();  // (the previous call's readers are done)
+    if (lane == 31) wtot[t >> 5] = incl;
+    __syncthreads();
+    for (int w = 0; w < (t >> 5); w++) incl += wtot[w];
+    if (incl >= rank && incl - c < rank) {
+        pick[0] = dgt;
+        pick[1] = incl - c;
+        pick[2] = c;
+    }
+    __syncthreads();
+    digit = pick[0];
+    before = pick[1];
+    in = pick[2];
 }
 
 // fixed_e > 0: no cluster lists; the fixed_e rows of largest min_dist go, in
@@ -675,8 +692,9 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
     const unsigned long long* mdb = reinterpret_cast<const unsigned long long*>(md);
     // 2. T, the E-th largest distance pattern, and A, the rows above it
     unsigned long long prefix = 0, mask = 0;
-    unsigned rank = (unsigned)E, above = 0;
-    for (int pass = 0; pass < 8; pass++) {
+    unsigned rank = (unsigned)E;
+    bool whole = false;  // every row whose pattern starts with the prefix is wanted
+    for (int pass = 0; pass < 8 && !whole; pass++) {
         const int shift = 56 - 8 * pass;
         sh[t] = 0;
         __syncthreads();
@@ -687,17 +705,17 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
         __syncthreads();
         if (sh[t]) atomicAdd(&es->hist[pass][t], sh[t]);
         if (!grid_barrier(es, nb, status)) return;
-        unsigned digit, before;
-        radix_pick(es->hist[pass], true, rank, digit, before);
-        above += before;
+        unsigned digit, before, in;
+        radix_pick(es->hist[pass], true, rank, digit, before, in);
         rank -= before;
+        whole = in == rank;
         prefix |= (unsigned long long)digit << shift;
         mask |= 255ull << shift;
     }
     const unsigned long long T = prefix;
     // 3. among the rows equal to T, the rank-th smallest index I (rank = E - A)
     unsigned iprefix = 0, imask = 0;
-    for (int pass = 0; pass < 4; pass++) {
+    for (int pass = 0; pass < 4 && !whole; pass++) {
         const int shift = 24 - 8 * pass;
         sh[t] = 0;
         __syncthreads();
@@ -707,13 +725,13 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
         __syncthreads();
         if (sh[t]) atomicAdd(&es->hist[8 + pass][t], sh[t]);
         if (!grid_barrier(es, nb, status)) return;
-        unsigned digit, before;
-        radix_pick(es->hist[8 + pass], false, rank, digit, before);
+        unsigned digit, before, in;
+        radix_pick(es->hist[8 + pass], false, rank, digit, before, in);
         rank -= before;
         iprefix |= digit << shift;
         imask |= 255u << shift;
     }
-    const unsigned I = iprefix;
+    const unsigned I = whole ? 0xffffffffu : iprefix;
     // 4. collect the E rows, rank them, fill the clusters
     for (int64_t i = gtid; i < n; i += gstride) {
         const unsigned long long key = mdb[i];
@@ -772,28 +790,58 @@ __global__ void k_shift(int k, int d, const float* __restrict__ C_old, const flo
     }
 }
 
-// Deterministic sum: fixed partition into `nparts` chunks, fixed in-block tree.
-__global__ void k_sum_parts(const double* __restrict__ v, int64_t n, double* __restrict__ parts) {
+// Deterministic sum: a fixed partition into nparts chunks; a chunk is summed
+// as 256 columns (column t adds rows t, t + 256, ... in order) folded by a
+// halving tree; one warp adds the parts (lane l adds parts l, l + 32, ... in
+// turn, then a butterfly).  The block that finishes last does that: one launch.
+// WARP: a warp per part, eight columns per lane, the same tree (few rows per
+// part: 1024 blocks of mostly idle threads took 7 us whatever n), else a
+// block.  Bound by launch latency for few rows, by the FP64 pipe for many.
+template <bool WARP>
+__global__ void __launch_bounds__(256) k_sum(const double* __restrict__ v, int64_t n, int nparts, double* parts,
+                                             double* __restrict__ out, unsigned* ticket) {
     __shared__ double red[256];
-    const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t b = (int64_t)blockIdx.x * chunk, e = min(n, b + chunk);
-    double s = 0.0;
-    for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) s += v[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+    __shared__ bool last;
+    const int t = threadIdx.x, lane = t & 31;
+    const int64_t chunk = (n + nparts - 1) / nparts;
+    if (WARP) {
+        const int part = blockIdx.x * 8 + (t >> 5);
+        const int64_t b = part * chunk, e = min(n, b + chunk);
+        double s[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) s[i] = 0.0;
+        for (int64_t r = b + lane; r < e; r += 256)
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+                if (r + 32 * i < e) s[i] += v[r + 32 * i];
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+            for (int i = 0; i < h; i++) s[i] += s[i + h];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s[0] += __shfl_down_sync(0xffffffffu, s[0], off);
+        if (lane == 0 && part < nparts) parts[part] = s[0];
+    } else {
+        const int64_t b = (int64_t)blockIdx.x * chunk, e = min(n, b + chunk);
+        double s = 0.0;
+        for (int64_t i = b + t; i < e; i += 256) s += v[i];
+        red[t] = s;
         __syncthreads();
+        for (int st = 128; st > 0; st >>= 1) {
+            if (t < st) red[t] += red[t + st];
+            __syncthreads();
+        }
+        if (t == 0) parts[blockIdx.x] = red[0];
     }
-    if (threadIdx.x == 0) parts[blockIdx.x] = red[0];
-}
-// One warp, a fixed order: lane l adds parts l, l + 32, ... in turn, then a
-// fixed butterfly (a serial sum over all parts would chain every binary64
-// addition's latency).
-__global__ void k_sum_final(const double* __restrict__ parts, int nparts, double* out) {
-    const int lane = threadIdx.x & 31;
+    __threadfence();
+    __syncthreads();
+    if (t == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;  // back to 0 for the next sum
+    __syncthreads();
+    if (!last || t >= 32) return;
+    __threadfence();
     double s = 0.0;
-    for (int i = lane; i < nparts; i += 32) s += parts[i];
+#pragma unroll 8
+    for (int i = lane; i < nparts; i += 32) s += __ldcg(parts + i);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if (lane == 0) *out = s;
@@ -997,11 +1045,11 @@ cudaError_t launch_farthest_rows(const double* min_dist, int64_t n, int e, long 
     return cudaLaunchCooperativeKernel((const void*)k_empty_select, dim3((unsigned)num_sms), dim3(256), args, 0, st);
 }
 
-cudaError_t launch_sum_f64(const double* v, int64_t n, double* partials, int nparts, double* out, cudaStream_t st) {
-    k_sum_parts<<<nparts, 256, 0, st>>>(v, n, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_sum_final<<<1, 32, 0, st>>>(partials, nparts, out);
+cudaError_t launch_sum_f64(const double* v, int64_t n, double* partials, int nparts, double* out, unsigned* ticket,
+                           cudaStream_t st) {
+    // up to four rows per column of a part, a warp keeps up with the loads
+    if (n <= (int64_t)nparts * 1024) k_sum<true><<<(nparts + 7) / 8, 256, 0, st>>>(v, n, nparts, partials, out, ticket);
+    else k_sum<false><<<nparts, 256, 0, st>>>(v, n, nparts, partials, out, ticket);
     return cudaGetLastError();
 }
 

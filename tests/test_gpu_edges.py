@@ -126,3 +126,53 @@ def test_refine_forms(ctx, low, n, d, k, scale):
     m = min(n, 20000)
     check_assign(lab[:m], md[:m], X[:m], C, oracle, RTOL_MD)
     check_assign(lab[-200:], md[-200:], X[-200:], C, oracle, RTOL_MD)
+
+
+# rows of unaligned or odd length quantise with the statistics of a full warp's tree (eight
+# lanes standing for 32): equal to the aligned form's up to the fp32 sums' own rounding
+@pytest.mark.parametrize("low", ["bf16", "fp16", "e4m3"])
+@pytest.mark.parametrize("d", [1, 7, 8, 9, 31, 32, 33, 40, 57, 63, 64, 65])
+def test_quantise_short_rows(ctx, low, d):
+    if low == "e4m3" and d < 16:
+        pytest.skip("E4M3 takes d >= 16")
+    r = np.random.Generator(np.random.PCG64(d))
+    X = r.normal(size=(1003, d)).astype(np.float32) * np.exp2(r.integers(-8, 8, size=(1003, 1))).astype(np.float32)
+    X[5] = 0
+    q, st, sc = (t.cpu().numpy() for t in ctx.quantize(_dev(X, 1), low))
+    x = X.astype(np.float64)
+    esz = 1 if low == "e4m3" else 2
+    dt = {"bf16": torch.bfloat16, "fp16": torch.float16, "e4m3": torch.float8_e4m3fn}[low]
+    xq = torch.from_numpy(q).view(dt).double().numpy()[:, :d] * sc[:, None]
+    assert q.shape[1] // esz >= d and not q[:, d * esz :].any()
+    infl = 1 + 2.0 ** -12
+    for got, want in ((st[:, 0], (x * x).sum(1)), (st[:, 1], infl * np.linalg.norm(x, axis=1)),
+                      (st[:, 2], infl * np.linalg.norm(xq, axis=1)), (st[:, 3], infl * np.linalg.norm(xq - x, axis=1))):
+        np.testing.assert_allclose(got, want, rtol=(d + 4) * 2.0 ** -24)
+
+
+# the deterministic sum: a warp or a block per part, parts of no, one and many rows
+@pytest.mark.parametrize("n", [1, 2, 1023, 1024, 1025, 300000, 1024 * 1024, 1024 * 1024 + 1, 1500007])
+def test_sse_sum(ctx, n):
+    import paper_2407_12208_gb300 as pkg
+    r = np.random.Generator(np.random.PCG64(n))
+    X = _dev(r.normal(size=(n, 3)).astype(np.float32))
+    _, md, _ = ctx.assign(X, X[:1].clone(), pkg.params("fp32"))
+    sse = ctx.stats()["sse"]
+    np.testing.assert_allclose(sse, md.sum().item(), rtol=n * 2.0 ** -53 + 1e-15)
+    ctx.assign(X, X[:1].clone(), pkg.params("fp32"))
+    assert ctx.stats()["sse"] == sse  # the same order whatever the launch
+
+
+# empty clusters: the rows of largest min_dist in order, ties to the lowest index, when the
+# radix selection can stop early (distinct distances) and when it cannot (ties at the threshold)
+@pytest.mark.parametrize("ties", [False, True])
+@pytest.mark.parametrize("n,e", [(300, 1), (5000, 7), (70000, 300)])
+def test_farthest_rows_selection(ctx, ties, n, e):
+    r = np.random.Generator(np.random.PCG64(n))
+    md = r.random(n)
+    if ties:
+        md = np.floor(md * 4)
+    rows, vals = ctx.farthest_rows(torch.from_numpy(md).cuda(), e)
+    want = np.lexsort((np.arange(n), -md))[:e]
+    assert np.array_equal(rows.cpu().numpy(), want)
+    assert np.array_equal(vals.cpu().numpy(), md[want])
