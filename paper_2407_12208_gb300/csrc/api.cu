@@ -1626,8 +1626,8 @@ extern "C" km_status km_seed_pp(km_ctx* ctx, const float* X, int64_t n, int d, i
     double* D2 = cv.take<double>((size_t)n);
     double* u = cv.take<double>((size_t)k);
     int64_t* idx = cv.take<int64_t>((size_t)k);
-    double* csum = cv.take<double>(seed_chunk_count(n));
-    int64_t* clast = cv.take<int64_t>(seed_chunk_count(n));
+    double* csum = cv.take<double>(seed_scratch_count(n, d));
+    int64_t* clast = cv.take<int64_t>(seed_scratch_count(n, d));
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));

@@ -176,3 +176,16 @@ def test_farthest_rows_selection(ctx, ties, n, e):
     want = np.lexsort((np.arange(n), -md))[:e]
     assert np.array_equal(rows.cpu().numpy(), want)
     assert np.array_equal(vals.cpu().numpy(), md[want])
+
+
+# seeding: chunks of 16 or 32 rows and their groups of eight, one and several lanes per row,
+# unaligned rows, more rows than one chunk size covers
+@pytest.mark.parametrize("n,d,offset", [(1, 3, 0), (33, 8, 0), (127, 9, 1), (129, 20, 0), (1025, 33, 1), (4099, 64, 0),
+                                        (2047, 130, 0), (900, 260, 1), (240001, 2, 0), (235000, 12, 1)])
+def test_seeding_chunks(ctx, n, d, offset):
+    X, _ = workloads.blobs(n, d, 1, seed=n)
+    k = min(n, 12)
+    C, idx = ctx.seed_pp(_dev(X, offset), workloads.seed_uniforms(k, seed=d))
+    oidx, margin = oracle.kmeanspp(X, workloads.seed_uniforms(k, seed=d), follow=idx)
+    assert np.array_equal(idx[margin > 1e-9], oidx[margin > 1e-9])
+    assert np.array_equal(C.cpu().numpy(), X[idx])
