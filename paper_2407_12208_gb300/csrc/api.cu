@@ -1228,6 +1228,7 @@ km_status km_lloyd_run(km_ctx* ctx, const float* X, int64_t n, int d, int k, con
 __global__ void k_record_iteration(const double* __restrict__ sse_slot, const DevCounters* __restrict__ cnt,
                                    double* __restrict__ sse_hist, unsigned long long* __restrict__ flag_hist,
                                    int* hist_len, int cap) {
+    chain_enter();
     const int i = *hist_len;
     if (i < cap) {
         sse_hist[i] = *sse_slot;
@@ -1253,7 +1254,7 @@ static km_status lloyd_iteration(km_ctx* ctx, const float* X, int64_t n, int d, 
     KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, graph ? L.sse_slot : sse_out, &L.a.cnt->sum_ticket, st));
     if ((s = finalize(ctx, L.u, n, k, d, cur, p, X, L.min_dist, nxt, L.counts, L.a.cnt, st, true)) != KM_OK) return s;
     if (graph) {
-        k_record_iteration<<<1, 1, 0, st>>>(L.sse_slot, L.a.cnt, L.sse_hist, L.flag_hist, L.hist_len, cap);
+        klaunch(k_record_iteration, 1, 1, 0, st, L.sse_slot, L.a.cnt, L.sse_hist, L.flag_hist, L.hist_len, cap);
         ctx->launches++;
         CK(cudaGetLastError());
     }
@@ -1600,6 +1601,7 @@ namespace {
 // The wait is the library's bounded one: it runs out after KM_WAIT_CYCLES,
 // sets the status word's timeout bit and returns; nothing faults or hangs.
 __global__ void k_wait_unsignalled(DevCounters* cnt) {
+    chain_enter();
     __shared__ __align__(8) uint64_t bar;
     __shared__ int abort_flag;
     if (threadIdx.x == 0) {
@@ -1649,7 +1651,7 @@ km_status km_selftest_timeout(km_ctx* ctx, void* ws, size_t ws_bytes, void* stre
     CK(cudaSetDevice(ctx->device));
     DevCounters* cnt = reinterpret_cast<DevCounters*>(ws);
     CK(cudaMemsetAsync(cnt, 0, sizeof(DevCounters), st));
-    k_wait_unsignalled<<<1, 32, 0, st>>>(cnt);
+    klaunch(k_wait_unsignalled, 1, 32, 0, st, cnt);
     CK(cudaGetLastError());
     ctx->launches++;
     return sync_status(ctx, cnt, st);

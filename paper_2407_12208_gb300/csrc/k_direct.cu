@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(DA_ROWS, 5) k_direct_assign(const float* __res
                                                          const float* __restrict__ C, int k, int d,
                                                          int32_t* __restrict__ labels, double* __restrict__ min_dist,
                                                          unsigned* __restrict__ absmax_out) {
+    chain_enter();
     extern __shared__ __align__(16) unsigned char smem[];
     float amx = 0.0f;  // largest |x| this thread stages (absmax_out)
     const int ldx = d + 1;
@@ -480,6 +481,7 @@ __global__ void __launch_bounds__(256, 2) k_direct_tiled(const float* __restrict
                                                          int32_t* __restrict__ labels, double* __restrict__ min_dist,
                                                          DevCounters* cnt,
                                                          float gamma32, unsigned* __restrict__ absmax_out) {
+    chain_enter();
     direct_tiled<RPT, 4>(X, n, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32, absmax_out);
 }
 // every other shape
@@ -491,6 +493,7 @@ __global__ void __launch_bounds__(256, 2) k_direct_assign(const float* __restric
                                                           int32_t* __restrict__ labels, double* __restrict__ min_dist,
                                                           DevCounters* cnt,
                                                           float gamma32, unsigned* __restrict__ absmax_out) {
+    chain_enter();
     static_assert(sizeof(T) == 4, "binary32 accumulation");
     direct_tiled<RPT, VEC>(X, n, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32, absmax_out);
 }
@@ -505,7 +508,7 @@ static cudaError_t launch_tiled(const float* X, int64_t n, const float* C, int k
     cudaError_t e = allow_max_smem(fn);
     if (e != cudaSuccess) return e;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 32 * RPT - 1) / (32 * RPT), (int64_t)num_sms * 2));
-    fn<<<(unsigned)grid, 256, sm, st>>>(X, n, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32,
+    klaunch(fn, (unsigned)grid, 256, sm, st, X, n, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32,
                                         absmax_out);
     return cudaGetLastError();
 }
@@ -523,6 +526,7 @@ __global__ void __launch_bounds__(256) k_direct_small(const float* __restrict__ 
                                                       int32_t* __restrict__ labels, double* __restrict__ min_dist,
                                                       DevCounters* cnt,
                                                       float gamma32, unsigned* __restrict__ absmax_out) {
+    chain_enter();
     extern __shared__ __align__(16) float Csm[];
     float amx = 0.0f;  // largest |x| of this thread's rows (absmax_out)
     for (int e = threadIdx.x; e < k * D; e += blockDim.x) Csm[e] = C[e];
@@ -620,7 +624,7 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
         switch (d) {
 #define KM_SMALL(DD)                                                                                                  \
     case DD:                                                                                                          \
-        k_direct_small<DD><<<(unsigned)grid, 256, csm, st>>>(X, n, C, k, row_list, row_count, labels, min_dist,      \
+        klaunch(k_direct_small<DD>, (unsigned)grid, 256, csm, st, X, n, C, k, row_list, row_count, labels, min_dist,      \
                                                               cnt, gamma32, absmax_out);                                \
         break;
             KM_SMALL(1) KM_SMALL(2) KM_SMALL(3) KM_SMALL(4) KM_SMALL(5) KM_SMALL(6) KM_SMALL(7) KM_SMALL(8)
@@ -650,7 +654,7 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
     void (*fn64)(const float*, int64_t, const float*, int, int, int32_t*, double*, unsigned*) = k_direct_assign<double>;
     cudaError_t e = allow_max_smem(fn64);
     if (e != cudaSuccess) return e;
-    fn64<<<(unsigned)grid, DA_ROWS, sm, st>>>(X, n, C, k, d, labels, min_dist, absmax_out);
+    klaunch(fn64, (unsigned)grid, DA_ROWS, sm, st, X, n, C, k, d, labels, min_dist, absmax_out);
     return cudaGetLastError();
 }
 
@@ -660,6 +664,7 @@ __global__ void __launch_bounds__(256) k_rows_full(const float* __restrict__ X, 
                                                    const int* __restrict__ row_count, int32_t* __restrict__ labels,
                                                    double* __restrict__ min_dist, DevCounters* cnt, float gamma32,
                                                    size_t bytes) {
+    chain_enter();
     extern __shared__ __align__(16) double shd[];
     const int64_t nrows = *row_count;
     unsigned long long ev32 = 0, ev64 = 0, open = 0;
@@ -684,7 +689,7 @@ cudaError_t launch_rows_full(const float* X, const float* C, int k, int d, const
     const size_t bytes = all <= (size_t)kMaxBlockSmem - fa.sharedSizeBytes ? all : resolve_bytes(d);
     e = allow_max_smem(k_rows_full);
     if (e != cudaSuccess) return e;
-    k_rows_full<<<num_sms * 2, 256, bytes, st>>>(X, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32, bytes);
+    klaunch(k_rows_full, num_sms * 2, 256, bytes, st, X, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32, bytes);
     return cudaGetLastError();
 }
 

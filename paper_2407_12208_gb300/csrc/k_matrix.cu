@@ -27,6 +27,7 @@ constexpr int MX_T = 16;  // pairs tile: 16 rows x 16 centres per block
 
 // out[i] = sum_l fl(a_il a_il) by recursive summation in binary32
 __global__ void k_rowdot_fp32(const float* __restrict__ A, int64_t m, int d, float* __restrict__ out) {
+    chain_enter();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const float* a = A + i * d;
         float s = 0.0f;
@@ -46,6 +47,7 @@ __global__ void __launch_bounds__(256) k_matrix(const float* __restrict__ X, int
                                                 uint32_t* __restrict__ flag_bits, int2* __restrict__ queue,
                                                 int64_t qcap, unsigned long long* __restrict__ qlen,
                                                 DevCounters* cnt) {
+    chain_enter();
     extern __shared__ float msh[];
     float* xs = msh;                    // MX_T x (d + 1)
     float* cs = msh + MX_T * (d + 1);   // MX_T x (d + 1)
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(256) k_matrix(const float* __restrict__ X, int
 
 cudaError_t launch_rowdot_fp32(const float* A, int64_t m, int d, float* out, int num_sms, cudaStream_t st) {
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((m + 255) / 256, (int64_t)num_sms * 8));
-    k_rowdot_fp32<<<blocks, 256, 0, st>>>(A, m, d, out);
+    klaunch(k_rowdot_fp32, blocks, 256, 0, st, A, m, d, out);
     return cudaGetLastError();
 }
 
@@ -131,7 +133,7 @@ cudaError_t launch_matrix(int mode, const float* X, int64_t n, const float* C, i
 #define KM_MX(M)                                                                                                 \
     e = allow_max_smem(k_matrix<M>);                                                                             \
     if (e != cudaSuccess) return e;                                                                              \
-    k_matrix<M><<<blocks, 256, sm, st>>>(X, n, C, k, d, dxx, dyy, test, rho, coef, kacc, kn, D, flag_bits, queue, \
+    klaunch(k_matrix<M>, blocks, 256, sm, st, X, n, C, k, d, dxx, dyy, test, rho, coef, kacc, kn, D, flag_bits, queue, \
                                          qcap, qlen, cnt);
     if (mode == 0) { KM_MX(0) }
     else if (mode == 1) { KM_MX(1) }
@@ -183,6 +185,7 @@ template <int FB, int FMT>
 __global__ void k_patch_flagged(const float* __restrict__ X, const float* __restrict__ C, int k, int d,
                                 const int2* __restrict__ queue, const unsigned long long* __restrict__ qlen,
                                 int64_t cap, float* __restrict__ D, int64_t n, DevCounters* cnt) {
+    chain_enter();
     const int64_t len = (int64_t)*qlen;
     const bool scan = len > cap;
     const int64_t total = scan ? n * (int64_t)k : len;
@@ -213,10 +216,10 @@ cudaError_t launch_patch_flagged(int fb, int fmt, const float* X, const float* C
                                  const int2* queue, const unsigned long long* qlen, int64_t cap, float* D,
                                  DevCounters* cnt, int num_sms, cudaStream_t st) {
     const unsigned blocks = (unsigned)num_sms * 8;
-    if (fb == 0) k_patch_flagged<0, 0><<<blocks, 256, 0, st>>>(X, C, k, d, queue, qlen, cap, D, n, cnt);
-    else if (fb == 1) k_patch_flagged<1, 0><<<blocks, 256, 0, st>>>(X, C, k, d, queue, qlen, cap, D, n, cnt);
-    else if (fmt == 0) k_patch_flagged<2, 0><<<blocks, 256, 0, st>>>(X, C, k, d, queue, qlen, cap, D, n, cnt);
-    else k_patch_flagged<2, 1><<<blocks, 256, 0, st>>>(X, C, k, d, queue, qlen, cap, D, n, cnt);
+    if (fb == 0) klaunch(k_patch_flagged<0, 0>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
+    else if (fb == 1) klaunch(k_patch_flagged<1, 0>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
+    else if (fmt == 0) klaunch(k_patch_flagged<2, 0>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
+    else klaunch(k_patch_flagged<2, 1>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
     return cudaGetLastError();
 }
 

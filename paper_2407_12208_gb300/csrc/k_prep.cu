@@ -478,6 +478,7 @@ constexpr int quant_blocks(int kind) { return kind == 0 ? 6 : (kind == 8 ? 3 : (
 template <int KIND>
 __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const QuantSide x, const QuantSide c, const ColSide col, int d, int fmt,
                                                   int ldq, int cblocks) {
+    chain_enter();
     __shared__ bool last;
     const bool cs = (int)blockIdx.x < cblocks;
     const QuantSide& q = cs ? c : x;
@@ -521,7 +522,7 @@ static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c
     const int64_t cb = c.m ? std::min<int64_t>((c.m + rows - 1) / rows, 152) : 0;
     switch (kind) {
 #define KM_Q(K)                                                                                       \
-    case K: k_quantize<K><<<(unsigned)(xb + cb), 256, 0, st>>>(x, c, col, d, fmt, ldq, (int)cb); break;
+    case K: klaunch(k_quantize<K>, (unsigned)(xb + cb), 256, 0, st, x, c, col, d, fmt, ldq, (int)cb); break;
         KM_Q(-1) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(17) KM_Q(18) KM_Q(20)
 #undef KM_Q
         default: return cudaErrorInvalidValue;
@@ -562,6 +563,7 @@ __global__ void __launch_bounds__(256) k_predict_candidates(const float* __restr
                                                             const float* __restrict__ C, int k, int fmt,
                                                             const ColMax* __restrict__ cmx, TestParams tp, int64_t stride,
                                                             int nsample, unsigned long long* acc) {
+    chain_enter();
     extern __shared__ float xs[];
     __shared__ float red[8];
     __shared__ float sh_stat[4];
@@ -651,7 +653,7 @@ cudaError_t launch_predict_candidates(const float* X, int64_t n, int d, const fl
     const size_t sm = (size_t)d * sizeof(float);
     cudaError_t e = allow_max_smem(k_predict_candidates);
     if (e != cudaSuccess) return e;
-    k_predict_candidates<<<(unsigned)std::max(1, std::min(ns, num_sms * 4)), 256, sm, st>>>(X, n, d, C, k, fmt, cmx, tp,
+    klaunch(k_predict_candidates, (unsigned)std::max(1, std::min(ns, num_sms * 4)), 256, sm, st, X, n, d, C, k, fmt, cmx, tp,
                                                                                            stride, ns, acc);
     return cudaGetLastError();
 }

@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(256) k_pair_eval(const float* __restrict__ X, 
                                                    const int2* __restrict__ pairs,
                                                    const unsigned long long* __restrict__ npairs, int64_t cap,
                                                    float* __restrict__ v32) {
+    chain_enter();
     const int lane = threadIdx.x & 31, sl = lane & 7, gbase = lane & ~7;
     const unsigned gmask = 0xFFu << gbase;
     const int64_t gid = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4 + (lane >> 3);
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(256) k_cand_select(const int4* __restrict__ ro
                                                      int2* __restrict__ pairs, int64_t cap,
                                                      int2* __restrict__ rowpair, int32_t* __restrict__ labels,
                                                      DevCounters* cnt) {
+    chain_enter();
     const int lane = threadIdx.x & 31;
     const uint32_t emask = (1u << ebits) - 1u;
     const float lscale = __uint_as_float((uint32_t)(127 + ebits - 23) << 23);  // 2^(ebits - 23)
@@ -228,6 +230,7 @@ __global__ void __launch_bounds__(256) k_certify(const int2* __restrict__ rowpai
                                                  float gamma32, int32_t* __restrict__ labels,
                                                  double* __restrict__ min_dist, int32_t* __restrict__ full_list,
                                                  int32_t* __restrict__ amb_list, DevCounters* cnt) {
+    chain_enter();
     unsigned long long ev32 = 0, amb = 0, ovf_rows = 0;
     const float g = gamma32;
     for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < n;
@@ -290,6 +293,7 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
                                                   const float* __restrict__ C, int d, float gamma32,
                                                   int32_t* __restrict__ labels, double* __restrict__ min_dist,
                                                   DevCounters* cnt) {
+    chain_enter();
     extern __shared__ double amb_sm[];  // per warp: AMB_B x d products
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     double* prod = amb_sm + (size_t)wib * AMB_B * d;
@@ -381,6 +385,7 @@ __global__ void __launch_bounds__(256) k_refine(const int4* __restrict__ rowinfo
                                                 const float* __restrict__ C, int d, float gamma32,
                                                 int32_t* __restrict__ labels, int32_t* __restrict__ ovf_list,
                                                 int* __restrict__ ovf_n, DevCounters* cnt) {
+    chain_enter();
     constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
     static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
     extern __shared__ double rc_sm[];  // per warp: d products
@@ -623,7 +628,7 @@ static cudaError_t launch_refine_batched(const float* X, const float* C, const T
     const int64_t rows_blocks = std::max<int64_t>(1, (a.n + 255) / 256);
     const int64_t rb = std::min<int64_t>(rows_blocks, (int64_t)num_sms * std::max(sel_per_sm, 1));
     const int64_t cb = std::min<int64_t>(rows_blocks, (int64_t)num_sms * std::max(cert_per_sm, 1));
-    k_cand_select<<<(unsigned)rb, 256, 0, st>>>(a.rowinfo, a.cand, a.n, a.ebits, a.pairs, a.pair_cap, a.rowpair, labels,
+    klaunch(k_cand_select, (unsigned)rb, 256, 0, st, a.rowinfo, a.cand, a.n, a.ebits, a.pairs, a.pair_cap, a.rowpair, labels,
                                                 a.cnt);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -638,20 +643,20 @@ static cudaError_t launch_refine_batched(const float* X, const float* C, const T
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)num_sms * (unsigned)std::max(per_sm, 1);
     const unsigned long long* np = &a.cnt->npairs;
-    if (!vec) k_pair_eval<0><<<blocks, 256, 0, st>>>(X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
-    else if (a.d <= 32) k_pair_eval<1><<<blocks, 256, 0, st>>>(X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
-    else if (a.d <= 128) k_pair_eval<4><<<blocks, 256, 0, st>>>(X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
-    else k_pair_eval<8><<<blocks, 256, 0, st>>>(X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
+    if (!vec) klaunch(k_pair_eval<0>, blocks, 256, 0, st, X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
+    else if (a.d <= 32) klaunch(k_pair_eval<1>, blocks, 256, 0, st, X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
+    else if (a.d <= 128) klaunch(k_pair_eval<4>, blocks, 256, 0, st, X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
+    else klaunch(k_pair_eval<8>, blocks, 256, 0, st, X, C, a.d, a.pairs, np, a.pair_cap, a.v32);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_certify<<<(unsigned)cb, 256, 0, st>>>(a.rowpair, a.n, a.pairs, a.v32, X, C, a.d, a.tp.gamma32, labels, min_dist,
+    klaunch(k_certify, (unsigned)cb, 256, 0, st, a.rowpair, a.n, a.pairs, a.v32, X, C, a.d, a.tp.gamma32, labels, min_dist,
                                              full_list, amb_list, a.cnt);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t amb_smem = (size_t)8 * AMB_B * a.d * sizeof(double);  // 8 warps per block
     e = allow_max_smem(k_amb_fp64);
     if (e != cudaSuccess) return e;
-    k_amb_fp64<<<(unsigned)num_sms, 256, amb_smem, st>>>(amb_list, &a.cnt->amb_count, a.rowpair, a.pairs, a.v32, X, C,
+    klaunch(k_amb_fp64, (unsigned)num_sms, 256, amb_smem, st, amb_list, &a.cnt->amb_count, a.rowpair, a.pairs, a.v32, X, C,
                                                           a.d, a.tp.gamma32, labels, min_dist, a.cnt);
     return cudaGetLastError();
 }
@@ -670,7 +675,7 @@ static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, sm);
     if (e != cudaSuccess) return e;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + threads - 1) / threads, (int64_t)num_sms * std::max(per_sm, 1)));
-    fn<<<(unsigned)blocks, threads, sm, st>>>(a.rowinfo, a.cand, a.n, a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,
+    klaunch(fn, (unsigned)blocks, threads, sm, st, a.rowinfo, a.cand, a.n, a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,
                                               labels, ovf_list, ovf_n, a.cnt);
     return cudaGetLastError();
 }
@@ -698,6 +703,7 @@ cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, const
 __global__ void __launch_bounds__(256) k_centre_rows(const int32_t* __restrict__ list, const int* __restrict__ list_n,
                                                      const float* __restrict__ X, const float* __restrict__ C, int k,
                                                      int d, const Centred cen, unsigned* ticket) {
+    chain_enter();
     const int nf = *list_n;
     if (nf == 0) return;
     __shared__ __align__(16) float mu[256];
@@ -728,7 +734,7 @@ __global__ void __launch_bounds__(256) k_centre_rows(const int32_t* __restrict__
 
 cudaError_t launch_centre_rows(const int32_t* list, const int* list_n, const float* X, const float* C, int k, int d,
                                const Centred& cen, unsigned* ticket, int num_sms, cudaStream_t st) {
-    k_centre_rows<<<(unsigned)num_sms * 4, 256, 0, st>>>(list, list_n, X, C, k, d, cen, ticket);
+    klaunch(k_centre_rows, (unsigned)num_sms * 4, 256, 0, st, list, list_n, X, C, k, d, cen, ticket);
     return cudaGetLastError();
 }
 

@@ -302,6 +302,7 @@ template <int NV4, int LPR, bool VEC, bool SMALL>
 __global__ void __launch_bounds__(256, NV4 == 1 || SMALL ? 3 : 2) k_seed_step(const float* __restrict__ X, int64_t n, int d, const SeedPlan pl,
                                                    const double* __restrict__ u, int t, float g, double* D2, double* csum,
                                                    int64_t* clast, int64_t* idx, unsigned* ticket) {
+    chain_enter();
     __shared__ double part_sh[SD_WARPS * 32];
     __shared__ int last_sh[SD_WARPS];
     __shared__ bool last_block;
@@ -366,6 +367,7 @@ __global__ void __launch_bounds__(256, NV4 == 1 || SMALL ? 3 : 2) k_seed_step(co
 // The picked rows (and the first pick's index).
 __global__ void k_seed_gather(const float* __restrict__ X, int64_t n, int d, const double* __restrict__ u, int64_t* idx,
                               int k, float* __restrict__ C) {
+    chain_enter();
     const int64_t first = uniform_pick(u[0], n);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)k * d;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -410,11 +412,11 @@ cudaError_t launch_seed_pp(const float* X, int64_t n, int d, int k, const double
     // Theorem 4.1's gamma_{d+2}(2^-24) with safety, and the double-float distance's own 2^-40
     const float g = (float)((d + 4) * std::ldexp(1.0, -24) * 1.01 + std::ldexp(1.0, -22));
     for (int t = 0; t + 1 < k; t++) {
-        kern<<<blocks, 256, 0, st>>>(X, n, d, pl, u_dev, t, g, D2, csum, clast, idx, ticket);
+        klaunch(kern, blocks, 256, 0, st, X, n, d, pl, u_dev, t, g, D2, csum, clast, idx, ticket);
         (*nlaunch)++;
     }
     const unsigned gb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)k * d + 255) / 256, 4096));
-    k_seed_gather<<<gb, 256, 0, st>>>(X, n, d, u_dev, idx, k, C_out);
+    klaunch(k_seed_gather, gb, 256, 0, st, X, n, d, u_dev, idx, k, C_out);
     (*nlaunch)++;
     return cudaGetLastError();
 }

@@ -163,6 +163,7 @@ KM_DEV float fmin3(float a, float b, float c) {
 template <int FMT, int BN, int MODE, int SV>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmC, const TcArgs a) {
+    chain_enter();
     extern __shared__ unsigned char smem_raw[];
     const int64_t nrows = a.nrows ? min((int64_t)*a.nrows, a.n) : a.n;
     if (nrows == 0) return;
@@ -665,7 +666,7 @@ static cudaError_t launch_one(const CUtensorMap& mx, const CUtensorMap& mc, cons
     if (e != cudaSuccess) return e;
     const int64_t nrb = (a.n + TC_BM - 1) / TC_BM;
     const int grid = (int)std::min<int64_t>(nrb, (int64_t)num_sms);
-    k_tc<FMT, BN, MODE, SV><<<grid, TC_THREADS, L.total, st>>>(mx, mc, a);
+    klaunch(k_tc<FMT, BN, MODE, SV>, grid, TC_THREADS, L.total, st, mx, mc, a);
     return cudaGetLastError();
 }
 

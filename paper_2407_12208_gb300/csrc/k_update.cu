@@ -22,6 +22,7 @@
 namespace km {
 
 __global__ void k_absmax(const float* __restrict__ X, int64_t count, unsigned* out) {
+    chain_enter();
     float m = 0.0f;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
         m = fmaxf(m, fabsf(X[e]));
@@ -37,6 +38,7 @@ template <bool SMEM>
 __global__ void k_accumulate(const float* __restrict__ X, int64_t n, int d, const int32_t* __restrict__ labels,
                              int k, const unsigned* __restrict__ amax_bits, int64_t nscale, long long* __restrict__ sums,
                              long long* __restrict__ counts) {
+    chain_enter();
     extern __shared__ long long acc[];
     const FixedScale fx(fixed_shift(*amax_bits, nscale));
     const int64_t kd = (int64_t)k * d;
@@ -82,6 +84,7 @@ constexpr int SCAT_ROWS = 4096;  // rows per block of the histogram / scatter ke
 
 // per-label counts (block histogram in shared memory, one global add per label)
 __global__ void k_label_hist(const int32_t* __restrict__ labels, int64_t n, int k, int* __restrict__ cnt32) {
+    chain_enter();
     extern __shared__ int h[];
     for (int j = threadIdx.x; j < k; j += blockDim.x) h[j] = 0;
     __syncthreads();
@@ -96,6 +99,7 @@ __global__ void k_label_hist(const int32_t* __restrict__ labels, int64_t n, int 
 // the offsets of each bucket's first work item; counts as int64.
 __global__ void k_bucket_scan(const int* __restrict__ cnt32, int k, int seg, int* __restrict__ off,
                               int* __restrict__ cursor, int* __restrict__ item_off, long long* __restrict__ counts) {
+    chain_enter();
     __shared__ int sa[1024], sb[1024];
     const int t = threadIdx.x, T = blockDim.x;
     const int per = (k + T - 1) / T;
@@ -134,6 +138,7 @@ __global__ void k_bucket_scan(const int* __restrict__ cnt32, int k, int seg, int
 // label present) and places its rows with shared-memory cursors.
 __global__ void k_bucket_scatter(const int32_t* __restrict__ labels, int64_t n, int k, int* __restrict__ cursor,
                                  int32_t* __restrict__ perm) {
+    chain_enter();
     extern __shared__ int sh[];
     int* h = sh;
     int* lc = sh + k;
@@ -171,6 +176,7 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
                              const int* __restrict__ item_off, const int32_t* __restrict__ perm,
                              const unsigned* __restrict__ amax_bits, int64_t nscale, long long* __restrict__ sums,
                              const float* __restrict__ C, double* __restrict__ md) {
+    chain_enter();
     static_assert(LPR == 32 || NV4 == 1, "rows narrower than a warp take one float4 per lane");
     constexpr int G = 32 / LPR;                            // rows per warp load
     // loads in flight per lane: 8 at full-warp rows of one float4 (three blocks
@@ -294,6 +300,7 @@ template <int D>
 __global__ void k_bucket_sum_small(const float* __restrict__ X, int64_t n, int k, int seg, const int* __restrict__ off,
                                    const int* __restrict__ item_off, const int32_t* __restrict__ perm,
                                    const unsigned* __restrict__ amax_bits, int64_t nscale, long long* __restrict__ sums) {
+    chain_enter();
     const FixedScale fx(fixed_shift(*amax_bits, nscale));
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -339,6 +346,7 @@ __global__ void __launch_bounds__(256) k_accum_small(const float* __restrict__ X
                                                      const unsigned* __restrict__ amax_bits, int64_t nscale,
                                                      long long* __restrict__ sums, long long* __restrict__ counts,
                                                      const float* __restrict__ C, double* __restrict__ md) {
+    chain_enter();
     extern __shared__ unsigned acc_sm[];  // per warp: 3 * k * D parts, then k counts; then C (WD)
     const FixedScale fx(fixed_shift(*amax_bits, nscale));
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -422,6 +430,7 @@ template <int NV4, int LPR, bool VEC>
 __global__ void __launch_bounds__(256) k_winner_dist(const float* __restrict__ X, int64_t n, int d,
                                                      const float* __restrict__ C, const int32_t* __restrict__ labels,
                                                      double* __restrict__ md) {
+    chain_enter();
     constexpr int G = 32 / LPR;
     constexpr int R = NV4 == 4 ? 2 : 4;  // 4 rows per pass: measured faster than 8 (occupancy)
     constexpr int STEP = R * G;
@@ -473,6 +482,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_winner_small(const float* __restrict__ X, int64_t n,
                                                       const float* __restrict__ C, const int32_t* __restrict__ labels,
                                                       double* __restrict__ md) {
+    chain_enter();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int j = labels[i];
         float xr[D];
@@ -489,7 +499,7 @@ cudaError_t launch_winner_dist(const float* X, int64_t n, int d, const float* C,
         const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)num_sms * 8));
         switch (d) {
 #define KM_WS(DD) \
-    case DD: k_winner_small<DD><<<blocks, 256, 0, st>>>(X, n, C, labels, md); break;
+    case DD: klaunch(k_winner_small<DD>, blocks, 256, 0, st, X, n, C, labels, md); break;
             KM_WS(1) KM_WS(2) KM_WS(3) KM_WS(4) KM_WS(5) KM_WS(6) KM_WS(7) KM_WS(8)
 #undef KM_WS
         }
@@ -515,7 +525,7 @@ cudaError_t launch_winner_dist(const float* X, int64_t n, int d, const float* C,
     const int64_t warps_needed = (n + rows_per_warp_pass - 1) / rows_per_warp_pass;
     const unsigned blocks = (unsigned)std::max<int64_t>(
         1, std::min<int64_t>((warps_needed + 7) / 8, (int64_t)num_sms * std::max(per_sm, 1)));
-    kern<<<blocks, 256, 0, st>>>(X, n, d, C, labels, md);
+    klaunch(kern, blocks, 256, 0, st, X, n, d, C, labels, md);
     return cudaGetLastError();
 }
 
@@ -523,6 +533,7 @@ cudaError_t launch_winner_dist(const float* X, int64_t n, int d, const float* C,
 __global__ void k_means(const long long* __restrict__ sums, const long long* __restrict__ counts,
                         const unsigned* __restrict__ amax_bits, int64_t nscale, int k, int d,
                         const float* __restrict__ C_old, float* __restrict__ C_new, int64_t* counts_out) {
+    chain_enter();
     const int S = fixed_shift(*amax_bits, nscale);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)k * d;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -640,6 +651,7 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
                                                       int* __restrict__ rows, int* __restrict__ order,
                                                       unsigned* status, int fixed_e, long long* __restrict__ rows_out,
                                                       double* __restrict__ vals_out) {
+    chain_enter();
     __shared__ unsigned sh[256];
     __shared__ int wsum[8];
     __shared__ int any_empty;
@@ -775,6 +787,7 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
 // an unsigned integer), so the result does not depend on the order.
 __global__ void k_shift(int k, int d, const float* __restrict__ C_old, const float* __restrict__ C_new,
                         unsigned long long* __restrict__ shift_bits) {
+    chain_enter();
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -800,6 +813,7 @@ __global__ void k_shift(int k, int d, const float* __restrict__ C_old, const flo
 template <bool WARP>
 __global__ void __launch_bounds__(256) k_sum(const double* __restrict__ v, int64_t n, int nparts, double* parts,
                                              double* __restrict__ out, unsigned* ticket) {
+    chain_enter();
     __shared__ double red[256];
     __shared__ bool last;
     const int t = threadIdx.x, lane = t & 31;
@@ -852,7 +866,7 @@ cudaError_t launch_absmax(const float* X, int64_t count, unsigned* out_bits, cud
     if (e != cudaSuccess) return e;
     int64_t blocks = min((int64_t)152 * 8, (count + 255) / 256);
     if (blocks < 1) blocks = 1;
-    k_absmax<<<(unsigned)blocks, 256, 0, st>>>(X, count, out_bits);
+    klaunch(k_absmax, (unsigned)blocks, 256, 0, st, X, count, out_bits);
     return cudaGetLastError();
 }
 
@@ -881,12 +895,12 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         if (want_wd) {                                                                                              \
             e = allow_max_smem(k_accum_small<DD, true>);                                                            \
             if (e != cudaSuccess) return e;                                                                         \
-            k_accum_small<DD, true><<<(unsigned)blocks, 256, sm, st>>>(X, n, k, labels, absmax_bits, nscale, sums, counts,  \
+            klaunch(k_accum_small<DD, true>, (unsigned)blocks, 256, sm, st, X, n, k, labels, absmax_bits, nscale, sums, counts,  \
                                                                        C_wd, md_out);                               \
         } else {                                                                                                    \
             e = allow_max_smem(k_accum_small<DD, false>);                                                           \
             if (e != cudaSuccess) return e;                                                                         \
-            k_accum_small<DD, false><<<(unsigned)blocks, 256, sm, st>>>(X, n, k, labels, absmax_bits, nscale, sums, counts, \
+            klaunch(k_accum_small<DD, false>, (unsigned)blocks, 256, sm, st, X, n, k, labels, absmax_bits, nscale, sums, counts, \
                                                                         nullptr, nullptr);                          \
         }                                                                                                           \
         break;
@@ -917,7 +931,7 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         const int64_t nblk = (n + SCAT_ROWS - 1) / SCAT_ROWS;
         e = allow_max_smem(k_label_hist);
         if (e != cudaSuccess) return e;
-        k_label_hist<<<(unsigned)nblk, 512, hsm, st>>>(labels, n, k, cnt32);
+        klaunch(k_label_hist, (unsigned)nblk, 512, hsm, st, labels, n, k, cnt32);
         // persistent grid: every block resident at once (a partial second wave
         // would leave SMs idle), the items strided over the warps; work items of
         // `seg` rows, about four per resident warp (fewer, longer items mean
@@ -938,18 +952,18 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         }
         const int64_t resident_warps = (int64_t)num_sms * std::max(per_sm, 1) * 8;
         const int seg = (int)std::min<int64_t>(SEG_MAX, std::max<int64_t>(64, n / (resident_warps * 4) / 32 * 32));
-        k_bucket_scan<<<1, 1024, 0, st>>>(cnt32, k, seg, off, cursor, item_off, counts);
+        klaunch(k_bucket_scan, 1, 1024, 0, st, cnt32, k, seg, off, cursor, item_off, counts);
         e = allow_max_smem(k_bucket_scatter);
         if (e != cudaSuccess) return e;
-        k_bucket_scatter<<<(unsigned)nblk, 512, 2 * hsm, st>>>(labels, n, k, cursor, perm);
+        klaunch(k_bucket_scatter, (unsigned)nblk, 512, 2 * hsm, st, labels, n, k, cursor, perm);
         const int64_t items = n / seg + k + 1;
         const unsigned blocks =
             (unsigned)std::max<int64_t>(1, std::min<int64_t>((items * 32 + 255) / 256, (int64_t)num_sms * std::max(per_sm, 1)));
-        if (d == 1) k_bucket_sum_small<1><<<blocks, 256, 0, st>>>(X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else if (d == 2) k_bucket_sum_small<2><<<blocks, 256, 0, st>>>(X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else if (d == 3) k_bucket_sum_small<3><<<blocks, 256, 0, st>>>(X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else if (d == 5) k_bucket_sum_small<5><<<blocks, 256, 0, st>>>(X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else bfn<<<blocks, 256, 0, st>>>(X, n, d, k, seg, off, item_off, perm, absmax_bits, nscale, sums, C_wd, md_out);
+        if (d == 1) klaunch(k_bucket_sum_small<1>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
+        else if (d == 2) klaunch(k_bucket_sum_small<2>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
+        else if (d == 3) klaunch(k_bucket_sum_small<3>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
+        else if (d == 5) klaunch(k_bucket_sum_small<5>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
+        else klaunch(bfn, blocks, 256, 0, st, X, n, d, k, seg, off, item_off, perm, absmax_bits, nscale, sums, C_wd, md_out);
         if (nlaunch) *nlaunch = nl + 4;
         return cudaGetLastError();
     }
@@ -961,11 +975,11 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         e = allow_max_smem(k_accumulate<true>);
         if (e != cudaSuccess) return e;
         const int64_t blk = std::min<int64_t>((int64_t)num_sms, (total + 511) / 512);
-        k_accumulate<true><<<(unsigned)std::max<int64_t>(blk, 1), 512, smem, st>>>(X, n, d, labels, k, absmax_bits,
+        klaunch(k_accumulate<true>, (unsigned)std::max<int64_t>(blk, 1), 512, smem, st, X, n, d, labels, k, absmax_bits,
                                                                                     nscale, sums, counts);
     } else {
         const int64_t blk = std::min<int64_t>((int64_t)num_sms * 8, (total + 511) / 512);
-        k_accumulate<false><<<(unsigned)std::max<int64_t>(blk, 1), 512, 0, st>>>(X, n, d, labels, k, absmax_bits,
+        klaunch(k_accumulate<false>, (unsigned)std::max<int64_t>(blk, 1), 512, 0, st, X, n, d, labels, k, absmax_bits,
                                                                                   nscale, sums, counts);
     }
     if (nlaunch) *nlaunch = nl + 1;
@@ -979,7 +993,7 @@ cudaError_t launch_finalize(const long long* sums, const long long* counts, cons
     int nl = 0;
     int64_t kd = (int64_t)k * d;
     int64_t blocks = min((int64_t)1024, (kd + 255) / 256);
-    k_means<<<(unsigned)blocks, 256, 0, st>>>(sums, counts, absmax_bits, nscale > 0 ? nscale : n, k, d, C_old, C_new,
+    klaunch(k_means, (unsigned)blocks, 256, 0, st, sums, counts, absmax_bits, nscale > 0 ? nscale : n, k, d, C_old, C_new,
                                                counts_out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1013,7 +1027,7 @@ cudaError_t launch_finalize(const long long* sums, const long long* counts, cons
         e = cudaMemsetAsync(shift, 0, sizeof(double), st);
         if (e != cudaSuccess) return e;
         const int64_t sblocks = std::min<int64_t>(((int64_t)k * 32 + 255) / 256, (int64_t)num_sms * 8);
-        k_shift<<<(unsigned)std::max<int64_t>(sblocks, 1), 256, 0, st>>>(k, d, C_old, C_new,
+        klaunch(k_shift, (unsigned)std::max<int64_t>(sblocks, 1), 256, 0, st, k, d, C_old, C_new,
                                                                        reinterpret_cast<unsigned long long*>(shift));
         nl++;
     }
@@ -1048,8 +1062,8 @@ cudaError_t launch_farthest_rows(const double* min_dist, int64_t n, int e, long 
 cudaError_t launch_sum_f64(const double* v, int64_t n, double* partials, int nparts, double* out, unsigned* ticket,
                            cudaStream_t st) {
     // up to four rows per column of a part, a warp keeps up with the loads
-    if (n <= (int64_t)nparts * 1024) k_sum<true><<<(nparts + 7) / 8, 256, 0, st>>>(v, n, nparts, partials, out, ticket);
-    else k_sum<false><<<nparts, 256, 0, st>>>(v, n, nparts, partials, out, ticket);
+    if (n <= (int64_t)nparts * 1024) klaunch(k_sum<true>, (nparts + 7) / 8, 256, 0, st, v, n, nparts, partials, out, ticket);
+    else klaunch(k_sum<false>, nparts, 256, 0, st, v, n, nparts, partials, out, ticket);
     return cudaGetLastError();
 }
 
