@@ -147,6 +147,7 @@ struct TcArgs {
     const ColMax* colmax;
     TestParams tp;
     int mode;
+    int csplit;               // mode 1: ranges of column tiles per row block (set by launch_tc)
     int variant;              // mode 0 epilogue variant TC_SV_FULL / HALF / C32
     uint32_t* cand;           // mode 0: TC_GROUPS x TC_LIST x n quad entries (group, slot, row), common.cuh
     int ebits;                // low bits of an entry holding the quad index and mask: ceil(log2 ceil(k / 4)) + 4

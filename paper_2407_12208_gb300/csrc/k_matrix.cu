@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "df.cuh"
 #include "internal.h"
 
 namespace km {
@@ -178,8 +179,8 @@ KM_DEV float fallback_value(const float* x, const float* c, int d) {
     }
 }
 
-// Flagged pairs of the distance matrix (marked -1): the fallback's values,
-// from the bounded queue, or, when more pairs were flagged than it holds, by
+// Flagged pairs of the distance matrix (marked -1): the values of the
+// binary32 and low-format fallbacks, from the bounded queue, or, when more pairs were flagged than it holds, by
 // a scan of D for the marks.
 template <int FB, int FMT>
 __global__ void k_patch_flagged(const float* __restrict__ X, const float* __restrict__ C, int k, int d,
@@ -206,17 +207,123 @@ __global__ void k_patch_flagged(const float* __restrict__ X, const float* __rest
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ev += __shfl_xor_sync(0xffffffffu, ev, off);
-    if ((threadIdx.x & 31) == 0 && ev) {
-        if (FB == 0) atomicAdd(&cnt->fp64_evals, ev);
-        else atomicAdd(&cnt->fp32_evals, ev);
+    if ((threadIdx.x & 31) == 0 && ev) atomicAdd(&cnt->fp32_evals, ev);
+}
+
+// The binary64 fallback's value, rounded to the matrix's binary32, without the
+// narrow FP64 pipe: the pair's double-float distance (df.cuh) lies within eps
+// (relative) of the binary64 sum, and where both ends of that interval round
+// to the same binary32 number, that is the value.  eps covers the chain of
+// `levels` combinations (below 3 2^-48 each), the squares (2^-46) and the
+// binary64 sum's own rounding ((d + 2) 2^-53).  Values near a rounding boundary
+// (one in about 2^17), tiny ones (squares below binary32's normal range) and
+// what is no number take binary64 in the oracle's order.
+KM_DEV float patch_eps(int d, int levels) { return (float)(3 * levels + 5) * 0x1p-48f + (float)(d + 2) * 0x1p-53f; }
+KM_DEV bool patch_sure(DF r, float eps) {
+    const float e = r.hi * eps * 1.01f;
+    return r.hi >= 0x1p-60f && r.hi < INFINITY && __fadd_rn(r.hi, __fadd_ru(r.lo, e)) == r.hi &&
+           __fadd_rn(r.hi, __fsub_rd(r.lo, e)) == r.hi;
+}
+
+constexpr int PT = 32;    // scan: tile of 32 rows x 32 centres, a thread per centre and four rows
+constexpr int PT_DK = 64;  // coordinates staged at a time
+constexpr int PT_LD = PT_DK + 4;
+// Flagged pairs from the queue (eight lanes each), or, when more were flagged
+// than it holds, by tiles of D that hold a mark (-1).  Bound by the FP32 pipe
+// (about 16 lane operations per pair and coordinate); 5000 x 5000, d = 128:
+// all pairs 31.2 -> 2.2 ms, 2500 pairs 50 -> 6.6 us (binary64 throughout before).
+__global__ void __launch_bounds__(256) k_patch_fp64(const float* __restrict__ X, const float* __restrict__ C, int k, int d,
+                                                    const int2* __restrict__ queue,
+                                                    const unsigned long long* __restrict__ qlen, int64_t cap,
+                                                    float* __restrict__ D, int64_t n, DevCounters* cnt) {
+    chain_enter();
+    __shared__ __align__(16) float xs[PT][PT_LD], cs[PT][PT_LD];
+    const int64_t len = (int64_t)*qlen;
+    const int lane = threadIdx.x & 31;
+    unsigned ev = 0;
+    if (len <= cap) {
+        const int sl = lane & 7;
+        const int64_t ng = (int64_t)gridDim.x * (blockDim.x / 8);
+        const float eps = patch_eps(d, ((d + 3) / 4 + 7) / 8 + 3);
+        const bool vec = d % 4 == 0 && (((uintptr_t)X | (uintptr_t)C) & 15) == 0;
+        for (int64_t t0 = (int64_t)blockIdx.x * (blockDim.x / 8) + (threadIdx.x / 32) * 4; t0 < len; t0 += ng) {
+            const int64_t t = t0 + (lane >> 3);
+            const int2 pr = queue[t < len ? t : t0];
+            const float* x = X + (int64_t)pr.x * d;
+            const float* c = C + (int64_t)pr.y * d;
+            DF r{0.0f, 0.0f};
+            for (int q = sl; 4 * q < d; q += 8) {
+                float4 xv, cv;
+                if (vec) {
+                    xv = reinterpret_cast<const float4*>(x)[q];
+                    cv = reinterpret_cast<const float4*>(c)[q];
+                } else {
+                    xv = make_float4(x[4 * q], 4 * q + 1 < d ? x[4 * q + 1] : 0.f, 4 * q + 2 < d ? x[4 * q + 2] : 0.f,
+                                     4 * q + 3 < d ? x[4 * q + 3] : 0.f);
+                    cv = make_float4(c[4 * q], 4 * q + 1 < d ? c[4 * q + 1] : 0.f, 4 * q + 2 < d ? c[4 * q + 2] : 0.f,
+                                     4 * q + 3 < d ? c[4 * q + 3] : 0.f);
+                }
+                r = df_combine(r, df_chunk(xv, cv));
+            }
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) r = df_combine(r, df_shfl_xor(r, off));
+            if (sl == 0 && t < len) {
+                D[(int64_t)pr.x * k + pr.y] = patch_sure(r, eps) ? r.hi : fallback_value<0, 0>(x, c, d);
+                ev++;
+            }
+        }
+    } else {
+        const int64_t ntr = (n + PT - 1) / PT, ntc = (k + PT - 1) / PT;
+        const int cj = threadIdx.x & 31, ri = threadIdx.x >> 5;  // centre cj, rows ri + 8 i
+        const float eps = patch_eps(d, (d + 3) / 4);
+        for (int64_t tile = blockIdx.x; tile < ntr * ntc; tile += gridDim.x) {
+            const int64_t i0 = tile / ntc * PT, j0 = tile % ntc * PT;
+            const int64_t j = j0 + cj;
+            bool mark[4], any = false;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const int64_t row = i0 + ri + 8 * i;
+                mark[i] = row < n && j < k && D[row * k + j] < 0.0f;
+                any |= mark[i];
+            }
+            if (!__syncthreads_or(any)) continue;
+            DF r[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) r[i] = DF{0.0f, 0.0f};
+            for (int l0 = 0; l0 < d; l0 += PT_DK) {
+                const int w = min(PT_DK, d - l0), w4 = (w + 3) & ~3;
+                __syncthreads();
+                for (int e = threadIdx.x; e < PT * w4; e += 256) {
+                    const int q = e / w4, l = e - q * w4;
+                    xs[q][l] = l < w && i0 + q < n ? X[(i0 + q) * d + l0 + l] : 0.0f;
+                    cs[q][l] = l < w && j0 + q < k ? C[(j0 + q) * d + l0 + l] : 0.0f;
+                }
+                __syncthreads();
+                for (int l = 0; l < w4; l += 4) {
+                    const float4 cv = *reinterpret_cast<const float4*>(&cs[cj][l]);
+#pragma unroll
+                    for (int i = 0; i < 4; i++)
+                        r[i] = df_combine(r[i], df_chunk(*reinterpret_cast<const float4*>(&xs[ri + 8 * i][l]), cv));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                if (mark[i]) {
+                    const int64_t row = i0 + ri + 8 * i;
+                    D[row * k + j] = patch_sure(r[i], eps) ? r[i].hi : fallback_value<0, 0>(X + row * d, C + j * d, d);
+                    ev++;
+                }
+        }
     }
+    ev = __reduce_add_sync(0xffffffffu, ev);
+    if (lane == 0 && ev) atomicAdd(&cnt->fp64_evals, (unsigned long long)ev);
 }
 
 cudaError_t launch_patch_flagged(int fb, int fmt, const float* X, const float* C, int64_t n, int k, int d,
                                  const int2* queue, const unsigned long long* qlen, int64_t cap, float* D,
                                  DevCounters* cnt, int num_sms, cudaStream_t st) {
     const unsigned blocks = (unsigned)num_sms * 8;
-    if (fb == 0) klaunch(k_patch_flagged<0, 0>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
+    if (fb == 0) klaunch(k_patch_fp64, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
     else if (fb == 1) klaunch(k_patch_flagged<1, 0>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
     else if (fmt == 0) klaunch(k_patch_flagged<2, 0>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);
     else klaunch(k_patch_flagged<2, 1>, blocks, 256, 0, st, X, C, k, d, queue, qlen, cap, D, n, cnt);

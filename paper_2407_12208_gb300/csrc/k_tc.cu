@@ -200,6 +200,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t nrb = (nrows + TC_BM - 1) / TC_BM;
     const int NT = (a.k + BN - 1) / BN;
+    // work items: a row block, or (distance matrix, few row blocks) one of
+    // a.csplit ranges of its column tiles
+    const int csplit = MODE == 1 ? a.csplit : 1;
+    const int64_t nitem = nrb * csplit;
+    auto item_rows = [&](int64_t it, int& t0, int& t1) -> int64_t {
+        if (MODE == 0) {
+            t0 = 0;
+            t1 = NT;
+            return it;
+        }
+        const int64_t rb = it / csplit;
+        const int part = (int)(it - rb * csplit);
+        t0 = (int)((int64_t)NT * part / csplit);
+        t1 = (int)((int64_t)NT * (part + 1) / csplit);
+        return rb;
+    };
     constexpr uint32_t ESIZE = (FMT == 2) ? 1 : 2;
     constexpr int ATOM_ELEMS = 128 / ESIZE;
     unsigned* status = &a.cnt->status;
@@ -230,7 +246,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             int64_t bload = 0;
             int iter = 0;
             bool ok = true;
-            for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, iter++) {
+            for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x, iter++) {
+                int t0, t1;
+                const int64_t rb = item_rows(it, t0, t1);
                 const int ab = iter % L.NA;
                 if (iter >= L.NA) ok = mbar_wait(&a_empty[ab], ((iter / L.NA) - 1) & 1, abort_flag, status);
                 if (!ok) break;
@@ -238,7 +256,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 for (int kc = 0; kc < a.kchunks; kc++)
                     tma_load_2d(sA + (size_t)ab * L.a_bytes + (size_t)kc * TC_BM * 128, &tmX, &a_full[ab],
                                 kc * ATOM_ELEMS, (int)(rb * TC_BM));
-                for (int nt = 0; nt < NT; nt++, bload++) {
+                for (int nt = t0; nt < t1; nt++, bload++) {
                     const int s = (int)(bload % L.NS);
                     if (bload >= L.NS) ok = mbar_wait(&b_empty[s], ((bload / L.NS) - 1) & 1, abort_flag, status);
                     if (!ok) break;
@@ -258,11 +276,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             int64_t bcons = 0, tcount = 0;
             int iter = 0;
             bool ok = true;
-            for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, iter++) {
+            for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x, iter++) {
+                int t0, t1;
+                item_rows(it, t0, t1);
                 const int ab = iter % L.NA;
                 ok = mbar_wait(&a_full[ab], (iter / L.NA) & 1, abort_flag, status);
                 if (!ok) break;
-                for (int nt = 0; nt < NT; nt++, bcons++, tcount++) {
+                for (int nt = t0; nt < t1; nt++, bcons++, tcount++) {
                     const int s = (int)(bcons % L.NS);
                     ok = mbar_wait(&b_full[s], (bcons / L.NS) & 1, abort_flag, status);
                     if (!ok) break;
@@ -311,8 +331,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const float lscale = __uint_as_float((uint32_t)(127 + a.ebits - 23) << 23);  // 2^(ebits - 23)
         unsigned long long nflag_total = 0;
         bool ok = true;
-        int iter = 0;
-        for (int64_t rb = blockIdx.x; rb < nrb && ok; rb += gridDim.x, iter++) {
+        int64_t tbase = 0;  // tiles of the items before this one
+        for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x) {
+            int t0, t1;
+            const int64_t rb = item_rows(it, t0, t1);
             const int64_t row = rb * TC_BM + r_in;
             const bool valid = row < nrows;
             float4 xs = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -347,15 +369,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             float m = INFINITY;
             int cnt = 0, ovf = 0, nflag = 0;
 
-            for (int nt = 0; nt < NT; nt++) {
-                const int64_t tc = (int64_t)iter * NT + nt;
+            for (int nt = t0; nt < t1; nt++) {
+                const int64_t tc = tbase + (nt - t0);
                 if ((int)(tc % TC_NG) != g) continue;
                 const int buf = (int)(tc % NBUF);
                 ok = mbar_wait(&acc_full[buf], (uint32_t)((tc / NBUF) & 1), abort_flag, status);
                 if (!ok) break;
                 tc_fence_after();
                 const int nch = min(BN / 32, (a.k - nt * BN + 31) / 32);
-                const uint32_t tbase = tmem_base + lane_addr + (uint32_t)(buf * BN);
+                const uint32_t tbase_addr = tmem_base + lane_addr + (uint32_t)(buf * BN);
                 if (MODE == 0) {
                     // TC_CW chunks of 32 columns per step (padded columns have q = +inf:
                     // they never qualify)
@@ -366,7 +388,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         uint32_t v[TC_CW][32];
                         __syncwarp();
 #pragma unroll
-                        for (int c = 0; c < TC_CW; c++) tmem_ld32_async(tbase + (uint32_t)((ch + c) * 32), v[c]);
+                        for (int c = 0; c < TC_CW; c++) tmem_ld32_async(tbase_addr + (uint32_t)((ch + c) * 32), v[c]);
                         const float4* q4 = reinterpret_cast<const float4*>(qg + col0);
                         float4 qv[NQ];
 #pragma unroll
@@ -536,55 +558,92 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     }
                 } else {
                     // distance-matrix mode: Alg. 2's d = max(d^, 0) and its flag, every
-                    // pair; when K fits two 128-byte atoms the warp's 32 rows x 32
-                    // columns go through shared memory (lane = row, stride 33:
-                    // conflict-free both ways) so that each store writes 32
-                    // consecutive columns of one row
-                    float* tr = reinterpret_cast<float*>(smem + L.stage_off) + (size_t)(warp - 2) * 32 * 33;
+                    // pair.  Flags as a 32-bit mask per row and chunk: the queue and the
+                    // flag words are updated once per warp and row.  When K fits two
+                    // 128-byte atoms the warp's 32 rows x 32 columns go through shared
+                    // memory (quad q of row r at q ^ (r mod 8): conflict-free 16-byte
+                    // accesses both ways) so that stores write whole lines.
+                    const uint32_t tr = smem_u32(smem) + (uint32_t)L.stage_off + (uint32_t)((warp - 2) * tc_stage_warp_bytes(SV));
                     const int64_t row_w = rb * TC_BM + quarter * 32;  // the warp's first row
+                    const bool vec = (a.k & 3) == 0 && ((uintptr_t)a.D & 15) == 0;
                     for (int ch = 0; ch < nch; ch++) {
                         const int col0 = nt * BN + ch * 32;
                         uint32_t v[32];
                         __syncwarp();
-                        tmem_ld32_async(tbase + (uint32_t)(ch * 32), v);
-                        tmem_wait_ld(v);
+                        tmem_ld32_async(tbase_addr + (uint32_t)(ch * 32), v);
                         const float4* q4 = reinterpret_cast<const float4*>(qg + col0);
                         const float4* s4 = reinterpret_cast<const float4*>(a.spad + col0);
+                        float4 qv[8];
+#pragma unroll
+                        for (int t4 = 0; t4 < 8; t4++) qv[t4] = __ldg(q4 + t4);
+                        tmem_wait_ld(v);
+                        float dh[32];
+                        float least = INFINITY;
 #pragma unroll
                         for (int t4 = 0; t4 < 8; t4++) {
-                            const float4 qq = __ldg(q4 + t4);
                             const float4 sc = FMT == 2 ? __ldg(s4 + t4) : make_float4(1.f, 1.f, 1.f, 1.f);
-                            const float ev[4] = {fmaf(__uint_as_float(v[4 * t4 + 0]) * sc.x, neg2s, qq.x),
-                                                 fmaf(__uint_as_float(v[4 * t4 + 1]) * sc.y, neg2s, qq.y),
-                                                 fmaf(__uint_as_float(v[4 * t4 + 2]) * sc.z, neg2s, qq.z),
-                                                 fmaf(__uint_as_float(v[4 * t4 + 3]) * sc.w, neg2s, qq.w)};
+                            dh[4 * t4 + 0] = fmaxf(p + fmaf(__uint_as_float(v[4 * t4 + 0]) * sc.x, neg2s, qv[t4].x), 0.0f);
+                            dh[4 * t4 + 1] = fmaxf(p + fmaf(__uint_as_float(v[4 * t4 + 1]) * sc.y, neg2s, qv[t4].y), 0.0f);
+                            dh[4 * t4 + 2] = fmaxf(p + fmaf(__uint_as_float(v[4 * t4 + 2]) * sc.z, neg2s, qv[t4].z), 0.0f);
+                            dh[4 * t4 + 3] = fmaxf(p + fmaf(__uint_as_float(v[4 * t4 + 3]) * sc.w, neg2s, qv[t4].w), 0.0f);
+                            least = fminf(fmin3(least, dh[4 * t4], dh[4 * t4 + 1]), fminf(dh[4 * t4 + 2], dh[4 * t4 + 3]));
+                        }
+                        // (F is -inf for rows past n; columns past k are +inf)
+                        if (__any_sync(0xffffffffu, least <= F)) {
+                            unsigned fl = 0;
 #pragma unroll
-                            for (int c = 0; c < 4; c++) {
-                                const int t = 4 * t4 + c;
-                                const int j = col0 + t;
-                                const float dh = fmaxf(p + ev[c], 0.0f);
-                                const bool fl = valid && j < a.k && (dh <= F) && KM_PAIR_FLAGGED(j, dh);
-                                if (fl) {
-                                    nflag++;
-                                    const unsigned long long pos = atomicAdd(a.flag_queue_len, 1ull);
-                                    if ((int64_t)pos < a.flag_queue_cap) a.flag_queue[pos] = make_int2((int)row, j);
-                                    if (a.flag_bits) {
-                                        const unsigned long long bit = (unsigned long long)row * a.k + j;
-                                        atomicOr(&a.flag_bits[bit >> 5], 1u << (bit & 31));
-                                    }
+                            for (int t = 0; t < 32; t++)
+                                if (dh[t] <= F && col0 + t < a.k && KM_PAIR_FLAGGED(col0 + t, dh[t])) {
+                                    fl |= 1u << t;
+                                    dh[t] = -1.0f;  // until the fallback's value replaces it
                                 }
-                                // a flagged pair is marked -1 until the fallback's value replaces it
-                                if constexpr (STG) tr[lane * 33 + t] = fl ? -1.0f : dh;
-                                else if (valid && j < a.k) a.D[(size_t)row * a.k + j] = fl ? -1.0f : dh;
+                            const int c = __popc(fl);
+                            nflag += c;
+                            int incl = c;
+#pragma unroll
+                            for (int off = 1; off < 32; off <<= 1) {
+                                const int o = __shfl_up_sync(0xffffffffu, incl, off);
+                                if (lane >= off) incl += o;
+                            }
+                            unsigned long long pos = 0;
+                            if (lane == 31 && incl) pos = atomicAdd(a.flag_queue_len, (unsigned long long)incl);
+                            pos = __shfl_sync(0xffffffffu, pos, 31) + (unsigned long long)(incl - c);
+                            for (unsigned m = fl; m; m &= m - 1, pos++)
+                                if ((int64_t)pos < a.flag_queue_cap) a.flag_queue[pos] = make_int2((int)row, col0 + __ffs(m) - 1);
+                            if (fl && a.flag_bits) {
+                                const unsigned long long bit = (unsigned long long)row * a.k + col0;
+                                const unsigned sh = (unsigned)(bit & 31);
+                                atomicOr(&a.flag_bits[bit >> 5], fl << sh);
+                                if (sh && fl >> (32 - sh)) atomicOr(&a.flag_bits[(bit >> 5) + 1], fl >> (32 - sh));
                             }
                         }
-                        if constexpr (!STG) continue;  // (wide rows: no room to stage)
+                        if constexpr (!STG) {  // (wide rows: no room to stage)
+                            if (valid)
+                                for (int t = 0; t < 32; t++)
+                                    if (col0 + t < a.k) a.D[(size_t)row * a.k + col0 + t] = dh[t];
+                            continue;
+                        }
+#pragma unroll
+                        for (int q = 0; q < 8; q++)
+                            st_shared_v4(tr + lane * 128 + ((q ^ (lane & 7)) << 4), dh[4 * q], dh[4 * q + 1], dh[4 * q + 2],
+                                         dh[4 * q + 3]);
                         __syncwarp();
-                        const int j = col0 + lane;
-#pragma unroll 4
-                        for (int r = 0; r < 32; r++) {
-                            const float val = tr[r * 33 + lane];
-                            if (row_w + r < a.n && j < a.k) a.D[(size_t)(row_w + r) * a.k + j] = val;
+                        const int q = lane & 7, j = col0 + 4 * q;
+#pragma unroll
+                        for (int r0 = 0; r0 < 32; r0 += 4) {
+                            const int r = r0 + (lane >> 3);
+                            const float4 val = ld_shared_v4(tr + r * 128 + ((q ^ (r & 7)) << 4));
+                            if (row_w + r < nrows) {
+                                float* dst = a.D + (size_t)(row_w + r) * a.k + j;
+                                if (vec) {
+                                    if (j < a.k) *reinterpret_cast<float4*>(dst) = val;
+                                } else {
+                                    if (j + 0 < a.k) dst[0] = val.x;
+                                    if (j + 1 < a.k) dst[1] = val.y;
+                                    if (j + 2 < a.k) dst[2] = val.z;
+                                    if (j + 3 < a.k) dst[3] = val.w;
+                                }
+                            }
                         }
                     }
                 }
@@ -592,6 +651,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[buf]);
             }
+            tbase += t1 - t0;
             if (!ok) break;
             if (valid && MODE == 0) {
                 // the row's list (slot-major: consecutive rows side by side), its
@@ -664,8 +724,8 @@ static cudaError_t launch_one(const CUtensorMap& mx, const CUtensorMap& mc, cons
     if (L.NS < 2) return cudaErrorInvalidConfiguration;
     cudaError_t e = allow_max_smem(k_tc<FMT, BN, MODE, SV>);
     if (e != cudaSuccess) return e;
-    const int64_t nrb = (a.n + TC_BM - 1) / TC_BM;
-    const int grid = (int)std::min<int64_t>(nrb, (int64_t)num_sms);
+    const int64_t nitem = (a.n + TC_BM - 1) / TC_BM * (MODE == 1 ? a.csplit : 1);
+    const int grid = (int)std::min<int64_t>(nitem, (int64_t)num_sms);
     klaunch(k_tc<FMT, BN, MODE, SV>, grid, TC_THREADS, L.total, st, mx, mc, a);
     return cudaGetLastError();
 }
@@ -687,8 +747,15 @@ static cudaError_t launch_fmt(const CUtensorMap& mx, const CUtensorMap& mc, cons
     }
 }
 
-cudaError_t launch_tc(const void* Xq, const void* Cq, int ldq, const TcArgs& a, int num_sms, cudaStream_t st) {
+cudaError_t launch_tc(const void* Xq, const void* Cq, int ldq, const TcArgs& args, int num_sms, cudaStream_t st) {
+    TcArgs a = args;
     const int bn = pick_bn(a.kchunks, a.k);
+    // the distance matrix of few row blocks: about eight items per SM, so that
+    // neither idle SMs nor the last round weigh (5000 x 5000, 40 row blocks: 267
+    // us with a block of rows per SM and a flag call per value; 38 us now)
+    const int64_t nrb = (a.n + TC_BM - 1) / TC_BM;
+    const int nt = (a.k + bn - 1) / bn;
+    a.csplit = (int)std::max<int64_t>(1, std::min<int64_t>(nt, (8 * (int64_t)num_sms + nrb - 1) / nrb));
     CUtensorMap mx, mc;
     cudaError_t e = make_map(&mx, Xq, a.fmt, a.n, ldq, TC_BM);
     if (e != cudaSuccess) return e;

@@ -189,3 +189,26 @@ def test_seeding_chunks(ctx, n, d, offset):
     oidx, margin = oracle.kmeanspp(X, workloads.seed_uniforms(k, seed=d), follow=idx)
     assert np.array_equal(idx[margin > 1e-9], oidx[margin > 1e-9])
     assert np.array_equal(C.cpu().numpy(), X[idx])
+
+
+# the distance matrix: column ranges of few row blocks, 16-byte and single stores (k % 4),
+# unstaged wide rows, flag masks that straddle words, and the binary64 fallback's values
+# (bit for bit the rounded binary64 sums) from the queue and by the scan of D
+@pytest.mark.parametrize("low,test,n,d,k,near", [("fp16", "tc", 130, 128, 129, 0.5), ("bf16", "tc", 300, 64, 300, 0.1),
+                                                 ("bf16", "paper", 257, 128, 255, 0.0), ("bf16", "paper", 1200, 100, 1100, 0.3),
+                                                 ("fp16", "tc", 5000, 37, 33, 0.9), ("fp16", "tc", 500, 200, 130, 0.5),
+                                                 ("e4m3", "tc", 200, 128, 131, 0.5), ("bf16", "tc", 64, 9, 1, 1.0),
+                                                 ("fp16", "tc", 20000, 16, 512, 0.02)])
+def test_distance_matrix_edges(ctx, low, test, n, d, k, near):
+    import paper_2407_12208_gb300 as pkg
+    X, C = workloads.near_far(n, d, near, seed=n + k)
+    C = C[:k].copy()
+    C[0] = X[0]
+    D, bits, nf = ctx.distances(_dev(X), _dev(C), pkg.params(low, test))
+    D, bits = D.cpu().numpy(), bits.cpu().numpy().view(np.uint32)
+    fl = np.unpackbits(bits.view(np.uint8), bitorder="little")[: n * k].reshape(n, k).astype(bool)
+    assert fl.sum() == nf and fl[0, 0] and not (D < 0).any()
+    want = oracle.dist_direct(X, C)
+    assert np.array_equal(D[fl], want[fl].astype(np.float32))
+    if low != "e4m3" and (~fl).any():  # Eq. (quantis-rel-bound-expand): unflagged pairs to 1 / (rho - 1)
+        assert (np.abs(D[~fl] - want[~fl]) <= 0.26 * want[~fl]).all()
