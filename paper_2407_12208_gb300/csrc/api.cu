@@ -259,19 +259,25 @@ struct UpdateWs {
     long long* sums;
     long long* counts;
     unsigned* absmax;
+    ZeroWords zero;  // what an update starts from zero: the four below and bar
     double* shift;
+    unsigned* bar;
     void* esel;
     int* iscratch;
     int32_t* perm;
 };
 UpdateWs carve_update(Carve& cv, int64_t n, int d, int k) {
     UpdateWs u{};
-    u.sums = cv.take<long long>((size_t)k * d);
-    u.counts = cv.take<long long>((size_t)k);
+    // (one span: sums, counts, shift, barrier, the label counts at iscratch's start)
+    const size_t words = 2 * ((size_t)k * d + k) + 4 + k;
+    u.sums = reinterpret_cast<long long*>(cv.take<unsigned>(words + 3 * (size_t)k + 2));
+    u.counts = u.sums + (size_t)k * d;
+    u.shift = reinterpret_cast<double*>(u.counts + k);
+    u.bar = reinterpret_cast<unsigned*>(u.shift + 1);
+    u.iscratch = reinterpret_cast<int*>(u.bar + 2);
+    u.zero = ZeroWords{{reinterpret_cast<unsigned*>(u.sums), nullptr}, {(int64_t)words, 0}};
     u.absmax = cv.take<unsigned>(1);
-    u.shift = cv.take<double>(1);
     u.esel = cv.take<unsigned char>(empty_select_bytes(k));
-    u.iscratch = cv.take<int>((size_t)4 * k + 2);
     u.perm = cv.take<int32_t>((size_t)n);
     return u;
 }
@@ -387,10 +393,10 @@ bool aligned256(const void* p) { return ((uintptr_t)p & 255) == 0; }
 // statistics (per-row power-of-two scales for E4M3), the column maxima of the
 // bound, q_j and the scales padded to the tile width.
 km_status prepare(km_ctx* ctx, const float* X, int64_t n, const float* C, int k, int d, int fmt, const AssignWs& w,
-                  unsigned* x_absmax, cudaStream_t st) {
+                  unsigned* x_absmax, const ZeroWords& zero, cudaStream_t st) {
     int nl = 0;
     CK(launch_prepare(X, n, w.Xq, w.xstat, w.xscale, x_absmax, C, k, w.Cq, w.cstat, w.cscale, w.colmax, w.qpad, w.spad,
-                      kpad_of(k), &w.cnt->prep_ticket, d, fmt, ldq_of(fmt, d), st, &nl));
+                      kpad_of(k), &w.cnt->prep_ticket, w.cnt->colacc, d, fmt, ldq_of(fmt, d), zero, st, &nl));
     ctx->launches += (uint64_t)nl;
     return KM_OK;
 }
@@ -412,18 +418,20 @@ int screen_variant(km_ctx* ctx, int fmt, int kchunks, int k, int64_t n) {
     return kchunks == 2 ? TC_SV_HALF : TC_SV_FULL;
 }
 
-// The caller has zeroed the counters of one assignment (zero_counters, or all).
+// zero: what the call's later kernels add to, cleared here; the counters of one
+// assignment must be zero, by the caller or by `zero`.
 // c_prepared: the workspace already holds C's low-precision copy, statistics
 // and column maxima for this C and format (later row chunks of one call).
 km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int k, int d, const km_params* p,
-                     int32_t* labels, double* min_dist, const AssignWs& w, const Centred& cen, bool x_prepared,
-                     cudaStream_t st, unsigned* x_absmax = nullptr, bool c_prepared = false) {
+                     int32_t* labels, double* min_dist, const AssignWs& w, const Centred& cen, const ZeroWords& zero,
+                     bool x_prepared, cudaStream_t st, unsigned* x_absmax = nullptr, bool c_prepared = false) {
     const TestParams tp = make_tp(p, d);
     km_status s = KM_OK;
     if (p->low == KM_FP64_DIRECT || p->low == KM_FP32_DIRECT) {
         const bool acc64 = p->low == KM_FP64_DIRECT;
         {
             PhaseScope ps(ctx, KM_PHASE_DIRECT, st);
+            if (zero.n[0]) CK(cudaMemsetAsync(zero.p[0], 0, 4 * (size_t)zero.n[0], st));
             KL(1, launch_direct_assign(acc64, X, n, C, k, d, nullptr, nullptr, labels, min_dist, w.cnt, tp.gamma32,
                                        ctx->num_sms, st, x_absmax));
         }
@@ -435,7 +443,7 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
     {
         PhaseScope ps(ctx, KM_PHASE_QUANTISE, st);
         if (!c_prepared) {
-            if ((s = prepare(ctx, x_prepared ? nullptr : X, n, C, k, d, fmt, w, x_absmax, st)) != KM_OK) return s;
+            if ((s = prepare(ctx, x_prepared ? nullptr : X, n, C, k, d, fmt, w, x_absmax, zero, st)) != KM_OK) return s;
         } else if (!x_prepared) {
             KL(1, launch_quantize(X, n, d, fmt, ldq, w.Xq, w.xstat, w.xscale, st, x_absmax));
         }
@@ -515,14 +523,14 @@ km_status refine_winners(km_ctx* ctx, const float* X, int64_t n, int d, const fl
     return KM_OK;
 }
 
-// The centre update's accumulation; md_wd (nullable) also receives the rows'
+// The centre update's accumulation (u.zero is zero); md_wd (nullable) also receives the rows'
 // distances to their centres C_wd (the winner refinement, from the same pass
 // over X where the kernel allows).
 km_status accumulate(km_ctx* ctx, const float* X, int64_t n, int d, const int32_t* labels, int k, const UpdateWs& u,
                      const float* C_wd, double* md_wd, cudaStream_t st) {
     int nl = 0;
     CK(launch_accumulate(X, n, d, labels, k, u.absmax, u.sums, u.counts, u.iscratch, u.perm, ctx->num_sms, st, C_wd,
-                         md_wd, &nl));
+                         md_wd, &nl, 0, true));
     ctx->launches += (uint64_t)nl;
     return KM_OK;
 }
@@ -533,7 +541,7 @@ km_status finalize(km_ctx* ctx, const UpdateWs& u, int64_t n, int k, int d, cons
                    bool want_shift) {
     int nl = 0;
     CK(launch_finalize(u.sums, u.counts, u.absmax, n, k, d, C_old, p->empty, X, md, C_new, counts,
-                       want_shift ? u.shift : nullptr, u.esel, &cnt->status, ctx->num_sms, st, &nl));
+                       want_shift ? u.shift : nullptr, u.bar, u.esel, &cnt->status, ctx->num_sms, st, &nl));
     ctx->launches += (uint64_t)nl;
     return KM_OK;
 }
@@ -643,7 +651,7 @@ km_status km_choose_low(km_ctx* ctx, const float* X, int64_t n, const float* C, 
         return fail(ctx, KM_EUNSUPPORTED, "no tensor-core path for d=%d, k=%d", d, k);
     constexpr int kSample = 2048;
     Carve cv{(char*)ws};
-    unsigned long long* acc = cv.take<unsigned long long>(5);
+    unsigned long long* acc = cv.take<unsigned long long>(10);
     unsigned* ticket = reinterpret_cast<unsigned*>(acc + 4);
     ColMax* colmax = cv.take<ColMax>(1);
     void* Cq = cv.take<char>((size_t)k * ldq_of(1, d) * 2);
@@ -654,7 +662,7 @@ km_status km_choose_low(km_ctx* ctx, const float* X, int64_t n, const float* C, 
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
-    CK(cudaMemsetAsync(acc, 0, 5 * sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(acc, 0, 10 * sizeof(unsigned long long), st));
     const int fmts[2] = {1, 2};  // bf16, E4M3
     for (int f = 0; f < 2; f++) {
         const int fmt = fmts[f];
@@ -664,7 +672,7 @@ km_status km_choose_low(km_ctx* ctx, const float* X, int64_t n, const float* C, 
         q.low = fmt == 2 ? KM_E4M3 : KM_BF16;
         int nl = 0;
         CK(launch_prepare(nullptr, 0, nullptr, nullptr, nullptr, nullptr, C, k, Cq, cstat, cscale, colmax, qpad, spad,
-                          kpad_of(k), ticket, d, fmt, ldq_of(fmt, d), st, &nl));
+                          kpad_of(k), ticket, ticket + 1, d, fmt, ldq_of(fmt, d), ZeroWords{}, st, &nl));
         ctx->launches += (uint64_t)nl;
         KL(1, launch_predict_candidates(X, n, d, C, k, fmt, colmax, make_tp(&q, d), kSample, acc + 2 * f,
                                         ctx->num_sms, st));
@@ -710,7 +718,7 @@ km_status km_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int 
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     CK(cudaMemsetAsync(w.cnt, 0, sizeof(DevCounters), st));
-    s = run_assign(ctx, X, n, C, k, d, p, labels, md, w, cen, false, st);
+    s = run_assign(ctx, X, n, C, k, d, p, labels, md, w, cen, ZeroWords{}, false, st);
     if (s != KM_OK) return s;
     if ((s = refine_winners(ctx, X, n, d, C, p, labels, md, st)) != KM_OK) return s;
     KL(1, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, &w.cnt->sum_ticket, st));
@@ -846,7 +854,7 @@ km_status km_distances(km_ctx* ctx, const float* X, int64_t n, const float* C, i
         const int fmt = fmt_of(p->low);
         const int ldq = ldq_of(fmt, d);
         const int esz = fmt == 2 ? 1 : 2;
-        if ((s = prepare(ctx, X, n, C, k, d, fmt, w, nullptr, st)) != KM_OK) return s;
+        if ((s = prepare(ctx, X, n, C, k, d, fmt, w, nullptr, ZeroWords{}, st)) != KM_OK) return s;
         TcArgs a{};
         a.n = n; a.k = k; a.d = d; a.fmt = fmt;
         a.kchunks = (ldq * esz + 127) / 128;
@@ -892,6 +900,7 @@ km_status km_update_centroids(km_ctx* ctx, const float* X, int64_t n, int d, con
     {
         PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
         KL(1, launch_absmax(X, n * (int64_t)d, u.absmax, st));
+        CK(cudaMemsetAsync(u.zero.p[0], 0, 4 * (size_t)u.zero.n[0], st));
         if ((s = accumulate(ctx, X, n, d, labels, k, u, nullptr, nullptr, st)) != KM_OK) return s;
         if ((s = finalize(ctx, u, n, k, d, C_old, p, X, min_dist, C_new, counts, cnt, st, shift_host != nullptr)) != KM_OK)
             return s;
@@ -961,10 +970,11 @@ km_status km_update_finalize(km_ctx* ctx, const int64_t* sums, const int64_t* co
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     CK(cudaMemsetAsync(cnt, 0, sizeof(DevCounters), st));
+    CK(cudaMemsetAsync(u.shift, 0, sizeof(double), st));
     CK(cudaMemcpyAsync(u.absmax, &absmax_bits, sizeof(unsigned), cudaMemcpyHostToDevice, st));
     int nl = 0;
     CK(launch_finalize(reinterpret_cast<const long long*>(sums), reinterpret_cast<const long long*>(counts), u.absmax,
-                       n_total, k, d, C_old, KM_EMPTY_KEEP, nullptr, nullptr, C_new, nullptr, u.shift, u.esel,
+                       n_total, k, d, C_old, KM_EMPTY_KEEP, nullptr, nullptr, C_new, nullptr, u.shift, u.bar, u.esel,
                        &cnt->status, ctx->num_sms, st, &nl, n_total));
     ctx->launches += (uint64_t)nl;
     if (shift_host) {
@@ -984,11 +994,12 @@ km_status km_farthest_rows(km_ctx* ctx, const double* min_dist, int64_t n, int e
     Carve cv{(char*)ws};
     DevCounters* cnt = cv.take<DevCounters>(1);
     void* esel = cv.take<unsigned char>(empty_select_bytes(e));
+    unsigned* bar = cnt->colacc;  // (two words that nothing else uses here)
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     CK(cudaMemsetAsync(cnt, 0, sizeof(DevCounters), st));
-    KL(1, launch_farthest_rows(min_dist, n, e, reinterpret_cast<long long*>(rows), vals, esel, &cnt->status,
+    KL(1, launch_farthest_rows(min_dist, n, e, reinterpret_cast<long long*>(rows), vals, bar, esel, &cnt->status,
                                ctx->num_sms, st));
     return sync_status(ctx, cnt, st);
 }
@@ -1012,8 +1023,8 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
     CK(cudaMemsetAsync(w.cnt, 0, sizeof(DevCounters), st));
     // assignment (Alg. 3 step 1); its pass over X (quantisation, or the direct
     // distances) also yields max |x|
-    CK(cudaMemsetAsync(u.absmax, 0, sizeof(unsigned), st));
-    s = run_assign(ctx, X, n, C_old, k, d, p, labels, md, w, cen, false, st, u.absmax);
+    u.absmax = &w.cnt->absmax;
+    s = run_assign(ctx, X, n, C_old, k, d, p, labels, md, w, cen, u.zero, false, st, u.absmax);
     if (s != KM_OK) return s;
     // centre update (Eq. (center)) on the labels just computed; its pass over
     // X also refines the winners' distances (min_dist, binary64 accuracy)
@@ -1119,15 +1130,15 @@ km_status km_lloyd_step_host(km_ctx* ctx, const float* X_host, int64_t n, int d,
             CK(cudaEventRecord(ev_in[c], cs));
         }
         CK(cudaMemsetAsync(w.cnt, 0, sizeof(DevCounters), st));
-        CK(cudaMemsetAsync(u.absmax, 0, sizeof(unsigned), st));
+        u.absmax = &w.cnt->absmax;
         for (int c = 0; c < nch; c++) {
             const int64_t r0 = chunk_r0(c), rows = cend[c] - r0;
             cudaStream_t cs = ctx->copy_st[1];
             CK(cudaStreamWaitEvent(st, ev_in[c], 0));
-            if ((s = zero_counters(ctx, w.cnt, st)) != KM_OK) return s;
+            if (c > 0 && (s = zero_counters(ctx, w.cnt, st)) != KM_OK) return s;
             // the centres are prepared once, with the first chunk
-            s = run_assign(ctx, h.X + r0 * d, rows, h.C, k, d, p, h.labels + r0, h.min_dist + r0, w, cen, false, st,
-                           u.absmax, c > 0);
+            s = run_assign(ctx, h.X + r0 * d, rows, h.C, k, d, p, h.labels + r0, h.min_dist + r0, w, cen,
+                           c == 0 ? u.zero : ZeroWords{}, false, st, u.absmax, c > 0);
             if (s != KM_OK) return s;
             // the chunk's winner distances (binary64 accuracy) while the next
             // chunk is still on its way: the update's pass then only sums
@@ -1243,9 +1254,10 @@ __global__ void k_record_iteration(const double* __restrict__ sse_slot, const De
 static km_status lloyd_iteration(km_ctx* ctx, const float* X, int64_t n, int d, int k, const km_params* p,
                                  int32_t* labels, const LloydWs& L, const float* cur, float* nxt, double* sse_out,
                                  unsigned long long* flag_out, bool graph, int cap, cudaStream_t st) {
-    km_status s = zero_counters(ctx, L.a.cnt, st);
-    if (s != KM_OK) return s;
-    s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, true, st);
+    ZeroWords zero = L.u.zero;
+    zero.p[1] = reinterpret_cast<unsigned*>(&L.a.cnt->amb_count);
+    zero.n[1] = kAssignCounterBytes / 4;
+    km_status s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, zero, true, st);
     if (s != KM_OK) return s;
     if (!graph) CK(cudaMemcpyAsync(flag_out, &L.a.cnt->flagged, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
     PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
@@ -1316,7 +1328,7 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
     if (is_tc(p->low)) {
         const int fmt = fmt_of(p->low);
         PhaseScope ps(ctx, KM_PHASE_QUANTISE, st);
-        CK(cudaMemsetAsync(L.u.absmax, 0, sizeof(unsigned), st));
+        L.u.absmax = &L.a.cnt->absmax;
         KL(1, launch_quantize(X, n, d, fmt, ldq_of(fmt, d), L.a.Xq, L.a.xstat, L.a.xscale, st, L.u.absmax));
     } else {
         KL(1, launch_absmax(X, n * (int64_t)d, L.u.absmax, st));
@@ -1388,7 +1400,7 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
         CK(cudaStreamWaitEvent(st, ctx->graph_ev[1], 0));
     }
     if ((s = zero_counters(ctx, L.a.cnt, st)) != KM_OK) return s;
-    s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, true, st);
+    s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, ZeroWords{}, true, st);
     if (s != KM_OK) return s;
     if ((s = refine_winners(ctx, X, n, d, cur, p, labels, L.min_dist, st)) != KM_OK) return s;
     KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.sse_hist + t, &L.a.cnt->sum_ticket, st));

@@ -27,7 +27,8 @@ struct DevCounters {
     unsigned status;     // KM_DEVERR_* bits
     unsigned sum_ticket;   // blocks of the deterministic sum that are done
     unsigned prep_ticket;  // blocks of the centre preparation that are done
-    unsigned pad;
+    unsigned absmax;       // max |x| of the call's points, as bits
+    unsigned colacc[10];   // column maxima being gathered
     // zeroed before every assignment (from amb_count on)
     int amb_count;       // rows whose fp32 argmin the refinement left open
     int ovf_count;       // rows whose candidate list overflowed
@@ -89,6 +90,12 @@ inline cudaError_t allow_max_smem(F* func) {
                                 kMaxBlockSmem - (int)fa.sharedSizeBytes);
 }
 
+// Two spans of 32-bit words to clear.
+struct ZeroWords {
+    unsigned* p[2];
+    int64_t n[2];
+};
+
 // ---- kernels (launch wrappers; all asynchronous on `st`) -----------------
 // quantise rows of A (m x d fp32) to fmt (0 fp16, 1 bf16, 2 e4m3) with row
 // stride ldq elements; stat[i] = (||a||^2 fp32, ||a||, ||a~||, ||a~ - a||);
@@ -100,11 +107,13 @@ cudaError_t launch_quantize(const float* A, int64_t m, int d, int fmt, int ldq, 
 // the points (X null: they are prepared already) and the centres quantised in
 // one launch where their rows take the same form (else two: *nlaunch), and the
 // centres' column data: maxima of the bound terms, q_j padded with +inf to
-// kpad entries, the E4M3 scales padded with 1; ticket: 0 before and after
+// kpad entries, the E4M3 scales padded with 1; ticket and the 10 words at
+// colacc: 0 before and after.  Also clears `zero` (what the call's later kernels
+// add to)
 cudaError_t launch_prepare(const float* X, int64_t n, void* Xq, float4* xstat, float* xscale, unsigned* absmax_out,
                            const float* C, int k, void* Cq, float4* cstat, float* cscale, ColMax* colmax, float* qpad,
-                           float* spad, int kpad, unsigned* ticket, int d, int fmt, int ldq, cudaStream_t st,
-                           int* nlaunch);
+                           float* spad, int kpad, unsigned* ticket, unsigned* colacc, int d, int fmt, int ldq,
+                           const ZeroWords& zero, cudaStream_t st, int* nlaunch);
 
 // candidates per sampled row under the format's certification window (the
 // choice of the low format): acc[0] += candidates, acc[1] += rows above one
@@ -204,12 +213,13 @@ cudaError_t launch_absmax(const float* X, int64_t count, unsigned* out_bits, cud
 // md_out (nullable): each row's ||x_i - C_wd[labels[i]]||^2 to binary64
 // accuracy (the winner distances of launch_winner_dist, bit for bit), fused
 // into the pass over X where the kernel allows.  *nlaunch: kernels launched.
+// zeroed: sums, counts and the first k ints of iscratch are zero already.
 // nscale (0: n): the row count that, with max |x|, fixes the fixed-point
 // scale (all shards' rows when the sums of several shards are added).
 cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* labels, int k,
                               const unsigned* absmax_bits, long long* sums, long long* counts, int* iscratch,
                               int32_t* perm, int num_sms, cudaStream_t st, const float* C_wd, double* md_out,
-                              int* nlaunch, int64_t nscale = 0);
+                              int* nlaunch, int64_t nscale = 0, bool zeroed = false);
 // md[i] = ||x_i - C[labels[i]]||^2, Eq. (dist-direct), to binary64 accuracy
 // on the fp32 pipe (double-float arithmetic of df.cuh)
 cudaError_t launch_winner_dist(const float* X, int64_t n, int d, const float* C, const int32_t* labels, double* md,
@@ -217,18 +227,20 @@ cudaError_t launch_winner_dist(const float* X, int64_t n, int d, const float* C,
 // bytes of scratch the empty-cluster selection needs (launch_finalize's esel)
 size_t empty_select_bytes(int k);
 // means (binary64 division, fp32 store), empty clusters (KM_EMPTY_FARTHEST:
-// the rows of largest min_dist, one cooperative launch), shift.
-// esel: empty_select_bytes(k) bytes, 256-byte aligned; status: the device
-// status word (a bounded wait that runs out sets its timeout bit).
+// the rows of largest min_dist, one cooperative launch), shift (nullable,
+// zeroed by the caller).
+// bar: two zeroed words; esel: empty_select_bytes(k) bytes, 256-byte aligned;
+// status: the device status word (a bounded wait that runs out sets its
+// timeout bit).
 cudaError_t launch_finalize(const long long* sums, const long long* counts, const unsigned* absmax_bits,
                             int64_t n, int k, int d, const float* C_old, int empty_policy, const float* X,
-                            const double* min_dist, float* C_new, int64_t* counts_out, double* shift,
+                            const double* min_dist, float* C_new, int64_t* counts_out, double* shift, unsigned* bar,
                             void* esel, unsigned* status, int num_sms, cudaStream_t st, int* nlaunch,
                             int64_t nscale = 0);
 // the e rows of largest min_dist (ties: lowest index), in that order, into
-// rows_out / vals_out; esel: empty_select_bytes(e) bytes
+// rows_out / vals_out; bar, esel as above
 cudaError_t launch_farthest_rows(const double* min_dist, int64_t n, int e, long long* rows_out, double* vals_out,
-                                 void* esel, unsigned* status, int num_sms, cudaStream_t st);
+                                 unsigned* bar, void* esel, unsigned* status, int num_sms, cudaStream_t st);
 // deterministic sum of n doubles (fixed two-level order); ticket: 0 before and after
 cudaError_t launch_sum_f64(const double* v, int64_t n, double* partials, int nparts, double* out, unsigned* ticket,
                            cudaStream_t st);

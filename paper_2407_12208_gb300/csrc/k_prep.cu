@@ -64,10 +64,41 @@ KM_DEV void block_absmax(float v, unsigned* out) {
     }
 }
 
+// Column maxima of the bound terms, gathered by all blocks that quantise
+// centres: maxima as bit patterns (non-negative floats order like integers;
+// zero to start with), minima as the complement of theirs.
+struct ColAcc {
+    unsigned v[10];
+};
+KM_DEV unsigned col_bits(float x, bool least) { return x >= 0.0f ? (least ? ~__float_as_uint(x) : __float_as_uint(x)) : 0u; }
+
+// Where a quantised row's statistics go: stat and (nullable) rscale, and for
+// centres q_j, the scale and the block's column maxima as well.
+struct RowOut {
+    float4* stat;
+    float* rscale;
+    float* qpad;    // null: points
+    float* spad;
+    unsigned* acc;  // shared, 10 words
+    KM_DEV void operator()(int64_t i, float4 o, float s) const {
+        stat[i] = o;
+        if (rscale) rscale[i] = s;
+        if (qpad) {
+            qpad[i] = o.x;
+            spad[i] = s;
+            const float m[5] = {o.y, o.w, o.z, o.x, o.z * o.z};
+#pragma unroll
+            for (int t = 0; t < 5; t++) {
+                atomicMax(&acc[t], col_bits(m[t], false));
+                atomicMax(&acc[5 + t], col_bits(m[t], true));
+            }
+        }
+    }
+};
+
 // Any d and alignment: one warp per row.
 KM_DEV void quantize_warp(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
-                          float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
-                          unsigned nblocks) {
+                          const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)block * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)nblocks * blockDim.x) >> 5;
@@ -125,8 +156,7 @@ KM_DEV void quantize_warp(const float* __restrict__ A, int64_t m, int d, int fmt
             // underflow, make the row unusable for the expanded formula: an
             // infinite bound flags all its pairs
             if (!isfinite(o.z) || (nzr && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
-            stat[i] = o;
-            if (rscale) rscale[i] = s;
+            out(i, o, s);
         }
     }
 }
@@ -137,8 +167,7 @@ KM_DEV void quantize_warp(const float* __restrict__ A, int64_t m, int d, int fmt
 // Lane l of a row's 8 holds float4 l, l + 8, ... (NV of them).
 template <int NV>
 KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
-                        float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
-                        unsigned nblocks) {
+                        const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
     const int lane = threadIdx.x & 31, sl = lane & 7;
     const unsigned gmask = 0xFFu << (lane & ~7);
     const int64_t gid = (((int64_t)block * blockDim.x + threadIdx.x) >> 5) * 4 + (lane >> 3);
@@ -271,8 +300,7 @@ KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, 
             // underflow, make the row unusable for the expanded formula: an
             // infinite bound flags all its pairs
             if (!isfinite(o.z) || (nzr && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
-            stat[i] = o;
-            if (rscale) rscale[i] = s;
+            out(i, o, s);
         }
         }
     }
@@ -282,8 +310,7 @@ KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, 
 // four float4 of the row in registers (coalesced 16-byte loads).
 template <int NV>
 KM_DEV void quantize_vec(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
-                         float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
-                         unsigned nblocks) {
+                         const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)block * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)nblocks * blockDim.x) >> 5;
@@ -363,8 +390,7 @@ KM_DEV void quantize_vec(const float* __restrict__ A, int64_t m, int d, int fmt,
             o.z = sqrtf(q2) * kNormInflate;
             o.w = sqrtf(r2) * kNormInflate;
             if (!isfinite(o.z) || (nzr && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
-            stat[i] = o;
-            if (rscale) rscale[i] = s;
+            out(i, o, s);
         }
     }
 }
@@ -375,8 +401,7 @@ KM_DEV void quantize_vec(const float* __restrict__ A, int64_t m, int d, int fmt,
 // per row spent its time on reductions of mostly idle lanes: 1e5 x 10 took 27 us
 // (now 16 with the centres in the same launch).
 KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
-                           float4* __restrict__ stat, float* __restrict__ rscale, float& amx, unsigned block,
-                           unsigned nblocks) {
+                           const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
     const int lane = threadIdx.x & 31, sl = lane & 7;
     const unsigned gmask = 0xFFu << (lane & ~7);
     const int64_t ng = (int64_t)nblocks * (blockDim.x / 8);
@@ -444,8 +469,7 @@ KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fm
             const float p = ph[0] + pl[0];
             float4 o = make_float4(p, sqrtf(p) * kNormInflate, sqrtf(q2[0]) * kNormInflate, sqrtf(r2[0]) * kNormInflate);
             if (!isfinite(o.z) || (nzr && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
-            stat[i] = o;
-            if (rscale) rscale[i] = s;
+            out(i, o, s);
         }
     }
 }
@@ -466,42 +490,67 @@ struct ColSide {
     float* spad;
     int kpad;
     unsigned* ticket;
+    unsigned* acc;  // 10 words, 0 before and after
 };
 
 // KIND: NV of quantize_g8 (1, 2, 4, 8), 16 + NV of quantize_vec, 0
 // quantize_warp, -1 quantize_short.  The first cblocks blocks take the centres
-// and the last of them to finish forms their column data (q_j, +inf on the
-// padding so padded columns never win; the E4M3 scales, 1 on the padding; the
-// column maxima); the rest take the points.  One launch instead of three: the
+// and form their column data (q_j, +inf on the padding so padded columns never
+// win; the E4M3 scales, 1 on the padding; the column maxima, written by the
+// last of them to finish); the rest take the points.  One launch instead of three: the
 // centres' part, 5 to 9 us of latency by itself, hides behind the points'.
 constexpr int quant_blocks(int kind) { return kind == 0 ? 6 : (kind == 8 ? 3 : (kind == 17 || kind == 18 ? 5 : 4)); }  // per SM
 template <int KIND>
 __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const QuantSide x, const QuantSide c, const ColSide col, int d, int fmt,
-                                                  int ldq, int cblocks) {
+                                                  int ldq, int cblocks, const ZeroWords zero) {
     chain_enter();
+#pragma unroll
+    for (int z = 0; z < 2; z++)
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < zero.n[z]; i += (int64_t)gridDim.x * blockDim.x)
+            zero.p[z][i] = 0u;
     __shared__ bool last;
+    __shared__ unsigned acc[10];
     const bool cs = (int)blockIdx.x < cblocks;
     const QuantSide& q = cs ? c : x;
     const unsigned block = cs ? blockIdx.x : blockIdx.x - cblocks, nblocks = cs ? cblocks : gridDim.x - cblocks;
+    const bool cols = cs && col.out;
+    if (cols) {
+        if (threadIdx.x < 10) acc[threadIdx.x] = 0u;
+        __syncthreads();
+    }
+    const RowOut out{q.stat, q.rscale, cols ? col.qpad : nullptr, col.spad, acc};
     float amx = 0.0f;  // largest |a| of this thread's elements
-    if constexpr (KIND == -1) quantize_short(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
-    else if constexpr (KIND == 0) quantize_warp(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
-    else if constexpr (KIND < 16) quantize_g8<KIND>(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
-    else quantize_vec<KIND - 16>(q.A, q.m, d, fmt, ldq, q.Aq, q.stat, q.rscale, amx, block, nblocks);
+    if constexpr (KIND == -1) quantize_short(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    else if constexpr (KIND == 0) quantize_warp(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    else if constexpr (KIND < 16) quantize_g8<KIND>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    else quantize_vec<KIND - 16>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     if (q.absmax) block_absmax(amx, q.absmax);
-    if (!cs || !col.out) return;
+    if (!cols) return;
+    if (block == 0)
+        for (int j = (int)c.m + threadIdx.x; j < col.kpad; j += blockDim.x) {
+            col.qpad[j] = INFINITY;
+            col.spad[j] = 1.0f;
+        }
+    __syncthreads();
+    if (threadIdx.x < 10) atomicMax(&col.acc[threadIdx.x], acc[threadIdx.x]);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) last = atomicInc(col.ticket, cblocks - 1) == (unsigned)cblocks - 1;  // back to 0 for the next call
     __syncthreads();
-    if (!last) return;
+    if (!last || threadIdx.x != 0) return;
     __threadfence();
-    const int k = (int)c.m;
-    for (int j = threadIdx.x; j < col.kpad; j += blockDim.x) {
-        col.qpad[j] = (j < k) ? __ldcg(c.stat + j).x : INFINITY;
-        col.spad[j] = (j < k && fmt == 2) ? __ldcg(c.rscale + j) : 1.0f;
+    float m[10];
+#pragma unroll
+    for (int t = 0; t < 10; t++) {
+        const unsigned u = atomicExch(&col.acc[t], 0u);
+        m[t] = __uint_as_float(t < 5 ? u : (u ? ~u : 0x7f800000u));
     }
-    colmax_block(c.stat, k, col.out);
+    ColMax o;
+    o.nc = m[0]; o.nrc = m[1]; o.ncq = m[2]; o.q = m[3]; o.ncq2 = m[4];
+    o.pad[0] = o.pad[1] = o.pad[2] = 0.0f;
+    o.nc_min = m[5]; o.nrc_min = m[6]; o.ncq_min = m[7]; o.q_min = m[8]; o.ncq2_min = m[9];
+    o.pad2[0] = o.pad2[1] = o.pad2[2] = 0.0f;
+    *col.out = o;
 }
 
 // The kernel form for rows at A: -1, 0, NV or 16 + NV (k_quantize).
@@ -514,7 +563,7 @@ static int quant_kind(const float* A, const void* Aq, int d, int ldq) {
 }
 
 static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c, const ColSide& col, int d, int fmt,
-                                int ldq, cudaStream_t st) {
+                                int ldq, const ZeroWords& zero, cudaStream_t st) {
     // 8 lanes or a warp per row, enough warps in flight to cover the memory latency
     const int rows = kind == 0 || kind >= 16 ? 8 : 32;  // per block and round
     const int64_t most = kind == 0 || kind >= 16 ? 152 * 64 : 152 * 16;
@@ -522,7 +571,7 @@ static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c
     const int64_t cb = c.m ? std::min<int64_t>((c.m + rows - 1) / rows, 152) : 0;
     switch (kind) {
 #define KM_Q(K)                                                                                       \
-    case K: klaunch(k_quantize<K>, (unsigned)(xb + cb), 256, 0, st, x, c, col, d, fmt, ldq, (int)cb); break;
+    case K: klaunch(k_quantize<K>, (unsigned)(xb + cb), 256, 0, st, x, c, col, d, fmt, ldq, (int)cb, zero); break;
         KM_Q(-1) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(17) KM_Q(18) KM_Q(20)
 #undef KM_Q
         default: return cudaErrorInvalidValue;
@@ -533,22 +582,22 @@ static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c
 cudaError_t launch_quantize(const float* A, int64_t m, int d, int fmt, int ldq, void* Aq, float4* stat,
                             float* rscale, cudaStream_t st, unsigned* absmax_out) {
     return launch_quant(quant_kind(A, Aq, d, ldq), QuantSide{A, m, Aq, stat, rscale, absmax_out}, QuantSide{}, ColSide{}, d,
-                        fmt, ldq, st);
+                        fmt, ldq, ZeroWords{}, st);
 }
 
 cudaError_t launch_prepare(const float* X, int64_t n, void* Xq, float4* xstat, float* xscale, unsigned* absmax_out,
                            const float* C, int k, void* Cq, float4* cstat, float* cscale, ColMax* colmax, float* qpad,
-                           float* spad, int kpad, unsigned* ticket, int d, int fmt, int ldq, cudaStream_t st,
-                           int* nlaunch) {
+                           float* spad, int kpad, unsigned* ticket, unsigned* colacc, int d, int fmt, int ldq,
+                           const ZeroWords& zero, cudaStream_t st, int* nlaunch) {
     const QuantSide x{X, X ? n : 0, Xq, xstat, xscale, absmax_out}, c{C, k, Cq, cstat, cscale, nullptr};
-    const ColSide col{colmax, qpad, spad, kpad, ticket};
+    const ColSide col{colmax, qpad, spad, kpad, ticket, colacc};
     const int kc = quant_kind(C, Cq, d, ldq), kx = X ? quant_kind(X, Xq, d, ldq) : kc;
     *nlaunch = 1;
-    if (kx == kc) return launch_quant(kc, x, c, col, d, fmt, ldq, st);
+    if (kx == kc) return launch_quant(kc, x, c, col, d, fmt, ldq, zero, st);
     // points and centres aligned differently: each in its own form
     *nlaunch = 2;
-    const cudaError_t e = launch_quant(kx, x, QuantSide{}, col, d, fmt, ldq, st);
-    return e != cudaSuccess ? e : launch_quant(kc, QuantSide{}, c, col, d, fmt, ldq, st);
+    const cudaError_t e = launch_quant(kx, x, QuantSide{}, col, d, fmt, ldq, ZeroWords{}, st);
+    return e != cudaSuccess ? e : launch_quant(kc, QuantSide{}, c, col, d, fmt, ldq, zero, st);
 }
 
 // ---- candidate-count prediction (the choice of the low format) ----------

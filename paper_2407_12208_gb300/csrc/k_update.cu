@@ -31,23 +31,14 @@ __global__ void k_absmax(const float* __restrict__ X, int64_t count, unsigned* o
     if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));  // non-negative floats order as uints
 }
 
-// Row-parallel accumulation for the shapes the bucketed path does not take:
-// shared-memory accumulators when k*d fits, else global atomics (integer, so
-// the result does not depend on the order of the adds).
-template <bool SMEM>
+// Row-parallel accumulation with global atomics, for the shapes that neither
+// the bucketed path nor shared memory takes (integer, so the result does not
+// depend on the order of the adds).
 __global__ void k_accumulate(const float* __restrict__ X, int64_t n, int d, const int32_t* __restrict__ labels,
                              int k, const unsigned* __restrict__ amax_bits, int64_t nscale, long long* __restrict__ sums,
                              long long* __restrict__ counts) {
     chain_enter();
-    extern __shared__ long long acc[];
     const FixedScale fx(fixed_shift(*amax_bits, nscale));
-    const int64_t kd = (int64_t)k * d;
-    if (SMEM) {
-        for (int64_t e = threadIdx.x; e < kd + k; e += blockDim.x) acc[e] = 0;
-        __syncthreads();
-    }
-    long long* sacc = SMEM ? acc : sums;
-    long long* cacc = SMEM ? acc + kd : counts;
     // rows spread over the warps; within a row the lanes walk the coordinates
     // (for d < 32 a warp covers 32 / d rows at once)
     const int lane = threadIdx.x & 31;
@@ -62,17 +53,93 @@ __global__ void k_accumulate(const float* __restrict__ X, int64_t n, int d, cons
         const float* x = X + i * d;
         for (int l = l_in; l < d; l += (d < 32 ? d : 32)) {
             const long long v = fx(x[l]);
-            atomicAdd(reinterpret_cast<unsigned long long*>(&sacc[(int64_t)j * d + l]), (unsigned long long)v);
+            atomicAdd(reinterpret_cast<unsigned long long*>(&sums[(int64_t)j * d + l]), (unsigned long long)v);
         }
-        if (l_in == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&cacc[j]), 1ull);
+        if (l_in == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&counts[j]), 1ull);
     }
-    if (SMEM) {
-        __syncthreads();
-        for (int64_t e = threadIdx.x; e < kd; e += blockDim.x)
-            if (acc[e]) atomicAdd(reinterpret_cast<unsigned long long*>(&sums[e]), (unsigned long long)acc[e]);
-        for (int e = threadIdx.x; e < k; e += blockDim.x)
-            if (acc[kd + e]) atomicAdd(reinterpret_cast<unsigned long long*>(&counts[e]), (unsigned long long)acc[kd + e]);
+}
+
+// The same in shared memory (the k d sums and k counts fit), rows spread over
+// LPR lanes of NV4 float4 as in k_winner_dist; WD: each row's distance to its
+// own centre (the same arithmetic, the same bits) from the same read of the
+// row.  One launch, where the bucketed path takes four: for few rows, and for
+// rows it does not take.  Bound by latency for few rows, by the shared atomics
+// for many: 1e4 x 16, k = 8 26 -> 9 us, 1e5 x 10, k = 100 26 -> 19 us.
+template <int NV4, int LPR, bool VEC, bool WD>
+__global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X, int64_t n, int d,
+                                                    const int32_t* __restrict__ labels, int k,
+                                                    const unsigned* __restrict__ amax_bits, int64_t nscale,
+                                                    long long* __restrict__ sums, long long* __restrict__ counts,
+                                                    const float* __restrict__ C, double* __restrict__ md) {
+    chain_enter();
+    extern __shared__ unsigned long long acc_rows[];  // k d sums, k counts
+    constexpr int G = 32 / LPR;
+    constexpr int R = NV4 == 4 ? 2 : 4;
+    constexpr int STEP = R * G;
+    const FixedScale fx(fixed_shift(*amax_bits, nscale));
+    const int kd = k * d;
+    unsigned long long* cacc = acc_rows + kd;
+    for (int e = threadIdx.x; e < kd + k; e += blockDim.x) acc_rows[e] = 0ull;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, sub = lane / LPR, cl = lane % LPR;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int d4 = (d + 3) >> 2;
+    for (int64_t base = w0 * STEP; base < n; base += nw * STEP) {
+        const int jl = (lane < STEP && base + lane < n) ? labels[base + lane] : 0;
+        float4 xv[R][NV4], cv[R][NV4];
+        int js[R];
+#pragma unroll
+        for (int b = 0; b < R; b++) {
+            const int64_t row = base + b * G + sub;
+            const int j = __shfl_sync(0xffffffffu, jl, b * G + sub);
+            js[b] = row < n ? j : -1;
+#pragma unroll
+            for (int u = 0; u < NV4; u++) {
+                const int cidx = cl + LPR * u;
+                const bool ok = row < n && cidx < d4;
+                xv[b][u] = cv[b][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (VEC) {
+                    if (ok) xv[b][u] = reinterpret_cast<const float4*>(X + row * d)[cidx];
+                    if (WD && ok) cv[b][u] = reinterpret_cast<const float4*>(C + (int64_t)j * d)[cidx];
+                } else if (ok) {
+                    const float* x = X + row * d + 4 * cidx;
+                    const float* c = C + (int64_t)j * d + 4 * cidx;
+                    const int m = d - 4 * cidx;
+                    xv[b][u] = make_float4(x[0], m > 1 ? x[1] : 0.f, m > 2 ? x[2] : 0.f, m > 3 ? x[3] : 0.f);
+                    if (WD) cv[b][u] = make_float4(c[0], m > 1 ? c[1] : 0.f, m > 2 ? c[2] : 0.f, m > 3 ? c[3] : 0.f);
+                }
+            }
+        }
+        if (WD) {
+            DF part[R];
+#pragma unroll
+            for (int b = 0; b < R; b++) part[b] = df_lane<NV4>(xv[b], cv[b]);
+            int rs;
+            const DF r = df_rows<R, LPR>(part, cl, rs);
+            const int64_t row = base + rs * G + sub;
+            if ((cl & (LPR / R - 1)) == 0 && row < n) md[row] = df_value(r);
+        }
+#pragma unroll
+        for (int b = 0; b < R; b++)
+            if (js[b] >= 0) {
+                unsigned long long* a = acc_rows + js[b] * d;
+#pragma unroll
+                for (int u = 0; u < NV4; u++) {
+                    const int l = 4 * (cl + LPR * u);
+                    const float xe[4] = {xv[b][u].x, xv[b][u].y, xv[b][u].z, xv[b][u].w};
+#pragma unroll
+                    for (int t = 0; t < 4; t++)
+                        if (l + t < d && xe[t] != 0.0f) atomicAdd(a + l + t, (unsigned long long)fx(xe[t]));
+                }
+                if (cl == 0) atomicAdd(cacc + js[b], 1ull);
+            }
     }
+    __syncthreads();
+    for (int e = threadIdx.x; e < kd; e += blockDim.x)
+        if (acc_rows[e]) atomicAdd(reinterpret_cast<unsigned long long*>(sums) + e, acc_rows[e]);
+    for (int e = threadIdx.x; e < k; e += blockDim.x)
+        if (cacc[e]) atomicAdd(reinterpret_cast<unsigned long long*>(counts) + e, cacc[e]);
 }
 
 // ---- bucketed reduction: rows grouped by label, summed in registers ------
@@ -529,23 +596,53 @@ cudaError_t launch_winner_dist(const float* X, int64_t n, int d, const float* C,
     return cudaGetLastError();
 }
 
-// mean = sum 2^-S / m in binary64, stored in fp32 (the working precision).
-__global__ void k_means(const long long* __restrict__ sums, const long long* __restrict__ counts,
-                        const unsigned* __restrict__ amax_bits, int64_t nscale, int k, int d,
-                        const float* __restrict__ C_old, float* __restrict__ C_new, int64_t* counts_out) {
+// mean = sum 2^-S / m in binary64, stored in fp32 (the working precision);
+// one warp per cluster.  shift_bits (nullable, zeroed): max_j ||c_new_j -
+// c_old_j|| over the clusters with rows, as the bit pattern of a non-negative
+// double (ordered like an integer, so the order does not matter); the reseeded
+// clusters follow in k_empty_select, the kept ones do not move.
+__global__ void __launch_bounds__(64) k_means(const long long* __restrict__ sums, const long long* __restrict__ counts,
+                                               const unsigned* __restrict__ amax_bits, int64_t nscale, int k, int d,
+                                               const float* __restrict__ C_old, float* __restrict__ C_new,
+                                               int64_t* counts_out, unsigned long long* shift_bits) {
     chain_enter();
     const int S = fixed_shift(*amax_bits, nscale);
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)k * d;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(e / d);
+    const double unit = __hiloint2double((1023 - S) << 20, 0);  // 2^-S, S in [-98, 209]: the product is exact
+    const int lane = threadIdx.x & 31;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t j = w0; j < k; j += nw) {
         const long long m = counts[j];
-        if (m > 0) {
-            double s = ldexp((double)sums[e], -S);  // int64 -> binary64 rounds once (2^-53 relative)
-            C_new[e] = (float)(s / (double)m);
-        } else {
-            C_new[e] = C_old[e];
+        double sq = 0.0;
+        for (int l0 = lane; l0 < d; l0 += 128) {
+            float old[4];
+            long long sm[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int l = l0 + 32 * u;
+                old[u] = l < d ? C_old[j * d + l] : 0.0f;
+                sm[u] = l < d ? sums[j * d + l] : 0;
+            }
+            float c[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++)  // int64 -> binary64 rounds once (2^-53 relative)
+                c[u] = m > 0 && l0 - lane + 32 * u < d ? (float)((double)sm[u] * unit / (double)m) : old[u];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int l = l0 + 32 * u;
+                if (l < d) C_new[j * d + l] = c[u];
+                if (shift_bits && m > 0 && l0 - lane + 32 * u < d) {
+                    const double df = (double)c[u] - (double)old[u];  // (0 past d)
+                    sq = fma(df, df, sq);
+                }
+            }
         }
-        if (e - (int64_t)j * d == 0 && counts_out) counts_out[j] = m;
+        if (lane == 0 && counts_out) counts_out[j] = m;
+        if (shift_bits && m > 0) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+            if (lane == 0) atomicMax(shift_bits, (unsigned long long)__double_as_longlong(sqrt(sq)));
+        }
     }
 }
 
@@ -571,7 +668,6 @@ __global__ void k_means(const long long* __restrict__ sums, const long long* __r
 // whose every wait is bounded: on timeout the status word's timeout bit is
 // set and the kernel winds down.
 struct EmptySel {
-    unsigned bar_count, bar_gen;  // grid barrier
     int nempty, ncollected;
     unsigned hist[12][256];       // 8 passes on the distance bits, 4 on the row index
 };
@@ -579,18 +675,19 @@ size_t empty_select_bytes(int k) {
     return ((sizeof(EmptySel) + 255) & ~(size_t)255) + (size_t)k * (sizeof(int) + 16 + sizeof(int));
 }
 
-KM_DEV bool grid_barrier(EmptySel* es, unsigned nblocks, unsigned* status) {
+// bar: count and generation, both 0 at the launch
+KM_DEV bool grid_barrier(unsigned* bar, unsigned nblocks, unsigned* status) {
     __shared__ int ok_sh;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        volatile unsigned* vgen = &es->bar_gen;
+        volatile unsigned* vgen = bar + 1;
         const unsigned g = *vgen;
         __threadfence();
-        if (atomicAdd(&es->bar_count, 1u) == nblocks - 1) {
-            es->bar_count = 0;
+        if (atomicAdd(bar, 1u) == nblocks - 1) {
+            bar[0] = 0;
             __threadfence();
-            atomicAdd(&es->bar_gen, 1u);
+            atomicAdd(bar + 1, 1u);
         } else {
             const long long t0 = clock64();
             while (*vgen == g) {
@@ -646,7 +743,8 @@ KM_DEV void radix_pick(const unsigned* hist, bool descending, unsigned rank, uns
 // clusters of a row-sharded update).
 __global__ void __launch_bounds__(256) k_empty_select(const long long* __restrict__ counts, int64_t n, int k, int d,
                                                       const float* __restrict__ X, const double* __restrict__ md,
-                                                      float* __restrict__ C_new, EmptySel* es,
+                                                      const float* __restrict__ C_old, float* __restrict__ C_new,
+                                                      unsigned long long* shift_bits, unsigned* bar, EmptySel* es,
                                                       int* __restrict__ empties, unsigned long long* __restrict__ keys,
                                                       int* __restrict__ rows, int* __restrict__ order,
                                                       unsigned* status, int fixed_e, long long* __restrict__ rows_out,
@@ -697,7 +795,7 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
             es->ncollected = 0;
         }
     }
-    if (!grid_barrier(es, nb, status)) return;
+    if (!grid_barrier(bar, nb, status)) return;
     const int E = *(volatile int*)&es->nempty;
     if (E == 0) return;
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + t, gstride = (int64_t)nb * blockDim.x;
@@ -716,7 +814,7 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
         }
         __syncthreads();
         if (sh[t]) atomicAdd(&es->hist[pass][t], sh[t]);
-        if (!grid_barrier(es, nb, status)) return;
+        if (!grid_barrier(bar, nb, status)) return;
         unsigned digit, before, in;
         radix_pick(es->hist[pass], true, rank, digit, before, in);
         rank -= before;
@@ -736,7 +834,7 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
         }
         __syncthreads();
         if (sh[t]) atomicAdd(&es->hist[8 + pass][t], sh[t]);
-        if (!grid_barrier(es, nb, status)) return;
+        if (!grid_barrier(bar, nb, status)) return;
         unsigned digit, before, in;
         radix_pick(es->hist[8 + pass], false, rank, digit, before, in);
         rank -= before;
@@ -755,7 +853,7 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
             }
         }
     }
-    if (!grid_barrier(es, nb, status)) return;
+    if (!grid_barrier(bar, nb, status)) return;
     // (the lists were written by other blocks: read through L2)
     for (int64_t s = gtid; s < E; s += gstride) {
         const unsigned long long ks = __ldcg(keys + s);
@@ -767,7 +865,7 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
         }
         order[r] = rs;
     }
-    if (!grid_barrier(es, nb, status)) return;
+    if (!grid_barrier(bar, nb, status)) return;
     if (fixed_e > 0) {
         for (int64_t r = gtid; r < E; r += gstride) {
             const int row = __ldcg(order + r);
@@ -776,30 +874,20 @@ __global__ void __launch_bounds__(256) k_empty_select(const long long* __restric
         }
         return;
     }
-    for (int64_t e = gtid; e < (int64_t)E * d; e += gstride) {
-        const int r = (int)(e / d), l = (int)(e - (int64_t)r * d);
-        C_new[(int64_t)__ldcg(empties + r) * d + l] = X[(int64_t)__ldcg(order + r) * d + l];
-    }
-}
-
-// shift = max_j ||c_new_j - c_old_j||: one warp per cluster, coalesced rows,
-// the maximum kept as the bit pattern of a non-negative double (ordered like
-// an unsigned integer), so the result does not depend on the order.
-__global__ void k_shift(int k, int d, const float* __restrict__ C_old, const float* __restrict__ C_new,
-                        unsigned long long* __restrict__ shift_bits) {
-    chain_enter();
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t j = w0; j < k; j += nw) {
-        double s = 0.0;
-        for (int l = lane; l < d; l += 32) {
-            const double df = (double)C_new[j * d + l] - (double)C_old[j * d + l];
-            s = fma(df, df, s);
+    for (int64_t r = gtid >> 5; r < E; r += gstride >> 5) {  // a warp per cluster
+        const int64_t j = __ldcg(empties + r), row = __ldcg(order + r);
+        double sq = 0.0;
+        for (int l = t & 31; l < d; l += 32) {
+            const float c = X[row * d + l];
+            C_new[j * d + l] = c;
+            const double df = (double)c - (double)C_old[j * d + l];
+            sq = fma(df, df, sq);
         }
+        if (shift_bits) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) atomicMax(shift_bits, (unsigned long long)__double_as_longlong(sqrt(s)));
+            for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+            if ((t & 31) == 0) atomicMax(shift_bits, (unsigned long long)__double_as_longlong(sqrt(sq)));
+        }
     }
 }
 
@@ -873,19 +961,22 @@ cudaError_t launch_absmax(const float* X, int64_t count, unsigned* out_bits, cud
 cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* labels, int k,
                               const unsigned* absmax_bits, long long* sums, long long* counts, int* iscratch,
                               int32_t* perm, int num_sms, cudaStream_t st, const float* C_wd, double* md_out,
-                              int* nlaunch, int64_t nscale) {
+                              int* nlaunch, int64_t nscale, bool zeroed) {
     if (nscale <= 0) nscale = n;  // the fixed-point scale of n rows (or of all shards' rows)
     // md_out: the rows' distances to their centres (C_wd) come out of the same
     // pass over X where the kernel has the row and its centre in hand, else
     // from the standalone kernel first (the same arithmetic either way)
     const bool want_wd = md_out != nullptr && C_wd != nullptr;
     int nl = 0;
-    cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(long long) * (size_t)k * d, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (!zeroed) {
+        e = cudaMemsetAsync(sums, 0, sizeof(long long) * (size_t)k * d, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(long long) * (size_t)k, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(iscratch, 0, sizeof(int) * (size_t)k, st);
+        if (e != cudaSuccess) return e;
+    }
     if (d <= 8 && (int64_t)k * d <= AS_MAX_KD) {
         // small d: rows in order, per-warp shared accumulators (+ C for the distances)
-        e = cudaMemsetAsync(counts, 0, sizeof(long long) * (size_t)k, st);
-        if (e != cudaSuccess) return e;
         const size_t sm = (((size_t)8 * (3 * (size_t)k * d + k) + 3) & ~(size_t)3) * sizeof(unsigned) +
                           (want_wd ? (size_t)k * 8 * sizeof(float) : 0);
         const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * 8, (n + 8 * AS_CHUNK - 1) / (8 * AS_CHUNK)));
@@ -912,7 +1003,33 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
     }
     const size_t hsm = sizeof(int) * (size_t)k;
     const bool vec = d % 4 == 0 && ((uintptr_t)X % 16) == 0;
-    const bool bucket = 2 * hsm <= 200 * 1024 && (d == 1 || d == 2 || d == 3 || d == 5 || (vec && d <= 512));
+    const bool can_bucket = 2 * hsm <= 200 * 1024 && (d == 1 || d == 2 || d == 3 || d == 5 || (vec && d <= 512));
+    const size_t smem = sizeof(long long) * ((size_t)k * d + k);
+    // shared-memory sums in one launch: what the bucketed path does not take, and
+    // few rows (n d <= 2^21, with at least 16 rows per cluster to pay for the
+    // blocks' folds): 1e4 x 16, k = 8 takes 9 us against 26 us in four launches;
+    // 1e5 x 128 would take 60 us of shared atomics against 51 us
+    if (smem <= 200 * 1024 && d <= 512 && (!can_bucket || (n * d <= (int64_t)1 << 21 && n >= 16 * (int64_t)k))) {
+        typedef void (*RowsFn)(const float*, int64_t, int, const int32_t*, int, const unsigned*, int64_t, long long*,
+                               long long*, const float*, double*);
+        RowsFn fn = nullptr;
+        const bool v4 = vec && (!want_wd || ((uintptr_t)C_wd % 16) == 0);
+        const int lpr = df_lpr(d), nv4 = df_nv4(d);
+#define KM_AR(NV, L)                                                                                      \
+    if (nv4 == NV && lpr == L)                                                                            \
+        fn = v4 ? (want_wd ? (RowsFn)k_accum_rows<NV, L, true, true> : (RowsFn)k_accum_rows<NV, L, true, false>) \
+                : (want_wd ? (RowsFn)k_accum_rows<NV, L, false, true> : (RowsFn)k_accum_rows<NV, L, false, false>);
+        KM_AR(1, 8) KM_AR(1, 16) KM_AR(1, 32) KM_AR(2, 32) KM_AR(4, 32)
+#undef KM_AR
+        if (!fn) return cudaErrorInvalidValue;
+        e = allow_max_smem(fn);
+        if (e != cudaSuccess) return e;
+        const int rows = (nv4 == 4 ? 2 : 4) * (32 / lpr) * 16;  // per block and pass
+        const int64_t blk = std::min<int64_t>(std::min<int64_t>((n + rows - 1) / rows, num_sms), std::max<int64_t>(1, n / (4 * (int64_t)k)));
+        *nlaunch = 1;
+        return klaunch(fn, (unsigned)blk, 512, smem, st, X, n, d, labels, k, absmax_bits, nscale, sums, counts, C_wd, md_out);
+    }
+    const bool bucket = can_bucket;
     // the bucket kernels of rows wider than 5 coordinates read the rows as
     // float4: they can take the distances along when C is aligned as well
     const bool fused = want_wd && bucket && d > 5 && ((uintptr_t)C_wd % 16) == 0;
@@ -926,8 +1043,6 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         int* off = iscratch + k;          // k + 1
         int* cursor = off + k + 1;        // k
         int* item_off = cursor + k;       // k + 1
-        e = cudaMemsetAsync(cnt32, 0, sizeof(int) * (size_t)k, st);
-        if (e != cudaSuccess) return e;
         const int64_t nblk = (n + SCAT_ROWS - 1) / SCAT_ROWS;
         e = allow_max_smem(k_label_hist);
         if (e != cudaSuccess) return e;
@@ -967,37 +1082,22 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         if (nlaunch) *nlaunch = nl + 4;
         return cudaGetLastError();
     }
-    e = cudaMemsetAsync(counts, 0, sizeof(long long) * (size_t)k, st);
-    if (e != cudaSuccess) return e;
-    const size_t smem = sizeof(long long) * ((size_t)k * d + k);
-    const int64_t total = n * d;
-    if (smem <= 200 * 1024) {
-        e = allow_max_smem(k_accumulate<true>);
-        if (e != cudaSuccess) return e;
-        const int64_t blk = std::min<int64_t>((int64_t)num_sms, (total + 511) / 512);
-        klaunch(k_accumulate<true>, (unsigned)std::max<int64_t>(blk, 1), 512, smem, st, X, n, d, labels, k, absmax_bits,
-                                                                                    nscale, sums, counts);
-    } else {
-        const int64_t blk = std::min<int64_t>((int64_t)num_sms * 8, (total + 511) / 512);
-        klaunch(k_accumulate<false>, (unsigned)std::max<int64_t>(blk, 1), 512, 0, st, X, n, d, labels, k, absmax_bits,
-                                                                                  nscale, sums, counts);
-    }
+    const int64_t blk = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * 8, (n * d + 511) / 512));
     if (nlaunch) *nlaunch = nl + 1;
-    return cudaGetLastError();
+    return klaunch(k_accumulate, (unsigned)blk, 512, 0, st, X, n, d, labels, k, absmax_bits, nscale, sums, counts);
 }
 
 cudaError_t launch_finalize(const long long* sums, const long long* counts, const unsigned* absmax_bits,
                             int64_t n, int k, int d, const float* C_old, int empty_policy, const float* X,
-                            const double* min_dist, float* C_new, int64_t* counts_out, double* shift,
+                            const double* min_dist, float* C_new, int64_t* counts_out, double* shift, unsigned* bar,
                             void* esel, unsigned* status, int num_sms, cudaStream_t st, int* nlaunch, int64_t nscale) {
-    int nl = 0;
-    int64_t kd = (int64_t)k * d;
-    int64_t blocks = min((int64_t)1024, (kd + 255) / 256);
-    klaunch(k_means, (unsigned)blocks, 256, 0, st, sums, counts, absmax_bits, nscale > 0 ? nscale : n, k, d, C_old, C_new,
-                                               counts_out);
-    cudaError_t e = cudaGetLastError();
+    unsigned long long* shift_bits = reinterpret_cast<unsigned long long*>(shift);
+    // (bound by the FP64 pipes: small blocks, so that few clusters reach all SMs)
+    const int64_t blocks = std::min<int64_t>(((int64_t)k * 32 + 63) / 64, (int64_t)num_sms * 16);
+    cudaError_t e = klaunch(k_means, (unsigned)blocks, 64, 0, st, sums, counts, absmax_bits, nscale > 0 ? nscale : n, k, d,
+                            C_old, C_new, counts_out, shift_bits);
     if (e != cudaSuccess) return e;
-    nl++;
+    *nlaunch = 1;
     if (empty_policy == 1 && min_dist != nullptr) {
         EmptySel* es = reinterpret_cast<EmptySel*>(esel);
         char* tail = reinterpret_cast<char*>(esel) + ((sizeof(EmptySel) + 255) & ~(size_t)255);
@@ -1005,57 +1105,38 @@ cudaError_t launch_finalize(const long long* sums, const long long* counts, cons
         unsigned long long* keys = reinterpret_cast<unsigned long long*>(empties + k + (k & 1));
         int* rows = reinterpret_cast<int*>(keys + k);
         int* order = rows + k;
-        e = cudaMemsetAsync(es, 0, 2 * sizeof(unsigned), st);
-        if (e != cudaSuccess) return e;
         // one block per SM: every block resident at once (cooperative launch)
-        int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_empty_select, 256, 0);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
         int fixed_e = 0;
         long long* rows_out = nullptr;
         double* vals_out = nullptr;
         void* args[] = {(void*)&counts, (void*)&n,     (void*)&k,     (void*)&d,      (void*)&X,
-                        (void*)&min_dist, (void*)&C_new, (void*)&es,   (void*)&empties, (void*)&keys,
-                        (void*)&rows,   (void*)&order, (void*)&status, (void*)&fixed_e, (void*)&rows_out,
-                        (void*)&vals_out};
+                        (void*)&min_dist, (void*)&C_old, (void*)&C_new, (void*)&shift_bits, (void*)&bar, (void*)&es,
+                        (void*)&empties, (void*)&keys, (void*)&rows,   (void*)&order, (void*)&status, (void*)&fixed_e,
+                        (void*)&rows_out, (void*)&vals_out};
         e = cudaLaunchCooperativeKernel((const void*)k_empty_select, dim3((unsigned)num_sms), dim3(256), args, 0, st);
         if (e != cudaSuccess) return e;
-        nl++;
+        ++*nlaunch;
     }
-    if (shift) {  // null: the caller does not want the shift
-        e = cudaMemsetAsync(shift, 0, sizeof(double), st);
-        if (e != cudaSuccess) return e;
-        const int64_t sblocks = std::min<int64_t>(((int64_t)k * 32 + 255) / 256, (int64_t)num_sms * 8);
-        klaunch(k_shift, (unsigned)std::max<int64_t>(sblocks, 1), 256, 0, st, k, d, C_old, C_new,
-                                                                       reinterpret_cast<unsigned long long*>(shift));
-        nl++;
-    }
-    if (nlaunch) *nlaunch = nl;
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 cudaError_t launch_farthest_rows(const double* min_dist, int64_t n, int e, long long* rows_out, double* vals_out,
-                                 void* esel, unsigned* status, int num_sms, cudaStream_t st) {
+                                 unsigned* bar, void* esel, unsigned* status, int num_sms, cudaStream_t st) {
     EmptySel* es = reinterpret_cast<EmptySel*>(esel);
     char* tail = reinterpret_cast<char*>(esel) + ((sizeof(EmptySel) + 255) & ~(size_t)255);
     int* empties = reinterpret_cast<int*>(tail);
     unsigned long long* keys = reinterpret_cast<unsigned long long*>(empties + e + (e & 1));
     int* rows = reinterpret_cast<int*>(keys + e);
     int* order = rows + e;
-    cudaError_t err = cudaMemsetAsync(es, 0, 2 * sizeof(unsigned), st);
-    if (err != cudaSuccess) return err;
-    int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_empty_select, 256, 0);
-    if (err != cudaSuccess) return err;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const long long* counts = nullptr;
     int k = e, d = 0;
-    const float* X = nullptr;
+    const float *X = nullptr, *C_old = nullptr;
     float* C_new = nullptr;
+    unsigned long long* shift_bits = nullptr;
     void* args[] = {(void*)&counts, (void*)&n,     (void*)&k,     (void*)&d,  (void*)&X,    (void*)&min_dist,
-                    (void*)&C_new,  (void*)&es,    (void*)&empties, (void*)&keys, (void*)&rows, (void*)&order,
-                    (void*)&status, (void*)&e,     (void*)&rows_out, (void*)&vals_out};
+                    (void*)&C_old,  (void*)&C_new,  (void*)&shift_bits, (void*)&bar, (void*)&es,    (void*)&empties,
+                    (void*)&keys, (void*)&rows, (void*)&order, (void*)&status, (void*)&e,     (void*)&rows_out,
+                    (void*)&vals_out};
     return cudaLaunchCooperativeKernel((const void*)k_empty_select, dim3((unsigned)num_sms), dim3(256), args, 0, st);
 }
 

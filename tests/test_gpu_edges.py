@@ -212,3 +212,36 @@ def test_distance_matrix_edges(ctx, low, test, n, d, k, near):
     assert np.array_equal(D[fl], want[fl].astype(np.float32))
     if low != "e4m3" and (~fl).any():  # Eq. (quantis-rel-bound-expand): unflagged pairs to 1 / (rho - 1)
         assert (np.abs(D[~fl] - want[~fl]) <= 0.26 * want[~fl]).all()
+
+
+# the centre update at the edges of its dispatch (shared sums in one launch, buckets, global
+# sums): counts and means against the oracle's within Lemma 4.4's fp32 store, kept, reseeded
+# and shifted centres; the fused distances equal a separate assignment's bit for bit
+@pytest.mark.parametrize("empty", ["keep", "farthest"])
+@pytest.mark.parametrize("n,d,k,offset", [(1, 9, 1, 0), (100, 10, 7, 0), (5000, 16, 8, 0), (5000, 16, 8, 1), (131072, 16, 4, 0),
+                                          (131073, 16, 4, 0), (3000, 130, 150, 1), (4000, 33, 250, 0), (2000, 129, 199, 0),
+                                          (2000, 129, 201, 0), (1500, 8, 90, 0), (700, 256, 40, 0)])
+def test_update_dispatch_edges(ctx, n, d, k, offset, empty):
+    import paper_2407_12208_gb300 as pkg
+    X, C = workloads.blobs(n, d, k, seed=n + k)
+    if k > 4:
+        C[1] += 1e3  # empty
+    p = pkg.params("fp32", empty=empty)
+    Xd, Cd = _dev(X, offset), _dev(C, offset)
+    lab, md, Cn, counts, shift = ctx.lloyd_step(Xd, Cd, p)
+    lab2, md2, _ = ctx.assign(Xd, Cd, p)
+    assert torch.equal(lab, lab2) and torch.equal(md, md2)
+    Cn2, counts2, shift2 = ctx.update_centroids(Xd, lab, Cd, p, min_dist=md)
+    assert torch.equal(Cn, Cn2) and torch.equal(counts, counts2) and shift == shift2
+    lab, md, Cn, counts = (t.cpu().numpy() for t in (lab, md, Cn, counts))
+    cnt = np.bincount(lab, minlength=k)
+    assert np.array_equal(counts, cnt)
+    want = C.astype(np.float64)
+    for j in np.nonzero(cnt)[0]:
+        want[j] = X[lab == j].astype(np.float64).mean(0)
+    if empty == "farthest":
+        far = np.lexsort((np.arange(n), -md))
+        for r, j in enumerate(np.nonzero(cnt == 0)[0]):
+            want[j] = X[far[r]]
+    np.testing.assert_allclose(Cn, want, rtol=2.0 ** -23, atol=np.abs(X).max() * 2.0 ** -30)
+    np.testing.assert_allclose(shift, np.linalg.norm(Cn.astype(np.float64) - C, axis=1).max(), rtol=1e-12)
