@@ -546,13 +546,18 @@ km_status finalize(km_ctx* ctx, const UpdateWs& u, int64_t n, int k, int d, cons
     return KM_OK;
 }
 
-km_status sync_status(km_ctx* ctx, DevCounters* cnt, cudaStream_t st) {
+// Reads the counters back and waits for the stream: one copy and one wait
+// (each separate read-back of a few bytes costs about 10 us).
+km_status sync_counters(km_ctx* ctx, const DevCounters* cnt, DevCounters* h, cudaStream_t st) {
+    CK(cudaMemcpyAsync(h, cnt, sizeof *h, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    unsigned status = 0;
-    CK(cudaMemcpy(&status, &cnt->status, sizeof status, cudaMemcpyDeviceToHost));
-    if (status & KM_DEVERR_TIMEOUT) return fail(ctx, KM_ETIMEOUT, "a device-side wait ran out of its budget");
-    if (status) return fail(ctx, KM_ECUDA, "device status word 0x%x", status);
+    if (h->status & KM_DEVERR_TIMEOUT) return fail(ctx, KM_ETIMEOUT, "a device-side wait ran out of its budget");
+    if (h->status) return fail(ctx, KM_ECUDA, "device status word 0x%x", h->status);
     return KM_OK;
+}
+km_status sync_status(km_ctx* ctx, const DevCounters* cnt, cudaStream_t st) {
+    DevCounters h;
+    return sync_counters(ctx, cnt, &h, st);
 }
 
 km_status check_common(km_ctx* ctx, const void* X, int64_t n, const void* C, int k, int d) {
@@ -727,10 +732,9 @@ km_status km_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int 
     ctx->last_stream = st;
     ctx->last_pairs = (uint64_t)n * (uint64_t)k;
     if (n_flagged_host) {
-        if ((s = sync_status(ctx, w.cnt, st)) != KM_OK) return s;
-        unsigned long long f = 0;
-        CK(cudaMemcpy(&f, &w.cnt->flagged, sizeof f, cudaMemcpyDeviceToHost));
-        *n_flagged_host = f;
+        DevCounters h;
+        if ((s = sync_counters(ctx, w.cnt, &h, st)) != KM_OK) return s;
+        *n_flagged_host = h.flagged;
     }
     return KM_OK;
 }
@@ -871,10 +875,9 @@ km_status km_distances(km_ctx* ctx, const float* X, int64_t n, const float* C, i
     ctx->last_stream = st;
     ctx->last_pairs = (uint64_t)n * (uint64_t)k;
     if (n_flagged_host) {
-        if ((s = sync_status(ctx, w.cnt, st)) != KM_OK) return s;
-        unsigned long long f = 0;
-        CK(cudaMemcpy(&f, &w.cnt->flagged, sizeof f, cudaMemcpyDeviceToHost));
-        *n_flagged_host = f;
+        DevCounters h;
+        if ((s = sync_counters(ctx, w.cnt, &h, st)) != KM_OK) return s;
+        *n_flagged_host = h.flagged;
     }
     return KM_OK;
 }
@@ -906,8 +909,10 @@ km_status km_update_centroids(km_ctx* ctx, const float* X, int64_t n, int d, con
             return s;
     }
     if (shift_host) {
+        double sh = 0.0;
+        CK(cudaMemcpyAsync(&sh, u.shift, sizeof sh, cudaMemcpyDeviceToHost, st));
         if ((s = sync_status(ctx, cnt, st)) != KM_OK) return s;
-        CK(cudaMemcpy(shift_host, u.shift, sizeof(double), cudaMemcpyDeviceToHost));
+        *shift_host = sh;
     }
     return KM_OK;
 }
@@ -978,9 +983,11 @@ km_status km_update_finalize(km_ctx* ctx, const int64_t* sums, const int64_t* co
                        &cnt->status, ctx->num_sms, st, &nl, n_total));
     ctx->launches += (uint64_t)nl;
     if (shift_host) {
+        double sh = 0.0;
+        CK(cudaMemcpyAsync(&sh, u.shift, sizeof sh, cudaMemcpyDeviceToHost, st));
         km_status s = sync_status(ctx, cnt, st);
         if (s != KM_OK) return s;
-        CK(cudaMemcpy(shift_host, u.shift, sizeof(double), cudaMemcpyDeviceToHost));
+        *shift_host = sh;
     }
     return KM_OK;
 }
@@ -1041,8 +1048,10 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
     ctx->last_stream = st;
     ctx->last_pairs = (uint64_t)n * (uint64_t)k;
     if (shift_host) {
+        double sh = 0.0;
+        CK(cudaMemcpyAsync(&sh, u.shift, sizeof sh, cudaMemcpyDeviceToHost, st));
         if ((s = sync_status(ctx, w.cnt, st)) != KM_OK) return s;
-        CK(cudaMemcpy(shift_host, u.shift, sizeof(double), cudaMemcpyDeviceToHost));
+        *shift_host = sh;
     }
     return KM_OK;
 }
@@ -1177,8 +1186,10 @@ km_status km_lloyd_step_host(km_ctx* ctx, const float* X_host, int64_t n, int d,
     ctx->last_sse = w.sse;
     ctx->last_stream = st;
     ctx->last_pairs = (uint64_t)n * (uint64_t)k;
+    double sh = 0.0;
+    if (shift_host) CK(cudaMemcpyAsync(&sh, u.shift, sizeof sh, cudaMemcpyDeviceToHost, st));
     if ((s = sync_status(ctx, w.cnt, st)) != KM_OK) return s;
-    if (shift_host) CK(cudaMemcpy(shift_host, u.shift, sizeof(double), cudaMemcpyDeviceToHost));
+    if (shift_host) *shift_host = sh;
     return KM_OK;
 }
 
@@ -1411,11 +1422,14 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
     ctx->last_sse = L.a.sse;
     ctx->last_stream = st;
     ctx->last_pairs = (uint64_t)n * (uint64_t)k * (uint64_t)(t + 1);
+    // both histories (side by side in the workspace) and the counters, one wait
+    std::vector<unsigned char> hist(reinterpret_cast<char*>(L.flag_hist + t + 1) - reinterpret_cast<char*>(L.sse_hist));
+    CK(cudaMemcpyAsync(hist.data(), L.sse_hist, hist.size(), cudaMemcpyDeviceToHost, st));
     if ((s = sync_status(ctx, L.a.cnt, st)) != KM_OK) return s;
     std::vector<double> sse(t + 1);
     std::vector<unsigned long long> fl(t + 1);
-    CK(cudaMemcpy(sse.data(), L.sse_hist, sizeof(double) * (t + 1), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(fl.data(), L.flag_hist, sizeof(unsigned long long) * (t + 1), cudaMemcpyDeviceToHost));
+    memcpy(sse.data(), hist.data(), sizeof(double) * (t + 1));
+    memcpy(fl.data(), hist.data() + hist.size() - sizeof(unsigned long long) * (t + 1), sizeof(unsigned long long) * (t + 1));
     const double pairs = (double)n * (double)k;
     for (int i = 0; i <= t; i++) {
         if (sse_per_iter) sse_per_iter[i] = sse[i];
@@ -1430,9 +1444,8 @@ extern "C" {
 km_status km_get_stats(km_ctx* ctx, km_stats* out) {
     if (!ctx || !out) return KM_EINVAL;
     if (!ctx->last_cnt) return fail(ctx, KM_EINVAL, "no call to report on");
-    km_status s = sync_status(ctx, ctx->last_cnt, ctx->last_stream);
     DevCounters c{};
-    CK(cudaMemcpy(&c, ctx->last_cnt, sizeof c, cudaMemcpyDeviceToHost));
+    km_status s = sync_counters(ctx, ctx->last_cnt, &c, ctx->last_stream);
     out->pairs = ctx->last_pairs;
     out->flagged = c.flagged;
     out->fp32_evals = c.fp32_evals;

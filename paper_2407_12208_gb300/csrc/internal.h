@@ -75,19 +75,23 @@ struct TestParams {
     float gamma32;   // gamma_{d+2}(2^-24) with safety, for fp32 direct certification
 };
 
-// Lets `func` take all the dynamic shared memory a block can have (the
-// per-block maximum less the kernel's static shared memory).  Every call sets
-// the same value: jobs of different shapes launched from several host threads
-// (the serving workers) cannot lower the limit under one another's launches;
-// the launch itself states the bytes it uses.
+// Facts of a kernel on the current device, asked of the runtime once per kernel,
+// device, block and shared-memory size (each question costs a call about a
+// microsecond): launch_facts.cu.  Safe from any thread.
+//
+// allow_max_smem lets `func` take all the dynamic shared memory a block can have
+// (the per-block maximum less the kernel's static shared memory): the same value
+// whatever the shape, so jobs launched from several host threads cannot lower
+// the limit under one another's launches; the launch itself states the bytes it
+// uses.  blocks_per_sm: resident blocks (at least 1).
 constexpr int kMaxBlockSmem = 227 * 1024;
+cudaError_t allow_max_smem_of(const void* func);
+cudaError_t blocks_per_sm_of(const void* func, int block, size_t smem, int* out);
 template <typename F>
-inline cudaError_t allow_max_smem(F* func) {
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(func));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(reinterpret_cast<const void*>(func), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kMaxBlockSmem - (int)fa.sharedSizeBytes);
+inline cudaError_t allow_max_smem(F* func) { return allow_max_smem_of(reinterpret_cast<const void*>(func)); }
+template <typename F>
+inline cudaError_t blocks_per_sm(F* func, int block, size_t smem, int* out) {
+    return blocks_per_sm_of(reinterpret_cast<const void*>(func), block, smem, out);
 }
 
 // Two spans of 32-bit words to clear.

@@ -618,7 +618,7 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
                               (const void*)k_direct_small<3>, (const void*)k_direct_small<4>,
                               (const void*)k_direct_small<5>, (const void*)k_direct_small<6>,
                               (const void*)k_direct_small<7>, (const void*)k_direct_small<8>};
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[d], 256, csm);
+        cudaError_t e = blocks_per_sm_of(fns[d], 256, csm, &per_sm);
         if (e != cudaSuccess) return e;
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)num_sms * std::max(per_sm, 1)));
         switch (d) {

@@ -621,9 +621,9 @@ static cudaError_t launch_refine_batched(const float* X, const float* C, const T
                                          cudaStream_t st, int* nlaunch) {
     // persistent grids: the resident blocks only
     int sel_per_sm = 1, cert_per_sm = 1;
-    cudaError_t e0 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sel_per_sm, k_cand_select, 256, 0);
+    cudaError_t e0 = blocks_per_sm(k_cand_select, 256, 0, &sel_per_sm);
     if (e0 != cudaSuccess) return e0;
-    e0 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cert_per_sm, k_certify, 256, 0);
+    e0 = blocks_per_sm(k_certify, 256, 0, &cert_per_sm);
     if (e0 != cudaSuccess) return e0;
     const int64_t rows_blocks = std::max<int64_t>(1, (a.n + 255) / 256);
     const int64_t rb = std::min<int64_t>(rows_blocks, (int64_t)num_sms * std::max(sel_per_sm, 1));
@@ -639,7 +639,7 @@ static cudaError_t launch_refine_batched(const float* X, const float* C, const T
                           : (a.d <= 32 ? (const void*)k_pair_eval<1>
                                        : (a.d <= 128 ? (const void*)k_pair_eval<4> : (const void*)k_pair_eval<8>));
     int per_sm = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, 0);
+    e = blocks_per_sm_of(fn, 256, 0, &per_sm);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)num_sms * (unsigned)std::max(per_sm, 1);
     const unsigned long long* np = &a.cnt->npairs;
@@ -672,7 +672,7 @@ static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs
     cudaError_t e = allow_max_smem(fn);
     if (e != cudaSuccess) return e;
     int per_sm = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, sm);
+    e = blocks_per_sm(fn, threads, sm, &per_sm);
     if (e != cudaSuccess) return e;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + threads - 1) / threads, (int64_t)num_sms * std::max(per_sm, 1)));
     klaunch(fn, (unsigned)blocks, threads, sm, st, a.rowinfo, a.cand, a.n, a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,

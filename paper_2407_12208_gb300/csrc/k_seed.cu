@@ -406,7 +406,7 @@ cudaError_t launch_seed_pp(const float* X, int64_t n, int d, int k, const double
     }
     if (!kern) return cudaErrorInvalidValue;
     int per_sm = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0);
+    e = blocks_per_sm(kern, 256, 0, &per_sm);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)std::min<int64_t>(pl.ng, (int64_t)num_sms * std::max(per_sm, 1));
     // Theorem 4.1's gamma_{d+2}(2^-24) with safety, and the double-float distance's own 2^-40

@@ -586,7 +586,7 @@ cudaError_t launch_winner_dist(const float* X, int64_t n, int d, const float* C,
     if (!kern) return cudaErrorInvalidValue;
     fn = (const void*)kern;
     int per_sm = 1;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, 0);
+    cudaError_t e = blocks_per_sm_of(fn, 256, 0, &per_sm);
     if (e != cudaSuccess) return e;
     const int rows_per_warp_pass = (nv4 == 4 ? 2 : 4) * (32 / lpr);
     const int64_t warps_needed = (n + rows_per_warp_pass - 1) / rows_per_warp_pass;
@@ -1062,7 +1062,7 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         }
         int per_sm = 8;
         if (bfn) {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)bfn, 256, 0);
+            e = blocks_per_sm_of((const void*)bfn, 256, 0, &per_sm);
             if (e != cudaSuccess) return e;
         }
         const int64_t resident_warps = (int64_t)num_sms * std::max(per_sm, 1) * 8;
