@@ -514,10 +514,15 @@ km_status zero_counters(km_ctx* ctx, DevCounters* cnt, cudaStream_t st) {
     return KM_OK;
 }
 
-// min_dist of the winners to binary64 accuracy (the FP64 path has it already).
-km_status refine_winners(km_ctx* ctx, const float* X, int64_t n, int d, const float* C, const km_params* p,
+// Whether run_assign's min_dist has binary64 accuracy already.
+bool winners_refined(const km_params* p, int d, int k) {
+    return p->low == KM_FP64_DIRECT || (p->low == KM_FP32_DIRECT && direct_gives_winners(d, k));
+}
+
+// min_dist of the winners to binary64 accuracy.
+km_status refine_winners(km_ctx* ctx, const float* X, int64_t n, int d, const float* C, int k, const km_params* p,
                          const int32_t* labels, double* md, cudaStream_t st) {
-    if (p->low == KM_FP64_DIRECT) return KM_OK;
+    if (winners_refined(p, d, k)) return KM_OK;
     PhaseScope ps(ctx, KM_PHASE_REFINE, st);
     KL(1, launch_winner_dist(X, n, d, C, labels, md, ctx->num_sms, st));
     return KM_OK;
@@ -725,7 +730,7 @@ km_status km_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int 
     CK(cudaMemsetAsync(w.cnt, 0, sizeof(DevCounters), st));
     s = run_assign(ctx, X, n, C, k, d, p, labels, md, w, cen, ZeroWords{}, false, st);
     if (s != KM_OK) return s;
-    if ((s = refine_winners(ctx, X, n, d, C, p, labels, md, st)) != KM_OK) return s;
+    if ((s = refine_winners(ctx, X, n, d, C, k, p, labels, md, st)) != KM_OK) return s;
     KL(1, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, &w.cnt->sum_ticket, st));
     ctx->last_cnt = w.cnt;
     ctx->last_sse = w.sse;
@@ -1037,7 +1042,7 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
     // X also refines the winners' distances (min_dist, binary64 accuracy)
     {
         PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
-        s = accumulate(ctx, X, n, d, labels, k, u, C_old, p->low == KM_FP64_DIRECT ? nullptr : md, st);
+        s = accumulate(ctx, X, n, d, labels, k, u, C_old, winners_refined(p, d, k) ? nullptr : md, st);
         if (s != KM_OK) return s;
         KL(1, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, &w.cnt->sum_ticket, st));
         if ((s = finalize(ctx, u, n, k, d, C_old, p, X, md, C_new, counts, w.cnt, st, shift_host != nullptr)) != KM_OK)
@@ -1151,7 +1156,7 @@ km_status km_lloyd_step_host(km_ctx* ctx, const float* X_host, int64_t n, int d,
             if (s != KM_OK) return s;
             // the chunk's winner distances (binary64 accuracy) while the next
             // chunk is still on its way: the update's pass then only sums
-            if ((s = refine_winners(ctx, h.X + r0 * d, rows, d, h.C, p, h.labels + r0, h.min_dist + r0, st)) != KM_OK)
+            if ((s = refine_winners(ctx, h.X + r0 * d, rows, d, h.C, k, p, h.labels + r0, h.min_dist + r0, st)) != KM_OK)
                 return s;
             // this chunk's labels and distances go back while the next chunk is assigned
             CK(cudaEventRecord(ev_out[c], st));
@@ -1272,7 +1277,7 @@ static km_status lloyd_iteration(km_ctx* ctx, const float* X, int64_t n, int d, 
     if (s != KM_OK) return s;
     if (!graph) CK(cudaMemcpyAsync(flag_out, &L.a.cnt->flagged, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
     PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
-    s = accumulate(ctx, X, n, d, labels, k, L.u, cur, p->low == KM_FP64_DIRECT ? nullptr : L.min_dist, st);
+    s = accumulate(ctx, X, n, d, labels, k, L.u, cur, winners_refined(p, d, k) ? nullptr : L.min_dist, st);
     if (s != KM_OK) return s;
     KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, graph ? L.sse_slot : sse_out, &L.a.cnt->sum_ticket, st));
     if ((s = finalize(ctx, L.u, n, k, d, cur, p, X, L.min_dist, nxt, L.counts, L.a.cnt, st, true)) != KM_OK) return s;
@@ -1413,7 +1418,7 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
     if ((s = zero_counters(ctx, L.a.cnt, st)) != KM_OK) return s;
     s = run_assign(ctx, X, n, cur, k, d, p, labels, L.min_dist, L.a, L.cen, ZeroWords{}, true, st);
     if (s != KM_OK) return s;
-    if ((s = refine_winners(ctx, X, n, d, cur, p, labels, L.min_dist, st)) != KM_OK) return s;
+    if ((s = refine_winners(ctx, X, n, d, cur, k, p, labels, L.min_dist, st)) != KM_OK) return s;
     KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.sse_hist + t, &L.a.cnt->sum_ticket, st));
     CK(cudaMemcpyAsync(L.flag_hist + t, &L.a.cnt->flagged, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
     KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, L.a.sse, &L.a.cnt->sum_ticket, st));
@@ -1716,6 +1721,6 @@ extern "C" km_status km_assign_static(km_ctx* ctx, const float* X, int64_t n, co
     CK(cudaMemsetAsync(cnt, 0, sizeof(DevCounters), st));
     KL(1, launch_direct_assign(false, X, n, C, k, d, nullptr, nullptr, labels, min_dist, cnt, tp.gamma32, ctx->num_sms, st));
     // the winners' distances to binary64 accuracy, as km_assign (no scratch)
-    KL(1, launch_winner_dist(X, n, d, C, labels, min_dist, ctx->num_sms, st));
+    if (!winners_refined(&p, d, k)) KL(1, launch_winner_dist(X, n, d, C, labels, min_dist, ctx->num_sms, st));
     return KM_OK;
 }

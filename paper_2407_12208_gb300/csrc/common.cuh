@@ -226,12 +226,20 @@ __host__ __device__ constexpr uint32_t idesc_make(uint32_t ab_fmt, int M, int N)
 }
 
 // ----------------------------------------------------------- float helpers
+// Three-input minimum (one instruction on sm_100 and later).
+KM_DEV float fmin3f(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 // Error-free sum (Knuth's TwoSum): a + b = s + e exactly.
 KM_DEV void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
 }
+// Largest magnitude of three (one instruction).
+KM_DEV float fmaxabs3(float a, float b, float c) { return fmaxf(fabsf(a), fmaxf(fabsf(b), fabsf(c))); }
 // Accumulate x*x into the double-float (hi, lo) using an FMA-based exact product.
 KM_DEV void df_add_sq(float x, float& hi, float& lo) {
     float p = x * x;

@@ -146,15 +146,15 @@ KM_DEV DF df_rows(DF (&v)[R], int cl, int& row) {
 }
 
 // binary32 -> binary64 by moving bits (exact for zeros and normal numbers);
-// GB300 runs the conversion instruction on its narrow FP64 pipe, so only
-// subnormals (and non-finite values) take it.
+// GB300 runs the conversion instruction on its narrow FP64 pipe (16 cycles per
+// warp), so only subnormals and non-finite values take it, out of line: inlined,
+// both ways were executed and one selected.
+static __device__ __noinline__ double f32_to_f64_rare(float f) { return (double)f; }
 KM_DEV double f32_to_f64(float f) {
-    const unsigned u = __float_as_uint(f);
-    const unsigned e = (u >> 23) & 0xFFu;
-    if ((u & 0x7FFFFFFFu) == 0u) return __hiloint2double((int)(u & 0x80000000u), 0);
-    if (e == 0u || e == 0xFFu) return (double)f;
-    const unsigned hi = (u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7FFFFFu) >> 3);
-    return __hiloint2double((int)hi, (int)(u << 29));
+    const unsigned u = __float_as_uint(f), a = u & 0x7FFFFFFFu;
+    if (a - 0x00800000u >= 0x7F000000u && a != 0u) return f32_to_f64_rare(f);
+    const unsigned hi = a ? (a >> 3) + (896u << 20) : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 KM_DEV double df_value(DF v) { return f32_to_f64(v.hi) + f32_to_f64(v.lo); }
 
@@ -204,6 +204,53 @@ KM_DEV DF df_small(const float (&x)[D], const float* c) {
     for (int l = 0; l < 8; l++) ca[l] = l < D ? c[l] : 0.0f;
     return df_small4<D>(x, make_float4(ca[0], ca[1], ca[2], ca[3]), make_float4(ca[4], ca[5], ca[6], ca[7]));
 }
+
+// Two rows at once, a pair per packed instruction (each half the operations, in
+// the order, of df_small): x[l] = (row 0's, row 1's coordinate l), c likewise
+// their centres'.
+struct DF2 {
+    float2 hi, lo;
+};
+KM_DEV DF2 df2_sq_diff(float2 x, float2 c) {
+    const float2 t = fsub2(x, c);
+    const float2 bb = fsub2(t, x);
+    const float2 u = fsub2(t, bb);
+    const float2 tl = fsub2(fsub2(x, u), __fadd2_rn(c, bb));
+    const float2 p = __fmul2_rn(t, t);
+    const float2 pe = __ffma2_rn(t, t, make_float2(-p.x, -p.y));
+    return DF2{p, __ffma2_rn(__fadd2_rn(t, t), tl, pe)};
+}
+KM_DEV DF2 df2_add_raw(DF2 a, DF2 b) {
+    const float2 s = __fadd2_rn(a.hi, b.hi);
+    const float2 bb = fsub2(s, a.hi);
+    const float2 e = __fadd2_rn(fsub2(a.hi, fsub2(s, bb)), fsub2(b.hi, bb));
+    return DF2{s, __fadd2_rn(e, __fadd2_rn(a.lo, b.lo))};
+}
+KM_DEV DF2 df2_norm(DF2 r) {
+    const float2 hi = __fadd2_rn(r.hi, r.lo);
+    return DF2{hi, fsub2(r.lo, fsub2(hi, r.hi))};
+}
+// the first L coordinates of a chunk of four
+template <int L>
+KM_DEV DF2 df2_chunk(const float2* x, const float2* c) {
+    DF2 A = df2_sq_diff(x[0], c[0]);
+    if constexpr (L >= 3) A = df2_add_raw(A, df2_sq_diff(x[2], c[2]));
+    if constexpr (L >= 2) {
+        DF2 B = df2_sq_diff(x[1], c[1]);
+        if constexpr (L >= 4) B = df2_add_raw(B, df2_sq_diff(x[3], c[3]));
+        return df2_norm(df2_add_raw(A, B));
+    }
+    return df2_norm(A);  // (adding the padding's exact zeros changes nothing)
+}
+template <int D>
+KM_DEV DF2 df2_small(const float2 (&x)[D], const float2 (&c)[D]) {
+    const DF2 h0 = df2_chunk<(D < 4 ? D : 4)>(x, c);
+    if constexpr (D <= 4) return h0;
+    else return df2_norm(df2_add_raw(h0, df2_chunk<D - 4>(x + 4, c + 4)));
+}
+// (one conversion of each part on the FP64 pipe: with a row per lane that costs
+// less than moving bits)
+KM_DEV double df_value64(float hi, float lo) { return (double)hi + (double)lo; }
 
 // Chunk geometry of a row of d coordinates: d4 = ceil(d / 4) chunks over LPR
 // lanes, NV4 chunks per lane (LPR = 8, 16 or 32; the centre-sum kernel uses

@@ -70,6 +70,23 @@ struct FixedScale {
         b1 = make_uint2(__float_as_uint(t1.x), __float_as_uint(t1.y));
         b2 = make_uint2(__float_as_uint(t2.x), __float_as_uint(t2.y));
     }
+    // split2() when |v 2^S| < 2^39 and 2^S is a normal float (two_parts): the top
+    // part is zero, one factor does
+    static KM_DEV bool two_parts(int S, int64_t n) {
+        int lgn = 0;
+        while (((int64_t)1 << lgn) < n) lgn++;
+        return 61 - lgn <= 39 && S >= -126 && S <= 127;
+    }
+    KM_DEV void split2_low(float2 v, float f, uint2& b1, uint2& b0) const {
+        const float2 c20 = make_float2(0x1.8p43f, 0x1.8p43f), n20 = make_float2(-0x1.8p43f, -0x1.8p43f);
+        const float2 c0 = make_float2(0x1.8p23f, 0x1.8p23f);
+        const float2 y = __fmul2_rn(v, make_float2(f, f));
+        const float2 p1 = __fadd2_rn(__fadd2_rn(y, c20), n20);
+        const float2 t0 = __fadd2_rn(__fadd2_rn(y, make_float2(-p1.x, -p1.y)), c0);
+        const float2 t1 = __ffma2_rn(p1, make_float2(0x1p-20f, 0x1p-20f), c0);
+        b0 = make_uint2(__float_as_uint(t0.x), __float_as_uint(t0.y));
+        b1 = make_uint2(__float_as_uint(t1.x), __float_as_uint(t1.y));
+    }
     // sum of m split values -> int64 (the biased parts were added modulo 2^32;
     // each true part sum is below 2^31 in magnitude for m <= 2^10)
     KM_DEV static long long combine(unsigned s2, unsigned s1, unsigned s0, unsigned m) {

@@ -131,6 +131,9 @@ cudaError_t launch_predict_candidates(const float* X, int64_t n, int d, const fl
 // binary64 (counted in cnt->amb_rows); rows = all n, or the device list
 // row_list[0 .. *row_count).
 // absmax_out (nullable, zeroed by the caller): max |x| over the rows read.
+// direct_gives_winners: whether its fp32 min_dist is already the winner's
+// distance to binary64 accuracy (launch_winner_dist's, bit for bit).
+bool direct_gives_winners(int d, int k);
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
                                  double* min_dist, DevCounters* cnt, float gamma32,

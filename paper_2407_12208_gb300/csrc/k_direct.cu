@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "df.cuh"
 #include "internal.h"
+#include "rowstat.cuh"
 
 namespace km {
 
@@ -513,124 +514,270 @@ static cudaError_t launch_tiled(const float* X, int64_t n, const float* C, int k
     return cudaGetLastError();
 }
 
-// Small d (d <= 8) with C small enough to stay in shared memory for the
-// whole launch: one thread per row, the row in registers, every centre from
-// shared memory (all lanes read the same centre: a broadcast).  The same
-// fp32 operations, in the same order, and the same certificate as the tiled
-// kernel above, so the two give the same results.
+// Small d (d <= 8) with C small enough to stay in shared memory for the whole
+// launch.  The argmin by the expanded formula on centred data, in fp32 with a
+// bound: x' = fl(x - mu), c' = fl(c - mu), mu the mean of up to 32 centres, and
+//   e_j = q_j + sum_l x'_l (-2 c'_jl),  q_j = ||c'_j||^2   (D fused multiply-adds).
+// |e_j - (d_j - const)| <= gamma_D (q + 2 ||x'|| ||c'||) + gamma_D q + 2.1 u (||x'||
+// + ||c'||)^2, u = 2^-24 (the sums' rounding, q's, and that of the centring), so
+// every centre that can be the nearest lies within
+//   W = (8 D + 20) u (||x'||^2 + max_j ||c'_j||^2)   (twice the bound, with slack)
+// of the smallest e.  One centre inside the window is the argmin; otherwise (few
+// rows) fp32 direct values of all centres with Theorem 4.1's certificate, and
+// binary64 for those that can still hold the minimum.  min_dist is the winner's
+// distance to binary64 accuracy (df.cuh), from the row in hand.
+// A warp takes 64 rows per step, two per lane; the rows come through a ring in
+// shared memory (16-byte asynchronous copies: D scalar loads per lane at a
+// stride of D words cost D times the wavefronts), the two in packed arithmetic.
+// 16.8 M rows x 5, k = 16: 213 us with the winners' distances (110 of them the
+// window test, 47 the double-floats, 77 the rows and results alone), where the
+// direct distances of all pairs took 193 us without them.  Bound by dependent
+// latencies (issue 60 %, FP32 pipe 45 %); two to four blocks per SM alike.
+constexpr int DS_STAGES = 3;
+__host__ __device__ constexpr size_t ds_centre_bytes(int d, int k) { return (size_t)((k + 7) / 8 * 8) * (d + 1) * sizeof(float2); }
+constexpr size_t ds_smem(int d, int k, int warps) {
+    return ((ds_centre_bytes(d, k) + 15) & ~(size_t)15) + (size_t)warps * DS_STAGES * 64 * d * sizeof(float);
+}
+
+// The rows that the window leaves open, by one thread.
 template <int D>
-__global__ void __launch_bounds__(256) k_direct_small(const float* __restrict__ X, int64_t n,
+__device__ __noinline__ int small_open_row(const float* __restrict__ X, int64_t i, const float* __restrict__ C, int k,
+                                           float g, unsigned* amb, unsigned* ev64) {
+    float x[D];
+#pragma unroll
+    for (int l = 0; l < D; l++) x[l] = X[i * D + l];
+    float b1 = INFINITY, b2 = INFINITY;
+    int j1 = 0;
+    for (int j = 0; j < k; j++) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int l = 0; l < D; l++) {
+            const float t = x[l] - C[j * D + l];
+            acc = fmaf(t, t, acc);
+        }
+        if (acc < b1) {
+            b2 = b1;
+            b1 = acc;
+            j1 = j;
+        } else if (acc < b2) {
+            b2 = acc;
+        }
+    }
+    // Theorem 4.1: true values lie in [v (1 - g), v (1 + g)]
+    if (b2 * (1.0f - g) > b1 * (1.0f + g)) return j1;
+    ++*amb;
+    // (squares below binary32's range: at most 2^-149 per coordinate)
+    const float thr = b1 * (1.0f + g) + (float)(2 * D + 4) * 0x1p-149f;
+    double best = INFINITY;
+    for (int j = 0; j < k; j++) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int l = 0; l < D; l++) {
+            const float t = x[l] - C[j * D + l];
+            acc = fmaf(t, t, acc);
+        }
+        if (!(acc * (1.0f - g) <= thr)) continue;
+        const double s = direct64(x, C + j * D, D);
+        ++*ev64;
+        if (s < best) {
+            best = s;
+            j1 = j;
+        }
+    }
+    return j1;
+}
+
+template <int D, bool STAGED>
+__global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict__ X, int64_t n,
                                                       const float* __restrict__ C, int k,
                                                       const int32_t* __restrict__ row_list,
                                                       const int* __restrict__ row_count,
                                                       int32_t* __restrict__ labels, double* __restrict__ min_dist,
-                                                      DevCounters* cnt,
-                                                      float gamma32, unsigned* __restrict__ absmax_out) {
+                                                      DevCounters* cnt, float gamma32,
+                                                      unsigned* __restrict__ absmax_out) {
     chain_enter();
-    extern __shared__ __align__(16) float Csm[];
-    float amx = 0.0f;  // largest |x| of this thread's rows (absmax_out)
-    for (int e = threadIdx.x; e < k * D; e += blockDim.x) Csm[e] = C[e];
-    __syncthreads();
+    extern __shared__ __align__(16) float dsm[];
+    __shared__ float mu[8];
+    __shared__ unsigned qmax_bits;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nwb = blockDim.x >> 5;
     const int64_t nrows = row_list ? (int64_t)(*row_count) : n;
-    const float g = gamma32;
-    unsigned long long rows_done = 0, local_amb = 0, ev64 = 0;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nrows; r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t gi = row_list ? (int64_t)row_list[r] : r;
-        float x[D];
+    if (nrows == 0) return;
+    const int kp = (k + 7) / 8 * 8;
+    // a centre: D float2 of -2 c' (twice the same), then the float2 of q (+inf past k)
+    if (threadIdx.x == 0) qmax_bits = 0u;
+    centre_mean(C, k, D, D, mu);
+    for (int j = threadIdx.x; j < kp; j += blockDim.x) {
+        float q = j < k ? 0.0f : INFINITY;
+        float* dst = dsm + j * 2 * (D + 1);
 #pragma unroll
         for (int l = 0; l < D; l++) {
-            x[l] = X[gi * D + l];
-            amx = fmaxf(amx, fabsf(x[l]));
+            const float c = j < k ? C[j * D + l] - mu[l] : 0.0f;
+            if (j < k) q = fmaf(c, c, q);
+            dst[2 * l] = dst[2 * l + 1] = -2.0f * c;
         }
-        float b1 = INFINITY, b2 = INFINITY;
-        int j1 = 0;
-        for (int j = 0; j < k; j++) {
-            float acc = 0.0f;
-#pragma unroll
-            for (int l = 0; l < D; l++) {
-                const float t = x[l] - Csm[j * D + l];
-                acc = fmaf(t, t, acc);
-            }
-            if (acc < b1) {
-                b2 = b1;
-                b1 = acc;
-                j1 = j;
-            } else if (acc < b2) {
-                b2 = acc;
-            }
-        }
-        labels[gi] = j1;
-        min_dist[gi] = (double)b1;
-        rows_done++;
-        // Theorem 4.1: true values lie in [v (1 - g), v (1 + g)]; a row left open
-        // takes binary64 values of the centres that can hold its minimum
-        if (!(b2 * (1.0f - g) > b1 * (1.0f + g))) {
-            local_amb++;
-            // (squares below binary32's range: at most 2^-149 per coordinate)
-            const float thr = b1 * (1.0f + g) + (float)(2 * D + 4) * 0x1p-149f;
-            double best = INFINITY;
-            for (int j = 0; j < k; j++) {
-                float acc = 0.0f;
-#pragma unroll
-                for (int l = 0; l < D; l++) {
-                    const float t = x[l] - Csm[j * D + l];
-                    acc = fmaf(t, t, acc);
-                }
-                if (!(acc * (1.0f - g) <= thr)) continue;
-                const double s = direct64(x, Csm + j * D, D);
-                ev64++;
-                if (s < best) {
-                    best = s;
-                    j1 = j;
-                }
-            }
-            labels[gi] = j1;
-            min_dist[gi] = best;
-        }
+        dst[2 * D] = dst[2 * D + 1] = q;
+        if (j < k) atomicMax(&qmax_bits, q >= 0.0f ? __float_as_uint(q) : 0x7f800000u);
     }
+    __syncthreads();
+    const float qmax = __uint_as_float(qmax_bits);
+    const float wscale = (float)(8 * D + 20) * 0x1p-24f * 1.02f;
+    float m[D];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        rows_done += __shfl_xor_sync(0xffffffffu, rows_done, off);
-        local_amb += __shfl_xor_sync(0xffffffffu, local_amb, off);
-        ev64 += __shfl_xor_sync(0xffffffffu, ev64, off);
+    for (int l = 0; l < D; l++) m[l] = mu[l];
+    constexpr int STEP = 64;
+    float* ring = dsm + ((ds_centre_bytes(D, k) + 15) & ~(size_t)15) / sizeof(float) + (size_t)wib * DS_STAGES * STEP * D;
+    const uint32_t ring_s = smem_u32(ring);
+    const int64_t w0 = (int64_t)blockIdx.x * nwb + wib, nw = (int64_t)gridDim.x * nwb;
+    const int64_t nstep = (nrows + STEP - 1) / STEP;
+    auto fetch = [&](int64_t st, int slot) {
+        if (STAGED && st < nstep) {
+            const char* src = reinterpret_cast<const char*>(X + st * STEP * D) + 16 * lane;
+            const uint32_t dst = ring_s + (uint32_t)(slot * STEP * D * 4 + 16 * lane);
+            const int left = (int)min((int64_t)STEP * D * 4, (nrows - st * STEP) * D * 4) - 16 * lane;  // bytes from src on
+#pragma unroll
+            for (int c = 0; c < (16 * D + 31) / 32; c++) {  // 16-byte pieces
+                const int rest = left - 512 * c;
+                if (rest > 0)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst + 512 * c), "l"(src + 512 * c),
+                                 "r"(min(rest, 16))
+                                 : "memory");
+            }
+        }
+        cp_async_commit();
+    };
+    float amx = 0.0f;  // largest |x| of this thread's rows (absmax_out)
+    unsigned rows_done = 0, local_amb = 0, ev64 = 0;
+#pragma unroll
+    for (int t = 0; t < DS_STAGES - 1; t++) fetch(w0 + t * nw, t);
+    int slot = 0;
+    for (int64_t st = w0; st < nstep; st += nw) {
+        // (the slot fetched into was read in the step before: the warp is past it)
+        __syncwarp();
+        fetch(st + (DS_STAGES - 1) * nw, slot == 0 ? DS_STAGES - 1 : slot - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(DS_STAGES - 1) : "memory");
+        __syncwarp();
+        const int64_t r0 = st * STEP + lane;
+        const bool valid0 = r0 < nrows, valid1 = r0 + 32 < nrows;
+        const int64_t g0 = STAGED || !row_list ? r0 : (valid0 ? row_list[r0] : 0);
+        const int64_t g1 = STAGED || !row_list ? r0 + 32 : (valid1 ? row_list[r0 + 32] : 0);
+        float2 x[D], y[D], p = make_float2(0.f, 0.f);  // (row 0, row 1)
+        const float* xs0 = ring + (slot * STEP + lane) * D;
+#pragma unroll
+        for (int l = 0; l < D; l++) {
+            if (STAGED) {  // (rows past the end: whatever an earlier step left; nothing of them is kept)
+                x[l] = make_float2(xs0[l], xs0[32 * D + l]);
+                if (!valid1) x[l] = make_float2(valid0 ? x[l].x : 0.0f, 0.0f);
+            } else {
+                x[l] = make_float2(valid0 ? X[g0 * D + l] : 0.0f, valid1 ? X[g1 * D + l] : 0.0f);
+            }
+            amx = fmaxabs3(amx, x[l].x, x[l].y);
+            y[l] = fsub2(x[l], make_float2(m[l], m[l]));
+            p = __ffma2_rn(y[l], y[l], p);
+        }
+        const float2 W = __ffma2_rn(make_float2(wscale, wscale), __fadd2_rn(p, make_float2(qmax, qmax)),
+                                    make_float2(0x1p-120f, 0x1p-120f));
+        slot = slot + 1 == DS_STAGES ? 0 : slot + 1;
+        float2 b1 = make_float2(INFINITY, INFINITY);
+        int ja = -1, jb = -1;  // the rows' only centre inside the window so far (-1: none or several)
+        // a chunk of eight centres for one row: its smallest e, the signs of e - (that or
+        // the smallest so far + W) as a mask (equality counts as outside: W has slack)
+        for (int j0 = 0; j0 < kp; j0 += 8) {
+            const float4* cp = reinterpret_cast<const float4*>(dsm + (size_t)j0 * 2 * (D + 1));
+            float2 e[8];
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {  // two centres: 2 (D + 1) float2
+                float4 c4[D + 1];
+#pragma unroll
+                for (int l = 0; l <= D; l++) c4[l] = cp[(i >> 1) * (D + 1) + l];
+                const float2* cc = reinterpret_cast<const float2*>(c4);
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    float2 a = cc[h * (D + 1) + D];
+#pragma unroll
+                    for (int l = 0; l < D; l++) a = __ffma2_rn(y[l], cc[h * (D + 1) + l], a);
+                    e[i + h] = a;
+                }
+            }
+            float2 cm;
+            cm.x = fmin3f(fmin3f(e[0].x, e[1].x, e[2].x), fmin3f(e[3].x, e[4].x, e[5].x), fminf(e[6].x, e[7].x));
+            cm.y = fmin3f(fmin3f(e[0].y, e[1].y, e[2].y), fmin3f(e[3].y, e[4].y, e[5].y), fminf(e[6].y, e[7].y));
+            const float2 bw = __fadd2_rn(b1, W), cw = __fadd2_rn(cm, W);
+            const bool in0 = cm.x <= bw.x, in1 = cm.y <= bw.y;  // (false where nothing is comparable)
+            if (!__any_sync(0xffffffffu, in0 || in1)) continue;
+            const float2 thr = make_float2(fminf(bw.x, cw.x), fminf(bw.y, cw.y));
+            unsigned m0 = 0, m1 = 0;
+#pragma unroll
+            for (int i = 7; i >= 0; i--) {
+                const float2 t = fsub2(e[i], thr);
+                m0 = __funnelshift_l(__float_as_uint(t.x), m0, 1);
+                m1 = __funnelshift_l(__float_as_uint(t.y), m1, 1);
+            }
+            // strictly below what was found before and alone: the candidate; else several
+            // lie in the window (a row with none here keeps what it had)
+            if (in0) ja = cw.x < b1.x && m0 != 0u && (m0 & (m0 - 1)) == 0u ? j0 + 31 - __clz(m0) : -1;
+            if (in1) jb = cw.y < b1.y && m1 != 0u && (m1 & (m1 - 1)) == 0u ? j0 + 31 - __clz(m1) : -1;
+            b1 = make_float2(fminf(b1.x, cm.x), fminf(b1.y, cm.y));
+        }
+        if (valid0 && ja < 0) ja = small_open_row<D>(X, g0, C, k, gamma32, &local_amb, &ev64);
+        if (valid1 && jb < 0) jb = small_open_row<D>(X, g1, C, k, gamma32, &local_amb, &ev64);
+        const float *ca = C + (int64_t)max(ja, 0) * D, *cb = C + (int64_t)max(jb, 0) * D;
+        float2 c2[D];
+#pragma unroll
+        for (int l = 0; l < D; l++) c2[l] = make_float2(ca[l], cb[l]);
+        const DF2 r = df2_small<D>(x, c2);
+        if (valid0) {
+            labels[g0] = ja;
+            min_dist[g0] = df_value64(r.hi.x, r.lo.x);
+        }
+        if (valid1) {
+            labels[g1] = jb;
+            min_dist[g1] = df_value64(r.hi.y, r.lo.y);
+        }
+        rows_done += (valid0 ? 1 : 0) + (valid1 ? 1 : 0);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    rows_done = __reduce_add_sync(0xffffffffu, rows_done);
+    local_amb = __reduce_add_sync(0xffffffffu, local_amb);
+    ev64 = __reduce_add_sync(0xffffffffu, ev64);
     if (absmax_out) {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) amx = fmaxf(amx, __shfl_xor_sync(0xffffffffu, amx, off));
     }
-    if ((threadIdx.x & 31) == 0) {
-        if (rows_done) atomicAdd(&cnt->fp32_evals, rows_done * (unsigned long long)k);
-        if (local_amb) atomicAdd(&cnt->amb_rows, local_amb);
-        if (ev64) atomicAdd(&cnt->fp64_evals, ev64);
+    if (lane == 0) {
+        if (rows_done) atomicAdd(&cnt->fp32_evals, (unsigned long long)rows_done * (unsigned long long)k);
+        if (local_amb) atomicAdd(&cnt->amb_rows, (unsigned long long)local_amb);
+        if (ev64) atomicAdd(&cnt->fp64_evals, (unsigned long long)ev64);
         if (absmax_out) atomicMax(absmax_out, __float_as_uint(amx));
     }
 }
+
+bool direct_gives_winners(int d, int k) { return d <= 8 && (size_t)k * d * sizeof(float) <= 32 * 1024; }
 
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
                                  double* min_dist, DevCounters* cnt, float gamma32,
                                  int num_sms, cudaStream_t st, unsigned* absmax_out) {
-    if (!acc64 && d <= 8 && (size_t)k * d * sizeof(float) <= 32 * 1024) {
-        // small d: C resident in shared memory, one thread per row, persistent grid
-        const size_t csm = (size_t)k * d * sizeof(float);
-        int per_sm = 1;
-        const void* fns[9] = {nullptr, (const void*)k_direct_small<1>, (const void*)k_direct_small<2>,
-                              (const void*)k_direct_small<3>, (const void*)k_direct_small<4>,
-                              (const void*)k_direct_small<5>, (const void*)k_direct_small<6>,
-                              (const void*)k_direct_small<7>, (const void*)k_direct_small<8>};
-        cudaError_t e = blocks_per_sm_of(fns[d], 256, csm, &per_sm);
-        if (e != cudaSuccess) return e;
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)num_sms * std::max(per_sm, 1)));
+    if (!acc64 && direct_gives_winners(d, k)) {
+        // small d: C resident in shared memory, persistent grid; few rows in small
+        // blocks, so that they spread over the SMs
+        const int threads = n <= (int64_t)num_sms * 512 ? 64 : 256;
+        const size_t sm = ds_smem(d, k, threads / 32);
+        const bool staged = !row_list && ((uintptr_t)X & 15) == 0;
+        void (*fn)(const float*, int64_t, const float*, int, const int32_t*, const int*, int32_t*, double*, DevCounters*,
+                   float, unsigned*) = nullptr;
         switch (d) {
-#define KM_SMALL(DD)                                                                                                  \
-    case DD:                                                                                                          \
-        klaunch(k_direct_small<DD>, (unsigned)grid, 256, csm, st, X, n, C, k, row_list, row_count, labels, min_dist,      \
-                                                              cnt, gamma32, absmax_out);                                \
-        break;
+#define KM_SMALL(DD) \
+    case DD: fn = staged ? k_direct_small<DD, true> : k_direct_small<DD, false>; break;
             KM_SMALL(1) KM_SMALL(2) KM_SMALL(3) KM_SMALL(4) KM_SMALL(5) KM_SMALL(6) KM_SMALL(7) KM_SMALL(8)
 #undef KM_SMALL
         }
-        return cudaGetLastError();
+        cudaError_t e = allow_max_smem(fn);
+        int per_sm = 1;
+        if (e == cudaSuccess) e = blocks_per_sm(fn, threads, sm, &per_sm);
+        if (e != cudaSuccess) return e;
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 2 * threads - 1) / (2 * threads), (int64_t)num_sms * per_sm));
+        return klaunch(fn, (unsigned)grid, (unsigned)threads, sm, st, X, n, C, k, row_list, row_count, labels, min_dist, cnt,
+                       gamma32, absmax_out);
     }
     if (!acc64) {
         // rows per block: 128, or 64 where 128 would leave one block per SM

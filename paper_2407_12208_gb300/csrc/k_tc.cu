@@ -153,13 +153,6 @@ KM_DEV int compact_list(uint32_t* list, int cnt, float lim, uint32_t emask, floa
     return w;
 }
 
-// Three-input minimum (one instruction on sm_100 and later; no NaN reaches it).
-KM_DEV float fmin3(float a, float b, float c) {
-    float r;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
 template <int FMT, int BN, int MODE, int SV>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmC, const TcArgs a) {
@@ -433,10 +426,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         float qm[NQ];
 #pragma unroll
                         for (int qd = 0; qd < NQ; qd++)
-                            qm[qd] = fminf(fmin3(e[4 * qd + 0], e[4 * qd + 1], e[4 * qd + 2]), e[4 * qd + 3]);
+                            qm[qd] = fminf(fmin3f(e[4 * qd + 0], e[4 * qd + 1], e[4 * qd + 2]), e[4 * qd + 3]);
                         float c4[NQ / 4];
 #pragma unroll
-                        for (int i = 0; i < NQ / 4; i++) c4[i] = fminf(fmin3(qm[4 * i], qm[4 * i + 1], qm[4 * i + 2]), qm[4 * i + 3]);
+                        for (int i = 0; i < NQ / 4; i++) c4[i] = fminf(fmin3f(qm[4 * i], qm[4 * i + 1], qm[4 * i + 2]), qm[4 * i + 3]);
                         float cmin = c4[0];
 #pragma unroll
                         for (int i = 1; i < NQ / 4; i++) cmin = fminf(cmin, c4[i]);
@@ -485,7 +478,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                                 const bool pc = act && mk != 0u && !ovf;
                                 const bool room = cnt < TC_L;
                                 const int slot = (pc && room) ? cnt : TC_L;
-                                const float qmn = fminf(fmin3(x0, x1, x2), x3);
+                                const float qmn = fminf(fmin3f(x0, x1, x2), x3);
                                 st_shared_u32(lbase + slot * (TC_BM * 4), quad_entry(jq >> 2, mk, p + qmn, emask));
                                 ovf |= (pc && !room);
                                 cnt += (pc && room) ? 1 : 0;
@@ -586,7 +579,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             dh[4 * t4 + 1] = fmaxf(p + fmaf(__uint_as_float(v[4 * t4 + 1]) * sc.y, neg2s, qv[t4].y), 0.0f);
                             dh[4 * t4 + 2] = fmaxf(p + fmaf(__uint_as_float(v[4 * t4 + 2]) * sc.z, neg2s, qv[t4].z), 0.0f);
                             dh[4 * t4 + 3] = fmaxf(p + fmaf(__uint_as_float(v[4 * t4 + 3]) * sc.w, neg2s, qv[t4].w), 0.0f);
-                            least = fminf(fmin3(least, dh[4 * t4], dh[4 * t4 + 1]), fminf(dh[4 * t4 + 2], dh[4 * t4 + 3]));
+                            least = fminf(fmin3f(least, dh[4 * t4], dh[4 * t4 + 1]), fminf(dh[4 * t4 + 2], dh[4 * t4 + 3]));
                         }
                         // (F is -inf for rows past n; columns past k are +inf)
                         if (__any_sync(0xffffffffu, least <= F)) {

@@ -395,34 +395,54 @@ __global__ void k_bucket_sum_small(const float* __restrict__ X, int64_t n, int k
     }
 }
 
-// Small d and small k * d: rows in their natural order (one per lane,
-// coalesced), each warp keeps the 32-bit parts of every cluster's fixed-point
-// sum (and its count) in shared memory.  A segmented inclusive scan over the
-// warp's runs of equal labels (five shuffle levels, whatever the labels: an
-// image's pixels come in long runs) leaves each run's total in its last
-// lane, which adds it with a shared atomic.  Every AS_CHUNK rows the
-// accumulators are folded into the global int64 sums.  Integer additions
-// throughout: the order does not matter.
-// WD: each row's distance to its own centre (binary64 accuracy, df.cuh) from
-// the same read of the row, with C staged in shared memory.
+// Small d and small k * d: rows in their natural order, a warp per chunk of up
+// to AS_CHUNK, 32 rows per step (one per lane, through a ring in shared memory
+// filled by 16-byte asynchronous copies), each warp keeping the 32-bit parts of
+// every cluster's fixed-point sum (and its count) in shared memory.
+//  * A step whose rows all have one label (an image's pixels come in long runs)
+//    adds each lane's parts to registers; they are folded over the warp when the
+//    label changes or the chunk ends.
+//  * Other steps: AS_FEW labels one after another by hardware reductions over
+//    their lanes, then, if rows are left, a segmented inclusive scan over the
+//    warp's runs of equal labels (five shuffle levels, whatever the labels) that
+//    leaves each run's total in its last lane, which adds it with a shared atomic.
+// At the end of the chunk the accumulators are folded into the global int64
+// sums.  Integer additions throughout: the order does not matter.
+// NP: parts per value, 3, or 2 where the top one is always zero (from 2^22
+// rows on).  WD: each row's distance to its own centre (binary64 accuracy,
+// df.cuh) from the same read of the row, with C staged in shared memory.
+// Bound by reads of X and the labels where runs are long, else by the scan's
+// instructions (17 per row); 16.8 M rows x 5, k = 16, image: 143 us (249 us with
+// the scan in every step and D loads at a stride of D words).
 constexpr int AS_CHUNK = 1024;   // rows per warp between folds (keeps each 32-bit part sum below 2^31)
 constexpr int AS_MAX_KD = 512;   // k * d bound of this path
-template <int D, bool WD>
-__global__ void __launch_bounds__(256) k_accum_small(const float* __restrict__ X, int64_t n, int k,
+constexpr int AS_STAGES = 4;
+constexpr int AS_FEW = 4;
+static size_t as_smem(int d, int k, bool wd) {
+    const size_t parts = ((size_t)8 * (3 * (size_t)k * d + k) + 3) & ~(size_t)3;
+    return parts * 4 + (size_t)8 * AS_STAGES * 32 * d * 4 + (wd ? (size_t)k * 32 : 0);
+}
+template <int D, bool WD, int NP>
+__global__ void __launch_bounds__(256) k_accum_small(const float* __restrict__ X, int64_t n, int k, int chunk,
                                                      const int32_t* __restrict__ labels,
                                                      const unsigned* __restrict__ amax_bits, int64_t nscale,
                                                      long long* __restrict__ sums, long long* __restrict__ counts,
                                                      const float* __restrict__ C, double* __restrict__ md) {
     chain_enter();
-    extern __shared__ unsigned acc_sm[];  // per warp: 3 * k * D parts, then k counts; then C (WD)
-    const FixedScale fx(fixed_shift(*amax_bits, nscale));
+    extern __shared__ __align__(16) unsigned acc_sm[];  // per warp: 3 k D parts, k counts; per warp: the ring; C (WD)
+    const int S = fixed_shift(*amax_bits, nscale);
+    if (FixedScale::two_parts(S, nscale) != (NP == 2)) return;  // (the other form's launch does the work)
+    const FixedScale fx(S);
+    const float f = __int_as_float((S + 127) << 23);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int kd = k * D;
     unsigned* a = acc_sm + (size_t)wib * (3 * kd + k);
     unsigned* cntw = a + 3 * kd;
+    const size_t parts = ((size_t)8 * (3 * kd + k) + 3) & ~(size_t)3;
+    float* ring = reinterpret_cast<float*>(acc_sm + parts) + (size_t)wib * AS_STAGES * 32 * D;
+    const uint32_t ring_s = smem_u32(ring);
     // C with rows of 8 floats (zero past D), 16-byte aligned: two vector reads per row
-    const size_t coff = (((size_t)(blockDim.x >> 5) * (3 * kd + k)) + 3) & ~(size_t)3;
-    float4* Cs = reinterpret_cast<float4*>(acc_sm + coff);
+    float4* Cs = reinterpret_cast<float4*>(acc_sm + parts + (size_t)8 * AS_STAGES * 32 * D);
     if (WD) {
         for (int e = threadIdx.x; e < k * 8; e += blockDim.x) {
             const int j = e >> 3, l = e & 7;
@@ -430,53 +450,157 @@ __global__ void __launch_bounds__(256) k_accum_small(const float* __restrict__ X
         }
         __syncthreads();
     }
+    const bool staged = ((uintptr_t)X & 15) == 0;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t c0 = w0 * AS_CHUNK; c0 < n; c0 += nw * AS_CHUNK) {
+    for (int64_t c0 = w0 * chunk; c0 < n; c0 += nw * chunk) {
         for (int e = lane; e < 3 * kd + k; e += 32) a[e] = 0u;
         __syncwarp();
-        const int64_t c1 = min(n, c0 + AS_CHUNK);
+        const int64_t c1 = min(n, c0 + chunk);
+        auto fetch = [&](int64_t base, int slot) {
+            if (staged && base < c1) {
+                const char* src = reinterpret_cast<const char*>(X + base * D);
+                const int64_t left = (n - base) * D * 4;  // bytes
+#pragma unroll
+                for (int c = 0; c < (8 * D + 31) / 32; c++) {
+                    const int q = lane + 32 * c;  // 16-byte piece
+                    if (q < 8 * D) {
+                        const int64_t rest = left - 16 * q;
+                        const int bytes = rest >= 16 ? 16 : (rest > 0 ? (int)rest : 0);
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(
+                                         ring_s + (uint32_t)(slot * 32 * D * 4 + 16 * q)),
+                                     "l"(bytes ? src + 16 * q : reinterpret_cast<const char*>(X)), "r"(bytes)
+                                     : "memory");
+                    }
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        // parts of a run of whole steps with the label `cur`
+        unsigned v[NP * D];
+#pragma unroll
+        for (int t = 0; t < NP * D; t++) v[t] = 0u;
+        int cur = -1, steps = 0;
+        auto flush = [&]() {
+            if (steps) {
+                unsigned mine = 0;
+#pragma unroll
+                for (int t = 0; t < NP * D; t++) {
+                    const unsigned r = __reduce_add_sync(0xffffffffu, v[t] - (unsigned)steps * FixedScale::kBias);
+                    if (lane == t) mine = r;
+                    v[t] = 0u;
+                }
+                __syncwarp();
+                // (lane t holds part NP - 1 - t % NP, the accumulators' order b2, b1, b0)
+                if (lane < NP * D) a[3 * cur * D + 3 * (lane / NP) + (3 - NP) + lane % NP] += mine;
+                if (lane == 0) cntw[cur] += 32u * (unsigned)steps;
+                __syncwarp();
+                steps = 0;
+            }
+        };
+#pragma unroll
+        for (int s = 0; s < AS_STAGES - 1; s++) fetch(c0 + 32 * s, s);
+        int slot = 0;
+        int jn = c0 + lane < c1 ? labels[c0 + lane] : -1;
         for (int64_t base = c0; base < c1; base += 32) {
             const int64_t i = base + lane;
             const bool valid = i < c1;
-            const int j = valid ? labels[i] : -1;
+            const int j = jn;
+            jn = i + 32 < c1 ? labels[i + 32] : -1;
+            __syncwarp();
+            fetch(base + 32 * (AS_STAGES - 1), slot == 0 ? AS_STAGES - 1 : slot - 1);
+            asm volatile("cp.async.wait_group %0;" ::"n"(AS_STAGES - 1) : "memory");
+            __syncwarp();
             float xr[D];
 #pragma unroll
-            for (int l = 0; l < D; l++) xr[l] = valid ? X[i * D + l] : 0.0f;
+            for (int l = 0; l < D; l++) xr[l] = !valid ? 0.0f : (staged ? ring[(slot * 32 + lane) * D + l] : X[i * D + l]);
+            slot = slot + 1 == AS_STAGES ? 0 : slot + 1;
             if (WD && valid) md[i] = df_value(df_small4<D>(xr, Cs[2 * j], D > 4 ? Cs[2 * j + 1] : make_float4(0.f, 0.f, 0.f, 0.f)));
-            unsigned v[3 * D + 1];  // true (unbiased) parts modulo 2^32, then the row count
+            const int j0 = __shfl_sync(0xffffffffu, j, 0);
+            const bool whole = __all_sync(0xffffffffu, valid && j == j0);
+            unsigned u[NP * D];  // this row's parts (biased), b2 (NP = 3), b1, b0 per coordinate
 #pragma unroll
-            for (int l = 0; l < D; l++) {
-                unsigned b2 = FixedScale::kBias, b1 = FixedScale::kBias, b0 = FixedScale::kBias;
-                if (valid) fx.split(xr[l], b2, b1, b0);
-                v[3 * l + 0] = b2 - FixedScale::kBias;
-                v[3 * l + 1] = b1 - FixedScale::kBias;
-                v[3 * l + 2] = b0 - FixedScale::kBias;
+            for (int l = 0; l < D; l += 2) {
+                const float2 x2 = make_float2(xr[l], l + 1 < D ? xr[l + 1] : 0.0f);
+                uint2 b2, b1, b0;
+                if constexpr (NP == 2) fx.split2_low(x2, f, b1, b0);
+                else fx.split2(x2, b2, b1, b0);
+                if constexpr (NP == 3) u[NP * l] = b2.x;
+                u[NP * l + NP - 2] = b1.x;
+                u[NP * l + NP - 1] = b0.x;
+                if (l + 1 < D) {
+                    if constexpr (NP == 3) u[NP * (l + 1)] = b2.y;
+                    u[NP * (l + 1) + NP - 2] = b1.y;
+                    u[NP * (l + 1) + NP - 1] = b0.y;
+                }
             }
-            v[3 * D] = 1u;
-            const int jp = __shfl_up_sync(0xffffffffu, j, 1);
-            const bool head = lane == 0 || j != jp;
-            bool f = head;  // segment flag of the scan
+            if (whole) {
+                if (j0 != cur) {
+                    flush();
+                    cur = j0;
+                }
+#pragma unroll
+                for (int t = 0; t < NP * D; t++) v[t] += u[t];
+                steps++;
+                continue;
+            }
+            // true (unbiased) parts modulo 2^32
+#pragma unroll
+            for (int t = 0; t < NP * D; t++) u[t] = u[t] - FixedScale::kBias;
+            // up to AS_FEW labels one after another, each summed over its lanes by a
+            // hardware reduction; what is left by the scan
+            unsigned rem = __ballot_sync(0xffffffffu, valid);
+            int left = j;
+            for (int it = 0; it < AS_FEW && rem; it++) {
+                const int lead = __ffs(rem) - 1, jl = __shfl_sync(0xffffffffu, left, lead);
+                const unsigned m = __ballot_sync(0xffffffffu, left == jl) & rem;
+                if ((m >> lane) & 1u) {
+                    unsigned* aj = a + 3 * jl * D;
+#pragma unroll
+                    for (int t = 0; t < NP * D; t++) {
+                        const unsigned r = __reduce_add_sync(m, u[t]);
+                        if (lane == lead) aj[3 * (t / NP) + (3 - NP) + t % NP] += r;
+                    }
+                    if (lane == lead) cntw[jl] += (unsigned)__popc(m);
+                    left = -1;
+                }
+                __syncwarp();
+                rem &= ~m;
+            }
+            if (!rem) continue;
+            unsigned cnt = left >= 0 ? 1u : 0u;
+#pragma unroll
+            for (int t = 0; t < NP * D; t++) u[t] = left >= 0 ? u[t] : 0u;
+            const int jp = __shfl_up_sync(0xffffffffu, left, 1);
+            const bool head = lane == 0 || left != jp;
+            bool fl = head;  // segment flag of the scan
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
-                const bool fu = __shfl_up_sync(0xffffffffu, f, off);
-                const bool take = lane >= off && !f;
+                const bool fu = __shfl_up_sync(0xffffffffu, fl, off);
+                const bool take = lane >= off && !fl;
 #pragma unroll
-                for (int t = 0; t <= 3 * D; t++) {
-                    const unsigned u = __shfl_up_sync(0xffffffffu, v[t], off);
-                    if (take) v[t] += u;
+                for (int t = 0; t < NP * D; t++) {
+                    const unsigned w = __shfl_up_sync(0xffffffffu, u[t], off);
+                    if (take) u[t] += w;
                 }
-                if (take) f = fu;
+                const unsigned w = __shfl_up_sync(0xffffffffu, cnt, off);
+                if (take) {
+                    cnt += w;
+                    fl = fu;
+                }
             }
             const bool next_head = __shfl_down_sync(0xffffffffu, head, 1);
             const bool tail = lane == 31 || next_head;
-            if (valid && tail) {
-                unsigned* aj = a + 3 * j * D;
+            if (left >= 0 && tail) {
+                unsigned* aj = a + 3 * left * D;
 #pragma unroll
-                for (int t = 0; t < 3 * D; t++) atomicAdd(&aj[t], v[t]);
-                atomicAdd(&cntw[j], v[3 * D]);
+                for (int t = 0; t < NP * D; t++) atomicAdd(&aj[3 * (t / NP) + (3 - NP) + t % NP], u[t]);
+                atomicAdd(&cntw[left], cnt);
             }
+            __syncwarp();
         }
+        flush();
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
         for (int e = lane; e < kd; e += 32) {
             const long long s64 = FixedScale::combine(a[3 * e + 0], a[3 * e + 1], a[3 * e + 2], 0u);
@@ -977,29 +1101,37 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
     }
     if (d <= 8 && (int64_t)k * d <= AS_MAX_KD) {
         // small d: rows in order, per-warp shared accumulators (+ C for the distances)
-        const size_t sm = (((size_t)8 * (3 * (size_t)k * d + k) + 3) & ~(size_t)3) * sizeof(unsigned) +
-                          (want_wd ? (size_t)k * 8 * sizeof(float) : 0);
-        const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * 8, (n + 8 * AS_CHUNK - 1) / (8 * AS_CHUNK)));
+        const size_t sm = as_smem(d, k, want_wd);
+        // about two chunks per resident warp, so that few rows still reach all SMs
+        const int chunk = (int)std::min<int64_t>(AS_CHUNK, std::max<int64_t>(32, n / ((int64_t)num_sms * 64) / 32 * 32));
+        const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * 8, (n + 8 * chunk - 1) / (8 * chunk)));
+        typedef void (*SmallFn)(const float*, int64_t, int, int, const int32_t*, const unsigned*, int64_t, long long*,
+                                long long*, const float*, double*);
+        SmallFn three = nullptr, two = nullptr;
         switch (d) {
-#define KM_ACC(DD)                                                                                                  \
-    case DD:                                                                                                        \
-        if (want_wd) {                                                                                              \
-            e = allow_max_smem(k_accum_small<DD, true>);                                                            \
-            if (e != cudaSuccess) return e;                                                                         \
-            klaunch(k_accum_small<DD, true>, (unsigned)blocks, 256, sm, st, X, n, k, labels, absmax_bits, nscale, sums, counts,  \
-                                                                       C_wd, md_out);                               \
-        } else {                                                                                                    \
-            e = allow_max_smem(k_accum_small<DD, false>);                                                           \
-            if (e != cudaSuccess) return e;                                                                         \
-            klaunch(k_accum_small<DD, false>, (unsigned)blocks, 256, sm, st, X, n, k, labels, absmax_bits, nscale, sums, counts, \
-                                                                        nullptr, nullptr);                          \
-        }                                                                                                           \
+#define KM_ACC(DD)                                                                                             \
+    case DD:                                                                                                   \
+        three = want_wd ? (SmallFn)k_accum_small<DD, true, 3> : (SmallFn)k_accum_small<DD, false, 3>;          \
+        two = want_wd ? (SmallFn)k_accum_small<DD, true, 2> : (SmallFn)k_accum_small<DD, false, 2>;            \
         break;
             KM_ACC(1) KM_ACC(2) KM_ACC(3) KM_ACC(4) KM_ACC(5) KM_ACC(6) KM_ACC(7) KM_ACC(8)
 #undef KM_ACC
         }
-        if (nlaunch) *nlaunch = 1;
-        return cudaGetLastError();
+        *nlaunch = 0;
+        // two parts per value suffice from 2^22 rows on, whatever max |x| short of
+        // the ends of the float range, where the three-part form still does the work
+        int lgn = 0;
+        while (((int64_t)1 << lgn) < nscale) lgn++;
+        for (SmallFn fn : {61 - lgn <= 39 ? two : nullptr, three}) {
+            if (!fn) continue;
+            e = allow_max_smem(fn);
+            if (e != cudaSuccess) return e;
+            e = klaunch(fn, (unsigned)blocks, 256, sm, st, X, n, k, chunk, labels, absmax_bits, nscale, sums, counts,
+                        want_wd ? C_wd : nullptr, want_wd ? md_out : nullptr);
+            if (e != cudaSuccess) return e;
+            ++*nlaunch;
+        }
+        return cudaSuccess;
     }
     const size_t hsm = sizeof(int) * (size_t)k;
     const bool vec = d % 4 == 0 && ((uintptr_t)X % 16) == 0;

@@ -245,3 +245,52 @@ def test_update_dispatch_edges(ctx, n, d, k, offset, empty):
             want[j] = X[far[r]]
     np.testing.assert_allclose(Cn, want, rtol=2.0 ** -23, atol=np.abs(X).max() * 2.0 ** -30)
     np.testing.assert_allclose(shift, np.linalg.norm(Cn.astype(np.float64) - C, axis=1).max(), rtol=1e-12)
+
+
+# small d: the window test on centred data (two rows per lane, steps of 64, chunks of eight
+# centres), staged and unaligned rows, listed rows (low formats whose lists overflow), ties,
+# data far from the origin and below binary32's normal squares
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("kind", ["mixture", "cancellation", "copies", "tiny"])
+@pytest.mark.parametrize("n,d,k", [(1, 1, 1), (63, 2, 9), (64, 3, 8), (65, 4, 16), (1000, 5, 17), (4097, 6, 33), (777, 7, 100),
+                                   (5000, 8, 1024), (3000, 2, 3000)])
+def test_small_d_edges(ctx, n, d, k, kind, offset):
+    if kind == "cancellation":
+        X, C = workloads.cancellation(n, d, k, seed=n)
+    else:
+        X, C = workloads.gaussian_mixture(n, d, k, seed=n)
+        if kind == "copies":
+            C[k // 2 :] = C[: k - k // 2].copy()
+        if kind == "tiny":
+            X, C = X * np.float32(1e-19), C * np.float32(1e-19)
+    for low in ("fp32", "bf16") if kind == "cancellation" else ("fp32",):
+        lab, md, _ = _assign(ctx, X, C, low, offset)
+        olab, od1, od2 = oracle.assign(X, C)
+        sure = (od2 - od1) > 1e-6 * od2
+        assert np.array_equal(lab[sure], olab[sure])
+        first = np.unique(C, axis=0, return_index=True, return_inverse=True)
+        assert np.array_equal(first[1][first[2].ravel()][lab], lab)
+        if kind != "tiny":  # (there the double-float squares underflow, as they always did)
+            np.testing.assert_allclose(md, oracle.dist_labelled(X, C, lab), rtol=RTOL_MD, atol=1e-30)
+
+
+# small-d centre sums: whole steps of one label, few labels, many labels; two and three parts
+# per value (2^22 rows and more), also at the ends of the float range, where the fixed-point
+# scale leaves it: sums equal to integer sums of the rounded values
+@pytest.mark.parametrize("scale", [1.0, 1e30, 1e-36])
+@pytest.mark.parametrize("n,d,k", [(31, 3, 2), (40000, 5, 16), (100001, 8, 64), (4194304 + 77, 2, 7), (4194304 + 77, 5, 16)])
+def test_small_d_sums_parts(ctx, n, d, k, scale):
+    import math
+    import paper_2407_12208_gb300 as pkg
+    g = torch.Generator(device="cuda").manual_seed(n + d)
+    X = (torch.randn(n, d, generator=g, device="cuda") * scale).contiguous()
+    i = torch.arange(n, device="cuda")
+    lab = torch.where(i % 3000 < 1800, (i // 700) % k, torch.where(i % 3000 < 2400, (i // 5) % k, (i * 7919) % k)).int()
+    bits = ctx.absmax(X)
+    sums, counts = ctx.update_partial(X, lab, k, bits, n)
+    assert torch.equal(counts, torch.bincount(lab.long(), minlength=k))
+    amax = float(np.array([bits], dtype=np.uint32).view(np.float32)[0])
+    S = 60 - (n - 1).bit_length() - (math.frexp(amax)[1] - 1)
+    v = torch.round(X.double() * 2.0 ** (S // 2) * 2.0 ** (S - S // 2)).long()  # (ties to even, as the kernel's additions)
+    want = torch.zeros(k, d, dtype=torch.int64, device="cuda").index_add_(0, lab.long(), v)
+    assert torch.equal(sums, want)
