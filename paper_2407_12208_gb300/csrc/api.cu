@@ -466,7 +466,7 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
         PhaseScope ps(ctx, KM_PHASE_REFINE, st);
         int nl = 0;
         CK(launch_refine(X, C, a, nullptr, nullptr, labels, min_dist, w.ovf_list, &w.cnt->ovf_count, w.amb_list,
-                         ctx->num_sms, st, &nl));
+                         cen.Xq != nullptr, ctx->num_sms, st, &nl));
         ctx->launches += (uint64_t)nl;
     }
     {
@@ -494,7 +494,7 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
             KL(1, launch_tc(cen.Xq, cen.Cq, cen.ldq, b, ctx->num_sms, st));
             int nl = 0;
             KL(1, launch_refine(X, C, b, list, list_n, labels, min_dist, cen.list2, &w.cnt->ovf2_count, w.amb_list,
-                                ctx->num_sms, st, &nl));
+                                false, ctx->num_sms, st, &nl));
             list = cen.list2;
             list_n = &w.cnt->ovf2_count;
         }

@@ -186,10 +186,11 @@ size_t tc_smem_bytes(int fmt, int d, int k);
 // candidate refinement: the certified argmin of every row from its candidates
 // (list, list_n null: row r of a.cand / a.rowinfo is row r of X; else row
 // list[r] for r < *list_n); rows whose list overflowed are appended to
-// ovf_list / *ovf_n (amb_list, min_dist: scratch, min_dist of the winners in fp32)
+// ovf_list / *ovf_n, as may be rows of many candidates (centred_follows: the
+// centred screen takes them next; amb_list, min_dist: scratch)
 cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, const int32_t* list, const int* list_n,
-                          int32_t* labels, double* min_dist, int32_t* ovf_list, int* ovf_n, int32_t* amb_list, int num_sms,
-                          cudaStream_t st, int* nlaunch);
+                          int32_t* labels, double* min_dist, int32_t* ovf_list, int* ovf_n, int32_t* amb_list,
+                          bool centred_follows, int num_sms, cudaStream_t st, int* nlaunch);
 // whether the refinement of n rows takes the flat pair list (a.pairs ..)
 bool refine_batched(int64_t n, int d);
 // centred bf16 copies of the listed rows and of the centres (d <= 256), when

@@ -10,6 +10,7 @@
 //    row), lowest index on ties; binary64 values with products and sums rounded
 //    separately (no FMA), equal to the CPU oracle's bit for bit.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "df.cuh"
@@ -282,12 +283,9 @@ constexpr int DT_C = 64;    // centres per tile
 constexpr int DT_DK = 64;   // coordinates per streamed chunk
 
 template <int BYTES>
-KM_DEV void cp_async(uint32_t dst, const void* src, bool full) {
-    if constexpr (BYTES == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(full ? 16 : 0) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(full ? BYTES : 0)
-                     : "memory");
+KM_DEV void cp_async(uint32_t dst, const void* src) {
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
 }
 KM_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 KM_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
@@ -312,11 +310,10 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
     float* Xs = dts;
     float* Cs = dts + R * ldx;  // [2][DT_C][ldc]
     const uint32_t cs0 = smem_u32(Cs);
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3, lane = tid & 31, wid = tid >> 5;
     const int64_t nrows = row_list ? (int64_t)(*row_count) : n;
     const int ntile = (k + DT_C - 1) / DT_C, nck = (dp + DT_DK - 1) / DT_DK, nstep = ntile * nck;
     const float g = gamma32;
-    const int dv = d / VEC;  // loads per row
     __shared__ int open_rows[R], nopen;
     float amx = 0.0f;
     unsigned long long local_amb = 0, ev64 = 0;
@@ -327,32 +324,40 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
     for (int64_t base = (int64_t)blockIdx.x * R; base < nrows; base += (int64_t)gridDim.x * R) {
         const int rows_here = (int)min((int64_t)R, nrows - base);
         __syncthreads();  // the previous round's readers are done with all buffers
-        for (int e = tid; e < R * dv; e += 256) {
-            const int r = e / dv, l = (e - r * dv) * VEC;
-            float v[VEC];
+        // a warp per row, lanes along it: coalesced, no index division
+#pragma unroll 2
+        for (int r = wid; r < R; r += 8) {
+            const bool have = r < rows_here;
+            const int64_t gi = !have ? 0 : (row_list ? (int64_t)row_list[base + r] : base + r);
+            const float* src = X + gi * d;
+#pragma unroll 4
+            for (int l = lane * VEC; l < d; l += 32 * VEC) {
+                float v[VEC];
 #pragma unroll
-            for (int t = 0; t < VEC; t++) v[t] = 0.0f;
-            if (r < rows_here) {
-                const int64_t gi = row_list ? (int64_t)row_list[base + r] : base + r;
-                const float* src = X + gi * d + l;
-                if constexpr (VEC == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(src);
-                else if constexpr (VEC == 2) *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(src);
-                else v[0] = *src;
+                for (int t = 0; t < VEC; t++) v[t] = 0.0f;
+                if (have) {
+                    if constexpr (VEC == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(src + l);
+                    else if constexpr (VEC == 2) *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(src + l);
+                    else v[0] = src[l];
+                }
 #pragma unroll
-                for (int t = 0; t < VEC; t++) amx = fmaxf(amx, fabsf(v[t]));
+                for (int t = 0; t < VEC; t++) {
+                    amx = fmaxf(amx, fabsf(v[t]));
+                    Xs[r * ldx + l + t] = v[t];
+                }
             }
-#pragma unroll
-            for (int t = 0; t < VEC; t++) Xs[r * ldx + l + t] = v[t];
         }
         // step s: coordinates [DT_DK (s % nck), ...) of the centres of tile s / nck
         auto load_step = [&](int s, int buf) {
             const int c0 = (s / nck) * DT_C, l0 = (s % nck) * DT_DK;
-            const int w = min(DT_DK, d - l0), wv = w / VEC;
-            for (int e = tid; e < DT_C * wv; e += 256) {
-                const int c = e / wv, l = (e - c * wv) * VEC;
-                const bool ok = c0 + c < k;
-                cp_async<4 * VEC>(cs0 + (uint32_t)(((buf * DT_C + c) * ldc + l) * 4),
-                                  ok ? (const void*)(C + (int64_t)(c0 + c) * d + l0 + l) : (const void*)C, ok);
+            const int w = min(DT_DK, d - l0);
+            // LPC lanes per centre (a chunk is at most 64 coordinates)
+            constexpr int LPC = 64 / VEC < 32 ? 64 / VEC : 32, CPW = 32 / LPC;
+            const int cmax = min(DT_C, k - c0);  // (what lies past k stays from an earlier tile: its values are not used)
+            for (int e = wid * CPW + lane / LPC; e < cmax * (64 / (LPC * VEC)); e += 8 * CPW) {
+                const int c = e / (64 / (LPC * VEC)), l = (lane % LPC + LPC * (e % (64 / (LPC * VEC)))) * VEC;
+                if (l >= w) continue;
+                cp_async<4 * VEC>(cs0 + (uint32_t)(((buf * DT_C + c) * ldc + l) * 4), C + (int64_t)(c0 + c) * d + l0 + l);
             }
             if (w & 3)  // the last chunk's padding
                 for (int c = tid; c < DT_C; c += 256)
@@ -379,24 +384,29 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
             }
             const float* xb = Xs + ty * ldx + ck * DT_DK;            // rows ty + 32 i
             const float* cb = Cs + (size_t)(buf * DT_C + tx) * ldc;  // centres tx + 8 c
-            const int w = min(DT_DK, dp - ck * DT_DK);
+            const int w = min(DT_DK, dp - ck * DT_DK), kleft = k - c0;
+            auto chunk = [&](auto whole) {
 #pragma unroll 1
-            for (int l = 0; l < w; l += 4) {
-                float4 xv[RPT];
+                for (int l = 0; l < w; l += 4) {
+                    float4 xv[RPT];
 #pragma unroll
-                for (int i = 0; i < RPT; i++) xv[i] = *reinterpret_cast<const float4*>(xb + 32 * i * ldx + l);
+                    for (int i = 0; i < RPT; i++) xv[i] = *reinterpret_cast<const float4*>(xb + 32 * i * ldx + l);
 #pragma unroll
-                for (int c = 0; c < 8; c++) {
-                    const float4 cv = *reinterpret_cast<const float4*>(cb + 8 * c * ldc + l);
+                    for (int c = 0; c < 8; c++) {
+                        if (!decltype(whole)::value && 8 * c >= kleft) break;  // (the last tile's missing centres)
+                        const float4 cv = *reinterpret_cast<const float4*>(cb + 8 * c * ldc + l);
 #pragma unroll
-                    for (int i = 0; i < RPT; i++) {
-                        const float2 t0 = fsub2(make_float2(xv[i].x, xv[i].y), make_float2(cv.x, cv.y));
-                        acc[i][c] = __ffma2_rn(t0, t0, acc[i][c]);
-                        const float2 t1 = fsub2(make_float2(xv[i].z, xv[i].w), make_float2(cv.z, cv.w));
-                        acc[i][c] = __ffma2_rn(t1, t1, acc[i][c]);
+                        for (int i = 0; i < RPT; i++) {
+                            const float2 t0 = fsub2(make_float2(xv[i].x, xv[i].y), make_float2(cv.x, cv.y));
+                            acc[i][c] = __ffma2_rn(t0, t0, acc[i][c]);
+                            const float2 t1 = fsub2(make_float2(xv[i].z, xv[i].w), make_float2(cv.z, cv.w));
+                            acc[i][c] = __ffma2_rn(t1, t1, acc[i][c]);
+                        }
                     }
                 }
-            }
+            };
+            if (kleft > 56) chunk(std::true_type{});
+            else chunk(std::false_type{});
             if (++ck < nck) continue;
             ck = 0;
 #pragma unroll

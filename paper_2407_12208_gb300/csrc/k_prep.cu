@@ -395,11 +395,12 @@ KM_DEV void quantize_vec(const float* __restrict__ A, int64_t m, int d, int fmt,
     }
 }
 
-// Any alignment, short rows (d <= 64): eight lanes per row, each standing for
-// four lanes of quantize_warp (lane l = sl + 8 i of 32: the same sums in the
-// same tree, so the same statistics bit for bit), four rows per warp.  A warp
+// Any alignment, rows of up to 32 NCH coordinates: eight lanes per row, each
+// standing for four lanes of quantize_warp (lane l = sl + 8 i of 32: the same
+// sums in the same tree, so the same statistics bit for bit), four rows per warp.  A warp
 // per row spent its time on reductions of mostly idle lanes: 1e5 x 10 took 27 us
-// (now 16 with the centres in the same launch).
+// (now 16 with the centres in the same launch), 700,000 x 77 290 us (now 137).
+template <int NCH>
 KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
                            const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
     const int lane = threadIdx.x & 31, sl = lane & 7;
@@ -407,9 +408,10 @@ KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fm
     const int64_t ng = (int64_t)nblocks * (blockDim.x / 8);
     for (int64_t i = (int64_t)block * (blockDim.x / 8) + threadIdx.x / 8; i < m; i += ng) {
         const float* a = A + i * d;
-        float v[8];  // coordinate sl + 8 t
+        constexpr int NT = 4 * NCH;
+        float v[NT];  // coordinate sl + 8 t
 #pragma unroll
-        for (int t = 0; t < 8; t++) {
+        for (int t = 0; t < NT; t++) {
             v[t] = sl + 8 * t < d ? a[sl + 8 * t] : 0.0f;
             amx = fmaxf(amx, fabsf(v[t]));
         }
@@ -417,7 +419,7 @@ KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fm
         if (fmt == 2) {
             float amax = 0.0f;
 #pragma unroll
-            for (int t = 0; t < 8; t++) amax = fmaxf(amax, fabsf(v[t]));
+            for (int t = 0; t < NT; t++) amax = fmaxf(amax, fabsf(v[t]));
 #pragma unroll
             for (int off = 4; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(gmask, amax, off));
             s = e4m3_row_scale(amax);
@@ -428,7 +430,7 @@ KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fm
 #pragma unroll
         for (int l = 0; l < 4; l++) ph[l] = pl[l] = q2[l] = r2[l] = 0.0f;
 #pragma unroll
-        for (int t = 0; t < 8; t++) {
+        for (int t = 0; t < NT; t++) {
             const int c = sl + 8 * t, l = t & 3;
             if (c < ldq) {
                 const float qv = quant_val(v[t] * inv, fmt);
@@ -494,12 +496,12 @@ struct ColSide {
 };
 
 // KIND: NV of quantize_g8 (1, 2, 4, 8), 16 + NV of quantize_vec, 0
-// quantize_warp, -1 quantize_short.  The first cblocks blocks take the centres
+// quantize_warp, -NCH of quantize_short (2, 4, 8).  The first cblocks blocks take the centres
 // and form their column data (q_j, +inf on the padding so padded columns never
 // win; the E4M3 scales, 1 on the padding; the column maxima, written by the
 // last of them to finish); the rest take the points.  One launch instead of three: the
 // centres' part, 5 to 9 us of latency by itself, hides behind the points'.
-constexpr int quant_blocks(int kind) { return kind == 0 ? 6 : (kind == 8 ? 3 : (kind == 17 || kind == 18 ? 5 : 4)); }  // per SM
+constexpr int quant_blocks(int kind) { return kind == 0 ? 6 : (kind == 8 || kind == -8 ? 3 : (kind == 17 || kind == 18 ? 5 : 4)); }  // per SM
 template <int KIND>
 __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const QuantSide x, const QuantSide c, const ColSide col, int d, int fmt,
                                                   int ldq, int cblocks, const ZeroWords zero) {
@@ -520,7 +522,7 @@ __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const Quan
     }
     const RowOut out{q.stat, q.rscale, cols ? col.qpad : nullptr, col.spad, acc};
     float amx = 0.0f;  // largest |a| of this thread's elements
-    if constexpr (KIND == -1) quantize_short(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    if constexpr (KIND < 0) quantize_short<-KIND>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     else if constexpr (KIND == 0) quantize_warp(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     else if constexpr (KIND < 16) quantize_g8<KIND>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     else quantize_vec<KIND - 16>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
@@ -553,13 +555,13 @@ __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const Quan
     *col.out = o;
 }
 
-// The kernel form for rows at A: -1, 0, NV or 16 + NV (k_quantize).
+// The kernel form for rows at A (k_quantize's KIND).
 static int quant_kind(const float* A, const void* Aq, int d, int ldq) {
     const bool vec = (d % 4 == 0) && (ldq % 4 == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)Aq % 16 == 0);
     const int nv = (ldq / 4 + 31) / 32, nv8 = (ldq / 4 + 7) / 8;
     if (vec && nv8 <= 8) return nv8 <= 1 ? 1 : (nv8 <= 2 ? 2 : (nv8 <= 4 ? 4 : 8));
     if (vec && nv <= 4) return 16 + (nv == 1 ? 1 : (nv == 2 ? 2 : 4));
-    return ldq <= 64 ? -1 : 0;
+    return ldq <= 64 ? -2 : (ldq <= 128 ? -4 : (ldq <= 256 ? -8 : 0));
 }
 
 static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c, const ColSide& col, int d, int fmt,
@@ -572,7 +574,7 @@ static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c
     switch (kind) {
 #define KM_Q(K)                                                                                       \
     case K: klaunch(k_quantize<K>, (unsigned)(xb + cb), 256, 0, st, x, c, col, d, fmt, ldq, (int)cb, zero); break;
-        KM_Q(-1) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(17) KM_Q(18) KM_Q(20)
+        KM_Q(-2) KM_Q(-4) KM_Q(-8) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(17) KM_Q(18) KM_Q(20)
 #undef KM_Q
         default: return cudaErrorInvalidValue;
     }

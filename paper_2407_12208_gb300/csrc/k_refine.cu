@@ -367,9 +367,12 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
 // the row's final d^ minimum, the smallest of the groups' minima.  Rows with 2
 // to RF_FEW candidates then take eight lanes each, four rows at a time: x in
 // registers (NV float4 per lane; NV = 0: any d and alignment, x read again per
-// candidate), two candidates' loads in flight.  Rows with more, and those
-// whose intervals overlap, take the whole warp, which ends in binary64
-// (products in parallel, one lane adds them in coordinate order).
+// candidate), two candidates' loads in flight.  Rows with more go with the
+// overflowed ones where that is cheaper (many_to_list: a centred screen follows,
+// or few centres: all of them in tiles take less than a row at a time; 89,201 x
+// 173, k = 28, all pairs open: 340 us one by one, 138 in tiles), else, like those whose intervals
+// overlap, they take the whole warp, which ends in binary64 (products in
+// parallel, one lane adds them in coordinate order).
 // Labels only: every caller refines the winner's distance afterwards, to
 // binary64 accuracy.
 // LIST: the rows are list[0 .. *list_n) of X (r indexes the lists), else all n.
@@ -384,7 +387,7 @@ __global__ void __launch_bounds__(256) k_refine(const int4* __restrict__ rowinfo
                                                 const int* __restrict__ list_n, const float* __restrict__ X,
                                                 const float* __restrict__ C, int d, float gamma32,
                                                 int32_t* __restrict__ labels, int32_t* __restrict__ ovf_list,
-                                                int* __restrict__ ovf_n, DevCounters* cnt) {
+                                                int* __restrict__ ovf_n, bool many_to_list, DevCounters* cnt) {
     chain_enter();
     constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
     static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
@@ -452,7 +455,8 @@ __global__ void __launch_bounds__(256) k_refine(const int4* __restrict__ rowinfo
         const unsigned fm = __ballot_sync(0xffffffffu, few);
         if (few) ord[__popc(fm & ((1u << lane) - 1u))] = lane;
         __syncwarp();
-        unsigned slow = __ballot_sync(0xffffffffu, c > RF_FEW);
+        if (many_to_list && c > RF_FEW) ovf_list[atomicAdd(ovf_n, 1)] = myrow;
+        unsigned slow = __ballot_sync(0xffffffffu, c > RF_FEW && !many_to_list);
         const int nfew = __popc(fm);
         for (int i0 = 0; i0 < nfew; i0 += 4) {
             const int i = i0 + (lane >> 3);
@@ -663,8 +667,8 @@ static cudaError_t launch_refine_batched(const float* X, const float* C, const T
 
 template <int NV, bool LIST>
 static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs& a, const int32_t* list,
-                                    const int* list_n, int32_t* labels, int32_t* ovf_list, int* ovf_n, int num_sms,
-                                    cudaStream_t st) {
+                                    const int* list_n, int32_t* labels, int32_t* ovf_list, int* ovf_n, bool many_to_list,
+                                    int num_sms, cudaStream_t st) {
     auto fn = k_refine<NV, LIST>;
     // few rows: one warp's 32 per block, so that they spread over the SMs
     const int threads = a.n <= (int64_t)num_sms * 256 ? 32 : 256;
@@ -676,22 +680,23 @@ static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs
     if (e != cudaSuccess) return e;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + threads - 1) / threads, (int64_t)num_sms * std::max(per_sm, 1)));
     klaunch(fn, (unsigned)blocks, threads, sm, st, a.rowinfo, a.cand, a.n, a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,
-                                              labels, ovf_list, ovf_n, a.cnt);
+                                              labels, ovf_list, ovf_n, many_to_list, a.cnt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_refine(const float* X, const float* C, const TcArgs& a, const int32_t* list, const int* list_n,
-                          int32_t* labels, double* min_dist, int32_t* ovf_list, int* ovf_n, int32_t* amb_list, int num_sms,
-                          cudaStream_t st, int* nlaunch) {
+                          int32_t* labels, double* min_dist, int32_t* ovf_list, int* ovf_n, int32_t* amb_list, bool centred_follows,
+                          int num_sms, cudaStream_t st, int* nlaunch) {
     if (!list && refine_batched(a.n, a.d) && a.pairs)
         return launch_refine_batched(X, C, a, labels, min_dist, ovf_list, amb_list, num_sms, st, nlaunch);
     *nlaunch = 1;
+    const bool many = centred_follows || (a.k <= 256 && a.d <= 256);
     const bool vec = a.d % 4 == 0 && a.d <= 256 && ((uintptr_t)X % 16 == 0) && ((uintptr_t)C % 16 == 0);
     const int nv = !vec ? 0 : (a.d <= 32 ? 1 : (a.d <= 64 ? 2 : (a.d <= 128 ? 4 : 8)));
 #define KM_RF(NV)                                                                                            \
     if (nv == NV)                                                                                            \
-        return list ? launch_refine_nv<NV, true>(X, C, a, list, list_n, labels, ovf_list, ovf_n, num_sms, st) \
-                    : launch_refine_nv<NV, false>(X, C, a, list, list_n, labels, ovf_list, ovf_n, num_sms, st);
+        return list ? launch_refine_nv<NV, true>(X, C, a, list, list_n, labels, ovf_list, ovf_n, many, num_sms, st) \
+                    : launch_refine_nv<NV, false>(X, C, a, list, list_n, labels, ovf_list, ovf_n, many, num_sms, st);
     KM_RF(0) KM_RF(1) KM_RF(2) KM_RF(4) KM_RF(8)
 #undef KM_RF
     return cudaErrorInvalidValue;

@@ -228,6 +228,15 @@ KM_DEV int bucket_of(const int* __restrict__ item_off, int k, int64_t it) {
     return lo;
 }
 
+// Coordinates 4c .. 4c + 3 of the row at `row` (zero past d).
+template <bool VEC>
+KM_DEV float4 load_chunk(const float* __restrict__ row, int d, int c) {
+    if (VEC) return reinterpret_cast<const float4*>(row)[c];
+    const float* x = row + 4 * c;
+    const int m = d - 4 * c;
+    return make_float4(x[0], m > 1 ? x[1] : 0.f, m > 2 ? x[2] : 0.f, m > 3 ? x[3] : 0.f);
+}
+
 // One warp per work item (bucket j, rows [c*CHUNK, (c+1)*CHUNK) of it); each
 // row is spread over LPR lanes (NV4 float4 each, d % 4 == 0), so a warp reads
 // 32 / LPR rows per load; exact sums in registers, folded across the row
@@ -237,7 +246,8 @@ KM_DEV int bucket_of(const int* __restrict__ item_off, int k, int64_t it) {
 // winner's ||x - c||^2, Eq. (dist-direct)) to binary64 accuracy (df.cuh: the
 // rows' chunk partials reduced over the row's lanes, eight rows at a time), so
 // the assignment's min_dist costs no second read of X.
-template <int NV4, int LPR, bool WD>
+// VEC: rows and centres are float4 (d % 4 == 0, aligned); else four loads each.
+template <int NV4, int LPR, bool WD, bool VEC>
 __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ? 1 : 2)) k_bucket_sum(const float* __restrict__ X, int64_t n, int d, int k, int seg,
                                                        const int* __restrict__ off,
                              const int* __restrict__ item_off, const int32_t* __restrict__ perm,
@@ -255,7 +265,7 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int nitems = item_off[k];
-    const int d4 = d >> 2;
+    const int d4 = (d + 3) >> 2;
     for (int64_t it = w0; it < nitems; it += nw) {
         const int j = bucket_of(item_off, k, it);
         const int c = (int)(it - item_off[j]);
@@ -266,8 +276,7 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
 #pragma unroll
             for (int u = 0; u < NV4; u++) {
                 const int cidx = cl + LPR * u;
-                cj[u] = (cidx < d4) ? reinterpret_cast<const float4*>(C + (int64_t)j * d)[cidx]
-                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+                cj[u] = (cidx < d4) ? load_chunk<VEC>(C + (int64_t)j * d, d, cidx) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
         // biased parts of the fixed-point values, summed modulo 2^32 (SEG_MAX rows at most)
@@ -295,11 +304,10 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
 #pragma unroll
                     for (int u = 0; u < NV4; u++) {
                         const int cidx = cl + LPR * u;
-                        v[b][u] = (i >= 0 && cidx < d4) ? reinterpret_cast<const float4*>(X + i * d)[cidx]
-                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+                        v[b][u] = (i >= 0 && cidx < d4) ? load_chunk<VEC>(X + i * d, d, cidx) : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                 }
-                if (LPR < 32 && pf) {  // narrow rows (measured: a loss at 512-byte rows)
+                if (VEC && LPR < 32 && pf) {  // narrow rows (measured: a loss at 512-byte rows)
                     if (next_i >= 0) prefetch_l2_bulk(X + next_i * d, (uint32_t)d * 4u);
                     pf = false;
                 }
@@ -353,7 +361,7 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
 #pragma unroll
                 for (int t = 0; t < 4; t++) {
                     const long long acc = FixedScale::combine(a2[u][t], a1[u][t], a0[u][t], m);
-                    if (acc)
+                    if (acc && (VEC || 4 * cidx + t < d))
                         atomicAdd(reinterpret_cast<unsigned long long*>(&sums[(int64_t)j * d + 4 * cidx + t]),
                                   (unsigned long long)acc);
                 }
@@ -1135,7 +1143,7 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
     }
     const size_t hsm = sizeof(int) * (size_t)k;
     const bool vec = d % 4 == 0 && ((uintptr_t)X % 16) == 0;
-    const bool can_bucket = 2 * hsm <= 200 * 1024 && (d == 1 || d == 2 || d == 3 || d == 5 || (vec && d <= 512));
+    const bool can_bucket = 2 * hsm <= 200 * 1024 && d <= 512;
     const size_t smem = sizeof(long long) * ((size_t)k * d + k);
     // shared-memory sums in one launch: what the bucketed path does not take, and
     // few rows (n d <= 2^21, with at least 16 rows per cluster to pay for the
@@ -1162,9 +1170,10 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         return klaunch(fn, (unsigned)blk, 512, smem, st, X, n, d, labels, k, absmax_bits, nscale, sums, counts, C_wd, md_out);
     }
     const bool bucket = can_bucket;
-    // the bucket kernels of rows wider than 5 coordinates read the rows as
-    // float4: they can take the distances along when C is aligned as well
-    const bool fused = want_wd && bucket && d > 5 && ((uintptr_t)C_wd % 16) == 0;
+    // the bucket kernels of rows wider than 5 coordinates take the distances along
+    const bool wide = d > 5 || d == 4;
+    const bool fused = want_wd && bucket && wide;
+    const bool bvec = vec && (!fused || ((uintptr_t)C_wd % 16) == 0);
     if (want_wd && !fused) {
         e = launch_winner_dist(X, n, d, C_wd, labels, md_out, num_sms, st);
         if (e != cudaSuccess) return e;
@@ -1186,8 +1195,10 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         typedef void (*BucketFn)(const float*, int64_t, int, int, int, const int*, const int*, const int32_t*,
                                  const unsigned*, int64_t, long long*, const float*, double*);
         BucketFn bfn = nullptr;
-        if (d > 5) {
-#define KM_BS(NV, L) (fused ? (BucketFn)k_bucket_sum<NV, L, true> : (BucketFn)k_bucket_sum<NV, L, false>)
+        if (wide) {
+#define KM_BS(NV, L)                                                                                              \
+    (fused ? (bvec ? (BucketFn)k_bucket_sum<NV, L, true, true> : (BucketFn)k_bucket_sum<NV, L, true, false>)      \
+           : (bvec ? (BucketFn)k_bucket_sum<NV, L, false, true> : (BucketFn)k_bucket_sum<NV, L, false, false>))
             bfn = d <= 32 ? KM_BS(1, 8) : d <= 64 ? KM_BS(1, 16) : d <= 128 ? KM_BS(1, 32) : d <= 256 ? KM_BS(2, 32)
                                                                                                  : KM_BS(4, 32);
 #undef KM_BS
