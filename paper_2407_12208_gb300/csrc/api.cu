@@ -164,7 +164,8 @@ struct AssignWs {
     float* v32;
     int2* rowpair;
     int64_t pair_cap;
-    int4* rowinfo;
+    int2* rowinfo;
+    float* roww;
     int32_t* ovf_list;
     int32_t* amb_list;
     double* partials;
@@ -202,7 +203,8 @@ AssignWs carve_assign(Carve& cv, int64_t n, int d, int k, int low, bool distance
         w.cscale = cv.take<float>((size_t)k);
         w.qpad = cv.take<float>((size_t)kpad_of(k));
         w.spad = cv.take<float>((size_t)kpad_of(k));
-        w.rowinfo = cv.take<int4>((size_t)n * TC_GROUPS);
+        w.rowinfo = cv.take<int2>((size_t)n * TC_GROUPS);
+        w.roww = cv.take<float>((size_t)n);
         w.ovf_list = cv.take<int32_t>((size_t)n);
         if (!distances) {
             w.cand = cv.take<uint32_t>((size_t)n * TC_GROUPS * TC_LIST);
@@ -452,7 +454,7 @@ km_status run_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int
     a.n = n; a.k = k; a.d = d; a.fmt = fmt;
     a.kchunks = (ldq * esz + 127) / 128;
     a.xstat = w.xstat; a.xscale = w.xscale; a.cstat = w.cstat; a.qpad = w.qpad; a.spad = w.spad; a.colmax = w.colmax;
-    a.tp = tp; a.mode = 0; a.cand = w.cand; a.rowinfo = w.rowinfo; a.cnt = w.cnt;
+    a.tp = tp; a.mode = 0; a.cand = w.cand; a.rowinfo = w.rowinfo; a.roww = w.roww; a.cnt = w.cnt;
     a.pairs = w.pairs; a.pair_cap = w.pair_cap; a.v32 = w.v32; a.rowpair = w.rowpair;
     a.variant = screen_variant(ctx, fmt, a.kchunks, k, n);
     int qbits = 0;
@@ -868,7 +870,7 @@ km_status km_distances(km_ctx* ctx, const float* X, int64_t n, const float* C, i
         a.n = n; a.k = k; a.d = d; a.fmt = fmt;
         a.kchunks = (ldq * esz + 127) / 128;
         a.xstat = w.xstat; a.xscale = w.xscale; a.cstat = w.cstat; a.qpad = w.qpad; a.spad = w.spad; a.colmax = w.colmax;
-        a.tp = make_tp(p, d); a.mode = 1; a.rowinfo = w.rowinfo; a.cnt = w.cnt;
+        a.tp = make_tp(p, d); a.mode = 1; a.cnt = w.cnt;
         a.D = D; a.flag_bits = flag_bits; a.flag_queue = w.queue; a.flag_queue_cap = w.qcap;
         a.flag_queue_len = w.qlen;
         KL(1, launch_tc(w.Xq, w.Cq, ldq, a, ctx->num_sms, st));

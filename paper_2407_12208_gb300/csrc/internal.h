@@ -12,6 +12,9 @@ namespace km {
 // row in all).
 constexpr int TC_GROUPS = 3;
 constexpr int TC_LIST = 48 / TC_GROUPS;
+constexpr int ROW_OVERFLOW = 1 << 16;
+// candidate lists in use per row: tile t of the 128-column tiles is in list t mod TC_GROUPS
+inline int tc_lists(int k) { return (k + 127) / 128 < TC_GROUPS ? (k + 127) / 128 : TC_GROUPS; }
 // Candidate pairs reserved per row in the workspace; rows past the capacity
 // are recomputed by the full-row kernel.
 constexpr int TC_PAIRS_PER_ROW = 8;
@@ -167,7 +170,8 @@ struct TcArgs {
     int variant;              // mode 0 epilogue variant TC_SV_FULL / HALF / C32
     uint32_t* cand;           // mode 0: TC_GROUPS x TC_LIST x n quad entries (group, slot, row), common.cuh
     int ebits;                // low bits of an entry holding the quad index and mask: ceil(log2 ceil(k / 4)) + 4
-    int4* rowinfo;            // n x TC_GROUPS: (count, overflow, window W bits, d^min bits) per epilogue group
+    int2* rowinfo;            // TC_GROUPS x n: (count, | ROW_OVERFLOW; d^min bits) of a row's list
+    float* roww;              // n: the row's window W
     int2* pairs;              // refinement: candidate pairs (row, j), each row's pairs contiguous
     int64_t pair_cap;         // capacity of pairs / v32
     float* v32;               // fp32 direct value of each pair

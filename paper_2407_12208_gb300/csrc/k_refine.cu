@@ -16,10 +16,9 @@
 // Two forms with the same results:
 //  * k_refine: one launch, 32 rows per warp;
 //  * more than 64 coordinates and n d > 2^25: k_cand_select (a flat list of
-//    (row, j) pairs, each row's contiguous, from rowinfo[TC_GROUPS i + g] =
-//    (count, overflow, W, d^min) per epilogue group), k_pair_eval (8 lanes per
-//    pair, 4 pairs per warp, no per-row bookkeeping), k_certify (one thread
-//    per row) and k_amb_fp64.
+//    (row, j) pairs, each row's contiguous, from the rows' lists), k_pair_eval
+//    (8 lanes per pair, 4 pairs per warp, no per-row bookkeeping), k_certify
+//    (one thread per row) and k_amb_fp64.
 // Measured, k_refine against the four launches (GPU time, without the gaps
 // between launches): 1000 x 32 7.9 / 15.0 us, 1e4 x 16 7.4 / 16.3 us, 1e5 x 128
 // 19.8 / 28.7 us, 4e6 x 64 206 / 260 us; 150,001 x 256 92 / 72 us, 1e6 x 128
@@ -105,8 +104,8 @@ __global__ void __launch_bounds__(256) k_pair_eval(const float* __restrict__ X, 
 // window holds every centre that can be the nearest, so that one is; its
 // label is written and its count is 0 (no evaluation: every caller refines
 // the winner's distance afterwards, to binary64 accuracy).
-__global__ void __launch_bounds__(256) k_cand_select(const int4* __restrict__ rowinfo,
-                                                     const uint32_t* __restrict__ cand, int64_t n, int ebits,
+__global__ void __launch_bounds__(256) k_cand_select(const int2* __restrict__ rowinfo, const float* __restrict__ roww,
+                                                     const uint32_t* __restrict__ cand, int64_t n, int ng, int ebits,
                                                      int2* __restrict__ pairs, int64_t cap,
                                                      int2* __restrict__ rowpair, int32_t* __restrict__ labels,
                                                      DevCounters* cnt) {
@@ -127,14 +126,14 @@ __global__ void __launch_bounds__(256) k_cand_select(const int4* __restrict__ ro
         const uint32_t* c0 = cand + row;
         unsigned msk[TC_GROUPS];  // entries inside the window, per group
         {
-            float dmin = INFINITY, W = 0.0f;
+            float dmin = INFINITY;
+            const float W = valid ? roww[row] : 0.0f;
 #pragma unroll
             for (int g = 0; g < TC_GROUPS; g++) {
-                const int4 ig = valid ? rowinfo[row * TC_GROUPS + g] : make_int4(0, 0, 0, __float_as_int(INFINITY));
-                full |= ig.y != 0;
-                cnt_g[g] = ig.x;
-                dmin = fminf(dmin, __int_as_float(ig.w));
-                W = __int_as_float(ig.z);
+                const int2 ig = valid && g < ng ? rowinfo[(size_t)g * n + row] : make_int2(0, __float_as_int(INFINITY));
+                full |= (ig.x & ROW_OVERFLOW) != 0;
+                cnt_g[g] = ig.x & (ROW_OVERFLOW - 1);
+                dmin = fminf(dmin, __int_as_float(ig.y));
             }
             lim = dmin + W;
             // an infinite window (or nothing comparable) takes in the columns' padding too: the whole row
@@ -144,19 +143,19 @@ __global__ void __launch_bounds__(256) k_cand_select(const int4* __restrict__ ro
         constexpr int SPEC = (16 / TC_GROUPS < TC_LIST) ? 16 / TC_GROUPS : TC_LIST;
 #pragma unroll
         for (int g = 0; g < TC_GROUPS; g++) {
-            const int ng = full ? 0 : cnt_g[g];
+            const int cg_n = full ? 0 : cnt_g[g];
             const uint32_t* cg = c0 + (size_t)g * TC_LIST * n;
             uint32_t eg[SPEC];
 #pragma unroll
-            for (int s = 0; s < SPEC; s++) eg[s] = (s < ng) ? cg[(size_t)s * n] : 0u;
+            for (int s = 0; s < SPEC; s++) eg[s] = (s < cg_n) ? cg[(size_t)s * n] : 0u;
             unsigned m = 0;
 #pragma unroll
             for (int s = 0; s < SPEC; s++) {
-                const bool in = s < ng && cand_lower(eg[s], emask, lscale) <= lim;
+                const bool in = s < cg_n && cand_lower(eg[s], emask, lscale) <= lim;
                 m |= in ? (1u << s) : 0u;
                 c += in ? __popc(entry_mask(eg[s])) : 0;
             }
-            for (int s = SPEC; s < ng; s++) {
+            for (int s = SPEC; s < cg_n; s++) {
                 const uint32_t e = cg[(size_t)s * n];
                 const bool in = cand_lower(e, emask, lscale) <= lim;
                 m |= in ? (1u << s) : 0u;
@@ -382,8 +381,8 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
 // 4e6 x 64 249 against 196 us: 48 registers for five blocks per SM spill).
 constexpr int RF_FEW = 12;
 template <int NV, bool LIST>
-__global__ void __launch_bounds__(256) k_refine(const int4* __restrict__ rowinfo, const uint32_t* __restrict__ cand,
-                                                int64_t n, int ebits, const int32_t* __restrict__ list,
+__global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo, const float* __restrict__ roww, const uint32_t* __restrict__ cand,
+                                                int64_t n, int ng, int ebits, const int32_t* __restrict__ list,
                                                 const int* __restrict__ list_n, const float* __restrict__ X,
                                                 const float* __restrict__ C, int d, float gamma32,
                                                 int32_t* __restrict__ labels, int32_t* __restrict__ ovf_list,
@@ -413,14 +412,14 @@ __global__ void __launch_bounds__(256) k_refine(const int4* __restrict__ rowinfo
         const int myrow = valid ? (LIST ? list[r] : (int)r) : 0;
         bool full = false;
         int cnt_g[TC_GROUPS];
-        float lim = INFINITY, W = 0.0f;
+        float lim = INFINITY;
+        const float W = valid ? roww[r] : 0.0f;
 #pragma unroll
         for (int q = 0; q < TC_GROUPS; q++) {
-            const int4 ig = valid ? rowinfo[r * TC_GROUPS + q] : make_int4(0, 0, 0, __float_as_int(INFINITY));
-            full |= ig.y != 0;
-            cnt_g[q] = ig.x;
-            lim = fminf(lim, __int_as_float(ig.w));
-            W = __int_as_float(ig.z);
+            const int2 ig = valid && q < ng ? rowinfo[(size_t)q * n + r] : make_int2(0, __float_as_int(INFINITY));
+            full |= (ig.x & ROW_OVERFLOW) != 0;
+            cnt_g[q] = ig.x & (ROW_OVERFLOW - 1);
+            lim = fminf(lim, __int_as_float(ig.y));
         }
         lim += W;
         // an overflowed list, or an infinite window (which takes in the columns'
@@ -632,7 +631,7 @@ static cudaError_t launch_refine_batched(const float* X, const float* C, const T
     const int64_t rows_blocks = std::max<int64_t>(1, (a.n + 255) / 256);
     const int64_t rb = std::min<int64_t>(rows_blocks, (int64_t)num_sms * std::max(sel_per_sm, 1));
     const int64_t cb = std::min<int64_t>(rows_blocks, (int64_t)num_sms * std::max(cert_per_sm, 1));
-    klaunch(k_cand_select, (unsigned)rb, 256, 0, st, a.rowinfo, a.cand, a.n, a.ebits, a.pairs, a.pair_cap, a.rowpair, labels,
+    klaunch(k_cand_select, (unsigned)rb, 256, 0, st, a.rowinfo, a.roww, a.cand, a.n, tc_lists(a.k), a.ebits, a.pairs, a.pair_cap, a.rowpair, labels,
                                                 a.cnt);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -679,7 +678,7 @@ static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs
     e = blocks_per_sm(fn, threads, sm, &per_sm);
     if (e != cudaSuccess) return e;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + threads - 1) / threads, (int64_t)num_sms * std::max(per_sm, 1)));
-    klaunch(fn, (unsigned)blocks, threads, sm, st, a.rowinfo, a.cand, a.n, a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,
+    klaunch(fn, (unsigned)blocks, threads, sm, st, a.rowinfo, a.roww, a.cand, a.n, tc_lists(a.k), a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,
                                               labels, ovf_list, ovf_n, many_to_list, a.cnt);
     return cudaGetLastError();
 }

@@ -21,6 +21,21 @@
 //               Candidates: every j with d^_j <= d^_min + 2 B_max, the only
 //               centres that can be the true argmin.
 //
+// What bounds it: the epilogue's instructions at three to four warps per
+// scheduler.  At 1e6 x 128 x 1024 (uniform, bf16) without any slow path 289
+// us, of which the MMA warp's chain of waits is 262 (the MMAs alone 117); the
+// walk over qualifying quads adds the rest, about 50 instructions an iteration
+// and a lane's worth of idle lanes.  Measured, with the row's numbers asked for
+// a block ahead (by the producer's L2 prefetch, then before the lists leave),
+// a group passing by the row blocks without a tile for it, lists written four
+// entries at a time, ring positions without divisions, and only undecided
+// pairs tested singly: 435 -> 402 us there, 583 -> 485 us at 4e6 x 64 x 256 (two
+// tiles per row block), 1109 -> 1045 us at 1e6 x 128 x 1024 with every list
+// overflowing (both screens).  Tried and slower: one queue of quads per lane
+// over a tile or more (450 / 709 us: registers spill), quads packed side by
+// side instead of at fixed places (424 / 531), releasing the accumulator
+// before the walk (416 / 532), four groups (96 registers a thread).
+//
 // All waits are bounded (common.cuh); a timeout sets the status word and the
 // CTA winds down.
 #include <cuda_bf16.h>
@@ -87,6 +102,21 @@ static int pick_bn(int kchunks, int k) {
     return 128;  // four accumulators: each epilogue group double-buffered
 }
 
+// A position in a ring of n buffers and how often it has come round, whose
+// parity the buffers' barriers wait for.  (The round only counts to 2: it
+// tells the first from the later ones, and its parity.)
+struct TcRing {
+    int n, at = 0;
+    uint32_t round = 0;
+    KM_DEV explicit TcRing(int n_) : n(n_) {}
+    KM_DEV void next() {
+        if (++at == n) {
+            at = 0;
+            round = round == 2 ? 1 : round + 1;
+        }
+    }
+};
+
 // Asynchronous TMEM load (32 lanes x 32 columns) and the matching wait; the
 // wait names the destination registers so no read of them is scheduled
 // before it.
@@ -120,21 +150,22 @@ KM_DEV void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
 }
 
-// Reliability test of one pair (rare path, kept out of line so the hot loop
-// stays small; scalar arguments, so nothing goes through the stack): tc form
-// rho * B(x, c) or Alg. 2's rho c_A gamma^l_{d+2} (||x~||^2 + ||c~||^2).
-__device__ __noinline__ bool pair_flagged(int test, float rho, float kn, float bsafe, float paper_coef,
-                                          const float4* cstat, int j, float dh, float a1, float a2, float a3, float p,
-                                          float nxq) {
-    const float4 cs = cstat[j];
+// Reliability test of one pair (rare path; it reads the row's numbers again so
+// that the hot loop need not hold them): tc form
+// rho * B(x, c) or Alg. 2's rho c_A gamma^l_{d+2} (||x~||^2 + ||c~||^2), with
+// B_ij = (a1 ||c_j|| + a2 ||c~_j - c_j|| + a3 ||c~_j|| + kn (p + q_j)) * bsafe.
+KM_DEV bool pair_flagged(int test, float rho, float kacc, float kn, float bsafe, float paper_coef,
+                         const float4* xstat, int64_t row, const float4* cstat, int j, float dh) {
+    const float4 cs = __ldg(cstat + j), xs = __ldg(xstat + row);
     if (test == 0) {
-        const float B = (a1 * cs.y + a2 * cs.w + a3 * cs.z + kn * (p + cs.x)) * bsafe;
+        const float a1 = 2.0f * xs.w, a2 = 2.0f * xs.z, a3 = kacc * xs.z;
+        const float B = (a1 * cs.y + a2 * cs.w + a3 * cs.z + kn * (xs.x + cs.x)) * bsafe;
         return dh <= rho * B;
     }
-    return dh <= paper_coef * (nxq * nxq + cs.z * cs.z);
+    return dh <= paper_coef * (xs.z * xs.z + cs.z * cs.z);
 }
 #define KM_PAIR_FLAGGED(j, dh) \
-    pair_flagged(tp.test, tp.rho, tp.kn, tp.bsafe, tp.paper_coef, a.cstat, (j), (dh), a1, a2, a3, p, xs.z)
+    pair_flagged(tp.test, tp.rho, tp.kacc, tp.kn, tp.bsafe, tp.paper_coef, a.xstat, row, a.cstat, (j), (dh))
 
 // Keep only the list entries still inside the window (slot-major layout):
 // all slots are read first (independent loads), then packed with predicated
@@ -236,22 +267,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (lane == 0) {
             tma_prefetch_desc(&tmX);
             tma_prefetch_desc(&tmC);
-            int64_t bload = 0;
-            int iter = 0;
+            TcRing ra(L.NA), rbs(L.NS);
             bool ok = true;
-            for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x, iter++) {
+            for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x, ra.next()) {
                 int t0, t1;
                 const int64_t rb = item_rows(it, t0, t1);
-                const int ab = iter % L.NA;
-                if (iter >= L.NA) ok = mbar_wait(&a_empty[ab], ((iter / L.NA) - 1) & 1, abort_flag, status);
+                const int ab = ra.at;
+                if (ra.round) ok = mbar_wait(&a_empty[ab], (ra.round - 1) & 1, abort_flag, status);
                 if (!ok) break;
                 mbar_arrive_expect_tx(&a_full[ab], (uint32_t)L.a_bytes);
+                // the epilogue's first load of these rows then finds them in L2
+                prefetch_l2_bulk(a.xstat + rb * TC_BM, (uint32_t)min((int64_t)TC_BM, nrows - rb * TC_BM) * 16u);
                 for (int kc = 0; kc < a.kchunks; kc++)
                     tma_load_2d(sA + (size_t)ab * L.a_bytes + (size_t)kc * TC_BM * 128, &tmX, &a_full[ab],
                                 kc * ATOM_ELEMS, (int)(rb * TC_BM));
-                for (int nt = t0; nt < t1; nt++, bload++) {
-                    const int s = (int)(bload % L.NS);
-                    if (bload >= L.NS) ok = mbar_wait(&b_empty[s], ((bload / L.NS) - 1) & 1, abort_flag, status);
+                for (int nt = t0; nt < t1; nt++, rbs.next()) {
+                    const int s = rbs.at;
+                    if (rbs.round) ok = mbar_wait(&b_empty[s], (rbs.round - 1) & 1, abort_flag, status);
                     if (!ok) break;
                     mbar_arrive_expect_tx(&b_full[s], (uint32_t)L.b_bytes);
                     for (int kc = 0; kc < a.kchunks; kc++)
@@ -266,21 +298,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_make(FMT == 1 ? 1u : 0u, TC_BM, BN);
             const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
-            int64_t bcons = 0, tcount = 0;
-            int iter = 0;
+            TcRing ra(L.NA), rbs(L.NS), rt(NBUF);
             bool ok = true;
-            for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x, iter++) {
+            for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x, ra.next()) {
                 int t0, t1;
                 item_rows(it, t0, t1);
-                const int ab = iter % L.NA;
-                ok = mbar_wait(&a_full[ab], (iter / L.NA) & 1, abort_flag, status);
+                const int ab = ra.at;
+                ok = mbar_wait(&a_full[ab], ra.round & 1, abort_flag, status);
                 if (!ok) break;
-                for (int nt = t0; nt < t1; nt++, bcons++, tcount++) {
-                    const int s = (int)(bcons % L.NS);
-                    ok = mbar_wait(&b_full[s], (bcons / L.NS) & 1, abort_flag, status);
+                for (int nt = t0; nt < t1; nt++, rbs.next(), rt.next()) {
+                    const int s = rbs.at;
+                    ok = mbar_wait(&b_full[s], rbs.round & 1, abort_flag, status);
                     if (!ok) break;
-                    const int accb = (int)(tcount % NBUF);
-                    if (tcount >= NBUF) ok = mbar_wait(&acc_empty[accb], ((tcount / NBUF) - 1) & 1, abort_flag, status);
+                    const int accb = rt.at;
+                    if (rt.round) ok = mbar_wait(&acc_empty[accb], (rt.round - 1) & 1, abort_flag, status);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t dt = tmem_base + (uint32_t)(accb * BN);
@@ -324,18 +355,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const float lscale = __uint_as_float((uint32_t)(127 + a.ebits - 23) << 23);  // 2^(ebits - 23)
         unsigned long long nflag_total = 0;
         bool ok = true;
-        int64_t tbase = 0;  // tiles of the items before this one
-        for (int64_t it = blockIdx.x; it < nitem && ok; it += gridDim.x) {
-            int t0, t1;
-            const int64_t rb = item_rows(it, t0, t1);
+        // this group's items: those with a tile t0 + slot, + TC_NG, ... for it (the
+        // rows' slot-th list); tn: the tiles before the item, modulo 2^32
+        int64_t it = blockIdx.x, rb = 0;
+        int t0 = 0, t1 = 0, slot = 0;
+        uint32_t tn = 0;
+        int tmod = 0;  // tiles before the item, modulo TC_NG
+        auto find_item = [&]() {
+            for (; it < nitem; it += gridDim.x) {
+                rb = item_rows(it, t0, t1);
+                slot = (g + TC_NG - tmod) % TC_NG;
+                if (t0 + slot < t1) break;
+                tn += t1 - t0;
+                tmod = (tmod + t1 - t0) % TC_NG;
+            }
+        };
+        float4 xs = make_float4(0.f, 0.f, 0.f, 0.f);
+        float rs = 1.0f;
+        auto load_row = [&]() {  // the row's statistics, a block ahead of their use
+            const int64_t r = rb * TC_BM + r_in;
+            xs = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (it < nitem && r < nrows) {
+                xs = __ldg(a.xstat + r);
+                if (FMT == 2) rs = __ldg(a.xscale + r);
+            }
+        };
+        find_item();
+        load_row();
+        while (it < nitem && ok) {
             const int64_t row = rb * TC_BM + r_in;
             const bool valid = row < nrows;
-            float4 xs = make_float4(0.f, 0.f, 0.f, 0.f);
-            float rs = 1.0f;
-            if (valid) {
-                xs = a.xstat[row];
-                if (FMT == 2) rs = a.xscale[row];
-            }
             const float p = xs.x;
             // e = q_j - 2 s_i s_j g (E4M3: row and column scales, powers of two)
             const float neg2s = -2.0f * rs;
@@ -362,11 +411,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             float m = INFINITY;
             int cnt = 0, ovf = 0, nflag = 0;
 
-            for (int nt = t0; nt < t1; nt++) {
-                const int64_t tc = tbase + (nt - t0);
-                if ((int)(tc % TC_NG) != g) continue;
+            for (int nt = t0 + slot; nt < t1; nt += TC_NG) {
+                const uint32_t tc = tn + (uint32_t)(nt - t0);
                 const int buf = (int)(tc % NBUF);
-                ok = mbar_wait(&acc_full[buf], (uint32_t)((tc / NBUF) & 1), abort_flag, status);
+                ok = mbar_wait(&acc_full[buf], (tc / NBUF) & 1, abort_flag, status);
                 if (!ok) break;
                 tc_fence_after();
                 const int nch = min(BN / 32, (a.k - nt * BN + 31) / 32);
@@ -473,22 +521,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             // with no pair near its flag threshold, carries no flag arithmetic
                             auto take_quad = [&](auto fs, float x0, float x1, float x2, float x3, int jq, bool act) {
                                 constexpr bool FS = decltype(fs)::value;
-                                const unsigned mk = (x0 <= cthr ? 1u : 0u) | (x1 <= cthr ? 2u : 0u) |
-                                                    (x2 <= cthr ? 4u : 0u) | (x3 <= cthr ? 8u : 0u);
-                                const bool pc = act && mk != 0u && !ovf;
-                                const bool room = cnt < TC_L;
+                                // the columns inside the window: the sign bits of cthr - x
+                                const float2 n1 = make_float2(-1.0f, -1.0f), ct = make_float2(cthr, cthr);
+                                const float2 t01 = __ffma2_rn(make_float2(x0, x1), n1, ct);
+                                const float2 t23 = __ffma2_rn(make_float2(x2, x3), n1, ct);
+                                unsigned mk = __float_as_uint(t23.y) >> 31;
+                                mk = __funnelshift_l(__float_as_uint(t23.x), mk, 1);
+                                mk = __funnelshift_l(__float_as_uint(t01.y), mk, 1);
+                                mk = __funnelshift_l(__float_as_uint(t01.x), mk, 1) ^ 15u;
+                                // (a row whose list overflowed keeps it full)
+                                const bool pc = act && mk != 0u, room = cnt < TC_L;
                                 const int slot = (pc && room) ? cnt : TC_L;
                                 const float qmn = fminf(fmin3f(x0, x1, x2), x3);
                                 st_shared_u32(lbase + slot * (TC_BM * 4), quad_entry(jq >> 2, mk, p + qmn, emask));
                                 ovf |= (pc && !room);
                                 cnt += (pc && room) ? 1 : 0;
                                 if constexpr (FS) {
-                                    const float xs4[4] = {x0, x1, x2, x3};
-#pragma unroll
-                                    for (int c = 0; c < 4; c++) {
-                                        const float dh = p + xs4[c];
-                                        if (act && !fwhole && dh <= F)
-                                            nflag += (dh <= Fall || KM_PAIR_FLAGGED(jq + c, dh)) ? 1 : 0;
+                                    // every d^ <= Fall is flagged whatever its column, none above F;
+                                    // those between are tested
+                                    const float d0 = p + x0, d1 = p + x1, d2 = p + x2, d3 = p + x3;
+                                    const unsigned all = (d0 <= Fall ? 1u : 0u) | (d1 <= Fall ? 2u : 0u) |
+                                                         (d2 <= Fall ? 4u : 0u) | (d3 <= Fall ? 8u : 0u);
+                                    const unsigned may = (d0 <= F ? 1u : 0u) | (d1 <= F ? 2u : 0u) |
+                                                         (d2 <= F ? 4u : 0u) | (d3 <= F ? 8u : 0u);
+                                    unsigned t = act && !fwhole ? may & ~all : 0u;
+                                    nflag += act && !fwhole ? __popc(may & all) : 0;
+                                    while (t) {
+                                        const float dh = t & 1u ? d0 : (t & 2u ? d1 : (t & 4u ? d2 : d3));
+                                        nflag += KM_PAIR_FLAGGED(jq + __ffs(t) - 1, dh) ? 1 : 0;
+                                        t &= t - 1;
                                     }
                                 }
                             };
@@ -513,9 +574,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                                             if ((ph >> qd) & 1u)
                                                 st_shared_v4(stg + qd * 512, e[4 * (QH * hh + qd)], e[4 * (QH * hh + qd) + 1],
                                                              e[4 * (QH * hh + qd) + 2], e[4 * (QH * hh + qd) + 3]);
-                                        while (__any_sync(0xffffffffu, ph)) {
+                                        const int most = __reduce_max_sync(0xffffffffu, __popc(ph));
+                                        for (int i = 0; i < most; i++) {
                                             const bool act = ph != 0;
-                                            const int qd = act ? __ffs(ph) - 1 : 0;
+                                            const int qd = __ffs(ph | (1u << (QH - 1))) - 1;
                                             ph &= ph - 1;
                                             const float4 ev = ld_shared_v4(stg + qd * 512);
                                             take_quad(fs, ev.x, ev.y, ev.z, ev.w, col0 + 4 * (QH * hh + qd), act);
@@ -644,14 +706,29 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[buf]);
             }
-            tbase += t1 - t0;
             if (!ok) break;
+            // the next item's rows are loaded before this one's lists leave
+            const int slot_done = slot;
+            tn += t1 - t0;
+            tmod = (tmod + t1 - t0) % TC_NG;
+            it += gridDim.x;
+            find_item();
+            load_row();
             if (valid && MODE == 0) {
                 // the row's list (slot-major: consecutive rows side by side), its
                 // window W and this group's d^ minimum
-                uint32_t* ccol = a.cand + (size_t)g * TC_L * a.n + row;
-                for (int sl = 0; sl < cnt; sl++) ccol[(size_t)sl * a.n] = list[sl * TC_BM];
-                a.rowinfo[row * TC_NG + g] = make_int4(cnt, ovf, __float_as_int(W), __float_as_int(p + m));
+                uint32_t* ccol = a.cand + (size_t)slot_done * TC_L * a.n + row;
+                static_assert(TC_L % 4 == 0, "four entries at a time");
+                for (int sl = 0; sl < cnt; sl += 4) {
+                    uint32_t en[4];
+#pragma unroll
+                    for (int t = 0; t < 4; t++) en[t] = list[(sl + t) * TC_BM];
+#pragma unroll
+                    for (int t = 0; t < 4; t++)
+                        if (sl + t < cnt) ccol[(size_t)(sl + t) * a.n] = en[t];
+                }
+                a.rowinfo[(size_t)slot_done * a.n + row] = make_int2(cnt | (ovf ? ROW_OVERFLOW : 0), __float_as_int(p + m));
+                if (slot_done == 0) a.roww[row] = W;
             }
             nflag_total += (unsigned long long)nflag;
         }

@@ -294,3 +294,28 @@ def test_small_d_sums_parts(ctx, n, d, k, scale):
     v = torch.round(X.double() * 2.0 ** (S // 2) * 2.0 ** (S - S // 2)).long()  # (ties to even, as the kernel's additions)
     want = torch.zeros(k, d, dtype=torch.int64, device="cuda").index_add_(0, lab.long(), v)
     assert torch.equal(sums, want)
+
+
+# the screen's epilogue groups: row blocks of 1, 2, 3, 4 and 7 column tiles, several per CTA, so
+# that groups pass by row blocks without a tile for them; every variant of the epilogue gives
+# the same flags and labels
+@pytest.mark.parametrize("low", ["bf16", "e4m3"])
+@pytest.mark.parametrize("k", [1, 128, 129, 256, 300, 385, 512, 800])
+def test_screen_groups(ctx, low, k):
+    import paper_2407_12208_gb300 as pkg
+    n, d = 152 * 128 * 3 + 5, 24
+    X, C = workloads.gaussian_mixture(n, d, k, seed=k)
+    Xd, Cd = _dev(X), _dev(C)
+    ref = torch.empty(n, dtype=torch.int64, device="cuda")
+    for s in range(0, n, 8192):
+        ref[s : s + 8192] = ((Xd[s : s + 8192, None, :].double() - Cd[None].double()) ** 2).sum(2).argmin(1)
+    flags = set()
+    try:
+        for variant in ("full", "half", "c32"):
+            ctx.set_screen_variant(n, d, k, low, variant)
+            lab, _, nf = ctx.assign(Xd, Cd, pkg.params(low))
+            assert torch.equal(lab.long(), ref)
+            flags.add(int(nf))
+    finally:
+        ctx.set_screen_variant(n, d, k, low, "auto")
+    assert len(flags) == 1
