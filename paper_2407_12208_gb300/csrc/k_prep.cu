@@ -164,8 +164,11 @@ KM_DEV void quantize_warp(const float* __restrict__ A, int64_t m, int d, int fmt
 
 // Group path (d % 4 == 0, padded width <= 256): 8 lanes per row, 4 rows per
 // warp, so the row reductions take 3 shuffle levels and serve 4 rows at once.
-// Lane l of a row's 8 holds float4 l, l + 8, ... (NV of them).
-template <int NV>
+// Lane l of a row's 8 holds float4 l, l + 8, ... (NV of them).  Bound by issue up
+// to 64 coordinates (50 instructions a row, of which 20 were the row's reduction
+// and square roots by itself): R rows' reductions together took 4e6 x 64 from 364
+// to 311 us (1.6 GB; 0.76 of the copy rate), 1e6 x 128 runs at 0.86 of it.
+template <int NV, bool FEW>
 KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
                         const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
     const int lane = threadIdx.x & 31, sl = lane & 7;
@@ -174,8 +177,8 @@ KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, 
     const int64_t ngroups = (((int64_t)nblocks * blockDim.x) >> 5) * 4;
     const int d4 = d >> 2, ldq4 = ldq >> 2;
     // R rows per group and round, all their loads issued first: at least four
-    // 16-byte loads in flight per lane
-    constexpr int R = NV >= 4 ? 1 : 4 / NV;
+    // 16-byte loads in flight per lane (FEW: no group has a second row)
+    constexpr int R = FEW || NV >= 4 ? 1 : 4 / NV;
     for (int64_t i0 = gid; i0 < m; i0 += ngroups * R) {
         float4 xr[R][NV];
 #pragma unroll
@@ -188,28 +191,31 @@ KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, 
                 xr[r][u] = (ir < m && c < d4) ? a4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
+        float vh[R], vl[R], vq[R], vr[R], vs[R];  // the lane's part of each row's sums, the row's scale
+        unsigned nzm = 0;
 #pragma unroll
         for (int r = 0; r < R; r++) {
         const int64_t i = i0 + (int64_t)r * ngroups;
-        if (i >= m) break;  // the same row for the group's eight lanes
         float4 x[NV];
-        bool nz = false;
+        float amax = 0.0f;
 #pragma unroll
         for (int u = 0; u < NV; u++) {
             x[u] = xr[r][u];
-            amx = fmaxf(amx, fmaxf(fmaxf(fabsf(x[u].x), fabsf(x[u].y)), fmaxf(fabsf(x[u].z), fabsf(x[u].w))));
-            nz |= (x[u].x != 0.0f) | (x[u].y != 0.0f) | (x[u].z != 0.0f) | (x[u].w != 0.0f);
+            amax = fmaxabs3(fmaxabs3(amax, x[u].x, x[u].y), x[u].z, x[u].w);
         }
-        const bool nzr = (__ballot_sync(gmask, nz) & gmask) != 0u;
+        amx = fmaxf(amx, amax);
+        // (a NaN alone leaves its row out here; its bound is infinite all the same)
+        nzm |= (__ballot_sync(gmask, amax > 0.0f) & gmask) != 0u ? 1u << r : 0u;
         float s = 1.0f;
         if (fmt == 2) {
-            float amax = 0.0f;
-#pragma unroll
-            for (int u = 0; u < NV; u++)
-                amax = fmaxf(amax, fmaxf(fmaxf(fabsf(x[u].x), fabsf(x[u].y)), fmaxf(fabsf(x[u].z), fabsf(x[u].w))));
 #pragma unroll
             for (int off = 4; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(gmask, amax, off));
             s = e4m3_row_scale(amax);
+        }
+        vs[r] = s;
+        if (r > 0 && i >= m) {  // past the last row (the same for the group's eight lanes)
+            vh[r] = vl[r] = vq[r] = vr[r] = 0.0f;
+            continue;
         }
         const float inv = 1.0f / s;
         float ph = 0.0f, pl = 0.0f, q2 = 0.0f, r2 = 0.0f;
@@ -281,27 +287,58 @@ KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, 
                 reinterpret_cast<uint32_t*>(Aq)[i * ldq4 + c] = w;
             }
         }
+        vh[r] = ph;
+        vl[r] = pl;
+        vq[r] = q2;
+        vr[r] = r2;
+        }
+        // The rows' sums over the eight lanes, the rows shared out on the way: at each
+        // level with rows left, half of the lanes go on with one half of them and hand
+        // over the other (the same additions as row by row, a third of the shuffles).
+        int rr = 0, left = R;  // this lane's row
 #pragma unroll
         for (int off = 4; off > 0; off >>= 1) {
-            float oh = __shfl_xor_sync(gmask, ph, off);
-            float ol = __shfl_xor_sync(gmask, pl, off);
-            df_add(ph, pl, oh, ol);
-            q2 += __shfl_xor_sync(gmask, q2, off);
-            r2 += __shfl_xor_sync(gmask, r2, off);
+            if (left > 1) {
+                left >>= 1;
+                const bool up = (sl & off) != 0;
+                rr += up ? left : 0;
+#pragma unroll
+                for (int r = 0; r < R / 2; r++) {
+                    if (r >= left) break;
+                    const float gh = up ? vh[r] : vh[r + left], gl = up ? vl[r] : vl[r + left];
+                    const float gq = up ? vq[r] : vq[r + left], gr = up ? vr[r] : vr[r + left];
+                    vh[r] = up ? vh[r + left] : vh[r];
+                    vl[r] = up ? vl[r + left] : vl[r];
+                    vq[r] = up ? vq[r + left] : vq[r];
+                    vr[r] = up ? vr[r + left] : vr[r];
+                    const float oh = __shfl_xor_sync(gmask, gh, off), ol = __shfl_xor_sync(gmask, gl, off);
+                    df_add(vh[r], vl[r], oh, ol);
+                    vq[r] += __shfl_xor_sync(gmask, gq, off);
+                    vr[r] += __shfl_xor_sync(gmask, gr, off);
+                }
+            } else {
+                const float oh = __shfl_xor_sync(gmask, vh[0], off), ol = __shfl_xor_sync(gmask, vl[0], off);
+                df_add(vh[0], vl[0], oh, ol);
+                vq[0] += __shfl_xor_sync(gmask, vq[0], off);
+                vr[0] += __shfl_xor_sync(gmask, vr[0], off);
+            }
         }
-        if (sl == 0) {
-            float p = ph + pl;
+        const int64_t i = i0 + (int64_t)rr * ngroups;
+        if ((sl & (8 / R - 1)) == 0 && i < m) {
+            const float p = vh[0] + vl[0];
             float4 o;
             o.x = p;
             o.y = sqrtf(p) * kNormInflate;
-            o.z = sqrtf(q2) * kNormInflate;
-            o.w = sqrtf(r2) * kNormInflate;
+            o.z = sqrtf(vq[0]) * kNormInflate;
+            o.w = sqrtf(vr[0]) * kNormInflate;
             // an element that overflowed the low format, or squares near the
             // underflow, make the row unusable for the expanded formula: an
             // infinite bound flags all its pairs
-            if (!isfinite(o.z) || (nzr && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
+            if (!isfinite(o.z) || (((nzm >> rr) & 1u) && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
+            float s = vs[0];
+#pragma unroll
+            for (int r = 1; r < R; r++) s = rr == r ? vs[r] : s;
             out(i, o, s);
-        }
         }
     }
 }
@@ -476,6 +513,113 @@ KM_DEV void quantize_short(const float* __restrict__ A, int64_t m, int d, int fm
     }
 }
 
+// Rows of at most 16 coordinates, a thread each: no shuffles, a row's low-format
+// copy leaves in one or two 16-byte stores.  The same sums in the same tree as
+// quantize_g8's (VEC: aligned rows, a float4 per lane there) or quantize_short's
+// (else), so the same statistics bit for bit.  Eight lanes a row, of which a
+// short row fills two to four, took 16.8 us at 1e5 x 10 and 59 us at 930,486 x
+// 16; this form 6.9 and 19.3.
+template <bool VEC>
+KM_DEV void quantize_row(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq, const RowOut& out,
+                         float& amx, unsigned block, unsigned nblocks) {
+    for (int64_t i = (int64_t)block * blockDim.x + threadIdx.x; i < m; i += (int64_t)nblocks * blockDim.x) {
+        float v[16];
+        if constexpr (VEC) {
+            const float4* a4 = reinterpret_cast<const float4*>(A + i * d);
+#pragma unroll
+            for (int f = 0; f < 4; f++) {
+                const float4 t = 4 * f < d ? a4[f] : make_float4(0.f, 0.f, 0.f, 0.f);
+                v[4 * f] = t.x; v[4 * f + 1] = t.y; v[4 * f + 2] = t.z; v[4 * f + 3] = t.w;
+            }
+        } else {
+            const float* a = A + i * d;
+#pragma unroll
+            for (int c = 0; c < 16; c++) v[c] = c < d ? a[c] : 0.0f;
+        }
+        float amax = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 16; c += 2) amax = fmaxabs3(amax, v[c], v[c + 1]);
+        amx = fmaxf(amx, amax);
+        const float s = fmt == 2 ? e4m3_row_scale(amax) : 1.0f, inv = 1.0f / s;
+        // partial sums: per float4 (VEC), else per coordinate pair (c, c + 8)
+        constexpr int NP = VEC ? 4 : 8;
+        float ph[NP], pl[NP], q2[NP], r2[NP];
+        uint32_t w[8];  // the row's low-format copy
+        auto put = [&](int c, float lo, float hi) {  // coordinates c, c + 1 (quantised values, scaled)
+            if (fmt == 0) {
+                const __half2 h = __floats2half2_rn(lo, hi);
+                w[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
+            } else if (fmt == 1) {
+                const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+                w[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
+            } else {
+                const uint32_t b = (uint32_t)__nv_cvt_float_to_fp8(lo, __NV_SATFINITE, __NV_E4M3) |
+                                   (uint32_t)__nv_cvt_float_to_fp8(hi, __NV_SATFINITE, __NV_E4M3) << 8;
+                w[c / 4] = (c & 2) ? w[c / 4] | b << 16 : b;
+            }
+        };
+#pragma unroll
+        for (int c = 0; c < 16; c += 2) put(c, v[c] * inv, v[c + 1] * inv);
+        if (VEC && fmt != 2) {
+#pragma unroll
+            for (int f = 0; f < 4; f++) {
+                float2 h2 = make_float2(0.f, 0.f), l2 = h2, qq2 = h2, rr2 = h2;
+#pragma unroll
+                for (int t = 0; t < 2; t++) {
+                    const uint32_t u = w[2 * f + t];
+                    const float2 q = fmt == 0 ? __half22float2(*reinterpret_cast<const __half2*>(&u))
+                                              : __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
+                    row_sums2(make_float2(v[4 * f + 2 * t], v[4 * f + 2 * t + 1]), q, h2, l2, qq2, rr2);
+                }
+                ph[f % NP] = h2.x;
+                pl[f % NP] = l2.x;
+                df_add(ph[f % NP], pl[f % NP], h2.y, l2.y);
+                q2[f % NP] = qq2.x + qq2.y;
+                r2[f % NP] = rr2.x + rr2.y;
+            }
+        } else {
+            auto term = [&](float x, float& h, float& l, float& qq, float& rr) {
+                const float qs = quant_val(x * inv, fmt) * s;
+                df_add_sq(x, h, l);
+                qq = fmaf(qs, qs, qq);
+                const float r = qs - x;
+                rr = fmaf(r, r, rr);
+            };
+#pragma unroll
+            for (int f = 0; f < NP; f++) {
+                ph[f] = pl[f] = q2[f] = r2[f] = 0.0f;
+                if constexpr (VEC) {
+#pragma unroll
+                    for (int t = 0; t < 4; t++) term(v[(4 * f + t) % 16], ph[f], pl[f], q2[f], r2[f]);
+                } else {
+                    float h = 0.0f, l = 0.0f, qq = 0.0f, rr = 0.0f;
+                    term(v[f], ph[f], pl[f], q2[f], r2[f]);
+                    term(v[f + 8], h, l, qq, rr);
+                    df_add(ph[f], pl[f], h, l);
+                    q2[f] += qq;
+                    r2[f] += rr;
+                }
+            }
+        }
+#pragma unroll
+        for (int off = NP / 2; off > 0; off >>= 1)
+#pragma unroll
+            for (int f = 0; f < off; f++) {
+                df_add(ph[f], pl[f], ph[f + off], pl[f + off]);
+                q2[f] += q2[f + off];
+                r2[f] += r2[f + off];
+            }
+        const int esz = fmt == 2 ? 1 : 2;
+        uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<char*>(Aq) + i * ldq * esz);
+        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        if (ldq * esz > 16) dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        const float p = ph[0] + pl[0];
+        float4 o = make_float4(p, sqrtf(p) * kNormInflate, sqrtf(q2[0]) * kNormInflate, sqrtf(r2[0]) * kNormInflate);
+        if (!isfinite(o.z) || (amax > 0.0f && !(p >= kTinyNorm2))) { o.z = INFINITY; o.w = INFINITY; }
+        out(i, o, s);
+    }
+}
+
 // The rows of a matrix, quantised (one side of a launch).
 struct QuantSide {
     const float* A;
@@ -495,8 +639,8 @@ struct ColSide {
     unsigned* acc;  // 10 words, 0 before and after
 };
 
-// KIND: NV of quantize_g8 (1, 2, 4, 8), 16 + NV of quantize_vec, 0
-// quantize_warp, -NCH of quantize_short (2, 4, 8).  The first cblocks blocks take the centres
+// KIND: NV of quantize_g8 (1, 2, 4, 8; few rows: 9, 10), 16 + NV of
+// quantize_vec, 0 quantize_warp, -NCH of quantize_short (2, 4, 8), 32 and 33 quantize_row.  The first cblocks blocks take the centres
 // and form their column data (q_j, +inf on the padding so padded columns never
 // win; the E4M3 scales, 1 on the padding; the column maxima, written by the
 // last of them to finish); the rest take the points.  One launch instead of three: the
@@ -524,8 +668,9 @@ __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const Quan
     float amx = 0.0f;  // largest |a| of this thread's elements
     if constexpr (KIND < 0) quantize_short<-KIND>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     else if constexpr (KIND == 0) quantize_warp(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
-    else if constexpr (KIND < 16) quantize_g8<KIND>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
-    else quantize_vec<KIND - 16>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    else if constexpr (KIND < 16) quantize_g8<(KIND < 9 ? KIND : KIND - 8), (KIND > 8)>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    else if constexpr (KIND < 32) quantize_vec<KIND - 16>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    else quantize_row<KIND == 32>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     if (q.absmax) block_absmax(amx, q.absmax);
     if (!cols) return;
     if (block == 0)
@@ -556,10 +701,14 @@ __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const Quan
 }
 
 // The kernel form for rows at A (k_quantize's KIND).
-static int quant_kind(const float* A, const void* Aq, int d, int ldq) {
+static int quant_kind(const float* A, const void* Aq, int d, int ldq, int64_t rows) {
     const bool vec = (d % 4 == 0) && (ldq % 4 == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)Aq % 16 == 0);
     const int nv = (ldq / 4 + 31) / 32, nv8 = (ldq / 4 + 7) / 8;
-    if (vec && nv8 <= 8) return nv8 <= 1 ? 1 : (nv8 <= 2 ? 2 : (nv8 <= 4 ? 4 : 8));
+    // a thread per short row once that makes a block for every SM: 6.9 against 16.8
+    // us at 1e5 x 10, 5.8 against 5.2 at 1e4 x 16
+    if (ldq <= 16 && (uintptr_t)Aq % 16 == 0 && rows >= 152 * 256) return vec ? 32 : 33;
+    const bool few = rows <= 152 * 16 * 32;  // groups of one round (launch_quant)
+    if (vec && nv8 <= 8) return nv8 <= 1 ? (few ? 9 : 1) : (nv8 <= 2 ? (few ? 10 : 2) : (nv8 <= 4 ? 4 : 8));
     if (vec && nv <= 4) return 16 + (nv == 1 ? 1 : (nv == 2 ? 2 : 4));
     return ldq <= 64 ? -2 : (ldq <= 128 ? -4 : (ldq <= 256 ? -8 : 0));
 }
@@ -567,14 +716,14 @@ static int quant_kind(const float* A, const void* Aq, int d, int ldq) {
 static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c, const ColSide& col, int d, int fmt,
                                 int ldq, const ZeroWords& zero, cudaStream_t st) {
     // 8 lanes or a warp per row, enough warps in flight to cover the memory latency
-    const int rows = kind == 0 || kind >= 16 ? 8 : 32;  // per block and round
-    const int64_t most = kind == 0 || kind >= 16 ? 152 * 64 : 152 * 16;
+    const int rows = kind >= 32 ? 256 : (kind == 0 || kind >= 16 ? 8 : 32);  // per block and round
+    const int64_t most = kind >= 32 ? 152 * 8 : (kind == 0 || kind >= 16 ? 152 * 64 : 152 * 16);
     const int64_t xb = x.m ? std::min<int64_t>((x.m + rows - 1) / rows, most) : 0;
     const int64_t cb = c.m ? std::min<int64_t>((c.m + rows - 1) / rows, 152) : 0;
     switch (kind) {
 #define KM_Q(K)                                                                                       \
     case K: klaunch(k_quantize<K>, (unsigned)(xb + cb), 256, 0, st, x, c, col, d, fmt, ldq, (int)cb, zero); break;
-        KM_Q(-2) KM_Q(-4) KM_Q(-8) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(17) KM_Q(18) KM_Q(20)
+        KM_Q(-2) KM_Q(-4) KM_Q(-8) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(9) KM_Q(10) KM_Q(17) KM_Q(18) KM_Q(20) KM_Q(32) KM_Q(33)
 #undef KM_Q
         default: return cudaErrorInvalidValue;
     }
@@ -583,7 +732,7 @@ static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c
 
 cudaError_t launch_quantize(const float* A, int64_t m, int d, int fmt, int ldq, void* Aq, float4* stat,
                             float* rscale, cudaStream_t st, unsigned* absmax_out) {
-    return launch_quant(quant_kind(A, Aq, d, ldq), QuantSide{A, m, Aq, stat, rscale, absmax_out}, QuantSide{}, ColSide{}, d,
+    return launch_quant(quant_kind(A, Aq, d, ldq, m), QuantSide{A, m, Aq, stat, rscale, absmax_out}, QuantSide{}, ColSide{}, d,
                         fmt, ldq, ZeroWords{}, st);
 }
 
@@ -593,7 +742,8 @@ cudaError_t launch_prepare(const float* X, int64_t n, void* Xq, float4* xstat, f
                            const ZeroWords& zero, cudaStream_t st, int* nlaunch) {
     const QuantSide x{X, X ? n : 0, Xq, xstat, xscale, absmax_out}, c{C, k, Cq, cstat, cscale, nullptr};
     const ColSide col{colmax, qpad, spad, kpad, ticket, colacc};
-    const int kc = quant_kind(C, Cq, d, ldq), kx = X ? quant_kind(X, Xq, d, ldq) : kc;
+    const int64_t rows = X ? n : k;
+    const int kc = quant_kind(C, Cq, d, ldq, rows), kx = X ? quant_kind(X, Xq, d, ldq, rows) : kc;
     *nlaunch = 1;
     if (kx == kc) return launch_quant(kc, x, c, col, d, fmt, ldq, zero, st);
     // points and centres aligned differently: each in its own form

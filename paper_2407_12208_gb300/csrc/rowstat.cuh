@@ -15,17 +15,19 @@ constexpr float kTinyNorm2 = 0x1p-100f;  // below this ||x||^2 the fp32 statisti
 // Two coordinates (scale 1, 16-bit formats) into the row's running sums, two
 // per packed instruction: ||x||^2 as a pair of double-floats (exact product,
 // two-sum), ||x~||^2 and ||x~ - x||^2 in fp32.
-KM_DEV float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 KM_DEV void row_sums2(float2 x, float2 q, float2& hi, float2& lo, float2& qq, float2& rr) {
-    const float2 p = __fmul2_rn(x, x);
-    const float2 pe = __ffma2_rn(x, x, neg2(p));
-    const float2 s = __fadd2_rn(hi, p);
-    const float2 bb = __fadd2_rn(s, neg2(hi));
-    const float2 e = __fadd2_rn(__fadd2_rn(hi, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
+    // (differences as fused products with -1: the packed operations take no sign)
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 nx = __fmul2_rn(x, m1), np = __fmul2_rn(nx, x);  // -x, -p with p = fl(x^2)
+    const float2 pe = __ffma2_rn(x, x, np);
+    const float2 s = __ffma2_rn(np, m1, hi);
+    const float2 bb = __ffma2_rn(hi, m1, s);
+    const float2 e1 = __ffma2_rn(__ffma2_rn(bb, m1, s), m1, hi);
+    const float2 e = __ffma2_rn(__fadd2_rn(np, bb), m1, e1);
     hi = s;
     lo = __fadd2_rn(lo, __fadd2_rn(e, pe));
     qq = __ffma2_rn(q, q, qq);
-    const float2 r = __fadd2_rn(q, neg2(x));  // exact (Sterbenz)
+    const float2 r = __fadd2_rn(q, nx);  // exact (Sterbenz)
     rr = __ffma2_rn(r, r, rr);
 }
 

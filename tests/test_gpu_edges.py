@@ -319,3 +319,23 @@ def test_screen_groups(ctx, low, k):
     finally:
         ctx.set_screen_variant(n, d, k, low, "auto")
     assert len(flags) == 1
+
+
+# quantisation, a thread per row (d <= 16, from 38,912 rows on) and several rows per eight lanes
+# (d <= 64 aligned, from 77,825 rows on), on both sides of the lines and past the end of a round
+@pytest.mark.parametrize("low", ["fp16", "bf16", "e4m3"])
+@pytest.mark.parametrize("n,d,offset", [(38911, 10, 0), (38912, 10, 0), (38913, 16, 0), (77824, 32, 0), (77825, 32, 0),
+                                        (155651, 24, 0), (311299, 20, 0), (90001, 64, 0), (160003, 40, 0), (60001, 12, 1),
+                                        (60001, 3, 0), (60001, 1, 0), (60002, 4, 0), (60003, 8, 2), (60005, 15, 0),
+                                        (50000, 16, 1)])
+def test_quantise_rows_per_thread(ctx, low, n, d, offset):
+    if low == "e4m3" and d < 16:
+        pytest.skip("E4M3 takes d >= 16")
+    k = 30
+    X, C = workloads.gaussian_mixture(n, d, k, seed=n + d)
+    lab, md, nf = _assign(ctx, X, C, low, offset)
+    check_assign(lab, md, X, C, oracle, RTOL_MD)
+    # the first rows by themselves, in the form for few rows: the same statistics, so the same flags
+    _, _, nf1 = _assign(ctx, X[:30000], C, low, offset)
+    _, _, nf2 = _assign(ctx, X[30000:], C, low, offset)
+    assert nf == nf1 + nf2
