@@ -792,12 +792,14 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
     if (!acc64) {
         // rows per block: 128, or 64 where 128 would leave one block per SM
         // (111 KB of dynamic shared memory, past d = 148) or too few blocks for two per
-        // SM, or 32 where 64 would; a row list's length is not known here
+        // SM, or 32 where 64 would; a row list is taken for as long as the call's rows
+        // (7265 x 128 x 436, most rows listed: 119 us with 128 rows per block, 66 with
+        // 32; 37,638 x 128 x 44: 40 and 30 with 64)
         const bool a16 = ((uintptr_t)X % 16) == 0 && ((uintptr_t)C % 16) == 0;
         const bool a8 = ((uintptr_t)X % 8) == 0 && ((uintptr_t)C % 8) == 0;
         const int vec = d % 4 == 0 && a16 ? 4 : (d % 2 == 0 && a8 ? 2 : 1);
         int rpt = dt_smem(4, d) <= 111 * 1024 ? 4 : 2;
-        while (rpt > 1 && !row_list && (n + 32 * rpt - 1) / (32 * rpt) < 2 * num_sms) rpt >>= 1;
+        while (rpt > 1 && (n + 32 * rpt - 1) / (32 * rpt) < 2 * num_sms) rpt >>= 1;
 #define KM_DT(RP, VE)                                                                                              \
     if (rpt == RP && vec == VE)                                                                                    \
         return launch_tiled<RP, VE>(X, n, C, k, d, row_list, row_count, labels, min_dist, cnt, gamma32, \

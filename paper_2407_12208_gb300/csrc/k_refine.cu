@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
                                                 const int* __restrict__ list_n, const float* __restrict__ X,
                                                 const float* __restrict__ C, int d, float gamma32,
                                                 int32_t* __restrict__ labels, int32_t* __restrict__ ovf_list,
-                                                int* __restrict__ ovf_n, bool many_to_list, DevCounters* cnt) {
+                                                int* __restrict__ ovf_n, bool many_to_list, int rpw, DevCounters* cnt) {
     chain_enter();
     constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
     static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
@@ -406,9 +406,9 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
     const int d4 = d >> 2;
     unsigned ev32 = 0, ev64 = 0, amb = 0, ovf = 0;
     const int nwb = blockDim.x >> 5;
-    for (int64_t r0 = ((int64_t)blockIdx.x * nwb + wib) * 32; r0 < nrows; r0 += (int64_t)gridDim.x * nwb * 32) {
+    for (int64_t r0 = ((int64_t)blockIdx.x * nwb + wib) * rpw; r0 < nrows; r0 += (int64_t)gridDim.x * nwb * rpw) {
         const int64_t r = r0 + lane;
-        const bool valid = r < nrows;
+        const bool valid = lane < rpw && r < nrows;
         const int myrow = valid ? (LIST ? list[r] : (int)r) : 0;
         bool full = false;
         int cnt_g[TC_GROUPS];
@@ -669,17 +669,22 @@ static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs
                                     const int* list_n, int32_t* labels, int32_t* ovf_list, int* ovf_n, bool many_to_list,
                                     int num_sms, cudaStream_t st) {
     auto fn = k_refine<NV, LIST>;
-    // few rows: one warp's 32 per block, so that they spread over the SMs
-    const int threads = a.n <= (int64_t)num_sms * 256 ? 32 : 256;
+    // rows per warp: few rows are spread over the SMs in rounds of the four that
+    // are evaluated together (a lane per row selects, so more rows want whole warps)
+    const int rpw = !LIST && a.n <= (int64_t)num_sms * 128 ? 4 : (!LIST && a.n <= (int64_t)num_sms * 256 ? 8 : 32);
+    const int64_t warps = (a.n + rpw - 1) / rpw;
+    const int threads = LIST ? (a.n <= (int64_t)num_sms * 256 ? 32 : 256)
+                             : 32 * (int)std::max<int64_t>(1, std::min<int64_t>(8, (warps + num_sms - 1) / num_sms));
+    const int per_block = threads / 32 * rpw;
     const size_t sm = (size_t)(threads / 32) * a.d * sizeof(double);
     cudaError_t e = allow_max_smem(fn);
     if (e != cudaSuccess) return e;
     int per_sm = 1;
     e = blocks_per_sm(fn, threads, sm, &per_sm);
     if (e != cudaSuccess) return e;
-    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + threads - 1) / threads, (int64_t)num_sms * std::max(per_sm, 1)));
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.n + per_block - 1) / per_block, (int64_t)num_sms * std::max(per_sm, 1)));
     klaunch(fn, (unsigned)blocks, threads, sm, st, a.rowinfo, a.roww, a.cand, a.n, tc_lists(a.k), a.ebits, list, list_n, X, C, a.d, a.tp.gamma32,
-                                              labels, ovf_list, ovf_n, many_to_list, a.cnt);
+                                              labels, ovf_list, ovf_n, many_to_list, rpw, a.cnt);
     return cudaGetLastError();
 }
 

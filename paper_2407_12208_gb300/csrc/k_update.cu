@@ -65,7 +65,7 @@ __global__ void k_accumulate(const float* __restrict__ X, int64_t n, int d, cons
 // row.  One launch, where the bucketed path takes four: for few rows, and for
 // rows it does not take.  Bound by latency for few rows, by the shared atomics
 // for many: 1e4 x 16, k = 8 26 -> 9 us, 1e5 x 10, k = 100 26 -> 19 us.
-template <int NV4, int LPR, bool VEC, bool WD>
+template <int NV4, int LPR, bool VEC, bool WD, bool SH>
 __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X, int64_t n, int d,
                                                     const int32_t* __restrict__ labels, int k,
                                                     const unsigned* __restrict__ amax_bits, int64_t nscale,
@@ -77,10 +77,13 @@ __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X,
     constexpr int R = NV4 == 4 ? 2 : 4;
     constexpr int STEP = R * G;
     const FixedScale fx(fixed_shift(*amax_bits, nscale));
-    const int kd = k * d;
-    unsigned long long* cacc = acc_rows + kd;
-    for (int e = threadIdx.x; e < kd + k; e += blockDim.x) acc_rows[e] = 0ull;
-    __syncthreads();
+    const int kd = SH ? k * d : 0;
+    unsigned long long* const acc = SH ? acc_rows : reinterpret_cast<unsigned long long*>(sums);
+    unsigned long long* const cacc = SH ? acc_rows + kd : reinterpret_cast<unsigned long long*>(counts);
+    if (SH) {
+        for (int e = threadIdx.x; e < kd + k; e += blockDim.x) acc_rows[e] = 0ull;
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31, sub = lane / LPR, cl = lane % LPR;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -123,7 +126,7 @@ __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X,
 #pragma unroll
         for (int b = 0; b < R; b++)
             if (js[b] >= 0) {
-                unsigned long long* a = acc_rows + js[b] * d;
+                unsigned long long* a = acc + (int64_t)js[b] * d;
 #pragma unroll
                 for (int u = 0; u < NV4; u++) {
                     const int l = 4 * (cl + LPR * u);
@@ -135,6 +138,7 @@ __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X,
                 if (cl == 0) atomicAdd(cacc + js[b], 1ull);
             }
     }
+    if (!SH) return;
     __syncthreads();
     for (int e = threadIdx.x; e < kd; e += blockDim.x)
         if (acc_rows[e]) atomicAdd(reinterpret_cast<unsigned long long*>(sums) + e, acc_rows[e]);
@@ -1090,6 +1094,13 @@ cudaError_t launch_absmax(const float* X, int64_t count, unsigned* out_bits, cud
     return cudaGetLastError();
 }
 
+// Rows whose sums go straight to L2 (k_accum_rows without shared memory): the
+// atomics leave at some 60 per ns, so up to 2^20 of them, while the clusters are
+// many enough to spread them (2371 x 70, k = 164: 8.6 us against 37.7 us in four
+// launches; 5814 x 30, k = 310: 7.4 against 34.7 us of shared sums in four blocks;
+// but 20,000 x 100, k = 90: 37.2 against 33, 45,905 x 8, k = 216: 17.8 against 16.5).
+static bool few_rows_direct(int64_t n, int d, int k) { return n * d <= (int64_t)1 << 20 && n <= 64 * (int64_t)k && d <= 512; }
+
 cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* labels, int k,
                               const unsigned* absmax_bits, long long* sums, long long* counts, int* iscratch,
                               int32_t* perm, int num_sms, cudaStream_t st, const float* C_wd, double* md_out,
@@ -1107,7 +1118,7 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         if (e == cudaSuccess) e = cudaMemsetAsync(iscratch, 0, sizeof(int) * (size_t)k, st);
         if (e != cudaSuccess) return e;
     }
-    if (d <= 8 && (int64_t)k * d <= AS_MAX_KD) {
+    if (d <= 8 && (int64_t)k * d <= AS_MAX_KD && !few_rows_direct(n, d, k)) {
         // small d: rows in order, per-warp shared accumulators (+ C for the distances)
         const size_t sm = as_smem(d, k, want_wd);
         // about two chunks per resident warp, so that few rows still reach all SMs
@@ -1145,27 +1156,37 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
     const bool vec = d % 4 == 0 && ((uintptr_t)X % 16) == 0;
     const bool can_bucket = 2 * hsm <= 200 * 1024 && d <= 512;
     const size_t smem = sizeof(long long) * ((size_t)k * d + k);
+    typedef void (*RowsFn)(const float*, int64_t, int, const int32_t*, int, const unsigned*, int64_t, long long*, long long*,
+                           const float*, double*);
+    const bool v4 = vec && (!want_wd || ((uintptr_t)C_wd % 16) == 0);
+    const int lpr = df_lpr(d), nv4 = df_nv4(d);
+    const int rows16 = (nv4 == 4 ? 2 : 4) * (32 / lpr) * 16;  // rows of 16 warps at once
+#define KM_AR(NV, L, SH)                                                                                      \
+    if (nv4 == NV && lpr == L)                                                                                \
+        fn = v4 ? (want_wd ? (RowsFn)k_accum_rows<NV, L, true, true, SH> : (RowsFn)k_accum_rows<NV, L, true, false, SH>) \
+                : (want_wd ? (RowsFn)k_accum_rows<NV, L, false, true, SH> : (RowsFn)k_accum_rows<NV, L, false, false, SH>);
+    // few rows, and few of them per cluster: straight to the sums in L2, whose
+    // atomics (one per coordinate) spread over the addresses
+    if (few_rows_direct(n, d, k)) {
+        RowsFn fn = nullptr;
+        KM_AR(1, 8, false) KM_AR(1, 16, false) KM_AR(1, 32, false) KM_AR(2, 32, false) KM_AR(4, 32, false)
+        if (!fn) return cudaErrorInvalidValue;
+        *nlaunch = 1;
+        return klaunch(fn, (unsigned)std::max<int64_t>(1, (8 * n + rows16 - 1) / rows16), 64, 0, st, X, n, d, labels, k,
+                       absmax_bits, nscale, sums, counts, C_wd, md_out);
+    }
     // shared-memory sums in one launch: what the bucketed path does not take, and
     // few rows (n d <= 2^21, with at least 16 rows per cluster to pay for the
     // blocks' folds): 1e4 x 16, k = 8 takes 9 us against 26 us in four launches;
     // 1e5 x 128 would take 60 us of shared atomics against 51 us
     if (smem <= 200 * 1024 && d <= 512 && (!can_bucket || (n * d <= (int64_t)1 << 21 && n >= 16 * (int64_t)k))) {
-        typedef void (*RowsFn)(const float*, int64_t, int, const int32_t*, int, const unsigned*, int64_t, long long*,
-                               long long*, const float*, double*);
         RowsFn fn = nullptr;
-        const bool v4 = vec && (!want_wd || ((uintptr_t)C_wd % 16) == 0);
-        const int lpr = df_lpr(d), nv4 = df_nv4(d);
-#define KM_AR(NV, L)                                                                                      \
-    if (nv4 == NV && lpr == L)                                                                            \
-        fn = v4 ? (want_wd ? (RowsFn)k_accum_rows<NV, L, true, true> : (RowsFn)k_accum_rows<NV, L, true, false>) \
-                : (want_wd ? (RowsFn)k_accum_rows<NV, L, false, true> : (RowsFn)k_accum_rows<NV, L, false, false>);
-        KM_AR(1, 8) KM_AR(1, 16) KM_AR(1, 32) KM_AR(2, 32) KM_AR(4, 32)
+        KM_AR(1, 8, true) KM_AR(1, 16, true) KM_AR(1, 32, true) KM_AR(2, 32, true) KM_AR(4, 32, true)
 #undef KM_AR
         if (!fn) return cudaErrorInvalidValue;
         e = allow_max_smem(fn);
         if (e != cudaSuccess) return e;
-        const int rows = (nv4 == 4 ? 2 : 4) * (32 / lpr) * 16;  // per block and pass
-        const int64_t blk = std::min<int64_t>(std::min<int64_t>((n + rows - 1) / rows, num_sms), std::max<int64_t>(1, n / (4 * (int64_t)k)));
+        const int64_t blk = std::min<int64_t>(std::min<int64_t>((n + rows16 - 1) / rows16, num_sms), std::max<int64_t>(1, n / (4 * (int64_t)k)));
         *nlaunch = 1;
         return klaunch(fn, (unsigned)blk, 512, smem, st, X, n, d, labels, k, absmax_bits, nscale, sums, counts, C_wd, md_out);
     }
@@ -1209,7 +1230,7 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
             if (e != cudaSuccess) return e;
         }
         const int64_t resident_warps = (int64_t)num_sms * std::max(per_sm, 1) * 8;
-        const int seg = (int)std::min<int64_t>(SEG_MAX, std::max<int64_t>(64, n / (resident_warps * 4) / 32 * 32));
+        const int seg = (int)std::min<int64_t>(SEG_MAX, std::max<int64_t>(32, n / (resident_warps * 4) / 32 * 32));
         klaunch(k_bucket_scan, 1, 1024, 0, st, cnt32, k, seg, off, cursor, item_off, counts);
         e = allow_max_smem(k_bucket_scatter);
         if (e != cudaSuccess) return e;

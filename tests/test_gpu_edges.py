@@ -339,3 +339,37 @@ def test_quantise_rows_per_thread(ctx, low, n, d, offset):
     _, _, nf1 = _assign(ctx, X[:30000], C, low, offset)
     _, _, nf2 = _assign(ctx, X[30000:], C, low, offset)
     assert nf == nf1 + nf2
+
+
+# centre sums of few rows straight in L2 (n <= 64 k, n d <= 2^20), on both sides of the lines, and
+# the bucketed sums' short segments: equal to integer sums of the rounded values, also when all
+# rows have one label
+@pytest.mark.parametrize("one_label", [False, True])
+@pytest.mark.parametrize("n,d,k,offset", [(1, 1, 1, 0), (64, 33, 1, 0), (65, 33, 1, 0), (6400, 70, 100, 0), (6401, 70, 100, 1),
+                                          (16384, 64, 300, 0), (16385, 64, 300, 0), (3000, 3, 200, 0), (2000, 512, 64, 0),
+                                          (2000, 513, 64, 0), (20000, 130, 90, 0), (37638, 128, 44, 0), (2371, 256, 164, 2)])
+def test_sums_of_few_rows(ctx, n, d, k, offset, one_label):
+    import math
+    import paper_2407_12208_gb300 as pkg
+    r = np.random.default_rng(n + d)
+    X = _dev(r.normal(size=(n, d)).astype(np.float32), offset)
+    lab = torch.from_numpy((np.full(n, k - 1) if one_label else r.integers(0, k, size=n)).astype(np.int32)).cuda()
+    bits = ctx.absmax(X)
+    sums, counts = ctx.update_partial(X, lab, k, bits, n)
+    assert torch.equal(counts, torch.bincount(lab.long(), minlength=k))
+    amax = float(np.array([bits], dtype=np.uint32).view(np.float32)[0])
+    S = 60 - (n - 1).bit_length() - (math.frexp(amax)[1] - 1)
+    v = torch.round(X.double() * 2.0 ** (S // 2) * 2.0 ** (S - S // 2)).long()
+    assert torch.equal(sums, torch.zeros(k, d, dtype=torch.int64, device="cuda").index_add_(0, lab.long(), v))
+
+
+# refinement, four, eight and 32 rows per warp: near-ties and many candidates on both sides of the lines
+@pytest.mark.parametrize("n", [130, 131, 133, 19456, 19457, 38912, 38913])
+@pytest.mark.parametrize("d", [16, 70])
+def test_refine_rows_per_warp(ctx, n, d):
+    r = np.random.default_rng(n + d)
+    C = r.uniform(size=(90, d)).astype(np.float32)
+    C = np.concatenate([C, C[:40] + np.float32(1e-7)]).astype(np.float32)  # near-ties
+    X = r.uniform(size=(n, d)).astype(np.float32)
+    lab, md, _ = _assign(ctx, X, C, "bf16")
+    check_assign(lab, md, X, C, oracle, RTOL_MD)
