@@ -20,7 +20,7 @@
 //    (8 lanes per pair, 4 pairs per warp, no per-row bookkeeping), k_certify
 //    (one thread per row) and k_amb_fp64.
 // Measured, k_refine against the four launches (GPU time, without the gaps
-// between launches): 1000 x 32 7.9 / 15.0 us, 1e4 x 16 7.4 / 16.3 us, 1e5 x 128
+// between launches): 1000 x 32 5.5 / 15.0 us, 1e4 x 16 5.6 / 16.3 us, 1e5 x 128
 // 19.8 / 28.7 us, 4e6 x 64 206 / 260 us; 150,001 x 256 92 / 72 us, 1e6 x 128
 // 293 / 219 us (x and two centres in registers leave three blocks per SM).
 
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
                                                 const int* __restrict__ list_n, const float* __restrict__ X,
                                                 const float* __restrict__ C, int d, float gamma32,
                                                 int32_t* __restrict__ labels, int32_t* __restrict__ ovf_list,
-                                                int* __restrict__ ovf_n, bool many_to_list, int rpw, DevCounters* cnt) {
+                                                int* __restrict__ ovf_n, bool many_to_list, int rpw_all, DevCounters* cnt) {
     chain_enter();
     constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
     static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
@@ -406,6 +406,10 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
     const int d4 = d >> 2;
     unsigned ev32 = 0, ev64 = 0, amb = 0, ovf = 0;
     const int nwb = blockDim.x >> 5;
+    // a list's rows, of unknown number, are spread evenly over the warps: a short
+    // one of rows with many candidates each (taken one by one) took 74 us at 32 rows
+    // per warp (1e5 x 128, k = 500), 9 now
+    const int rpw = !LIST ? rpw_all : (int)max((int64_t)1, min((int64_t)32, (nrows + (int64_t)gridDim.x * nwb - 1) / ((int64_t)gridDim.x * nwb)));
     for (int64_t r0 = ((int64_t)blockIdx.x * nwb + wib) * rpw; r0 < nrows; r0 += (int64_t)gridDim.x * nwb * rpw) {
         const int64_t r = r0 + lane;
         const bool valid = lane < rpw && r < nrows;
@@ -454,8 +458,15 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
         const unsigned fm = __ballot_sync(0xffffffffu, few);
         if (few) ord[__popc(fm & ((1u << lane) - 1u))] = lane;
         __syncwarp();
-        if (many_to_list && c > RF_FEW) ovf_list[atomicAdd(ovf_n, 1)] = myrow;
-        unsigned slow = __ballot_sync(0xffffffffu, c > RF_FEW && !many_to_list);
+        // rows of many candidates: up to four are taken here, one by one; more of them
+        // leave for the next pass, whose launches (30 to 40 us once a row is listed)
+        // a handful in all would not be worth (133,333 x 128 x 1024 uniform, 12 and more
+        // candidates in one row of a thousand)
+        unsigned slow = __ballot_sync(0xffffffffu, c > RF_FEW);
+        if (many_to_list && __popc(slow) > 4) {
+            if (c > RF_FEW) ovf_list[atomicAdd(ovf_n, 1)] = myrow;
+            slow = 0;
+        }
         const int nfew = __popc(fm);
         for (int i0 = 0; i0 < nfew; i0 += 4) {
             const int i = i0 + (lane >> 3);
