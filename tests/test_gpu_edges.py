@@ -373,3 +373,19 @@ def test_refine_rows_per_warp(ctx, n, d):
     X = r.uniform(size=(n, d)).astype(np.float32)
     lab, md, _ = _assign(ctx, X, C, "bf16")
     check_assign(lab, md, X, C, oracle, RTOL_MD)
+
+
+# rows of more than twelve candidates: none, a few per warp (decided in the first pass) and many
+# (listed), among rows of one candidate, with and without a centred screen after
+@pytest.mark.parametrize("every", [0, 40, 9, 6, 2])
+@pytest.mark.parametrize("n,d,k", [(20000, 24, 300), (60000, 40, 600), (6000, 16, 200)])
+def test_rows_of_many_candidates(ctx, n, d, k, every):
+    r = np.random.default_rng(n + every)
+    C = (20 * r.normal(size=(k, d))).astype(np.float32)
+    C[: 40] = C[0] + (0.02 * r.normal(size=(40, d))).astype(np.float32)  # forty centres close together
+    at = r.integers(40, k, size=n)
+    if every:
+        at[::every] = r.integers(0, 40, size=len(at[::every]))
+    X = (C[at] + 0.05 * r.normal(size=(n, d))).astype(np.float32)
+    lab, md, _ = _assign(ctx, X, C, "bf16")
+    check_assign(lab, md, X, C, oracle, RTOL_MD)
