@@ -213,12 +213,16 @@ __global__ void k_patch_flagged(const float* __restrict__ X, const float* __rest
 // The binary64 fallback's value, rounded to the matrix's binary32, without the
 // narrow FP64 pipe: the pair's double-float distance (df.cuh) lies within eps
 // (relative) of the binary64 sum, and where both ends of that interval round
-// to the same binary32 number, that is the value.  eps covers the chain of
-// `levels` combinations (below 3 2^-48 each), the squares (2^-46) and the
-// binary64 sum's own rounding ((d + 2) 2^-53).  Values near a rounding boundary
-// (one in about 2^17), tiny ones (squares below binary32's normal range) and
-// what is no number take binary64 in the oracle's order.
-KM_DEV float patch_eps(int d, int levels) { return (float)(3 * levels + 5) * 0x1p-48f + (float)(d + 2) * 0x1p-53f; }
+// to the same binary32 number, that is the value.  With u = 2^-24, relative to
+// the true sum and to first order in u^2: the squares 4 u^2 (their trailing
+// parts reach 3 u); a chunk's two sums of unnormalised squares 7 u^2 (trailing
+// parts added 3, the leading parts' error added 4; they reach 4 u) and their
+// combination 9 u^2 (4 and 5): 20 u^2 a chunk; each of the `levels`
+// combinations of normalised pairs 3 u^2 (1 and 2); the binary64 sum's own
+// rounding (d + 2) 2^-53.  Values near a rounding boundary (one in about 2^16),
+// tiny ones (squares below binary32's normal range) and what is no number take
+// binary64 in the oracle's order.
+KM_DEV float patch_eps(int d, int levels) { return (float)(3 * levels + 20) * 0x1p-48f + (float)(d + 2) * 0x1p-53f; }
 KM_DEV bool patch_sure(DF r, float eps) {
     const float e = r.hi * eps * 1.01f;
     return r.hi >= 0x1p-60f && r.hi < INFINITY && __fadd_rn(r.hi, __fadd_ru(r.lo, e)) == r.hi &&
