@@ -232,6 +232,14 @@ KM_DEV float fmin3f(float a, float b, float c) {
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
+// Theorem 4.1 for an fp32 direct value v of d coordinates: the true value lies
+// in [direct_lower, direct_upper].  g, relative, covers the roundings of normal
+// numbers; tiny = direct_tiny(d) those of squares and sums below binary32's
+// normal range, which are absolute, 2^-150 each (0.49 and 0.51 of the least
+// subnormal become 0 and 1 of it).
+KM_DEV float direct_tiny(int d) { return (float)(2 * d + 4) * 0x1p-149f; }
+KM_DEV float direct_lower(float v, float g) { return v * (1.0f - g); }
+KM_DEV float direct_upper(float v, float g, float tiny) { return fmaf(v, 1.0f + g, tiny); }
 // Error-free sum (Knuth's TwoSum): a + b = s + e exactly.
 KM_DEV void two_sum(float a, float b, float& s, float& e) {
     s = a + b;

@@ -182,20 +182,19 @@ __device__ __noinline__ bool resolve_row(const float* __restrict__ X, const floa
     __syncthreads();
     t = red[0];
     for (int q = 1; q < 8; q++) t = top2_merge(t, red[q]);
-    if (t.b2 * (1.0f - gamma32) > t.b1 * (1.0f + gamma32)) {
+    const float thr = direct_upper(t.b1, gamma32, direct_tiny(d));
+    if (direct_lower(t.b2, gamma32) > thr) {
         if (tid == 0) {
             labels[i] = t.j1;
             min_dist[i] = (double)t.b1;
         }
         return false;
     }
-    // squares below binary32's range: each coordinate adds at most 2^-149 of absolute error
-    const float thr = t.b1 * (1.0f + gamma32) + (float)(2 * d + 4) * 0x1p-149f;
     double best = INFINITY;
     int arg = 0x7fffffff;
     if (keep_vals) {
         for (int j = tid; j < k; j += 256)
-            if (vs[j] * (1.0f - gamma32) <= thr) {
+            if (direct_lower(vs[j], gamma32) <= thr) {
                 const int p = atomicAdd(&nopen, 1);
                 if (p < RF_OPEN) open_j[p] = j;
             }
@@ -205,7 +204,7 @@ __device__ __noinline__ bool resolve_row(const float* __restrict__ X, const floa
             warp_direct4(xs, C, k, d, j, lane, v);
 #pragma unroll
             for (int q = 0; q < 4; q++)
-                if (lane == 0 && j + q < k && v[q] * (1.0f - gamma32) <= thr) {
+                if (lane == 0 && j + q < k && direct_lower(v[q], gamma32) <= thr) {
                     const int p = atomicAdd(&nopen, 1);
                     if (p < RF_OPEN) open_j[p] = j + q;
                 }
@@ -235,7 +234,7 @@ __device__ __noinline__ bool resolve_row(const float* __restrict__ X, const floa
     } else {
         // (the open list did not fit: every centre it would have held)
         for (int j = tid; j < k; j += 256) {
-            if (keep_vals && !(vs[j] * (1.0f - gamma32) <= thr)) continue;
+            if (keep_vals && !(direct_lower(vs[j], gamma32) <= thr)) continue;
             const double s = direct64(xs, C + (int64_t)j * d, d);
             ++*ev64;
             if (s < best) { best = s; arg = j; }
@@ -451,8 +450,7 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
                     const int64_t gi = row_list ? (int64_t)row_list[base + r] : base + r;
                     labels[gi] = j1[i];
                     min_dist[gi] = (double)b1[i];
-                    // Theorem 4.1: true values lie in [v (1 - g), v (1 + g)]
-                    if (!(b2[i] * (1.0f - g) > b1[i] * (1.0f + g))) {
+                    if (!(direct_lower(b2[i], g) > direct_upper(b1[i], g, direct_tiny(d)))) {  // (Theorem 4.1)
                         open_rows[atomicAdd(&nopen, 1)] = (int)gi;
                         local_amb++;
                     }
@@ -573,11 +571,9 @@ __device__ __noinline__ int small_open_row(const float* __restrict__ X, int64_t 
             b2 = acc;
         }
     }
-    // Theorem 4.1: true values lie in [v (1 - g), v (1 + g)]
-    if (b2 * (1.0f - g) > b1 * (1.0f + g)) return j1;
+    const float thr = direct_upper(b1, g, direct_tiny(D));
+    if (direct_lower(b2, g) > thr) return j1;
     ++*amb;
-    // (squares below binary32's range: at most 2^-149 per coordinate)
-    const float thr = b1 * (1.0f + g) + (float)(2 * D + 4) * 0x1p-149f;
     double best = INFINITY;
     for (int j = 0; j < k; j++) {
         float acc = 0.0f;
@@ -586,7 +582,7 @@ __device__ __noinline__ int small_open_row(const float* __restrict__ X, int64_t 
             const float t = x[l] - C[j * D + l];
             acc = fmaf(t, t, acc);
         }
-        if (!(acc * (1.0f - g) <= thr)) continue;
+        if (!(direct_lower(acc, g) <= thr)) continue;
         const double s = direct64(x, C + j * D, D);
         ++*ev64;
         if (s < best) {

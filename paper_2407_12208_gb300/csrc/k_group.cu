@@ -81,13 +81,13 @@ KM_DEV void grp_assign(const float* __restrict__ X, int n, int k, const float* C
             else if (v < b2) b2 = v;
         }
         int lab = j1;
-        if (!(b2 * (1.0f - g) > b1 * (1.0f + g))) {  // not certified: binary64 over the open centres
-            const float thr = b1 * (1.0f + g);
+        const float thr = direct_upper(b1, g, direct_tiny(D));
+        if (!(direct_lower(b2, g) > thr)) {  // not certified: binary64 over the open centres
             double best = INFINITY;
             int arg = 0x7fffffff;
             for (int j = 0; j < k; j++) {
                 const float v = grp_direct32<D>(x, Cc + j * D);
-                if (!(v * (1.0f - g) <= thr)) continue;
+                if (!(direct_lower(v, g) <= thr)) continue;
                 const double s = grp_direct64<D>(x, Cc + j * D);
                 if (s < best) { best = s; arg = j; }
             }

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_certify(const int2* __restrict__ rowpai
                                                  int32_t* __restrict__ amb_list, DevCounters* cnt) {
     chain_enter();
     unsigned long long ev32 = 0, amb = 0, ovf_rows = 0;
-    const float g = gamma32;
+    const float g = gamma32, tiny = direct_tiny(d);
     for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < n;
          row += (int64_t)gridDim.x * blockDim.x) {
         const int2 rp = rowpair[row];
@@ -243,12 +243,12 @@ __global__ void __launch_bounds__(256) k_certify(const int2* __restrict__ rowpai
             continue;
         }
         float up = INFINITY;
-        for (int r = 0; r < rp.y; r++) up = fminf(up, v32[rp.x + r] * (1.0f + g));
+        for (int r = 0; r < rp.y; r++) up = fminf(up, direct_upper(v32[rp.x + r], g, tiny));
         int open = 0, bj = 0x7fffffff;
         float bv = INFINITY;
         for (int r = 0; r < rp.y; r++) {
             const float v = v32[rp.x + r];
-            if (v * (1.0f - g) <= up) {
+            if (direct_lower(v, g) <= up) {
                 open++;
                 const int j = pairs[rp.x + r].y;
                 if (v < bv || (v == bv && j < bj)) { bv = v; bj = j; }
@@ -299,13 +299,13 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int na = *amb_count;
-    const float g = gamma32;
+    const float g = gamma32, tiny = direct_tiny(d);
     unsigned long long ev64 = 0;
     for (int64_t t = w0; t < na; t += nw) {
         const int64_t row = amb_list[t];
         const int2 rp = rowpair[row];
         float up = INFINITY;
-        for (int r = lane; r < rp.y; r += 32) up = fminf(up, v32[rp.x + r] * (1.0f + g));
+        for (int r = lane; r < rp.y; r += 32) up = fminf(up, direct_upper(v32[rp.x + r], g, tiny));
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) up = fminf(up, __shfl_xor_sync(0xffffffffu, up, off));
         const float* x = X + row * d;
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
             int js[AMB_B] = {};
             int nb = 0;
             for (; r < rp.y && nb < AMB_B; r++)
-                if (v32[rp.x + r] * (1.0f - g) <= up) js[nb++] = pairs[rp.x + r].y;
+                if (direct_lower(v32[rp.x + r], g) <= up) js[nb++] = pairs[rp.x + r].y;
             if (nb == 0) break;
             __syncwarp();
             // lanes over the coordinates (coalesced loads, no index division)
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
     int *jl = jl_sh[wib], *ord = ord_sh[wib];
     const uint32_t emask = (1u << ebits) - 1u;
     const float lscale = __uint_as_float((uint32_t)(127 + ebits - 23) << 23);  // 2^(ebits - 23)
-    const float g = gamma32;
+    const float g = gamma32, tiny = direct_tiny(d);
     const int d4 = d >> 2;
     unsigned ev32 = 0, ev64 = 0, amb = 0, ovf = 0;
     const int nwb = blockDim.x >> 5;
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
                     keep(acc, j, t < cc);
                 }
             }
-            const bool sure = b2 * (1.0f - g) > b1 * (1.0f + g);  // false where nothing is comparable
+            const bool sure = direct_lower(b2, g) > direct_upper(b1, g, tiny);  // false where nothing is comparable
             if (sl == 0 && cc) {
                 ev32 += cc;
                 if (sure) labels[row] = j1;
@@ -578,12 +578,12 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
             __syncwarp();
             if (lane == 0 && total > RF_FEW) ev32 += total;
             float up = INFINITY;
-            for (int t = lane; t < total; t += 32) up = fminf(up, vs[t] * (1.0f + g));
+            for (int t = lane; t < total; t += 32) up = fminf(up, direct_upper(vs[t], g, tiny));
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) up = fminf(up, __shfl_xor_sync(0xffffffffu, up, off));
             int open = 0, bj = 0x7fffffff;
             for (int t = lane; t < total; t += 32)
-                if (vs[t] * (1.0f - g) <= up) {
+                if (direct_lower(vs[t], g) <= up) {
                     open++;
                     bj = js[t];  // (the only one, when open is 1 over the warp)
                 }
@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo
             double best = INFINITY;
             bj = 0x7fffffff;
             for (int t = 0; t < total; t++) {
-                if (!(vs[t] * (1.0f - g) <= up)) continue;
+                if (!(direct_lower(vs[t], g) <= up)) continue;
                 const int j = js[t];
                 const float* cj = C + (int64_t)j * d;
                 for (int l = lane; l < d; l += 32) {

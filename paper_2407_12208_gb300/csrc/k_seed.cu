@@ -84,11 +84,12 @@ KM_DEV double dmin_bits(double a, double b) {
     return __longlong_as_double(x < y ? x : y);
 }
 KM_DEV bool dpos(double a) { return __double_as_longlong(a) > 0; }
-// A float at or above the non-negative double a.
+// A float at or above the non-negative double a (2^-100 at least, unless a is 0:
+// there the fp32 distance's absolute roundings, 2^-150 each, are below its own).
 KM_DEV float dround_up(double a) {
     const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
     const unsigned e = hi >> 20;
-    if (e < 897u) return e == 0u && lo == 0u && hi == 0u ? 0.0f : 0x1p-126f;  // (below 2^-126)
+    if (e < 923u) return e == 0u && lo == 0u && hi == 0u ? 0.0f : 0x1p-100f;  // (below 2^-100)
     if (e > 1150u) return INFINITY;                                          // (2^128 or more, not a number)
     return __uint_as_float(((hi - (896u << 20)) << 3 | lo >> 29) + 1u);
 }
