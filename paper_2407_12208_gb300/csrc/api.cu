@@ -1534,14 +1534,16 @@ km_status km_cancel(km_ctx* ctx, uint64_t job_id) {
 
 }  // extern "C"
 
-size_t km_internal_ws_bytes(int64_t n, int d, int k, const km_params* p) {
+size_t km_internal_ws_bytes(int64_t n, int d, int k, const km_params* p, bool centred) {
     Carve a{nullptr};
     carve_lloyd(a, n, d, k, p->low, std::max(0, (int)p->max_iter));
-    carve_centred(a, n, d, k, p->low);
     Carve b{nullptr};
     carve_assign(b, n, d, k, p->low, false);
     b.take<double>((size_t)n);
-    carve_centred(b, n, d, k, p->low);
+    if (centred) {
+        carve_centred(a, n, d, k, p->low);
+        carve_centred(b, n, d, k, p->low);
+    }
     return std::max(a.off, b.off) + 256;
 }
 

@@ -29,7 +29,6 @@
 #include "group.h"
 #include "serve.h"
 
-size_t km_internal_ws_bytes(int64_t n, int d, int k, const km_params* p);
 
 namespace {
 
@@ -41,7 +40,8 @@ struct Job {
     uint64_t id = 0;
     km_job spec{};
     std::vector<float> X, C;
-    size_t bytes = 0, off = 0;
+    size_t bytes = 0, off = 0;  // what the job needs; once admitted, what it holds
+    size_t bytes_roomy = 0;     // with the centred screen's buffers, where the arena has room to spare
     bool has_mem = false;
     JobState state = JobState::Queued;
     volatile int cancel = 0;
@@ -123,7 +123,10 @@ struct km_serve {
             const bool g = km_internal_groupable(j->spec);
             if (!has_room(g)) break;
             size_t off = 0;
-            if (alloc(j->bytes, &off)) {
+            bool got = alloc(j->bytes_roomy, &off);
+            if (got) j->bytes = j->bytes_roomy;
+            else got = alloc(j->bytes, &off);
+            if (got) {
                 j->off = off;
                 j->has_mem = true;
                 j->t_admit = Clock::now();
@@ -326,8 +329,12 @@ km_status serve_submit(km_serve* s, const km_job* job, uint64_t* job_id, std::st
     const bool resident = (job->flags & KM_JOB_DEVICE_DATA) != 0;
     const size_t data = (resident ? 0 : up256(sizeof(float) * (size_t)job->n * job->d)) +
                         2 * up256(sizeof(float) * (size_t)job->k * job->d) + up256(sizeof(int32_t) * (size_t)job->n);
-    const size_t ws = km_internal_ws_bytes(job->n, job->d, job->k, &job->p);
-    const size_t bytes = up256(data + ws);
+    const size_t bytes = up256(data + km_internal_ws_bytes(job->n, job->d, job->k, &job->p, false));
+    // The centred screen's buffers are optional (without them rows whose lists
+    // overflow take the direct kernel) and up to as large as the rest: a job gets
+    // them only where one such job for every worker fits in the arena, so that jobs
+    // of its size or less keep none of their kind out.
+    const size_t roomy = up256(data + km_internal_ws_bytes(job->n, job->d, job->k, &job->p, true));
     // a job larger than the whole arena can never be admitted (checked before
     // the host arrays are copied)
     if (bytes > s->arena_usable) {
@@ -337,6 +344,7 @@ km_status serve_submit(km_serve* s, const km_job* job, uint64_t* job_id, std::st
     Job* j = new Job();
     j->spec = *job;
     j->bytes = bytes;
+    j->bytes_roomy = roomy <= s->arena_usable / (size_t)s->n_workers ? roomy : bytes;
     if (!resident) {
         j->X.assign(job->X, job->X + (size_t)job->n * job->d);
         j->C.assign(job->C_init, job->C_init + (size_t)job->k * job->d);

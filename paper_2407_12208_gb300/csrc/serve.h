@@ -23,6 +23,9 @@ km_status serve_poll(km_serve* s, uint64_t job_id, km_result* out);
 km_status serve_release(km_serve* s, uint64_t job_id);
 km_status serve_cancel(km_serve* s, uint64_t job_id);
 
+// Workspace of a job (defined in api.cu), with or without the buffers of the
+// centred screen, which a run does without when they are not there.
+size_t km_internal_ws_bytes(int64_t n, int d, int k, const km_params* p, bool centred);
 // Runs one job to completion on `st` (defined in api.cu).  `cancel` is polled
 // between Lloyd iterations.
 // Whether a job can run inside a grouped launch (km_lloyd_run_batch's limits),

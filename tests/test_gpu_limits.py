@@ -64,3 +64,43 @@ def test_squares_below_the_range_grouped(ctx):
     X, C = _subnormal_squares(50, 4, 6, 0.0)
     (out,) = ctx.lloyd_run_batch([(_dev(X), _dev(C))], pkg.params("fp32", max_iter=0))
     assert (out[1] == 5).all()
+
+
+def _smallest_workspace(ctx, run, ws):
+    """Bytes of the smallest workspace that `run` accepts, to 256."""
+    import paper_2407_12208_gb300 as pkg
+    lo, hi = 0, ws.numel()  # refused at lo, accepted at hi
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        try:
+            run(ws[:mid])
+            hi = mid
+        except pkg.KmError:
+            lo = mid
+    return hi
+
+
+# the serving engine takes a job, and two side by side, when the arena holds what they need: the
+# buffers of the centred screen (n k d >= 2^30) are no part of that
+def test_admission_without_optional_buffers(ctx):
+    import time
+    import paper_2407_12208_gb300 as pkg
+    n, d, k = 17000, 64, 1000
+    X, C = workloads.cancellation(n, d, k, seed=6)
+    Xd, Cd, p = _dev(X), _dev(C), pkg.params("bf16", max_iter=2)
+    need = _smallest_workspace(ctx, lambda ws: ctx.lloyd_run(Xd, Cd, p, ws=ws), ctx.workspace(n, d, k, p))
+    want = ctx.lloyd_run(Xd, Cd, p)
+    job = need + 4 * (n + 2 * k * d) + 2048  # labels, centres and their rounding to 256
+    s = pkg.Context(0, arena_bytes=2 * job + 1024)
+    try:
+        ids = [s.submit(Xd, Cd, p) for _ in range(2)]
+        for i in ids:  # both run although neither result is released
+            t0 = time.time()
+            while (r := s.poll(i)) is None:
+                assert time.time() - t0 < 60, "not admitted"
+                time.sleep(0.002)
+            assert r["status"] == pkg._binding.KM_OK
+            assert torch.equal(pkg.device_array(r["labels"], (n,), "<i4"), want[1])
+            assert torch.equal(pkg.device_array(r["C"], (k, d), "<f4"), want[0])
+    finally:
+        s.close()
