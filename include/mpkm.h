@@ -127,7 +127,10 @@ const char* km_last_error(const km_ctx* ctx);
 /* Bytes of workspace the synchronous calls (km_distances, km_assign,
  * km_update_centroids, km_lloyd_step, km_lloyd_run with p->max_iter) need for
  * these sizes: the largest of their layouts, all O(n (d + k_slots)) -- about
- * 0.66 GB at n = 1e6, d = 128, k = 1024 with a 16-bit low format. */
+ * 0.80 GB at n = 1e6, d = 128, k = 1024 with a 16-bit low format.  Part of it
+ * (there 0.17 GB) is optional, the buffers of the centred screen for rows whose
+ * candidate lists overflow: a workspace without them is taken, and such rows
+ * then cost more. */
 km_status km_workspace_size(const km_ctx* ctx, int64_t n, int d, int k, const km_params* p,
                             size_t* bytes);
 

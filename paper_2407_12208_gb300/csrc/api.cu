@@ -208,12 +208,6 @@ AssignWs carve_assign(Carve& cv, int64_t n, int d, int k, int low, bool distance
         w.ovf_list = cv.take<int32_t>((size_t)n);
         if (!distances) {
             w.cand = cv.take<uint32_t>((size_t)n * TC_GROUPS * TC_LIST);
-            if (refine_batched(n, d)) {
-                w.rowpair = cv.take<int2>((size_t)n);
-                w.pair_cap = std::min<int64_t>((int64_t)n * TC_PAIRS_PER_ROW, (int64_t)INT32_MAX);
-                w.pairs = cv.take<int2>((size_t)w.pair_cap);
-                w.v32 = cv.take<float>((size_t)w.pair_cap);
-            }
         } else {
             w.qcap = flag_queue_cap(n, k);
             w.queue = cv.take<int2>((size_t)w.qcap);
@@ -235,8 +229,6 @@ AssignWs carve_assign(Carve& cv, int64_t n, int d, int k, int low, bool distance
 bool centred_applies(int64_t n, int d, int k, int low) {
     return is_tc(low) && d <= 256 && (double)n * k * d >= (double)(1 << 30) && tc_smem_bytes(1, d, 1) != 0;
 }
-// Its buffers come last in every workspace: a workspace without room for them
-// does without (the rows then go to the full-row kernel).
 Centred carve_centred(Carve& cv, int64_t n, int d, int k, int low) {
     Centred c{};
     if (!centred_applies(n, d, k, low)) return c;
@@ -250,11 +242,29 @@ Centred carve_centred(Carve& cv, int64_t n, int d, int k, int low) {
     c.list2 = cv.take<int32_t>((size_t)n);
     return c;
 }
-// cv stands at the end of what the call needs
-Centred take_centred(const Carve& cv, size_t ws_bytes, int64_t n, int d, int k, int low) {
+// The last span of an assignment's workspace: the flat pair list of the first
+// refinement and, once that is done with it, the buffers of the centred screen.
+// cv: past the call's other buffers; left at the end of what it needs.  A
+// workspace without room for the larger, optional set does without (the rows
+// then go to the full-row kernel).  Returns the bytes with both.
+size_t carve_tail(Carve& cv, size_t ws_bytes, int64_t n, int d, int k, int low, AssignWs& w, Centred& cen) {
     Carve t = cv;
-    const Centred c = carve_centred(t, n, d, k, low);
-    return t.off <= ws_bytes ? c : Centred{};
+    cen = carve_centred(t, n, d, k, low);
+    if (t.off > ws_bytes) cen = Centred{};
+    if (is_tc(low) && refine_batched(n, d)) {
+        w.rowpair = cv.take<int2>((size_t)n);
+        w.pair_cap = std::min<int64_t>((int64_t)n * TC_PAIRS_PER_ROW, (int64_t)INT32_MAX);
+        w.pairs = cv.take<int2>((size_t)w.pair_cap);
+        w.v32 = cv.take<float>((size_t)w.pair_cap);
+    }
+    return std::max(cv.off, t.off);
+}
+// The bytes of that span past cv, with or without the optional buffers.
+size_t tail_end(Carve cv, int64_t n, int d, int k, int low, bool centred) {
+    AssignWs w{};
+    Centred cen;
+    const size_t both = carve_tail(cv, 0, n, d, k, low, w, cen);
+    return centred ? both : cv.off;
 }
 
 struct UpdateWs {
@@ -628,10 +638,9 @@ km_status km_workspace_size(const km_ctx* cctx, int64_t n, int d, int k, const k
     if (n < 1 || d < 1 || k < 1) return fail(ctx, KM_EINVAL, "need n, d, k >= 1");
     Carve a{nullptr};
     carve_lloyd(a, n, d, k, p->low, std::max(0, (int)p->max_iter));
-    carve_centred(a, n, d, k, p->low);
     Carve b{nullptr};
     carve_assign(b, n, d, k, p->low, true);
-    *bytes = std::max(a.off, b.off) + 256;
+    *bytes = std::max(tail_end(a, n, d, k, p->low, true), b.off) + 256;
     return KM_OK;
 }
 
@@ -714,19 +723,10 @@ km_status km_assign(km_ctx* ctx, const float* X, int64_t n, const float* C, int 
     if (!aligned256(ws)) return fail(ctx, KM_EINVAL, "workspace must be 256-byte aligned");
     Carve cv{(char*)ws};
     AssignWs w = carve_assign(cv, n, d, k, p->low, false);
-    double* md = min_dist;
-    Carve tmp{nullptr};
-    carve_assign(tmp, n, d, k, p->low, false);
-    size_t need = tmp.off;
-    if (!md) {  // scratch min_dist when the caller does not want it
-        Carve c2{(char*)ws};
-        c2.off = tmp.off;
-        md = c2.take<double>((size_t)n);
-        need = c2.off;
-    }
-    cv.off = need;
-    const Centred cen = take_centred(cv, ws_bytes, n, d, k, p->low);
-    if (ws_bytes < need) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, need);
+    double* md = min_dist ? min_dist : cv.take<double>((size_t)n);  // (scratch when the caller does not want it)
+    Centred cen;
+    carve_tail(cv, ws_bytes, n, d, k, p->low, w, cen);
+    if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
     CK(cudaMemsetAsync(w.cnt, 0, sizeof(DevCounters), st));
@@ -1030,7 +1030,8 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
     AssignWs w = carve_assign(cv, n, d, k, p->low, false);
     UpdateWs u = carve_update(cv, n, d, k);
     double* md = min_dist ? min_dist : cv.take<double>((size_t)n);
-    const Centred cen = take_centred(cv, ws_bytes, n, d, k, p->low);
+    Centred cen;
+    carve_tail(cv, ws_bytes, n, d, k, p->low, w, cen);
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
@@ -1071,8 +1072,7 @@ km_status km_host_workspace_size(const km_ctx* cctx, int64_t n, int d, int k, co
     carve_host(a, n, d, k);
     carve_assign(a, n, d, k, p->low, false);
     carve_update(a, n, d, k);
-    carve_centred(a, n, d, k, p->low);
-    *bytes = a.off + 256;
+    *bytes = tail_end(a, n, d, k, p->low, true) + 256;
     return KM_OK;
 }
 
@@ -1089,7 +1089,8 @@ km_status km_lloyd_step_host(km_ctx* ctx, const float* X_host, int64_t n, int d,
     HostWs h = carve_host(cv, n, d, k);
     AssignWs w = carve_assign(cv, n, d, k, p->low, false);
     UpdateWs u = carve_update(cv, n, d, k);
-    const Centred cen = take_centred(cv, ws_bytes, n, d, k, p->low);
+    Centred cen;
+    carve_tail(cv, ws_bytes, n, d, k, p->low, w, cen);
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
@@ -1334,7 +1335,7 @@ static km_status lloyd_impl(km_ctx* ctx, const float* X, int64_t n, int d, int k
     if (!aligned256(ws)) return fail(ctx, KM_EINVAL, "workspace must be 256-byte aligned");
     Carve cv{(char*)ws};
     LloydWs L = carve_lloyd(cv, n, d, k, p->low, p->max_iter);
-    L.cen = take_centred(cv, ws_bytes, n, d, k, p->low);
+    carve_tail(cv, ws_bytes, n, d, k, p->low, L.a, L.cen);
     if (ws_bytes < cv.off) return fail(ctx, KM_ENOMEM, "workspace too small: %zu < %zu", ws_bytes, cv.off);
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaSetDevice(ctx->device));
@@ -1540,11 +1541,7 @@ size_t km_internal_ws_bytes(int64_t n, int d, int k, const km_params* p, bool ce
     Carve b{nullptr};
     carve_assign(b, n, d, k, p->low, false);
     b.take<double>((size_t)n);
-    if (centred) {
-        carve_centred(a, n, d, k, p->low);
-        carve_centred(b, n, d, k, p->low);
-    }
-    return std::max(a.off, b.off) + 256;
+    return std::max(tail_end(a, n, d, k, p->low, centred), tail_end(b, n, d, k, p->low, centred)) + 256;
 }
 
 bool km_internal_groupable(const km_job& job) {

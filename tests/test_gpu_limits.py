@@ -104,3 +104,40 @@ def test_admission_without_optional_buffers(ctx):
             assert torch.equal(pkg.device_array(r["C"], (k, d), "<f4"), want[0])
     finally:
         s.close()
+
+
+# the flat pair list (n d > 2^25, d > 64) and the centred screen's buffers share a span: rows
+# decided by the one, by the other and by neither in the same call and the same run, with and
+# without room for the larger of the two
+def test_workspace_of_the_largest_step(ctx):
+    import paper_2407_12208_gb300 as pkg
+    n, d = 10 ** 6, 128
+    screen = n * (2 * d + 16) + n * 4 * (48 + 16)   # X in bf16, statistics, lists and per-row words
+    tail = n * (2 * d + 16 + 4)                      # the larger of the two sets
+    assert ctx.workspace_size(n, d, 1024, pkg.params("bf16")) < screen + tail + (8 << 20)
+
+
+@pytest.mark.parametrize("call", ["assign", "run", "host"])
+def test_shared_scratch_span(ctx, call):
+    import paper_2407_12208_gb300 as pkg
+    n, d, k = 270001, 128, 40
+    X, C = workloads.gaussian_mixture(n, d, k, seed=8)
+    far, near = workloads.cancellation(90000, d, 20, seed=9)
+    C[:20] = near  # a third of the rows: lists that overflow
+    X[::3][:90000] = far
+    C[39] = C[38]
+    p = pkg.params("bf16", max_iter=3)
+    Xd, Cd = _dev(X), _dev(C)
+    if call == "host":
+        got = ctx.lloyd_step_host(torch.from_numpy(X), torch.from_numpy(C), p)
+        want = ctx.lloyd_step(Xd, Cd, p)
+        assert torch.equal(got[0], want[0].cpu()) and torch.equal(got[2], want[2].cpu()) and got[4] == want[4]
+        return
+    f = (lambda ws: ctx.assign(Xd, Cd, p, ws=ws)[:2]) if call == "assign" else (lambda ws: ctx.lloyd_run(Xd, Cd, p, ws=ws)[:3])
+    ws = ctx.workspace(n, d, k, p)
+    hi = _smallest_workspace(ctx, f, ws)
+    assert hi < ws.numel() - n * 100
+    a, b = f(ws), f(ws[:hi])
+    assert all(np.array_equal(torch.as_tensor(u).cpu().numpy(), torch.as_tensor(v).cpu().numpy()) for u, v in zip(a, b))
+    if call == "assign":
+        check_assign(a[0].cpu().numpy()[:3000], a[1].cpu().numpy()[:3000], X[:3000], C, oracle, RTOL_MD)
