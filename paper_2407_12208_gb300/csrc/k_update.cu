@@ -59,13 +59,58 @@ __global__ void k_accumulate(const float* __restrict__ X, int64_t n, int d, cons
     }
 }
 
-// The same in shared memory (the k d sums and k counts fit), rows spread over
-// LPR lanes of NV4 float4 as in k_winner_dist; WD: each row's distance to its
-// own centre (the same arithmetic, the same bits) from the same read of the
-// row.  One launch, where the bucketed path takes four: for few rows, and for
-// rows it does not take.  Bound by latency for few rows, by the shared atomics
-// for many: 1e4 x 16, k = 8 26 -> 9 us, 1e5 x 10, k = 100 26 -> 19 us.
-template <int NV4, int LPR, bool VEC, bool WD, bool SH>
+// A warp's pass over STEP rows, each on LPR lanes of NV4 float4 as in
+// k_winner_dist: the rows' labels (js, -1 past the end) and coordinates (xv);
+// WD: each row's distance to its own centre (the same arithmetic, the same
+// bits) from the same read of the row.
+template <int NV4, int LPR, bool VEC, bool WD, int R>
+KM_DEV void rows_pass(const float* __restrict__ X, int64_t n, int d, const int32_t* __restrict__ labels, int64_t base,
+                      const float* __restrict__ C, double* __restrict__ md, int lane, int (&js)[R], float4 (&xv)[R][NV4]) {
+    constexpr int G = 32 / LPR, STEP = R * G;
+    const int sub = lane / LPR, cl = lane % LPR;
+    const int d4 = (d + 3) >> 2;
+    const int jl = (lane < STEP && base + lane < n) ? labels[base + lane] : 0;
+    float4 cv[R][NV4];
+#pragma unroll
+    for (int b = 0; b < R; b++) {
+        const int64_t row = base + b * G + sub;
+        const int j = __shfl_sync(0xffffffffu, jl, b * G + sub);
+        js[b] = row < n ? j : -1;
+#pragma unroll
+        for (int u = 0; u < NV4; u++) {
+            const int cidx = cl + LPR * u;
+            const bool ok = row < n && cidx < d4;
+            xv[b][u] = cv[b][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (VEC) {
+                if (ok) xv[b][u] = reinterpret_cast<const float4*>(X + row * d)[cidx];
+                if (WD && ok) cv[b][u] = reinterpret_cast<const float4*>(C + (int64_t)j * d)[cidx];
+            } else if (ok) {
+                const float* x = X + row * d + 4 * cidx;
+                const float* c = C + (int64_t)j * d + 4 * cidx;
+                const int m = d - 4 * cidx;
+                xv[b][u] = make_float4(x[0], m > 1 ? x[1] : 0.f, m > 2 ? x[2] : 0.f, m > 3 ? x[3] : 0.f);
+                if (WD) cv[b][u] = make_float4(c[0], m > 1 ? c[1] : 0.f, m > 2 ? c[2] : 0.f, m > 3 ? c[3] : 0.f);
+            }
+        }
+    }
+    if (WD) {
+        DF part[R];
+#pragma unroll
+        for (int b = 0; b < R; b++) part[b] = df_lane<NV4>(xv[b], cv[b]);
+        int rs;
+        const DF r = df_rows<R, LPR>(part, cl, rs);
+        const int64_t row = base + rs * G + sub;
+        if ((cl & (LPR / R - 1)) == 0 && row < n) md[row] = df_value(r);
+    }
+}
+
+// k_accumulate in shared memory (the k d sums and k counts), with the winners'
+// distances (WD, rows_pass), in one launch where the bucketed path takes four.
+// Bound by the shared atomics: 1e5 x 10, k = 100 26 -> 19 us with the distances.
+// Rows of one label take turns at its addresses, so a warp adds up several of
+// them first: an update call with all rows in one of the 100 clusters took 64 us
+// without that, 31 with (54 bucketed).
+template <int NV4, int LPR, bool VEC, bool WD>
 __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X, int64_t n, int d,
                                                     const int32_t* __restrict__ labels, int k,
                                                     const unsigned* __restrict__ amax_bits, int64_t nscale,
@@ -77,56 +122,56 @@ __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X,
     constexpr int R = NV4 == 4 ? 2 : 4;
     constexpr int STEP = R * G;
     const FixedScale fx(fixed_shift(*amax_bits, nscale));
-    const int kd = SH ? k * d : 0;
-    unsigned long long* const acc = SH ? acc_rows : reinterpret_cast<unsigned long long*>(sums);
-    unsigned long long* const cacc = SH ? acc_rows + kd : reinterpret_cast<unsigned long long*>(counts);
-    if (SH) {
-        for (int e = threadIdx.x; e < kd + k; e += blockDim.x) acc_rows[e] = 0ull;
-        __syncthreads();
-    }
-    const int lane = threadIdx.x & 31, sub = lane / LPR, cl = lane % LPR;
+    const int kd = k * d;
+    unsigned long long* const cacc = acc_rows + kd;
+    for (int e = threadIdx.x; e < kd + k; e += blockDim.x) acc_rows[e] = 0ull;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, cl = lane % LPR;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int d4 = (d + 3) >> 2;
     for (int64_t base = w0 * STEP; base < n; base += nw * STEP) {
-        const int jl = (lane < STEP && base + lane < n) ? labels[base + lane] : 0;
-        float4 xv[R][NV4], cv[R][NV4];
+        float4 xv[R][NV4];
         int js[R];
+        rows_pass<NV4, LPR, VEC, WD>(X, n, d, labels, base, C, md, lane, js, xv);
+        // several rows of one label (the first row's, the last one's) are added up in
+        // registers first: shared atomics on one address take turns
+        const int lead[2] = {__shfl_sync(0xffffffffu, js[0], 0), __shfl_sync(0xffffffffu, js[R - 1], 31)};
+        unsigned same = 0;  // the rows of either, 16 bits each
 #pragma unroll
-        for (int b = 0; b < R; b++) {
-            const int64_t row = base + b * G + sub;
-            const int j = __shfl_sync(0xffffffffu, jl, b * G + sub);
-            js[b] = row < n ? j : -1;
+        for (int b = 0; b < R; b++) same += (js[b] == lead[0] ? 1u : 0u) + (js[b] == lead[1] ? 65536u : 0u);
+        same = __reduce_add_sync(0xffffffffu, cl == 0 ? same : 0u);
+        if ((same & 0xfffcfffcu) != 0u) {
+#pragma unroll 1
+            for (int h = 0; h < 2; h++) {
+                const int j = lead[h];
+                const unsigned m = h ? same >> 16 : same & 65535u;
+                if (j < 0 || m < 4 || (h && j == lead[0])) continue;
 #pragma unroll
-            for (int u = 0; u < NV4; u++) {
-                const int cidx = cl + LPR * u;
-                const bool ok = row < n && cidx < d4;
-                xv[b][u] = cv[b][u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (VEC) {
-                    if (ok) xv[b][u] = reinterpret_cast<const float4*>(X + row * d)[cidx];
-                    if (WD && ok) cv[b][u] = reinterpret_cast<const float4*>(C + (int64_t)j * d)[cidx];
-                } else if (ok) {
-                    const float* x = X + row * d + 4 * cidx;
-                    const float* c = C + (int64_t)j * d + 4 * cidx;
-                    const int m = d - 4 * cidx;
-                    xv[b][u] = make_float4(x[0], m > 1 ? x[1] : 0.f, m > 2 ? x[2] : 0.f, m > 3 ? x[3] : 0.f);
-                    if (WD) cv[b][u] = make_float4(c[0], m > 1 ? c[1] : 0.f, m > 2 ? c[2] : 0.f, m > 3 ? c[3] : 0.f);
+                for (int u = 0; u < NV4; u++) {
+                    unsigned long long v[4] = {};
+#pragma unroll
+                    for (int b = 0; b < R; b++) {
+                        const float xe[4] = {xv[b][u].x, xv[b][u].y, xv[b][u].z, xv[b][u].w};
+#pragma unroll
+                        for (int t = 0; t < 4; t++) v[t] += js[b] == j ? (unsigned long long)fx(xe[t]) : 0ull;
+                    }
+#pragma unroll
+                    for (int t = 0; t < 4; t++) {
+#pragma unroll
+                        for (int o = LPR; o < 32; o <<= 1) v[t] += __shfl_xor_sync(0xffffffffu, v[t], o);
+                        const int l = 4 * (cl + LPR * u) + t;
+                        if (lane < LPR && l < d && v[t]) atomicAdd(acc_rows + (int64_t)j * d + l, v[t]);
+                    }
                 }
-            }
-        }
-        if (WD) {
-            DF part[R];
+                if (lane == 0) atomicAdd(cacc + j, (unsigned long long)m);
 #pragma unroll
-            for (int b = 0; b < R; b++) part[b] = df_lane<NV4>(xv[b], cv[b]);
-            int rs;
-            const DF r = df_rows<R, LPR>(part, cl, rs);
-            const int64_t row = base + rs * G + sub;
-            if ((cl & (LPR / R - 1)) == 0 && row < n) md[row] = df_value(r);
+                for (int b = 0; b < R; b++) js[b] = js[b] == j ? -1 : js[b];
+            }
         }
 #pragma unroll
         for (int b = 0; b < R; b++)
             if (js[b] >= 0) {
-                unsigned long long* a = acc + (int64_t)js[b] * d;
+                unsigned long long* a = acc_rows + (int64_t)js[b] * d;
 #pragma unroll
                 for (int u = 0; u < NV4; u++) {
                     const int l = 4 * (cl + LPR * u);
@@ -138,12 +183,129 @@ __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X,
                 if (cl == 0) atomicAdd(cacc + js[b], 1ull);
             }
     }
-    if (!SH) return;
     __syncthreads();
     for (int e = threadIdx.x; e < kd; e += blockDim.x)
         if (acc_rows[e]) atomicAdd(reinterpret_cast<unsigned long long*>(sums) + e, acc_rows[e]);
     for (int e = threadIdx.x; e < k; e += blockDim.x)
         if (cacc[e]) atomicAdd(reinterpret_cast<unsigned long long*>(counts) + e, cacc[e]);
+}
+
+// The same straight to the sums in L2, whatever the labels: a block takes rb
+// rows (a power of two, 16 to AO_ROWS) into shared
+// memory, ranks them by label (each row against all) and sums them in that
+// order, a thread per coordinate and slice of the order, so that a label costs
+// one atomic per coordinate and block however many rows have it.  A run of one
+// label that goes on from slice to slice is handed along through shared memory
+// and added by the slice it ends in.
+// Bound by latency, about four dependent stages, and for many rows of few
+// coordinates by ranking and by the atomics.  An update call of 65,536 x 16 takes
+// 31 us whether the rows spread over 1024 clusters or lie in one (53 and 58 in
+// the four bucketed launches; atomics row by row, some 60 per ns on spread
+// addresses but 2 on shared ones, took 31 and 671).  256 rows a block were
+// slower (131,072 x 16, k = 4: 40 us against 34).
+constexpr int AO_ROWS = 128;       // most rows per block
+constexpr int AO_FLOATS = 8192;    // coordinates per block
+template <int NV4, int LPR, bool VEC, bool WD>
+__global__ void __launch_bounds__(256) k_accum_ordered(const float* __restrict__ X, int64_t n, int d,
+                                                       const int32_t* __restrict__ labels, int rb,
+                                                       const unsigned* __restrict__ amax_bits, int64_t nscale,
+                                                       long long* __restrict__ sums, long long* __restrict__ counts,
+                                                       const float* __restrict__ C, double* __restrict__ md) {
+    chain_enter();
+    extern __shared__ __align__(16) float ord_xs[];  // rb rows of ldx floats
+    __shared__ __align__(16) int lab[AO_ROWS];
+    __shared__ int order[AO_ROWS], slab[AO_ROWS];
+    __shared__ unsigned long long part[256];
+    constexpr int G = 32 / LPR;
+    constexpr int R = NV4 == 4 ? 2 : 4;
+    constexpr int STEP = R * G;
+    const FixedScale fx(fixed_shift(*amax_bits, nscale));
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, sub = lane / LPR, cl = lane % LPR;
+    const int d4 = (d + 3) >> 2, ldx = 4 * d4;
+    const int64_t r0 = (int64_t)blockIdx.x * rb;
+    const int rows = (int)min((int64_t)rb, n - r0);
+    if (t >= rows && t < AO_ROWS) lab[t] = 0x7fffffff;  // (past the last row: above every label)
+    for (int base = wid * STEP; base < rows; base += 8 * STEP) {
+        float4 xv[R][NV4];
+        int js[R];
+        rows_pass<NV4, LPR, VEC, WD>(X, r0 + rows, d, labels, r0 + base, C, md, lane, js, xv);
+#pragma unroll
+        for (int b = 0; b < R; b++)
+            if (js[b] >= 0) {
+                const int r = base + b * G + sub;
+#pragma unroll
+                for (int u = 0; u < NV4; u++)
+                    if (cl + LPR * u < d4) reinterpret_cast<float4*>(ord_xs + r * ldx)[cl + LPR * u] = xv[b][u];
+                if (cl == 0) lab[r] = js[b];
+            }
+    }
+    __syncthreads();
+    if (t < rows) {
+        const int my = lab[t];
+        int rank = 0, before = 0, same = 0;  // smaller labels, equal ones before this row, equal ones
+        for (int q = 0; q < rows; q += 4) {
+            const int4 o4 = *reinterpret_cast<const int4*>(lab + q);
+            const int o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                rank += o[i] < my ? 1 : 0;
+                same += o[i] == my ? 1 : 0;
+                before += o[i] == my && q + i < t ? 1 : 0;
+            }
+        }
+        order[rank + before] = t;
+        slab[rank + before] = my;
+        if (before == 0) atomicAdd(reinterpret_cast<unsigned long long*>(counts) + my, (unsigned long long)same);
+    }
+    __syncthreads();
+    const int ns = max(1, min(256 / d, (rows + 7) / 8)), per = (rows + ns - 1) / ns;  // slices, rows of a slice
+    const int s = d <= 256 ? t / d : 0, p0 = s * per, p1 = min(rows, p0 + per);
+    const bool work = s < ns && p0 < p1;
+    auto flush = [&](int j, int l, unsigned long long v) {
+        if (v) atomicAdd(reinterpret_cast<unsigned long long*>(sums) + (int64_t)j * d + l, v);
+    };
+    for (int l0 = 0; l0 < d; l0 += 256) {  // (one round up to 256 coordinates; one slice past them)
+        const int l = d <= 256 ? t - s * d : l0 + t;
+        const bool on = work && l < d;
+        bool closes = false;     // a run from an earlier slice ends in this one
+        unsigned long long acc = 0ull, first = 0ull;
+        if (on) {
+            int cur = slab[p0];
+            bool joined = p0 > 0 && slab[p0 - 1] == cur;  // the current run came from an earlier slice
+            for (int p = p0; p < p1; p++) {
+                const int j = slab[p];
+                if (j != cur) {
+                    if (joined) {
+                        first = acc;
+                        closes = true;
+                    } else {
+                        flush(cur, l, acc);
+                    }
+                    joined = false;
+                    cur = j;
+                    acc = 0ull;
+                }
+                acc += (unsigned long long)fx(ord_xs[order[p] * ldx + l]);
+            }
+            if (p1 < rows && slab[p1] == cur) {
+                part[t] = acc;  // goes on in the next slice
+            } else if (joined) {
+                first = acc;
+                closes = true;
+            } else {
+                flush(cur, l, acc);
+            }
+        }
+        if (ns > 1) __syncthreads();
+        if (closes) {
+            const int j = slab[p0];
+            for (int q = s - 1; q >= 0; q--) {
+                first += part[q * d + l];
+                if (q == 0 || slab[q * per] != j || slab[q * per - 1] != j) break;
+            }
+            flush(j, l, first);
+        }
+    }
 }
 
 // ---- bucketed reduction: rows grouped by label, summed in registers ------
@@ -152,6 +314,17 @@ __global__ void __launch_bounds__(512) k_accum_rows(const float* __restrict__ X,
 // result.
 constexpr int SEG_MAX = 512;     // most rows per warp work item (the 32-bit part sums stay exact)
 constexpr int SCAT_ROWS = 4096;  // rows per block of the histogram / scatter kernels
+
+// Rows of a work item of a bucket of cnt rows: seg, but at least 64 where the
+// bucket holds a quarter of all rows and more, whose items' sums all go to the
+// same addresses (200,000 x 32 with all rows in one of 30 clusters: 159 us a call
+// with items of 32 rows, 98 of 64; 150,001 x 256 with clusters of uneven size: 12
+// us more in items of 64 for every cluster of 2048 rows).
+KM_DEV int bucket_seg(int cnt, int64_t n, int seg) { return seg < 64 && cnt >= n / 4 ? 64 : seg; }
+KM_DEV int bucket_items(int cnt, int64_t n, int seg) {
+    const int s = bucket_seg(cnt, n, seg);
+    return (cnt + s - 1) / s;
+}
 
 // per-label counts (block histogram in shared memory, one global add per label)
 __global__ void k_label_hist(const int32_t* __restrict__ labels, int64_t n, int k, int* __restrict__ cnt32) {
@@ -168,7 +341,7 @@ __global__ void k_label_hist(const int32_t* __restrict__ labels, int64_t n, int 
 
 // Exclusive scans (one block of 1024 threads): bucket offsets, cursors, and
 // the offsets of each bucket's first work item; counts as int64.
-__global__ void k_bucket_scan(const int* __restrict__ cnt32, int k, int seg, int* __restrict__ off,
+__global__ void k_bucket_scan(const int* __restrict__ cnt32, int64_t n, int k, int seg, int* __restrict__ off,
                               int* __restrict__ cursor, int* __restrict__ item_off, long long* __restrict__ counts) {
     chain_enter();
     __shared__ int sa[1024], sb[1024];
@@ -178,7 +351,7 @@ __global__ void k_bucket_scan(const int* __restrict__ cnt32, int k, int seg, int
     int a = 0, b = 0;
     for (int j = j0; j < j1; j++) {
         a += cnt32[j];
-        b += (cnt32[j] + seg - 1) / seg;
+        b += bucket_items(cnt32[j], n, seg);
     }
     sa[t] = a;
     sb[t] = b;
@@ -197,7 +370,7 @@ __global__ void k_bucket_scan(const int* __restrict__ cnt32, int k, int seg, int
         item_off[j] = ob;
         counts[j] = cnt32[j];
         oa += cnt32[j];
-        ob += (cnt32[j] + seg - 1) / seg;
+        ob += bucket_items(cnt32[j], n, seg);
     }
     if (t == T - 1) {
         off[k] = sa[T - 1];
@@ -273,7 +446,8 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
     for (int64_t it = w0; it < nitems; it += nw) {
         const int j = bucket_of(item_off, k, it);
         const int c = (int)(it - item_off[j]);
-        const int r0 = off[j] + c * seg, r1 = min(off[j + 1], r0 + seg);
+        const int sj = bucket_seg(off[j + 1] - off[j], n, seg);
+        const int r0 = off[j] + c * sj, r1 = min(off[j + 1], r0 + sj);
         // the bucket's centre: this lane's chunks of c_j (WD)
         float4 cj[NV4];
         if (WD) {
@@ -388,7 +562,8 @@ __global__ void k_bucket_sum_small(const float* __restrict__ X, int64_t n, int k
     for (int64_t it = w0; it < nitems; it += nw) {
         const int j = bucket_of(item_off, k, it);
         const int c = (int)(it - item_off[j]);
-        const int r0 = off[j] + c * seg, r1 = min(off[j + 1], r0 + seg);
+        const int sj = bucket_seg(off[j + 1] - off[j], n, seg);
+        const int r0 = off[j] + c * sj, r1 = min(off[j + 1], r0 + sj);
         long long acc[D];
 #pragma unroll
         for (int l = 0; l < D; l++) acc[l] = 0;
@@ -1094,13 +1269,6 @@ cudaError_t launch_absmax(const float* X, int64_t count, unsigned* out_bits, cud
     return cudaGetLastError();
 }
 
-// Rows whose sums go straight to L2 (k_accum_rows without shared memory): the
-// atomics leave at some 60 per ns, so up to 2^20 of them, while the clusters are
-// many enough to spread them (2371 x 70, k = 164: 8.6 us against 37.7 us in four
-// launches; 5814 x 30, k = 310: 7.4 against 34.7 us of shared sums in four blocks;
-// but 20,000 x 100, k = 90: 37.2 against 33, 45,905 x 8, k = 216: 17.8 against 16.5).
-static bool few_rows_direct(int64_t n, int d, int k) { return n * d <= (int64_t)1 << 20 && n <= 64 * (int64_t)k && d <= 512; }
-
 cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* labels, int k,
                               const unsigned* absmax_bits, long long* sums, long long* counts, int* iscratch,
                               int32_t* perm, int num_sms, cudaStream_t st, const float* C_wd, double* md_out,
@@ -1118,7 +1286,9 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         if (e == cudaSuccess) e = cudaMemsetAsync(iscratch, 0, sizeof(int) * (size_t)k, st);
         if (e != cudaSuccess) return e;
     }
-    if (d <= 8 && (int64_t)k * d <= AS_MAX_KD && !few_rows_direct(n, d, k)) {
+    // d <= 8: few rows of many clusters go to the general forms below
+    const bool sparse = n <= 64 * (int64_t)k && n * d <= (int64_t)1 << 20;
+    if (d <= 8 && (int64_t)k * d <= AS_MAX_KD && !sparse) {
         // small d: rows in order, per-warp shared accumulators (+ C for the distances)
         const size_t sm = as_smem(d, k, want_wd);
         // about two chunks per resident warp, so that few rows still reach all SMs
@@ -1160,35 +1330,41 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
                            const float*, double*);
     const bool v4 = vec && (!want_wd || ((uintptr_t)C_wd % 16) == 0);
     const int lpr = df_lpr(d), nv4 = df_nv4(d);
-    const int rows16 = (nv4 == 4 ? 2 : 4) * (32 / lpr) * 16;  // rows of 16 warps at once
-#define KM_AR(NV, L, SH)                                                                                      \
-    if (nv4 == NV && lpr == L)                                                                                \
-        fn = v4 ? (want_wd ? (RowsFn)k_accum_rows<NV, L, true, true, SH> : (RowsFn)k_accum_rows<NV, L, true, false, SH>) \
-                : (want_wd ? (RowsFn)k_accum_rows<NV, L, false, true, SH> : (RowsFn)k_accum_rows<NV, L, false, false, SH>);
-    // few rows, and few of them per cluster: straight to the sums in L2, whose
-    // atomics (one per coordinate) spread over the addresses
-    if (few_rows_direct(n, d, k)) {
-        RowsFn fn = nullptr;
-        KM_AR(1, 8, false) KM_AR(1, 16, false) KM_AR(1, 32, false) KM_AR(2, 32, false) KM_AR(4, 32, false)
-        if (!fn) return cudaErrorInvalidValue;
-        *nlaunch = 1;
-        return klaunch(fn, (unsigned)std::max<int64_t>(1, (8 * n + rows16 - 1) / rows16), 64, 0, st, X, n, d, labels, k,
-                       absmax_bits, nscale, sums, counts, C_wd, md_out);
-    }
-    // shared-memory sums in one launch: what the bucketed path does not take, and
-    // few rows (n d <= 2^21, with at least 16 rows per cluster to pay for the
-    // blocks' folds): 1e4 x 16, k = 8 takes 9 us against 26 us in four launches;
-    // 1e5 x 128 would take 60 us of shared atomics against 51 us
-    if (smem <= 200 * 1024 && d <= 512 && (!can_bucket || (n * d <= (int64_t)1 << 21 && n >= 16 * (int64_t)k))) {
-        RowsFn fn = nullptr;
-        KM_AR(1, 8, true) KM_AR(1, 16, true) KM_AR(1, 32, true) KM_AR(2, 32, true) KM_AR(4, 32, true)
-#undef KM_AR
-        if (!fn) return cudaErrorInvalidValue;
+    // few coordinates per row and not too few clusters: shared sums, folded once per
+    // block.  An update call of 100,000 x 10, k = 100 takes 32 us, 36 in the ordered
+    // form below; 200,000 x 10, k = 200: 43 and 52.  With fewer clusters too many rows
+    // share their addresses (131,072 x 16, k = 4: 46 and 34), with more the blocks'
+    // folds weigh (131,072 x 16, k = 1000: 69 and 37).
+    if (d <= 16 && k >= 32 && k * d <= 2048 && n >= 16 * (int64_t)k && n * d <= (int64_t)1 << 21) {
+        const RowsFn fn = v4 ? (want_wd ? (RowsFn)k_accum_rows<1, 8, true, true> : (RowsFn)k_accum_rows<1, 8, true, false>)
+                             : (want_wd ? (RowsFn)k_accum_rows<1, 8, false, true> : (RowsFn)k_accum_rows<1, 8, false, false>);
         e = allow_max_smem(fn);
         if (e != cudaSuccess) return e;
-        const int64_t blk = std::min<int64_t>(std::min<int64_t>((n + rows16 - 1) / rows16, num_sms), std::max<int64_t>(1, n / (4 * (int64_t)k)));
+        const int64_t blk = std::min<int64_t>(std::min<int64_t>((n + 255) / 256, num_sms), std::max<int64_t>(1, n / (4 * (int64_t)k)));
         *nlaunch = 1;
         return klaunch(fn, (unsigned)blk, 512, smem, st, X, n, d, labels, k, absmax_bits, nscale, sums, counts, C_wd, md_out);
+    }
+    // up to 2^21 coordinates, one launch of ordered sums in place of four bucketed
+    // ones (16,384 x 64, k = 300: 30 against 47 us a call); up to 2^22 where the rows
+    // are few (8000 x 512, k = 100: 45 and 54; 60,000 x 35, k = 4000: 47 and 63; but
+    // 200,000 x 20, k = 200: 53 and 42; 400,000 x 10, k = 100: 89 and 53)
+    if (d <= 512 && (n * d <= (int64_t)1 << 21 || (n * d <= (int64_t)1 << 22 && n <= (v4 ? 1 << 15 : 1 << 16)))) {
+        RowsFn fn = nullptr;
+#define KM_AO(NV, L)                                                                                                       \
+    if (nv4 == NV && lpr == L)                                                                                             \
+        fn = v4 ? (want_wd ? (RowsFn)k_accum_ordered<NV, L, true, true> : (RowsFn)k_accum_ordered<NV, L, true, false>)     \
+                : (want_wd ? (RowsFn)k_accum_ordered<NV, L, false, true> : (RowsFn)k_accum_ordered<NV, L, false, false>);
+        KM_AO(1, 8) KM_AO(1, 16) KM_AO(1, 32) KM_AO(2, 32) KM_AO(4, 32)
+#undef KM_AO
+        if (!fn) return cudaErrorInvalidValue;
+        // as many rows per block as its shared memory takes, halved while the SMs
+        // would not all have a block
+        const int ldx = (d + 3) / 4 * 4;
+        int rb = AO_ROWS;
+        while (rb > 16 && (rb * ldx > AO_FLOATS || (n + rb - 1) / rb < num_sms)) rb >>= 1;
+        *nlaunch = 1;
+        return klaunch(fn, (unsigned)((n + rb - 1) / rb), 256, (size_t)rb * ldx * sizeof(float), st, X, n, d, labels, rb,
+                       absmax_bits, nscale, sums, counts, C_wd, md_out);
     }
     const bool bucket = can_bucket;
     // the bucket kernels of rows wider than 5 coordinates take the distances along
@@ -1231,7 +1407,7 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         }
         const int64_t resident_warps = (int64_t)num_sms * std::max(per_sm, 1) * 8;
         const int seg = (int)std::min<int64_t>(SEG_MAX, std::max<int64_t>(32, n / (resident_warps * 4) / 32 * 32));
-        klaunch(k_bucket_scan, 1, 1024, 0, st, cnt32, k, seg, off, cursor, item_off, counts);
+        klaunch(k_bucket_scan, 1, 1024, 0, st, cnt32, n, k, seg, off, cursor, item_off, counts);
         e = allow_max_smem(k_bucket_scatter);
         if (e != cudaSuccess) return e;
         klaunch(k_bucket_scatter, (unsigned)nblk, 512, 2 * hsm, st, labels, n, k, cursor, perm);

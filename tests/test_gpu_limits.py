@@ -141,3 +141,60 @@ def test_shared_scratch_span(ctx, call):
     assert all(np.array_equal(torch.as_tensor(u).cpu().numpy(), torch.as_tensor(v).cpu().numpy()) for u, v in zip(a, b))
     if call == "assign":
         check_assign(a[0].cpu().numpy()[:3000], a[1].cpu().numpy()[:3000], X[:3000], C, oracle, RTOL_MD)
+
+
+def _sums(X, lab, k, bits, n):
+    """Integer sums of the rounded fixed-point values."""
+    import math
+    amax = float(np.array([bits], dtype=np.uint32).view(np.float32)[0])
+    S = 60 - (n - 1).bit_length() - (math.frexp(amax)[1] - 1)
+    v = torch.round(X.double() * 2.0 ** (S // 2) * 2.0 ** (S - S // 2)).long()
+    return torch.zeros(k, X.shape[1], dtype=torch.int64, device="cuda").index_add_(0, lab.long(), v)
+
+
+def _labels(kind, n, k, r):
+    u = r.integers(0, k, size=n)
+    return {"spread": u, "sorted": np.sort(u), "one": np.full(n, k - 1), "two": np.where(r.random(n) < 0.5, 0, k - 1),
+            "most": np.where(r.random(n) < 0.9, k // 2, u), "runs": (np.arange(n) // 11) % k}[kind].astype(np.int32)
+
+
+# centre sums in one launch: blocks of 16 to 128 rows ordered by label and their slices (runs of one
+# label that end in, cross and fill slices, in the last block's few rows too), the shared sums with
+# several rows of a label added up first, and the bucketed sums' long segments, on both sides of
+# the dispatch's lines
+@pytest.mark.parametrize("kind", ["spread", "sorted", "one", "two", "most", "runs"])
+@pytest.mark.parametrize("n,d,k,offset", [(1, 9, 1, 0), (15, 20, 3, 0), (17, 33, 5, 1), (2447, 70, 164, 0), (19457, 24, 37, 0),
+                                          (19585, 64, 40, 1), (3000, 257, 9, 0), (1500, 512, 30, 0), (5000, 3, 700, 0),
+                                          (100003, 10, 100, 0), (100003, 20, 500, 0), (20001, 16, 128, 1), (20001, 16, 129, 0),
+                                          (30000, 130, 31, 0), (33001, 127, 20, 0), (70001, 64, 12, 0), (9000, 250, 26000, 0)])
+def test_sums_of_any_labels(ctx, n, d, k, offset, kind):
+    r = np.random.default_rng(n + d + k)
+    X = _dev(r.normal(size=(n, d)).astype(np.float32), offset)
+    lab = torch.from_numpy(_labels(kind, n, k, r)).cuda()
+    bits = ctx.absmax(X)
+    sums, counts = ctx.update_partial(X, lab, k, bits, n)
+    assert torch.equal(counts, torch.bincount(lab.long(), minlength=k))
+    assert torch.equal(sums, _sums(X, lab, k, bits, n))
+
+
+# and none of them takes much longer when most rows have one label (atomics on one address take
+# turns: up to 20 times as long, were they left to)
+@pytest.mark.parametrize("n,d,k", [(16384, 64, 300), (65536, 16, 1024), (8192, 128, 128), (100000, 10, 100), (100000, 20, 500),
+                                   (200000, 10, 1000), (20000, 10, 1000)])
+def test_sums_time_of_any_labels(ctx, n, d, k):
+    import paper_2407_12208_gb300 as pkg
+    r = np.random.default_rng(n)
+    X, p, times = _dev(r.normal(size=(n, d)).astype(np.float32)), pkg.params("fp32", empty="keep"), {}
+    for kind in ("spread", "one", "two", "most"):
+        lab = torch.from_numpy(_labels(kind, n, k, r)).cuda()
+        best = float("inf")
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                ctx.update_centroids(X, lab, X[:k], p, want_shift=False)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) / 20)
+        times[kind] = best
+    assert max(times.values()) < 1.8 * times["spread"], times
