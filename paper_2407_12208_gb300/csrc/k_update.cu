@@ -320,9 +320,10 @@ constexpr int SCAT_ROWS = 4096;  // rows per block of the histogram / scatter ke
 // same addresses (200,000 x 32 with all rows in one of 30 clusters: 159 us a call
 // with items of 32 rows, 98 of 64; 150,001 x 256 with clusters of uneven size: 12
 // us more in items of 64 for every cluster of 2048 rows).
-KM_DEV int bucket_seg(int cnt, int64_t n, int seg) { return seg < 64 && cnt >= n / 4 ? 64 : seg; }
-KM_DEV int bucket_items(int cnt, int64_t n, int seg) {
-    const int s = bucket_seg(cnt, n, seg);
+// (big: a quarter of the rows where seg is below 64, else above all counts.)
+KM_DEV int bucket_seg(int cnt, int big, int seg) { return cnt >= big ? 64 : seg; }
+KM_DEV int bucket_items(int cnt, int big, int seg) {
+    const int s = bucket_seg(cnt, big, seg);
     return (cnt + s - 1) / s;
 }
 
@@ -341,7 +342,7 @@ __global__ void k_label_hist(const int32_t* __restrict__ labels, int64_t n, int 
 
 // Exclusive scans (one block of 1024 threads): bucket offsets, cursors, and
 // the offsets of each bucket's first work item; counts as int64.
-__global__ void k_bucket_scan(const int* __restrict__ cnt32, int64_t n, int k, int seg, int* __restrict__ off,
+__global__ void k_bucket_scan(const int* __restrict__ cnt32, int k, int seg, int big, int* __restrict__ off,
                               int* __restrict__ cursor, int* __restrict__ item_off, long long* __restrict__ counts) {
     chain_enter();
     __shared__ int sa[1024], sb[1024];
@@ -351,7 +352,7 @@ __global__ void k_bucket_scan(const int* __restrict__ cnt32, int64_t n, int k, i
     int a = 0, b = 0;
     for (int j = j0; j < j1; j++) {
         a += cnt32[j];
-        b += bucket_items(cnt32[j], n, seg);
+        b += bucket_items(cnt32[j], big, seg);
     }
     sa[t] = a;
     sb[t] = b;
@@ -370,7 +371,7 @@ __global__ void k_bucket_scan(const int* __restrict__ cnt32, int64_t n, int k, i
         item_off[j] = ob;
         counts[j] = cnt32[j];
         oa += cnt32[j];
-        ob += bucket_items(cnt32[j], n, seg);
+        ob += bucket_items(cnt32[j], big, seg);
     }
     if (t == T - 1) {
         off[k] = sa[T - 1];
@@ -425,7 +426,7 @@ KM_DEV float4 load_chunk(const float* __restrict__ row, int d, int c) {
 // the assignment's min_dist costs no second read of X.
 // VEC: rows and centres are float4 (d % 4 == 0, aligned); else four loads each.
 template <int NV4, int LPR, bool WD, bool VEC>
-__global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ? 1 : 2)) k_bucket_sum(const float* __restrict__ X, int64_t n, int d, int k, int seg,
+__global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ? 1 : 2)) k_bucket_sum(const float* __restrict__ X, int d, int k, int seg, int big,
                                                        const int* __restrict__ off,
                              const int* __restrict__ item_off, const int32_t* __restrict__ perm,
                              const unsigned* __restrict__ amax_bits, int64_t nscale, long long* __restrict__ sums,
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
     for (int64_t it = w0; it < nitems; it += nw) {
         const int j = bucket_of(item_off, k, it);
         const int c = (int)(it - item_off[j]);
-        const int sj = bucket_seg(off[j + 1] - off[j], n, seg);
+        const int sj = bucket_seg(off[j + 1] - off[j], big, seg);
         const int r0 = off[j] + c * sj, r1 = min(off[j + 1], r0 + sj);
         // the bucket's centre: this lane's chunks of c_j (WD)
         float4 cj[NV4];
@@ -550,7 +551,7 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
 // Small d (d <= 16): lanes over rows, each lane sums its rows' d coordinates,
 // then a warp reduction.
 template <int D>
-__global__ void k_bucket_sum_small(const float* __restrict__ X, int64_t n, int k, int seg, const int* __restrict__ off,
+__global__ void k_bucket_sum_small(const float* __restrict__ X, int k, int seg, int big, const int* __restrict__ off,
                                    const int* __restrict__ item_off, const int32_t* __restrict__ perm,
                                    const unsigned* __restrict__ amax_bits, int64_t nscale, long long* __restrict__ sums) {
     chain_enter();
@@ -562,7 +563,7 @@ __global__ void k_bucket_sum_small(const float* __restrict__ X, int64_t n, int k
     for (int64_t it = w0; it < nitems; it += nw) {
         const int j = bucket_of(item_off, k, it);
         const int c = (int)(it - item_off[j]);
-        const int sj = bucket_seg(off[j + 1] - off[j], n, seg);
+        const int sj = bucket_seg(off[j + 1] - off[j], big, seg);
         const int r0 = off[j] + c * sj, r1 = min(off[j + 1], r0 + sj);
         long long acc[D];
 #pragma unroll
@@ -1389,7 +1390,7 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         // would leave SMs idle), the items strided over the warps; work items of
         // `seg` rows, about four per resident warp (fewer, longer items mean
         // fewer atomic adds per centre coordinate)
-        typedef void (*BucketFn)(const float*, int64_t, int, int, int, const int*, const int*, const int32_t*,
+        typedef void (*BucketFn)(const float*, int, int, int, int, const int*, const int*, const int32_t*,
                                  const unsigned*, int64_t, long long*, const float*, double*);
         BucketFn bfn = nullptr;
         if (wide) {
@@ -1407,18 +1408,19 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
         }
         const int64_t resident_warps = (int64_t)num_sms * std::max(per_sm, 1) * 8;
         const int seg = (int)std::min<int64_t>(SEG_MAX, std::max<int64_t>(32, n / (resident_warps * 4) / 32 * 32));
-        klaunch(k_bucket_scan, 1, 1024, 0, st, cnt32, n, k, seg, off, cursor, item_off, counts);
+        const int big = seg < 64 ? (int)std::max<int64_t>(1, n / 4) : INT32_MAX;
+        klaunch(k_bucket_scan, 1, 1024, 0, st, cnt32, k, seg, big, off, cursor, item_off, counts);
         e = allow_max_smem(k_bucket_scatter);
         if (e != cudaSuccess) return e;
         klaunch(k_bucket_scatter, (unsigned)nblk, 512, 2 * hsm, st, labels, n, k, cursor, perm);
         const int64_t items = n / seg + k + 1;
         const unsigned blocks =
             (unsigned)std::max<int64_t>(1, std::min<int64_t>((items * 32 + 255) / 256, (int64_t)num_sms * std::max(per_sm, 1)));
-        if (d == 1) klaunch(k_bucket_sum_small<1>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else if (d == 2) klaunch(k_bucket_sum_small<2>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else if (d == 3) klaunch(k_bucket_sum_small<3>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else if (d == 5) klaunch(k_bucket_sum_small<5>, blocks, 256, 0, st, X, n, k, seg, off, item_off, perm, absmax_bits, nscale, sums);
-        else klaunch(bfn, blocks, 256, 0, st, X, n, d, k, seg, off, item_off, perm, absmax_bits, nscale, sums, C_wd, md_out);
+        if (d == 1) klaunch(k_bucket_sum_small<1>, blocks, 256, 0, st, X, k, seg, big, off, item_off, perm, absmax_bits, nscale, sums);
+        else if (d == 2) klaunch(k_bucket_sum_small<2>, blocks, 256, 0, st, X, k, seg, big, off, item_off, perm, absmax_bits, nscale, sums);
+        else if (d == 3) klaunch(k_bucket_sum_small<3>, blocks, 256, 0, st, X, k, seg, big, off, item_off, perm, absmax_bits, nscale, sums);
+        else if (d == 5) klaunch(k_bucket_sum_small<5>, blocks, 256, 0, st, X, k, seg, big, off, item_off, perm, absmax_bits, nscale, sums);
+        else klaunch(bfn, blocks, 256, 0, st, X, d, k, seg, big, off, item_off, perm, absmax_bits, nscale, sums, C_wd, md_out);
         if (nlaunch) *nlaunch = nl + 4;
         return cudaGetLastError();
     }
