@@ -523,66 +523,156 @@ static cudaError_t launch_tiled(const float* X, int64_t n, const float* C, int k
 }
 
 // Small d (d <= 8) with C small enough to stay in shared memory for the whole
-// launch.  The argmin by the expanded formula on centred data, in fp32 with a
-// bound: x' = fl(x - mu), c' = fl(c - mu), mu the mean of up to 32 centres, and
-//   e_j = q_j + sum_l x'_l (-2 c'_jl),  q_j = ||c'_j||^2   (D fused multiply-adds).
-// |e_j - (d_j - const)| <= gamma_D (q + 2 ||x'|| ||c'||) + gamma_D q + 2.1 u (||x'||
-// + ||c'||)^2, u = 2^-24 (the sums' rounding, q's, and that of the centring), so
-// every centre that can be the nearest lies within
-//   W = (8 D + 20) u (||x'||^2 + max_j ||c'_j||^2)   (twice the bound, with slack)
-// of the smallest e.  One centre inside the window is the argmin; otherwise (few
-// rows) fp32 direct values of all centres with Theorem 4.1's certificate, and
-// binary64 for those that can still hold the minimum.  min_dist is the winner's
-// distance to binary64 accuracy (df.cuh), from the row in hand.
-// A warp takes 64 rows per step, two per lane; the rows come through a ring in
-// shared memory (16-byte asynchronous copies: D scalar loads per lane at a
-// stride of D words cost D times the wavefronts), the two in packed arithmetic.
-// 16.8 M rows x 5, k = 16: 213 us with the winners' distances (110 of them the
-// window test, 47 the double-floats, 77 the rows and results alone), where the
-// direct distances of all pairs took 193 us without them.  Bound by dependent
-// latencies (issue 60 %, FP32 pipe 45 %); two to four blocks per SM alike.
+// launch.  Two passes over the centres, both in fp32 with a bound, decide a row
+// when one centre alone can be the nearest:
+//  * direct (d <= 2, and where the other decides too little): Eq. (dist-direct),
+//    2 D operations a centre; every centre that can be the nearest has a value of
+//    at most (1 + 3 g) times the smallest (Theorem 4.1, g = gamma_{D+2}(2^-24)).
+//  * window: the expanded formula on centred data, x' = fl(x - mu), c' = fl(c -
+//    mu), mu the mean of up to 32 centres,
+//      e_j = q_j + sum_l x'_l (-2 c'_jl),  q_j = ||c'_j||^2   (D operations).
+//    |e_j - (d_j - const)| <= gamma_D (q + 2 ||x'|| ||c'||) + gamma_D q + 2.1 u (||x'||
+//    + ||c'||)^2, u = 2^-24 (the sums' rounding, q's, and that of the centring), so
+//    every centre that can be the nearest lies within
+//      W = (8 D + 20) u (||x'||^2 + max_j ||c'_j||^2)   (twice the bound, with slack)
+//    of the smallest e.  W is absolute: it leaves most rows open when the centres
+//    lie close together for their spread (k of them in 1-d: one row in seven at k =
+//    256), or when one lies far away.
+// A step whose rows the window leaves open in number is passed over directly, as
+// are the next DS_SKIP steps of the warp; a few open rows take the warp each, lanes
+// over the centres.  What the direct values leave open (near-ties) is decided in
+// binary64.  min_dist is the winner's distance to binary64 accuracy (df.cuh), from
+// the row in hand.
+// A warp takes 64 rows per step, two per lane, the centres in pairs (packed
+// arithmetic, each pair read once for both rows); the rows come through a ring in
+// shared memory (16-byte asynchronous copies: D scalar loads per lane at a stride
+// of D words cost D times the wavefronts) unless it would cost resident blocks.
+// 16.8 M rows x 5, k = 16: 202 us with the winners' distances.  1e6 rows, uniform,
+// against direct values of every centre for every row in shared memory without the
+// distances, and against a window for every row whose open rows one thread each
+// took: d = 1, k = 1024 168 us (300, 733), d = 2, k = 1024 231 (364, 546), d = 3, k =
+// 64 30 (50, 59), d = 8, k = 1024 441 (756, 1162), the same with one centre at 1e4
+// 706 (756, 2900), d = 5, k = 16 on eight pairs of equal centres 116 (11,350, 692).
+// Still slower than the first: few rows against many centres, a latency of about
+// 50 us however few the rows (20,000 x 8, k = 1024: 66 us against 54).
+// Bound by dependent latencies at few centres, else by the FP32 pipe and the
+// chunks that hold a new minimum for one of a warp's 64 rows.
 constexpr int DS_STAGES = 3;
-__host__ __device__ constexpr size_t ds_centre_bytes(int d, int k) { return (size_t)((k + 7) / 8 * 8) * (d + 1) * sizeof(float2); }
-constexpr size_t ds_smem(int d, int k, int warps) {
-    return ((ds_centre_bytes(d, k) + 15) & ~(size_t)15) + (size_t)warps * DS_STAGES * 64 * d * sizeof(float);
+constexpr int DS_SKIP = 8;  // steps without the window after one it was not worth
+__host__ __device__ constexpr bool ds_window(int d) { return d > 2; }
+// chunks of eight centres, coordinate by coordinate: the window's -2 c' and q, then c
+__host__ __device__ constexpr size_t ds_window_floats(int d, int k) { return ds_window(d) ? (size_t)((k + 7) / 8 * 8) * (d + 1) : 0; }
+__host__ __device__ constexpr size_t ds_centre_floats(int d, int k) { return ds_window_floats(d, k) + (size_t)((k + 7) / 8 * 8) * d; }
+constexpr size_t ds_smem(int d, int k, int warps, bool staged) {
+    return (ds_centre_floats(d, k) + (staged ? (size_t)warps * DS_STAGES * 64 * d : 0)) * sizeof(float);
 }
 
-// The rows that the window leaves open, by one thread.
+// A lane's two rows u (row 0, row 1) against all centres: for each row the only
+// centre that can be the nearest, -1 when there are several.  DIRECT: squared
+// distances to the chunks at cs, those up to rel times the smallest (and W) count;
+// else e, those within W of it.
+template <int D, bool DIRECT>
+KM_DEV void ds_scan(const float* cs, int kp, const float2 (&u)[D], float2 W, float rel, int& ja, int& jb) {
+    constexpr int L = DIRECT ? D : D + 1;
+    float2 u0[D], u1[D];
+#pragma unroll
+    for (int l = 0; l < D; l++) {
+        u0[l] = make_float2(u[l].x, u[l].x);
+        u1[l] = make_float2(u[l].y, u[l].y);
+    }
+    float2 b1 = make_float2(INFINITY, INFINITY);
+    ja = jb = -1;
+    for (int j0 = 0; j0 < kp; j0 += 8) {
+        const float4* cp = reinterpret_cast<const float4*>(cs + (size_t)j0 * L);
+        float2 e0[4], e1[4];  // the chunk's values, two centres each
+        if constexpr (!DIRECT) {
+            const float4 qa = cp[2 * D], qb = cp[2 * D + 1];
+            e0[0] = e1[0] = make_float2(qa.x, qa.y);
+            e0[1] = e1[1] = make_float2(qa.z, qa.w);
+            e0[2] = e1[2] = make_float2(qb.x, qb.y);
+            e0[3] = e1[3] = make_float2(qb.z, qb.w);
+        }
+#pragma unroll
+        for (int l = 0; l < D; l++) {
+            const float4 ca = cp[2 * l], cb = cp[2 * l + 1];
+            const float2 c[4] = {make_float2(ca.x, ca.y), make_float2(ca.z, ca.w), make_float2(cb.x, cb.y), make_float2(cb.z, cb.w)};
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                if constexpr (DIRECT) {
+                    const float2 t0 = fsub2(u0[l], c[i]), t1 = fsub2(u1[l], c[i]);
+                    e0[i] = l == 0 ? __fmul2_rn(t0, t0) : __ffma2_rn(t0, t0, e0[i]);
+                    e1[i] = l == 0 ? __fmul2_rn(t1, t1) : __ffma2_rn(t1, t1, e1[i]);
+                } else {
+                    e0[i] = __ffma2_rn(u0[l], c[i], e0[i]);
+                    e1[i] = __ffma2_rn(u1[l], c[i], e1[i]);
+                }
+            }
+        }
+        float2 cm;
+        cm.x = fmin3f(fmin3f(e0[0].x, e0[0].y, e0[1].x), fmin3f(e0[1].y, e0[2].x, e0[2].y), fminf(e0[3].x, e0[3].y));
+        cm.y = fmin3f(fmin3f(e1[0].x, e1[0].y, e1[1].x), fmin3f(e1[1].y, e1[2].x, e1[2].y), fminf(e1[3].x, e1[3].y));
+        const float2 r2 = make_float2(rel, rel);
+        const float2 bw = DIRECT ? __ffma2_rn(b1, r2, W) : __fadd2_rn(b1, W);
+        const bool in0 = cm.x <= bw.x, in1 = cm.y <= bw.y;  // (false where nothing is comparable)
+        if (!__any_sync(0xffffffffu, in0 || in1)) continue;
+        const float2 cw = DIRECT ? __ffma2_rn(cm, r2, W) : __fadd2_rn(cm, W);
+        const float2 thr = make_float2(fminf(bw.x, cw.x), fminf(bw.y, cw.y));
+        const float2 ta = make_float2(thr.x, thr.x), tb = make_float2(thr.y, thr.y);
+        // the signs of the values less that as masks (equality counts as outside: there is slack)
+        unsigned m0 = 0, m1 = 0;
+#pragma unroll
+        for (int i = 3; i >= 0; i--) {
+            const float2 t0 = fsub2(e0[i], ta), t1 = fsub2(e1[i], tb);
+            m0 = __funnelshift_l(__float_as_uint(t0.x), __funnelshift_l(__float_as_uint(t0.y), m0, 1), 1);
+            m1 = __funnelshift_l(__float_as_uint(t1.x), __funnelshift_l(__float_as_uint(t1.y), m1, 1), 1);
+        }
+        // strictly below what was found before and alone: the candidate; else several
+        // lie in the window (a row with none here keeps what it had)
+        if (in0) ja = cw.x < b1.x && m0 != 0u && (m0 & (m0 - 1)) == 0u ? j0 + 31 - __clz(m0) : -1;
+        if (in1) jb = cw.y < b1.y && m1 != 0u && (m1 & (m1 - 1)) == 0u ? j0 + 31 - __clz(m1) : -1;
+        b1 = make_float2(fminf(b1.x, cm.x), fminf(b1.y, cm.y));
+    }
+}
+
+// A row that is open still, by one thread; live: the lanes that call.
 template <int D>
-__device__ __noinline__ int small_open_row(const float* __restrict__ X, int64_t i, const float* __restrict__ C, int k,
-                                           float g, unsigned* amb, unsigned* ev64) {
+__device__ __noinline__ int small_open_row(unsigned live, const float* __restrict__ X, int64_t i, const float* __restrict__ C,
+                                           int k, float g, unsigned* amb, unsigned* ev64) {
     float x[D];
 #pragma unroll
     for (int l = 0; l < D; l++) x[l] = X[i * D + l];
+    auto value = [&](int j) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int l = 0; l < D; l++) {
+            const float t = x[l] - C[j * D + l];
+            acc = fmaf(t, t, acc);
+        }
+        return acc;
+    };
     float b1 = INFINITY, b2 = INFINITY;
     int j1 = 0;
     for (int j = 0; j < k; j++) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int l = 0; l < D; l++) {
-            const float t = x[l] - C[j * D + l];
-            acc = fmaf(t, t, acc);
-        }
-        if (acc < b1) {
+        const float v = value(j);
+        if (v < b1) {
             b2 = b1;
-            b1 = acc;
+            b1 = v;
             j1 = j;
-        } else if (acc < b2) {
-            b2 = acc;
+        } else if (v < b2) {
+            b2 = v;
         }
     }
     const float thr = direct_upper(b1, g, direct_tiny(D));
-    if (direct_lower(b2, g) > thr) return j1;
-    ++*amb;
+    const bool open = !(direct_lower(b2, g) > thr);
+    *amb += open ? 1u : 0u;
+    // each lane goes on to its next candidate, then the lanes evaluate theirs together
+    // (each at its own index, where almost every index is some lane's, 1e6 rows x 5 on
+    // eight pairs of equal centres took 750 us, 115 so)
     double best = INFINITY;
-    for (int j = 0; j < k; j++) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int l = 0; l < D; l++) {
-            const float t = x[l] - C[j * D + l];
-            acc = fmaf(t, t, acc);
-        }
-        if (!(direct_lower(acc, g) <= thr)) continue;
+    for (int j = open ? 0 : k;; j++) {
+        while (j < k && !(direct_lower(value(j), g) <= thr)) j++;
+        if (!__any_sync(live, j < k)) break;
+        if (j >= k) continue;
         const double s = direct64(x, C + j * D, D);
         ++*ev64;
         if (s < best) {
@@ -591,6 +681,49 @@ __device__ __noinline__ int small_open_row(const float* __restrict__ X, int64_t 
         }
     }
     return j1;
+}
+
+// The same by a warp, lanes over the centres.
+template <int D>
+__device__ __noinline__ int warp_open_row(const float* __restrict__ X, int64_t i, const float* __restrict__ C, int k, float g,
+                                          unsigned* amb, unsigned* ev64) {
+    const int lane = threadIdx.x & 31;
+    float x[D];
+#pragma unroll
+    for (int l = 0; l < D; l++) x[l] = X[i * D + l];
+    auto value = [&](int j) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int l = 0; l < D; l++) {
+            const float t = x[l] - C[j * D + l];
+            acc = fmaf(t, t, acc);
+        }
+        return acc;
+    };
+    Top2 t{INFINITY, INFINITY, 0x7fffffff};
+    for (int j = lane; j < k; j += 32) t = top2_merge(t, Top2{value(j), INFINITY, j});
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        t = top2_merge(t, Top2{__shfl_xor_sync(0xffffffffu, t.b1, off), __shfl_xor_sync(0xffffffffu, t.b2, off),
+                               __shfl_xor_sync(0xffffffffu, t.j1, off)});
+    const float thr = direct_upper(t.b1, g, direct_tiny(D));
+    if (direct_lower(t.b2, g) > thr) return t.j1;
+    *amb += lane == 0 ? 1u : 0u;
+    double best = INFINITY;
+    int arg = 0x7fffffff;
+    for (int j = lane; j < k; j += 32) {
+        if (!(direct_lower(value(j), g) <= thr)) continue;
+        const double s = direct64(x, C + j * D, D);
+        ++*ev64;
+        if (s < best) { best = s; arg = j; }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+        const int oa = __shfl_xor_sync(0xffffffffu, arg, off);
+        if (ob < best || (ob == best && oa < arg)) { best = ob; arg = oa; }
+    }
+    return arg < k ? arg : 0;  // (no value to compare, NaN: a valid label all the same)
 }
 
 template <int D, bool STAGED>
@@ -609,29 +742,40 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
     const int64_t nrows = row_list ? (int64_t)(*row_count) : n;
     if (nrows == 0) return;
     const int kp = (k + 7) / 8 * 8;
-    // a centre: D float2 of -2 c' (twice the same), then the float2 of q (+inf past k)
+    float* const cdir = dsm + ds_window_floats(D, k);
     if (threadIdx.x == 0) qmax_bits = 0u;
-    centre_mean(C, k, D, D, mu);
+    if (ds_window(D)) centre_mean(C, k, D, D, mu);
     for (int j = threadIdx.x; j < kp; j += blockDim.x) {
-        float q = j < k ? 0.0f : INFINITY;
-        float* dst = dsm + j * 2 * (D + 1);
+        float q = j < k ? 0.0f : INFINITY;  // (padding never wins)
+        float* const cw = dsm + (size_t)(j & ~7) * (D + 1) + (j & 7);
 #pragma unroll
         for (int l = 0; l < D; l++) {
-            const float c = j < k ? C[j * D + l] - mu[l] : 0.0f;
-            if (j < k) q = fmaf(c, c, q);
-            dst[2 * l] = dst[2 * l + 1] = -2.0f * c;
+            const float c0 = j < k ? C[j * D + l] : INFINITY;
+            cdir[(size_t)(j & ~7) * D + 8 * l + (j & 7)] = c0;
+            if (ds_window(D)) {
+                const float c = j < k ? c0 - mu[l] : 0.0f;
+                if (j < k) q = fmaf(c, c, q);
+                cw[8 * l] = -2.0f * c;
+            }
         }
-        dst[2 * D] = dst[2 * D + 1] = q;
-        if (j < k) atomicMax(&qmax_bits, q >= 0.0f ? __float_as_uint(q) : 0x7f800000u);
+        if (ds_window(D)) {
+            cw[8 * D] = q;
+            if (j < k) atomicMax(&qmax_bits, q >= 0.0f ? __float_as_uint(q) : 0x7f800000u);
+        }
     }
     __syncthreads();
     const float qmax = __uint_as_float(qmax_bits);
     const float wscale = (float)(8 * D + 20) * 0x1p-24f * 1.02f;
     float m[D];
 #pragma unroll
-    for (int l = 0; l < D; l++) m[l] = mu[l];
+    for (int l = 0; l < D; l++) m[l] = ds_window(D) ? mu[l] : 0.0f;
+    // the direct pass: (1 + g) / (1 - g) < 1 + 3 g with the rounding of the product
+    const float rel = 1.0f + 3.0f * gamma32, wdir = 2.0f * direct_tiny(D);
+    // open rows that cost less by the warp (instructions, about) than the direct pass
+    const int few = (int)((unsigned)k * (2 * D + 6) / ((unsigned)(k >> 5) * (3 * D + 6) + 100u));
+    int skip = 0;  // steps to take without the window
     constexpr int STEP = 64;
-    float* ring = dsm + ((ds_centre_bytes(D, k) + 15) & ~(size_t)15) / sizeof(float) + (size_t)wib * DS_STAGES * STEP * D;
+    float* ring = dsm + ds_centre_floats(D, k) + (size_t)wib * DS_STAGES * STEP * D;
     const uint32_t ring_s = smem_u32(ring);
     const int64_t w0 = (int64_t)blockIdx.x * nwb + wib, nw = (int64_t)gridDim.x * nwb;
     const int64_t nstep = (nrows + STEP - 1) / STEP;
@@ -666,7 +810,7 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
         const bool valid0 = r0 < nrows, valid1 = r0 + 32 < nrows;
         const int64_t g0 = STAGED || !row_list ? r0 : (valid0 ? row_list[r0] : 0);
         const int64_t g1 = STAGED || !row_list ? r0 + 32 : (valid1 ? row_list[r0 + 32] : 0);
-        float2 x[D], y[D], p = make_float2(0.f, 0.f);  // (row 0, row 1)
+        float2 x[D];  // (row 0, row 1)
         const float* xs0 = ring + (slot * STEP + lane) * D;
 #pragma unroll
         for (int l = 0; l < D; l++) {
@@ -677,55 +821,43 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
                 x[l] = make_float2(valid0 ? X[g0 * D + l] : 0.0f, valid1 ? X[g1 * D + l] : 0.0f);
             }
             amx = fmaxabs3(amx, x[l].x, x[l].y);
-            y[l] = fsub2(x[l], make_float2(m[l], m[l]));
-            p = __ffma2_rn(y[l], y[l], p);
         }
-        const float2 W = __ffma2_rn(make_float2(wscale, wscale), __fadd2_rn(p, make_float2(qmax, qmax)),
-                                    make_float2(0x1p-120f, 0x1p-120f));
         slot = slot + 1 == DS_STAGES ? 0 : slot + 1;
-        float2 b1 = make_float2(INFINITY, INFINITY);
-        int ja = -1, jb = -1;  // the rows' only centre inside the window so far (-1: none or several)
-        // a chunk of eight centres for one row: its smallest e, the signs of e - (that or
-        // the smallest so far + W) as a mask (equality counts as outside: W has slack)
-        for (int j0 = 0; j0 < kp; j0 += 8) {
-            const float4* cp = reinterpret_cast<const float4*>(dsm + (size_t)j0 * 2 * (D + 1));
-            float2 e[8];
+        int ja = -1, jb = -1;
+        bool direct = !ds_window(D) || skip > 0;
+        if constexpr (ds_window(D)) {
+            if (!direct) {
+                float2 y[D], p = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) {  // two centres: 2 (D + 1) float2
-                float4 c4[D + 1];
-#pragma unroll
-                for (int l = 0; l <= D; l++) c4[l] = cp[(i >> 1) * (D + 1) + l];
-                const float2* cc = reinterpret_cast<const float2*>(c4);
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    float2 a = cc[h * (D + 1) + D];
-#pragma unroll
-                    for (int l = 0; l < D; l++) a = __ffma2_rn(y[l], cc[h * (D + 1) + l], a);
-                    e[i + h] = a;
+                for (int l = 0; l < D; l++) {
+                    y[l] = fsub2(x[l], make_float2(m[l], m[l]));
+                    p = __ffma2_rn(y[l], y[l], p);
+                }
+                const float2 W = __ffma2_rn(make_float2(wscale, wscale), __fadd2_rn(p, make_float2(qmax, qmax)),
+                                            make_float2(0x1p-120f, 0x1p-120f));
+                ds_scan<D, false>(dsm, kp, y, W, 0.0f, ja, jb);
+                const unsigned o0 = __ballot_sync(0xffffffffu, valid0 && ja < 0), o1 = __ballot_sync(0xffffffffu, valid1 && jb < 0);
+                if (__popc(o0) + __popc(o1) > few) {
+                    direct = true;
+                    skip = DS_SKIP + 1;
                 }
             }
-            float2 cm;
-            cm.x = fmin3f(fmin3f(e[0].x, e[1].x, e[2].x), fmin3f(e[3].x, e[4].x, e[5].x), fminf(e[6].x, e[7].x));
-            cm.y = fmin3f(fmin3f(e[0].y, e[1].y, e[2].y), fmin3f(e[3].y, e[4].y, e[5].y), fminf(e[6].y, e[7].y));
-            const float2 bw = __fadd2_rn(b1, W), cw = __fadd2_rn(cm, W);
-            const bool in0 = cm.x <= bw.x, in1 = cm.y <= bw.y;  // (false where nothing is comparable)
-            if (!__any_sync(0xffffffffu, in0 || in1)) continue;
-            const float2 thr = make_float2(fminf(bw.x, cw.x), fminf(bw.y, cw.y));
-            unsigned m0 = 0, m1 = 0;
-#pragma unroll
-            for (int i = 7; i >= 0; i--) {
-                const float2 t = fsub2(e[i], thr);
-                m0 = __funnelshift_l(__float_as_uint(t.x), m0, 1);
-                m1 = __funnelshift_l(__float_as_uint(t.y), m1, 1);
-            }
-            // strictly below what was found before and alone: the candidate; else several
-            // lie in the window (a row with none here keeps what it had)
-            if (in0) ja = cw.x < b1.x && m0 != 0u && (m0 & (m0 - 1)) == 0u ? j0 + 31 - __clz(m0) : -1;
-            if (in1) jb = cw.y < b1.y && m1 != 0u && (m1 & (m1 - 1)) == 0u ? j0 + 31 - __clz(m1) : -1;
-            b1 = make_float2(fminf(b1.x, cm.x), fminf(b1.y, cm.y));
         }
-        if (valid0 && ja < 0) ja = small_open_row<D>(X, g0, C, k, gamma32, &local_amb, &ev64);
-        if (valid1 && jb < 0) jb = small_open_row<D>(X, g1, C, k, gamma32, &local_amb, &ev64);
+        if (direct) {
+            ds_scan<D, true>(cdir, kp, x, make_float2(wdir, wdir), rel, ja, jb);
+            skip -= skip > 0 ? 1 : 0;
+        }
+        unsigned o0 = __ballot_sync(0xffffffffu, valid0 && ja < 0), o1 = __ballot_sync(0xffffffffu, valid1 && jb < 0);
+        if (__popc(o0) + __popc(o1) > few) {
+            if ((o0 >> lane) & 1u) ja = small_open_row<D>(o0, X, g0, C, k, gamma32, &local_amb, &ev64);
+            if ((o1 >> lane) & 1u) jb = small_open_row<D>(o1, X, g1, C, k, gamma32, &local_amb, &ev64);
+        } else {
+            for (; o0 | o1; o0 ? o0 &= o0 - 1 : o1 &= o1 - 1) {
+                const int b = __ffs(o0 ? o0 : o1) - 1;
+                const int j = warp_open_row<D>(X, __shfl_sync(0xffffffffu, o0 ? g0 : g1, b), C, k, gamma32, &local_amb, &ev64);
+                if (lane == b) (o0 ? ja : jb) = j;
+            }
+        }
         const float *ca = C + (int64_t)max(ja, 0) * D, *cb = C + (int64_t)max(jb, 0) * D;
         float2 c2[D];
 #pragma unroll
@@ -765,21 +897,35 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
                                  int num_sms, cudaStream_t st, unsigned* absmax_out) {
     if (!acc64 && direct_gives_winners(d, k)) {
         // small d: C resident in shared memory, persistent grid; few rows in small
-        // blocks, so that they spread over the SMs
-        const int threads = n <= (int64_t)num_sms * 512 ? 64 : 256;
-        const size_t sm = ds_smem(d, k, threads / 32);
-        const bool staged = !row_list && ((uintptr_t)X & 15) == 0;
-        void (*fn)(const float*, int64_t, const float*, int, const int32_t*, const int*, int32_t*, double*, DevCounters*,
-                   float, unsigned*) = nullptr;
+        // blocks, so that they spread over the SMs (but not too small for the table of
+        // many centres that each block makes: 60,000 x 8, k = 1024: 114 us in blocks of
+        // 64 threads, 71 of 128; 8192 x 1, k = 8192: 187 and 175)
+        const int threads = n > (int64_t)num_sms * 512 ? 256 : (k * d <= 1024 ? 64 : 128);
+        typedef void (*SmallFn)(const float*, int64_t, const float*, int, const int32_t*, const int*, int32_t*, double*,
+                                DevCounters*, float, unsigned*);
+        SmallFn ring = nullptr, plain = nullptr;
         switch (d) {
 #define KM_SMALL(DD) \
-    case DD: fn = staged ? k_direct_small<DD, true> : k_direct_small<DD, false>; break;
+    case DD: ring = k_direct_small<DD, true>; plain = k_direct_small<DD, false>; break;
             KM_SMALL(1) KM_SMALL(2) KM_SMALL(3) KM_SMALL(4) KM_SMALL(5) KM_SMALL(6) KM_SMALL(7) KM_SMALL(8)
 #undef KM_SMALL
         }
+        SmallFn fn = plain;
+        size_t sm = ds_smem(d, k, threads / 32, false);
         cudaError_t e = allow_max_smem(fn);
         int per_sm = 1;
         if (e == cudaSuccess) e = blocks_per_sm(fn, threads, sm, &per_sm);
+        if (e == cudaSuccess && !row_list && ((uintptr_t)X & 15) == 0) {
+            const size_t sr = ds_smem(d, k, threads / 32, true);
+            int pr = 1;
+            e = allow_max_smem(ring);
+            if (e == cudaSuccess) e = blocks_per_sm(ring, threads, sr, &pr);
+            if (pr >= per_sm && sr <= (size_t)kMaxBlockSmem - 1024) {
+                fn = ring;
+                sm = sr;
+                per_sm = pr;
+            }
+        }
         if (e != cudaSuccess) return e;
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 2 * threads - 1) / (2 * threads), (int64_t)num_sms * per_sm));
         return klaunch(fn, (unsigned)grid, (unsigned)threads, sm, st, X, n, C, k, row_list, row_count, labels, min_dist, cnt,

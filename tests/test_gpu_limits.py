@@ -198,3 +198,93 @@ def test_sums_time_of_any_labels(ctx, n, d, k):
             best = min(best, a.elapsed_time(b) / 20)
         times[kind] = best
     assert max(times.values()) < 1.8 * times["spread"], times
+
+
+def _small(kind, n, d, k, r):
+    X = r.random(size=(n, d)).astype(np.float32)
+    C = X[r.permutation(n)[:k]].copy()
+    if kind == "outlier":      # one centre far away: the window of every row is wide
+        C[k // 2] = 1e4
+    elif kind == "rows":       # a few rows far away
+        X[::100] *= np.float32(1e4)
+    elif kind == "grey":       # few distinct values, ties everywhere
+        X = np.round(X * 16) / np.float32(16)
+        C = X[:k].copy()
+    elif kind == "blocks":     # warps whose rows all need more than the window, among others that do not
+        C[: k // 2] = C[0] + np.float32(1e-4) * r.random(size=(k // 2, d)).astype(np.float32)
+        X[: n // 2] = C[0]
+        X[n // 4 : n // 4 + 3] = C[k - 1]
+    return X.astype(np.float32), C.astype(np.float32)
+
+
+# small d: rows that the window test leaves open, by the warp, by the direct pass and in the steps
+# after it, and its near-ties; one and two dimensions, which take the direct pass throughout
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("kind", ["uniform", "outlier", "rows", "grey", "blocks"])
+@pytest.mark.parametrize("n,d,k", [(2, 1, 1), (64, 1, 9), (9000, 1, 300), (9001, 1, 8192), (30000, 2, 700), (5000, 2, 4096),
+                                   (129, 3, 8), (40001, 3, 16), (9000, 3, 2730), (30000, 5, 17), (20000, 8, 1024)])
+def test_small_d_open_rows(ctx, n, d, k, kind, offset):
+    import paper_2407_12208_gb300 as pkg
+    k = min(k, n)
+    X, C = _small(kind, n, d, k, np.random.default_rng(n + d + k))
+    lab, md, _ = ctx.assign(_dev(X, offset), _dev(C, offset), pkg.params("fp32"))
+    lab, md = lab.cpu().numpy(), md.cpu().numpy()
+    m = min(n, 1 + (1 << 23) // (k * d))  # (the rows that the oracle is asked about: evenly spread)
+    at = np.unique(np.linspace(0, n - 1, m).astype(np.int64))
+    check_assign(lab[at], md[at], X[at], C, oracle, RTOL_MD)
+    _, first, inverse = np.unique(C, axis=0, return_index=True, return_inverse=True)
+    assert np.array_equal(first[inverse.ravel()][lab], lab)  # the lowest index of identical centres
+
+
+def _time(f):
+    best = float("inf")
+    for _ in range(6):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            f()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / 10)
+    return best
+
+
+# and it costs little when the window decides little: many centres on a line (64 times the centres
+# of the other), one centre far away
+@pytest.mark.parametrize("d,k,kind,than,most", [(1, 1024, "uniform", (1, 16, "uniform"), 20), (2, 1024, "uniform", (2, 16, "uniform"), 22),
+                                                (8, 1024, "outlier", (8, 1024, "uniform"), 1.8),
+                                                (8, 64, "outlier", (8, 64, "uniform"), 1.8)])
+def test_small_d_time(ctx, d, k, kind, than, most):
+    r, n, times = np.random.default_rng(d), 1000000, []
+    lab = torch.empty(n, dtype=torch.int32, device="cuda")
+    md = torch.empty(n, dtype=torch.float64, device="cuda")
+    for dd, kk, kind in ((d, k, kind), than):
+        X, C = (_dev(a) for a in _small(kind, n, dd, kk, r))
+        times.append(_time(lambda: ctx.assign_static(X, C, lab, md)))
+    assert times[0] < most * times[1], times
+
+
+# rows and centres that are no numbers or infinite: the other rows' results are not touched, their
+# own labels are valid
+@pytest.mark.parametrize("low,n,d,k", [("fp32", 3000, 1, 40), ("fp32", 3000, 5, 40), ("fp32", 3000, 20, 70), ("fp32", 3000, 130, 9),
+                                       ("bf16", 3000, 32, 40), ("fp16", 3001, 33, 300), ("e4m3", 3000, 200, 40),
+                                       ("e4m3", 900, 300, 40), ("bf16", 20000, 64, 1000), ("bf16", 270000, 128, 40)])
+@pytest.mark.parametrize("centre", [False, True])
+def test_not_numbers(ctx, low, n, d, k, centre):
+    import paper_2407_12208_gb300 as pkg
+    X, C = workloads.gaussian_mixture(n, d, k, seed=n + d)
+    bad = np.arange(5, n, 97)
+    for i, v in enumerate((np.nan, np.inf, -np.inf, 3e38)):
+        X[bad[i::4], i % d] = np.float32(v)
+    X[bad[::8]] = np.float32(np.nan)
+    if centre:
+        C[k // 2] = np.float32(np.nan)
+        C[k // 3, 0] = np.float32(np.inf)
+    lab, md, _ = ctx.assign(_dev(X), _dev(C), pkg.params(low))
+    lab, md = lab.cpu().numpy(), md.cpu().numpy()
+    assert lab.min() >= 0 and lab.max() < k
+    good = np.setdiff1d(np.arange(n), bad)[:: max(1, n // 6000)]
+    fin = np.isfinite(C).all(1)
+    want = np.nonzero(fin)[0][oracle.assign(X[good], C[fin])[0]]
+    assert np.array_equal(lab[good], want)
+    np.testing.assert_allclose(md[good], oracle.dist_labelled(X[good], C, want), rtol=RTOL_MD)
