@@ -547,16 +547,14 @@ static cudaError_t launch_tiled(const float* X, int64_t n, const float* C, int k
 // arithmetic, each pair read once for both rows); the rows come through a ring in
 // shared memory (16-byte asynchronous copies: D scalar loads per lane at a stride
 // of D words cost D times the wavefronts) unless it would cost resident blocks.
-// 16.8 M rows x 5, k = 16: 202 us with the winners' distances.  1e6 rows, uniform,
-// against direct values of every centre for every row in shared memory without the
-// distances, and against a window for every row whose open rows one thread each
-// took: d = 1, k = 1024 168 us (300, 733), d = 2, k = 1024 231 (364, 546), d = 3, k =
-// 64 30 (50, 59), d = 8, k = 1024 441 (756, 1162), the same with one centre at 1e4
-// 706 (756, 2900), d = 5, k = 16 on eight pairs of equal centres 116 (11,350, 692).
-// Still slower than the first: few rows against many centres, a latency of about
-// 50 us however few the rows (20,000 x 8, k = 1024: 66 us against 54).
-// Bound by dependent latencies at few centres, else by the FP32 pipe and the
-// chunks that hold a new minimum for one of a warp's 64 rows.
+// 16.8 M rows x 5, k = 16: 201 us with the winners' distances.  1e6 rows, uniform
+// (in brackets: direct values of every centre for every row, without the distances,
+// and a window for every row whose open rows one thread each took): d = 1, k = 1024
+// 99 us (300, 733), d = 2, k = 1024 168 (364, 546), d = 3, k = 64 30 (50, 59), d = 8,
+// k = 1024 414 (756, 1162), the same with one centre at 1e4 658 (756, 2900), d = 5, k
+// = 16 on eight pairs of equal centres 116 (11,350, 692); 20,000 x 8, k = 1024 a
+// latency of 55 (54, 136).
+// Bound by dependent latencies at few centres or few rows, else by the FP32 pipe.
 constexpr int DS_STAGES = 3;
 constexpr int DS_SKIP = 8;  // steps without the window after one it was not worth
 __host__ __device__ constexpr bool ds_window(int d) { return d > 2; }
@@ -567,70 +565,113 @@ constexpr size_t ds_smem(int d, int k, int warps, bool staged) {
     return (ds_centre_floats(d, k) + (staged ? (size_t)warps * DS_STAGES * 64 * d : 0)) * sizeof(float);
 }
 
+// The values of a chunk's eight centres for NR rows, two per packed operation.
+template <int D, bool DIRECT, int NR>
+KM_DEV void ds_chunk(const float4* cp, const float2 (&u)[2][D], float2 (&e)[2][4], int r0 = 0) {
+    if constexpr (!DIRECT) {
+        const float4 qa = cp[2 * D], qb = cp[2 * D + 1];
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+            e[r][0] = make_float2(qa.x, qa.y);
+            e[r][1] = make_float2(qa.z, qa.w);
+            e[r][2] = make_float2(qb.x, qb.y);
+            e[r][3] = make_float2(qb.z, qb.w);
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < D; l++) {
+        const float4 ca = cp[2 * l], cb = cp[2 * l + 1];
+        const float2 c[4] = {make_float2(ca.x, ca.y), make_float2(ca.z, ca.w), make_float2(cb.x, cb.y), make_float2(cb.z, cb.w)};
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                const float2 x = u[NR == 1 ? r0 : r][l];
+                if constexpr (DIRECT) {
+                    const float2 t = fsub2(x, c[i]);
+                    e[r][i] = l == 0 ? __fmul2_rn(t, t) : __ffma2_rn(t, t, e[r][i]);
+                } else {
+                    e[r][i] = __ffma2_rn(x, c[i], e[r][i]);
+                }
+            }
+    }
+}
+KM_DEV float ds_least(const float2 (&e)[4]) {
+    return fmin3f(fmin3f(e[0].x, e[0].y, e[1].x), fmin3f(e[1].y, e[2].x, e[2].y), fminf(e[3].x, e[3].y));
+}
+// The signs of a chunk's values less thr as a mask (equality counts as outside:
+// there is slack; so does what is not comparable).
+KM_DEV unsigned ds_below(const float2 (&e)[4], float thr) {
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 3; i >= 0; i--) {
+        const float2 t = fsub2(e[i], make_float2(thr, thr));
+        m = __funnelshift_l(__float_as_uint(t.x), __funnelshift_l(__float_as_uint(t.y), m, 1), 1);
+    }
+    return m;
+}
+
 // A lane's two rows u (row 0, row 1) against all centres: for each row the only
 // centre that can be the nearest, -1 when there are several.  DIRECT: squared
 // distances to the chunks at cs, those up to rel times the smallest (and W) count;
 // else e, those within W of it.
-template <int D, bool DIRECT>
+// Few centres (ds_few): the chunks that hold a row's smallest value so far, or one
+// near it, are looked at at once.  MANY: most chunks would be for one of the warp's
+// 64 rows; the smallest value, its chunk and the smallest of the other chunks are
+// kept, and that one chunk is formed again at the end (1e6 rows: d = 1, k = 64 24 ->
+// 18 us, k = 1024 168 -> 100; d = 3, k = 1024 242 -> 195, but k = 64 31 -> 37; d = 7,
+// k = 100 60 -> 84).
+__host__ __device__ constexpr int ds_few(int d) { return d <= 2 ? 32 : 128; }
+template <int D, bool DIRECT, bool MANY>
 KM_DEV void ds_scan(const float* cs, int kp, const float2 (&u)[D], float2 W, float rel, int& ja, int& jb) {
     constexpr int L = DIRECT ? D : D + 1;
-    float2 u0[D], u1[D];
+    float2 uu[2][D], e[2][4];
 #pragma unroll
     for (int l = 0; l < D; l++) {
-        u0[l] = make_float2(u[l].x, u[l].x);
-        u1[l] = make_float2(u[l].y, u[l].y);
+        uu[0][l] = make_float2(u[l].x, u[l].x);
+        uu[1][l] = make_float2(u[l].y, u[l].y);
     }
+    const float2 r2 = make_float2(rel, rel);
+    auto upper = [&](float2 v) { return DIRECT ? __ffma2_rn(v, r2, W) : __fadd2_rn(v, W); };
+    auto only = [](unsigned m) { return m != 0u && (m & (m - 1)) == 0u; };
     float2 b1 = make_float2(INFINITY, INFINITY);
     ja = jb = -1;
-    for (int j0 = 0; j0 < kp; j0 += 8) {
-        const float4* cp = reinterpret_cast<const float4*>(cs + (size_t)j0 * L);
-        float2 e0[4], e1[4];  // the chunk's values, two centres each
-        if constexpr (!DIRECT) {
-            const float4 qa = cp[2 * D], qb = cp[2 * D + 1];
-            e0[0] = e1[0] = make_float2(qa.x, qa.y);
-            e0[1] = e1[1] = make_float2(qa.z, qa.w);
-            e0[2] = e1[2] = make_float2(qb.x, qb.y);
-            e0[3] = e1[3] = make_float2(qb.z, qb.w);
+    if constexpr (!MANY) {
+        for (int j0 = 0; j0 < kp; j0 += 8) {
+            const float4* cp = reinterpret_cast<const float4*>(cs + (size_t)j0 * L);
+            ds_chunk<D, DIRECT, 2>(cp, uu, e);
+            const float2 cm = make_float2(ds_least(e[0]), ds_least(e[1]));
+            const float2 bw = upper(b1);
+            const bool in0 = cm.x <= bw.x, in1 = cm.y <= bw.y;  // (false where nothing is comparable)
+            if (!__any_sync(0xffffffffu, in0 || in1)) continue;
+            const float2 cw = upper(cm);
+            const unsigned m0 = ds_below(e[0], fminf(bw.x, cw.x)), m1 = ds_below(e[1], fminf(bw.y, cw.y));
+            // strictly below what was found before and alone: the candidate; else several
+            // lie in the window (a row with none here keeps what it had)
+            if (in0) ja = cw.x < b1.x && only(m0) ? j0 + 31 - __clz(m0) : -1;
+            if (in1) jb = cw.y < b1.y && only(m1) ? j0 + 31 - __clz(m1) : -1;
+            b1 = make_float2(fminf(b1.x, cm.x), fminf(b1.y, cm.y));
         }
-#pragma unroll
-        for (int l = 0; l < D; l++) {
-            const float4 ca = cp[2 * l], cb = cp[2 * l + 1];
-            const float2 c[4] = {make_float2(ca.x, ca.y), make_float2(ca.z, ca.w), make_float2(cb.x, cb.y), make_float2(cb.z, cb.w)};
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                if constexpr (DIRECT) {
-                    const float2 t0 = fsub2(u0[l], c[i]), t1 = fsub2(u1[l], c[i]);
-                    e0[i] = l == 0 ? __fmul2_rn(t0, t0) : __ffma2_rn(t0, t0, e0[i]);
-                    e1[i] = l == 0 ? __fmul2_rn(t1, t1) : __ffma2_rn(t1, t1, e1[i]);
-                } else {
-                    e0[i] = __ffma2_rn(u0[l], c[i], e0[i]);
-                    e1[i] = __ffma2_rn(u1[l], c[i], e1[i]);
-                }
-            }
+    } else {
+        float2 b2 = b1;
+        int c0 = 0, c1 = 0;
+#pragma unroll(D <= 2 ? 2 : 1)
+        for (int j0 = 0; j0 < kp; j0 += 8) {
+            ds_chunk<D, DIRECT, 2>(reinterpret_cast<const float4*>(cs + (size_t)j0 * L), uu, e);
+            const float2 cm = make_float2(ds_least(e[0]), ds_least(e[1]));
+            // (nothing comparable in the chunk: the row stays open)
+            b2 = make_float2(fminf(b2.x, fmaxf(b1.x, cm.x)), fminf(b2.y, fmaxf(b1.y, cm.y)));
+            c0 = cm.x < b1.x ? j0 : c0;
+            c1 = cm.y < b1.y ? j0 : c1;
+            b1 = make_float2(fminf(b1.x, cm.x), fminf(b1.y, cm.y));
         }
-        float2 cm;
-        cm.x = fmin3f(fmin3f(e0[0].x, e0[0].y, e0[1].x), fmin3f(e0[1].y, e0[2].x, e0[2].y), fminf(e0[3].x, e0[3].y));
-        cm.y = fmin3f(fmin3f(e1[0].x, e1[0].y, e1[1].x), fmin3f(e1[1].y, e1[2].x, e1[2].y), fminf(e1[3].x, e1[3].y));
-        const float2 r2 = make_float2(rel, rel);
-        const float2 bw = DIRECT ? __ffma2_rn(b1, r2, W) : __fadd2_rn(b1, W);
-        const bool in0 = cm.x <= bw.x, in1 = cm.y <= bw.y;  // (false where nothing is comparable)
-        if (!__any_sync(0xffffffffu, in0 || in1)) continue;
-        const float2 cw = DIRECT ? __ffma2_rn(cm, r2, W) : __fadd2_rn(cm, W);
-        const float2 thr = make_float2(fminf(bw.x, cw.x), fminf(bw.y, cw.y));
-        const float2 ta = make_float2(thr.x, thr.x), tb = make_float2(thr.y, thr.y);
-        // the signs of the values less that as masks (equality counts as outside: there is slack)
-        unsigned m0 = 0, m1 = 0;
-#pragma unroll
-        for (int i = 3; i >= 0; i--) {
-            const float2 t0 = fsub2(e0[i], ta), t1 = fsub2(e1[i], tb);
-            m0 = __funnelshift_l(__float_as_uint(t0.x), __funnelshift_l(__float_as_uint(t0.y), m0, 1), 1);
-            m1 = __funnelshift_l(__float_as_uint(t1.x), __funnelshift_l(__float_as_uint(t1.y), m1, 1), 1);
-        }
-        // strictly below what was found before and alone: the candidate; else several
-        // lie in the window (a row with none here keeps what it had)
-        if (in0) ja = cw.x < b1.x && m0 != 0u && (m0 & (m0 - 1)) == 0u ? j0 + 31 - __clz(m0) : -1;
-        if (in1) jb = cw.y < b1.y && m1 != 0u && (m1 & (m1 - 1)) == 0u ? j0 + 31 - __clz(m1) : -1;
-        b1 = make_float2(fminf(b1.x, cm.x), fminf(b1.y, cm.y));
+        const float2 thr = upper(b1);
+        ds_chunk<D, DIRECT, 1>(reinterpret_cast<const float4*>(cs + (size_t)c0 * L), uu, e, 0);
+        const unsigned m0 = ds_below(e[0], thr.x);
+        ds_chunk<D, DIRECT, 1>(reinterpret_cast<const float4*>(cs + (size_t)c1 * L), uu, e, 1);
+        const unsigned m1 = ds_below(e[0], thr.y);
+        if (!(b2.x < thr.x) && only(m0)) ja = c0 + 31 - __clz(m0);
+        if (!(b2.y < thr.y) && only(m1)) jb = c1 + 31 - __clz(m1);
     }
 }
 
@@ -726,7 +767,7 @@ __device__ __noinline__ int warp_open_row(const float* __restrict__ X, int64_t i
     return arg < k ? arg : 0;  // (no value to compare, NaN: a valid label all the same)
 }
 
-template <int D, bool STAGED>
+template <int D, bool STAGED, bool MANY>
 __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict__ X, int64_t n,
                                                       const float* __restrict__ C, int k,
                                                       const int32_t* __restrict__ row_list,
@@ -835,7 +876,7 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
                 }
                 const float2 W = __ffma2_rn(make_float2(wscale, wscale), __fadd2_rn(p, make_float2(qmax, qmax)),
                                             make_float2(0x1p-120f, 0x1p-120f));
-                ds_scan<D, false>(dsm, kp, y, W, 0.0f, ja, jb);
+                ds_scan<D, false, MANY>(dsm, kp, y, W, 0.0f, ja, jb);
                 const unsigned o0 = __ballot_sync(0xffffffffu, valid0 && ja < 0), o1 = __ballot_sync(0xffffffffu, valid1 && jb < 0);
                 if (__popc(o0) + __popc(o1) > few) {
                     direct = true;
@@ -844,7 +885,7 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
             }
         }
         if (direct) {
-            ds_scan<D, true>(cdir, kp, x, make_float2(wdir, wdir), rel, ja, jb);
+            ds_scan<D, true, MANY>(cdir, kp, x, make_float2(wdir, wdir), rel, ja, jb);
             skip -= skip > 0 ? 1 : 0;
         }
         unsigned o0 = __ballot_sync(0xffffffffu, valid0 && ja < 0), o1 = __ballot_sync(0xffffffffu, valid1 && jb < 0);
@@ -906,7 +947,10 @@ cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const fl
         SmallFn ring = nullptr, plain = nullptr;
         switch (d) {
 #define KM_SMALL(DD) \
-    case DD: ring = k_direct_small<DD, true>; plain = k_direct_small<DD, false>; break;
+    case DD:                                                                                  \
+        ring = k > ds_few(DD) ? k_direct_small<DD, true, true> : k_direct_small<DD, true, false>;  \
+        plain = k > ds_few(DD) ? k_direct_small<DD, false, true> : k_direct_small<DD, false, false>; \
+        break;
             KM_SMALL(1) KM_SMALL(2) KM_SMALL(3) KM_SMALL(4) KM_SMALL(5) KM_SMALL(6) KM_SMALL(7) KM_SMALL(8)
 #undef KM_SMALL
         }

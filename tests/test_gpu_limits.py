@@ -222,7 +222,8 @@ def _small(kind, n, d, k, r):
 @pytest.mark.parametrize("offset", [0, 1])
 @pytest.mark.parametrize("kind", ["uniform", "outlier", "rows", "grey", "blocks"])
 @pytest.mark.parametrize("n,d,k", [(2, 1, 1), (64, 1, 9), (9000, 1, 300), (9001, 1, 8192), (30000, 2, 700), (5000, 2, 4096),
-                                   (129, 3, 8), (40001, 3, 16), (9000, 3, 2730), (30000, 5, 17), (20000, 8, 1024)])
+                                   (129, 3, 8), (40001, 3, 16), (9000, 3, 2730), (30000, 5, 17), (20000, 8, 1024),
+                                   (5000, 1, 32), (5000, 2, 33), (5001, 3, 128), (5001, 6, 129), (70, 8, 70), (700, 4, 700)])
 def test_small_d_open_rows(ctx, n, d, k, kind, offset):
     import paper_2407_12208_gb300 as pkg
     k = min(k, n)
