@@ -7,7 +7,8 @@ test, direct-formula refinement and certified argmin (labels, min_dist),
 then the centre update (Eq. (center)).  Default workload: X uniform[0,1)
 1e6 x 128 fp32, C = 1024 distinct rows of X, BF16 cross term, rho = 5.
 
-Prints one JSON line (rank 0): the device-resident step rate (`value`), the
+Prints one JSON line (rank 0), short enough for a log that keeps the last 3000
+characters; the side legs are summarised in it and printed in full on stderr: the device-resident step rate (`value`), the
 screening kernel against the measured BF16 roofline (`roofline`), the same
 step end to end from pinned host buffers through km_lloyd_step_host (`e2e`),
 the oracle on the host cores (`cpu_baseline`), the plain FP64 path on a row
@@ -407,7 +408,7 @@ def run_ours(args):
             "vs_baseline": None, "dtype": args.low, "data": "synthetic",
             "config": {"workload": args.workload + ": " + desc, "n": n, "d": d, "k": k, "low": args.low,
                        "test": "tc", "rho": 5.0, "parallelism": "replicas" if world > 1 else "single",
-                       "step": "km_lloyd_step: quantise X (+ max |x|), screen, refine, certified argmin, min_dist, exact centre update",
+                       "step": "km_lloyd_step: assignment (labels, min_dist) and centre update",
                        "l2": "inputs larger than L2 (X %d MB fp32, L2 126 MB)" % (n * d * 4 // 1000000)},
             "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": int(launches), "clocks": clocks,
             "fp64_path": fp64, "serving": serving, "table6": table6, "quality": quality, "c3_trajectory": c3, "autotune": tuned,
@@ -415,10 +416,58 @@ def run_ours(args):
             "eta": stats["flagged"] / max(stats["pairs"], 1),
             "assign_stats": {kk: stats[kk] for kk in ("fp32_evals", "fp64_evals", "ambiguous_rows", "overflow_rows")},
         }
-        print(json.dumps(line), flush=True)
+        print("details " + json.dumps({leg: line[leg] for leg in LEG_SUMMARIES}), file=sys.stderr, flush=True)
+        print(json.dumps(compact(line)), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
+
+
+def _serving_summary(leg: dict) -> dict:
+    loads = [load for load in leg if load == "saturated" or load.startswith("poisson")]
+    return {"jobs": leg["jobs"], "pairs_per_s": leg["saturated"]["pairs_per_s"],
+            "p50_p99_ms": {load: [leg[load]["p50_ms"], leg[load]["p99_ms"]] for load in loads}}
+
+
+def _table6_summary(leg: dict) -> dict:
+    """The longest times of the two mixed modes that fall back to FP64."""
+    return {mode + " ms": max(rows[mode]["ms"] for rows in leg["modes"].values()) for mode in ("FP16->FP64", "BF16->FP64")}
+
+
+def _quality_summary(leg: dict) -> dict:
+    rows = [m for part in ("blobs", "image") for m in leg[part].values()]
+    speedups = [m["FP64"]["time_s"] / m["BF16->FP64 rho=5"]["time_s"] for m in rows]
+    return {"bf16_speedup_vs_fp64": [min(speedups), max(speedups)],
+            "worst_diff_vs_fp64": max(r["diff_vs_fp64"] for m in rows for r in m.values())}
+
+
+def _fp64_summary(leg: dict) -> dict:
+    return {**leg, "ms_per_call": statistics.median(leg["ms_per_call"])}
+
+
+def _c3_summary(leg: dict) -> dict:
+    return {"time_s": {low: r["time_s"] for low, r in leg.items()},
+            "labels_equal_fp64": all(r["labels_equal_fp64"] for r in leg.values()),
+            "max_rel_sse_diff_vs_fp64": max(r["max_rel_sse_diff_vs_fp64"] for r in leg.values())}
+
+
+LEG_SUMMARIES = {"serving": _serving_summary, "table6": _table6_summary, "quality": _quality_summary,
+                 "c3_trajectory": _c3_summary, "fp64_path": _fp64_summary}
+
+
+def _short(v):
+    """v with its floats to seven digits."""
+    if isinstance(v, float):
+        return float("%.7g" % v)
+    if isinstance(v, dict):
+        return {k: _short(x) for k, x in v.items()}
+    return [_short(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def compact(line: dict) -> dict:
+    """The benchmark's line with the side legs (None: skipped, or an error) summarised."""
+    return _short({key: LEG_SUMMARIES[key](v) if key in LEG_SUMMARIES and v and "error" not in v else v
+                   for key, v in line.items()})
 
 
 TABLE6_MODES = [
