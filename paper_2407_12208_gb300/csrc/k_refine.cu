@@ -379,9 +379,11 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
 // Evaluating the warp's pairs from one flat list in shared memory instead,
 // eight at a time, was slower (1e6 x 128 listed rows 172 against 137 us,
 // 4e6 x 64 249 against 196 us: 48 registers for five blocks per SM spill).
+// (NV = 0 keeps 64 registers: given its own way the compiler took 48 and spilled,
+// 300,000 x 77 134 us against 106.)
 constexpr int RF_FEW = 12;
 template <int NV, bool LIST>
-__global__ void __launch_bounds__(256) k_refine(const int2* __restrict__ rowinfo, const float* __restrict__ roww, const uint32_t* __restrict__ cand,
+__global__ void __launch_bounds__(256, NV == 0 ? 4 : 0) k_refine(const int2* __restrict__ rowinfo, const float* __restrict__ roww, const uint32_t* __restrict__ cand,
                                                 int64_t n, int ng, int ebits, const int32_t* __restrict__ list,
                                                 const int* __restrict__ list_n, const float* __restrict__ X,
                                                 const float* __restrict__ C, int d, float gamma32,
