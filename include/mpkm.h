@@ -415,7 +415,8 @@ km_status km_get_launch_count(const km_ctx* ctx, uint64_t* launches);
  * that must not call cudaMalloc/cudaFree (cudaFree can synchronise the whole
  * device).  It takes no workspace.  Its scratch (the device counters) is a
  * file-scope device array of the library, 256 B per device.
- *  - n > KM_STATIC_MAX_ROWS returns KM_ENOMEM before any launch; the other
+ *  - n > KM_STATIC_MAX_ROWS, a limit of this call, returns KM_ENOMEM before any
+ *    launch; the other
  *    argument errors are km_assign's (d <= 256 as on every direct path).
  *  - labels (n int32) and min_dist (n doubles) are required device outputs.
  *  - On success the call allocates nothing, host or device.  A rejected call
@@ -426,8 +427,8 @@ km_status km_get_launch_count(const km_ctx* ctx, uint64_t* launches);
  *    capture begins.
  *  - Each call clears the scratch counters on `stream` before its kernels.
  *  - There is one scratch per device and process.  Calls whose work overlaps
- *    in time on one device (other streams, threads or contexts) race on it
- *    and give wrong results: order them on one stream or with events.
+ *    in time on one device (other streams, threads or contexts) mix their
+ *    counts; labels and min_dist do not depend on them.
  *  - km_get_stats and the phase timers do not report on this call. */
 #define KM_STATIC_MAX_ROWS 1048576
 km_status km_assign_static(km_ctx* ctx, const float* X, int64_t n, const float* C, int k, int d,

@@ -1616,7 +1616,8 @@ km_status km_internal_run_job(km_ctx_view* v, const float* X, int64_t n, int d, 
 // memory held by another pool, where cudaMalloc fails; loops that must not
 // pay for cudaMalloc/cudaFree, which can synchronise the device).  The
 // scratch is a file-scope device array of the counters.  There is one copy per
-// device, so calls that overlap in time on one device race on it.
+// device; calls that overlap in time mix their counts, which no result depends on
+// and nothing reads.
 namespace {
 constexpr size_t kStaticCntBytes = 256;
 static_assert(sizeof(DevCounters) <= kStaticCntBytes, "counters exceed their slot");
@@ -1694,7 +1695,7 @@ extern "C" km_status km_assign_static(km_ctx* ctx, const float* X, int64_t n, co
     if (s != KM_OK) return s;
     if (!labels || !min_dist) return fail(ctx, KM_EINVAL, "km_assign_static needs labels and min_dist");
     if (n > (int64_t)KM_STATIC_MAX_ROWS)
-        return fail(ctx, KM_ENOMEM, "km_assign_static: n=%lld exceeds its static scratch of %d rows (use km_assign)",
+        return fail(ctx, KM_ENOMEM, "km_assign_static: n=%lld exceeds the %d rows of a call on static scratch (use km_assign)",
                     (long long)n, KM_STATIC_MAX_ROWS);
     km_params p;
     km_default_params(&p);

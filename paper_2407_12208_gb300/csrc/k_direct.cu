@@ -2,13 +2,14 @@
 //
 //  * k_direct_assign<double>: the plain FP64 path (every pair in binary64).
 //  * k_direct_tiled, its general form k_direct_assign<float> and (d <= 8, few
-//    centres) k_direct_small: fp32 direct distances for the fp32 path and for rows whose tensor-core candidate list
-//    overflowed.  Theorem 4.1 bounds each value's relative error by
-//    gamma_{d+2}(2^-24); a row whose best and second-best intervals overlap is
-//    not certified and goes to
-//  * k_rows_full: the exact argmin of one row over all centres (a block per
-//    row), lowest index on ties; binary64 values with products and sums rounded
+//    centres) k_direct_small: fp32 direct distances for the fp32 path and for rows
+//    whose tensor-core candidate list overflowed.  Theorem 4.1 bounds each value's
+//    error (common.cuh); a row whose best and second-best intervals overlap is
+//    not certified and its open centres are decided in binary64 by the same block
+//    (resolve_row) or warp, lowest index on ties: products and sums rounded
 //    separately (no FMA), equal to the CPU oracle's bit for bit.
+//  * k_rows_full: the same for listed rows of more than 256 coordinates, a block
+//    per row.
 #include <algorithm>
 #include <type_traits>
 

@@ -2,7 +2,8 @@
 // line 1: x~ = fl_l(x)), and the norms the expanded formula reuses
 // (Section 3.2: p_i = x_i^T x_i "precomputed and stored").
 //
-// One warp per row.  Output per row: the quantised row (fp16 / bf16, or
+// A thread, eight lanes or a warp per row, by d, alignment and the number of rows
+// (quant_kind).  Output per row: the quantised row (fp16 / bf16, or
 // E4M3 scaled by a power of two), and stat = (p, ||x||, ||x~||, ||x~ - x||):
 //   p is ||x||^2 accumulated as an fp32 double-float (error ~2^-44) and then
 //   rounded to fp32 -- the same value as binary64 rounded to fp32 except in
@@ -167,7 +168,7 @@ KM_DEV void quantize_warp(const float* __restrict__ A, int64_t m, int d, int fmt
 // Lane l of a row's 8 holds float4 l, l + 8, ... (NV of them).  Bound by issue up
 // to 64 coordinates (50 instructions a row, of which 20 were the row's reduction
 // and square roots by itself): R rows' reductions together took 4e6 x 64 from 364
-// to 311 us (1.6 GB; 0.76 of the copy rate), 1e6 x 128 runs at 0.86 of it.
+// to 311 us (1.6 GB; 0.76 of the copy rate), 1e6 x 128 runs at 0.83 of it.
 template <int NV, bool FEW>
 KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
                         const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
@@ -267,25 +268,11 @@ KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, 
                 const float rr = qs - xv[t];
                 r2 = fmaf(rr, rr, r2);
             }
-            if (fmt == 0) {
-                __half2 h0 = __floats2half2_rn(qv[0], qv[1]), h1 = __floats2half2_rn(qv[2], qv[3]);
-                uint2 w;
-                w.x = *reinterpret_cast<uint32_t*>(&h0);
-                w.y = *reinterpret_cast<uint32_t*>(&h1);
-                reinterpret_cast<uint2*>(Aq)[i * ldq4 + c] = w;
-            } else if (fmt == 1) {
-                __nv_bfloat162 h0 = __floats2bfloat162_rn(qv[0], qv[1]), h1 = __floats2bfloat162_rn(qv[2], qv[3]);
-                uint2 w;
-                w.x = *reinterpret_cast<uint32_t*>(&h0);
-                w.y = *reinterpret_cast<uint32_t*>(&h1);
-                reinterpret_cast<uint2*>(Aq)[i * ldq4 + c] = w;
-            } else {
-                uint32_t w = 0;
+            uint32_t w = 0;
 #pragma unroll
-                for (int t = 0; t < 4; t++)
-                    w |= (uint32_t)__nv_cvt_float_to_fp8(xv[t] * inv, __NV_SATFINITE, __NV_E4M3) << (8 * t);
-                reinterpret_cast<uint32_t*>(Aq)[i * ldq4 + c] = w;
-            }
+            for (int t = 0; t < 4; t++)
+                w |= (uint32_t)__nv_cvt_float_to_fp8(xv[t] * inv, __NV_SATFINITE, __NV_E4M3) << (8 * t);
+            reinterpret_cast<uint32_t*>(Aq)[i * ldq4 + c] = w;
         }
         vh[r] = ph;
         vl[r] = pl;
@@ -343,11 +330,11 @@ KM_DEV void quantize_g8(const float* __restrict__ A, int64_t m, int d, int fmt, 
     }
 }
 
-// Vector path (d % 4 == 0, d <= 512): one warp per row, each lane holds up to
-// four float4 of the row in registers (coalesced 16-byte loads).
-template <int NV>
+// Vector path (d % 4 == 0, 256 < d <= 512): one warp per row, each lane holds up to
+// NV float4 of the row in registers (coalesced 16-byte loads).
 KM_DEV void quantize_vec(const float* __restrict__ A, int64_t m, int d, int fmt, int ldq, void* Aq,
                          const RowOut& out, float& amx, unsigned block, unsigned nblocks) {
+    constexpr int NV = 4;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)block * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)nblocks * blockDim.x) >> 5;
@@ -639,13 +626,13 @@ struct ColSide {
     unsigned* acc;  // 10 words, 0 before and after
 };
 
-// KIND: NV of quantize_g8 (1, 2, 4, 8; few rows: 9, 10), 16 + NV of
+// KIND: NV of quantize_g8 (1, 2, 4, 8; few rows: 9, 10), 16
 // quantize_vec, 0 quantize_warp, -NCH of quantize_short (2, 4, 8), 32 and 33 quantize_row.  The first cblocks blocks take the centres
 // and form their column data (q_j, +inf on the padding so padded columns never
 // win; the E4M3 scales, 1 on the padding; the column maxima, written by the
 // last of them to finish); the rest take the points.  One launch instead of three: the
 // centres' part, 5 to 9 us of latency by itself, hides behind the points'.
-constexpr int quant_blocks(int kind) { return kind == 0 ? 6 : (kind == 8 || kind == -8 ? 3 : (kind == 17 || kind == 18 ? 5 : 4)); }  // per SM
+constexpr int quant_blocks(int kind) { return kind == 0 ? 6 : (kind == 8 || kind == -8 ? 3 : 4); }  // per SM
 template <int KIND>
 __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const QuantSide x, const QuantSide c, const ColSide col, int d, int fmt,
                                                   int ldq, int cblocks, const ZeroWords zero) {
@@ -669,7 +656,7 @@ __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const Quan
     if constexpr (KIND < 0) quantize_short<-KIND>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     else if constexpr (KIND == 0) quantize_warp(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     else if constexpr (KIND < 16) quantize_g8<(KIND < 9 ? KIND : KIND - 8), (KIND > 8)>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
-    else if constexpr (KIND < 32) quantize_vec<KIND - 16>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
+    else if constexpr (KIND == 16) quantize_vec(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     else quantize_row<KIND == 32>(q.A, q.m, d, fmt, ldq, q.Aq, out, amx, block, nblocks);
     if (q.absmax) block_absmax(amx, q.absmax);
     if (!cols) return;
@@ -703,13 +690,13 @@ __global__ void __launch_bounds__(256, quant_blocks(KIND)) k_quantize(const Quan
 // The kernel form for rows at A (k_quantize's KIND).
 static int quant_kind(const float* A, const void* Aq, int d, int ldq, int64_t rows) {
     const bool vec = (d % 4 == 0) && (ldq % 4 == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)Aq % 16 == 0);
-    const int nv = (ldq / 4 + 31) / 32, nv8 = (ldq / 4 + 7) / 8;
+    const int nv8 = (ldq / 4 + 7) / 8;
     // a thread per short row once that makes a block for every SM: 6.9 against 16.8
     // us at 1e5 x 10, 5.8 against 5.2 at 1e4 x 16
     if (ldq <= 16 && (uintptr_t)Aq % 16 == 0 && rows >= 152 * 256) return vec ? 32 : 33;
     const bool few = rows <= 152 * 16 * 32;  // groups of one round (launch_quant)
     if (vec && nv8 <= 8) return nv8 <= 1 ? (few ? 9 : 1) : (nv8 <= 2 ? (few ? 10 : 2) : (nv8 <= 4 ? 4 : 8));
-    if (vec && nv <= 4) return 16 + (nv == 1 ? 1 : (nv == 2 ? 2 : 4));
+    if (vec && ldq <= 512) return 16;
     return ldq <= 64 ? -2 : (ldq <= 128 ? -4 : (ldq <= 256 ? -8 : 0));
 }
 
@@ -723,7 +710,7 @@ static cudaError_t launch_quant(int kind, const QuantSide& x, const QuantSide& c
     switch (kind) {
 #define KM_Q(K)                                                                                       \
     case K: klaunch(k_quantize<K>, (unsigned)(xb + cb), 256, 0, st, x, c, col, d, fmt, ldq, (int)cb, zero); break;
-        KM_Q(-2) KM_Q(-4) KM_Q(-8) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(9) KM_Q(10) KM_Q(17) KM_Q(18) KM_Q(20) KM_Q(32) KM_Q(33)
+        KM_Q(-2) KM_Q(-4) KM_Q(-8) KM_Q(0) KM_Q(1) KM_Q(2) KM_Q(4) KM_Q(8) KM_Q(9) KM_Q(10) KM_Q(16) KM_Q(32) KM_Q(33)
 #undef KM_Q
         default: return cudaErrorInvalidValue;
     }

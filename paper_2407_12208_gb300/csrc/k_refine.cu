@@ -14,7 +14,7 @@
 // (k_centre_rows prepares them) or the full-row kernel.
 //
 // Two forms with the same results:
-//  * k_refine: one launch, 32 rows per warp;
+//  * k_refine: one launch, 4, 8 or 32 rows per warp;
 //  * more than 64 coordinates and n d > 2^25: k_cand_select (a flat list of
 //    (row, j) pairs, each row's contiguous, from the rows' lists), k_pair_eval
 //    (8 lanes per pair, 4 pairs per warp, no per-row bookkeeping), k_certify

@@ -23,7 +23,10 @@
 //
 // What bounds it: the epilogue's instructions at three to four warps per
 // scheduler.  At 1e6 x 128 x 1024 (uniform, bf16) without any slow path 289
-// us, of which the MMA warp's chain of waits is 262 (the MMAs alone 117); the
+// us, with an epilogue that only releases its accumulators 262, and then 236 at
+// 4e6 x 64 x 256, whose tiles have half the MMAs: 1320 and 1190 cycles a tile of
+// the 411 per SM.  So that part is the tile's own (two bounded waits, a commit, an
+// accumulator's round trip), not the MMAs (117 us at the measured rate); the
 // walk over qualifying quads adds the rest, about 50 instructions an iteration
 // and a lane's worth of idle lanes.  Measured, with the row's numbers asked for
 // a block ahead (by the producer's L2 prefetch, then before the lists leave),
@@ -64,7 +67,7 @@ struct TcLayout {
 // for C32) and the shared-memory staging of the walked quads: a float4 per
 // quad and lane, quad-major, for the step's 16 quads (FULL: 8 KB per warp) or
 // 8 quads at a time (HALF, C32: 4352 bytes per warp, which also holds the
-// distance-matrix mode's 32 x 33 transposed tile); REG stages nothing (quads
+// distance-matrix mode's 32 x 32 tile, its 16-byte pieces permuted); REG stages nothing (quads
 // picked from registers).  Smaller staging leaves room for a second A stage.
 __host__ __device__ constexpr int tc_cw(int sv) { return sv == TC_SV_C32 ? 1 : 2; }
 __host__ __device__ constexpr size_t tc_stage_warp_bytes(int sv) {

@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(256, (NV4 == 1 && LPR == 32) ? 3 : (NV4 == 4 ?
     }
 }
 
-// Small d (d <= 16): lanes over rows, each lane sums its rows' d coordinates,
+// d = 1, 2, 3 or 5: lanes over rows, each lane sums its rows' d coordinates,
 // then a warp reduction.
 template <int D>
 __global__ void k_bucket_sum_small(const float* __restrict__ X, int k, int seg, int big, const int* __restrict__ off,
