@@ -59,7 +59,8 @@ def _direct_kernel_name(low: str, d: int, k: int) -> str:
     FP32 kernel for 16 <= d <= 128 with d % 4 == 0, else its general form)."""
     if low == "fp64":
         return "k_direct_assign<double>"
-    if d <= 8 and k * d * 4 <= 32 * 1024:
+    floats = (2 * d + 1 if d > 2 else d) * ((k + 7) // 8 * 8)  # its tables (for some 10,000 rows and more)
+    if d <= 8 and 4 * floats <= (128 if d > 2 else 200) * 1024:
         return "k_direct_small<%d>" % d
     if d % 4 == 0 and 16 <= d <= 128:
         return "k_direct_tiled"

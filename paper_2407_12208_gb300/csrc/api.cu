@@ -527,14 +527,14 @@ km_status zero_counters(km_ctx* ctx, DevCounters* cnt, cudaStream_t st) {
 }
 
 // Whether run_assign's min_dist has binary64 accuracy already.
-bool winners_refined(const km_params* p, int d, int k) {
-    return p->low == KM_FP64_DIRECT || (p->low == KM_FP32_DIRECT && direct_gives_winners(d, k));
+bool winners_refined(const km_params* p, int64_t n, int d, int k) {
+    return p->low == KM_FP64_DIRECT || (p->low == KM_FP32_DIRECT && direct_gives_winners(n, d, k));
 }
 
 // min_dist of the winners to binary64 accuracy.
 km_status refine_winners(km_ctx* ctx, const float* X, int64_t n, int d, const float* C, int k, const km_params* p,
                          const int32_t* labels, double* md, cudaStream_t st) {
-    if (winners_refined(p, d, k)) return KM_OK;
+    if (winners_refined(p, n, d, k)) return KM_OK;
     PhaseScope ps(ctx, KM_PHASE_REFINE, st);
     KL(1, launch_winner_dist(X, n, d, C, labels, md, ctx->num_sms, st));
     return KM_OK;
@@ -1045,7 +1045,7 @@ km_status km_lloyd_step(km_ctx* ctx, const float* X, int64_t n, int d, int k, co
     // X also refines the winners' distances (min_dist, binary64 accuracy)
     {
         PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
-        s = accumulate(ctx, X, n, d, labels, k, u, C_old, winners_refined(p, d, k) ? nullptr : md, st);
+        s = accumulate(ctx, X, n, d, labels, k, u, C_old, winners_refined(p, n, d, k) ? nullptr : md, st);
         if (s != KM_OK) return s;
         KL(1, launch_sum_f64(md, n, w.partials, kSumParts, w.sse, &w.cnt->sum_ticket, st));
         if ((s = finalize(ctx, u, n, k, d, C_old, p, X, md, C_new, counts, w.cnt, st, shift_host != nullptr)) != KM_OK)
@@ -1280,7 +1280,7 @@ static km_status lloyd_iteration(km_ctx* ctx, const float* X, int64_t n, int d, 
     if (s != KM_OK) return s;
     if (!graph) CK(cudaMemcpyAsync(flag_out, &L.a.cnt->flagged, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
     PhaseScope ps(ctx, KM_PHASE_UPDATE, st);
-    s = accumulate(ctx, X, n, d, labels, k, L.u, cur, winners_refined(p, d, k) ? nullptr : L.min_dist, st);
+    s = accumulate(ctx, X, n, d, labels, k, L.u, cur, winners_refined(p, n, d, k) ? nullptr : L.min_dist, st);
     if (s != KM_OK) return s;
     KL(1, launch_sum_f64(L.min_dist, n, L.a.partials, kSumParts, graph ? L.sse_slot : sse_out, &L.a.cnt->sum_ticket, st));
     if ((s = finalize(ctx, L.u, n, k, d, cur, p, X, L.min_dist, nxt, L.counts, L.a.cnt, st, true)) != KM_OK) return s;
@@ -1723,6 +1723,6 @@ extern "C" km_status km_assign_static(km_ctx* ctx, const float* X, int64_t n, co
     CK(cudaMemsetAsync(cnt, 0, sizeof(DevCounters), st));
     KL(1, launch_direct_assign(false, X, n, C, k, d, nullptr, nullptr, labels, min_dist, cnt, tp.gamma32, ctx->num_sms, st));
     // the winners' distances to binary64 accuracy, as km_assign (no scratch)
-    if (!winners_refined(&p, d, k)) KL(1, launch_winner_dist(X, n, d, C, labels, min_dist, ctx->num_sms, st));
+    if (!winners_refined(&p, n, d, k)) KL(1, launch_winner_dist(X, n, d, C, labels, min_dist, ctx->num_sms, st));
     return KM_OK;
 }

@@ -136,7 +136,7 @@ cudaError_t launch_predict_candidates(const float* X, int64_t n, int d, const fl
 // absmax_out (nullable, zeroed by the caller): max |x| over the rows read.
 // direct_gives_winners: whether its fp32 min_dist is already the winner's
 // distance to binary64 accuracy (launch_winner_dist's, bit for bit).
-bool direct_gives_winners(int d, int k);
+bool direct_gives_winners(int64_t n, int d, int k);
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
                                  double* min_dist, DevCounters* cnt, float gamma32,

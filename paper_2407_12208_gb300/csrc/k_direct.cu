@@ -324,7 +324,30 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
     for (int64_t base = (int64_t)blockIdx.x * R; base < nrows; base += (int64_t)gridDim.x * R) {
         const int rows_here = (int)min((int64_t)R, nrows - base);
         __syncthreads();  // the previous round's readers are done with all buffers
-        // a warp per row, lanes along it: coalesced, no index division
+        // few coordinates: the rows' floats one after another; else a warp per row, lanes
+        // along it, coalesced without an index division (100,000 x 9, k = 10: 33 us
+        // with nine of a warp's lanes, 27 so)
+        if (d < 32 && !row_list) {
+            const float* src = X + base * d;
+            const int have = rows_here * d;
+#pragma unroll 4
+            for (int e = tid * VEC; e < R * d; e += 256 * VEC) {  // (VEC divides d)
+                float v[VEC];
+#pragma unroll
+                for (int t = 0; t < VEC; t++) v[t] = 0.0f;
+                if (e < have) {
+                    if constexpr (VEC == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(src + e);
+                    else if constexpr (VEC == 2) *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(src + e);
+                    else v[0] = src[e];
+                }
+                const int r = e / d;
+#pragma unroll
+                for (int t = 0; t < VEC; t++) {
+                    amx = fmaxf(amx, fabsf(v[t]));
+                    Xs[r * ldx + e - r * d + t] = v[t];
+                }
+            }
+        } else
 #pragma unroll 2
         for (int r = wid; r < R; r += 8) {
             const bool have = r < rows_here;
@@ -931,13 +954,22 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
     }
 }
 
-bool direct_gives_winners(int d, int k) { return d <= 8 && (size_t)k * d * sizeof(float) <= 32 * 1024; }
+// The small-d kernel where the centres' tables fit in shared memory (128 KB still
+// beat the tiles with one block per SM: 1e6 x 4, k = 3600 733 us against 4495, 1e6 x
+// 1, k = 10,000 912 against 16,520: tiles of 64 centres of so few coordinates wait
+// for each other), but for few rows of seven or eight coordinates, where a warp's
+// walk over all centres takes longer than the tiles (5000 x 8, k = 1032: 51 us
+// against 34; 20,000 rows: 56 against 68).
+bool direct_gives_winners(int64_t n, int d, int k) {
+    if (d > 8 || ds_centre_floats(d, k) * sizeof(float) > (size_t)(ds_window(d) ? 128 : 200) * 1024) return false;
+    return !(d >= 7 && k * d > 8192 && n <= 9728);
+}
 
 cudaError_t launch_direct_assign(bool acc64, const float* X, int64_t n, const float* C, int k, int d,
                                  const int32_t* row_list, const int* row_count, int32_t* labels,
                                  double* min_dist, DevCounters* cnt, float gamma32,
                                  int num_sms, cudaStream_t st, unsigned* absmax_out) {
-    if (!acc64 && direct_gives_winners(d, k)) {
+    if (!acc64 && direct_gives_winners(n, d, k)) {
         // small d: C resident in shared memory, persistent grid; few rows in small
         // blocks, so that they spread over the SMs (but not too small for the table of
         // many centres that each block makes: 60,000 x 8, k = 1024: 114 us in blocks of

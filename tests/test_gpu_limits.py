@@ -223,7 +223,9 @@ def _small(kind, n, d, k, r):
 @pytest.mark.parametrize("kind", ["uniform", "outlier", "rows", "grey", "blocks"])
 @pytest.mark.parametrize("n,d,k", [(2, 1, 1), (64, 1, 9), (9000, 1, 300), (9001, 1, 8192), (30000, 2, 700), (5000, 2, 4096),
                                    (129, 3, 8), (40001, 3, 16), (9000, 3, 2730), (30000, 5, 17), (20000, 8, 1024),
-                                   (5000, 1, 32), (5000, 2, 33), (5001, 3, 128), (5001, 6, 129), (70, 8, 70), (700, 4, 700)])
+                                   (5000, 1, 32), (5000, 2, 33), (5001, 3, 128), (5001, 6, 129), (70, 8, 70), (700, 4, 700),
+                                   (9300, 1, 9100), (30000, 2, 25000), (4000, 4, 3600), (9728, 8, 1100), (9729, 8, 1100),
+                                   (2000, 7, 1300), (9729, 8, 1920), (9729, 8, 1936)])
 def test_small_d_open_rows(ctx, n, d, k, kind, offset):
     import paper_2407_12208_gb300 as pkg
     k = min(k, n)
@@ -289,3 +291,18 @@ def test_not_numbers(ctx, low, n, d, k, centre):
     want = np.nonzero(fin)[0][oracle.assign(X[good], C[fin])[0]]
     assert np.array_equal(lab[good], want)
     np.testing.assert_allclose(md[good], oracle.dist_labelled(X[good], C, want), rtol=RTOL_MD)
+
+
+# few coordinates against more centres than 32 KB hold, and rows of 9 to 31 coordinates against a
+# few centres: the time per row and centre stays near that of fewer centres and of more coordinates
+@pytest.mark.parametrize("d,k,than,most", [(1, 10000, (1, 5000), 3), (2, 5000, (2, 2500), 3), (4, 2100, (4, 1050), 3),
+                                           (9, 10, (32, 10), 1.0), (12, 8, (32, 8), 0.5)])
+def test_few_coordinates_time(ctx, d, k, than, most):
+    n, times = 500000, []
+    lab = torch.empty(n, dtype=torch.int32, device="cuda")
+    md = torch.empty(n, dtype=torch.float64, device="cuda")
+    for dd, kk in ((d, k), than):
+        X = torch.rand(n, dd, generator=torch.Generator(device="cuda").manual_seed(dd), device="cuda")
+        C = X[:kk].clone()
+        times.append(_time(lambda: ctx.assign_static(X, C, lab, md)))
+    assert times[0] < most * times[1], times
