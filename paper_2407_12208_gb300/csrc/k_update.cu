@@ -590,22 +590,28 @@ __global__ void k_bucket_sum_small(const float* __restrict__ X, int k, int seg, 
 //  * A step whose rows all have one label (an image's pixels come in long runs)
 //    adds each lane's parts to registers; they are folded over the warp when the
 //    label changes or the chunk ends.
-//  * Other steps: AS_FEW labels one after another by hardware reductions over
-//    their lanes, then, if rows are left, a segmented inclusive scan over the
-//    warp's runs of equal labels (five shuffle levels, whatever the labels) that
-//    leaves each run's total in its last lane, which adds it with a shared atomic.
-// At the end of the chunk the accumulators are folded into the global int64
-// sums.  Integer additions throughout: the order does not matter.
+//  * Other steps: up to AS_FEW labels one after another by hardware reductions
+//    over their lanes; more of them, in at most AS_RUNS runs, by a segmented
+//    inclusive scan over the runs (five shuffle levels) that leaves each run's total
+//    in its last lane, which adds it with a shared atomic; in no order, each row by
+//    its own shared atomics.
+// At the end of a chunk the block's eight accumulators are folded into the global
+// int64 sums together, k d + k atomics on addresses that all blocks share: chunks
+// as long as two blocks per SM allow.  Integer additions throughout: the order
+// does not matter.
 // NP: parts per value, 3, or 2 where the top one is always zero (from 2^22
 // rows on).  WD: each row's distance to its own centre (binary64 accuracy,
 // df.cuh) from the same read of the row, with C staged in shared memory.
-// Bound by reads of X and the labels where runs are long, else by the scan's
-// instructions (17 per row); 16.8 M rows x 5, k = 16, image: 143 us (249 us with
-// the scan in every step and D loads at a stride of D words).
+// Bound by reads of X and the labels where runs are long, else by the steps'
+// instructions; 16.8 M rows x 5, k = 16, image: 128 us (249 us with the scan in
+// every step and D loads at a stride of D words).  An update call of 409,360 x 5,
+// k = 19, labels in no order: 29 us (134 with a fold per warp and 32 rows, labels
+// by reductions first; 57 with 1024 rows per warp), 1e6 x 5, k = 16 36 (121, 60).
 constexpr int AS_CHUNK = 1024;   // rows per warp between folds (keeps each 32-bit part sum below 2^31)
 constexpr int AS_MAX_KD = 512;   // k * d bound of this path
 constexpr int AS_STAGES = 4;
 constexpr int AS_FEW = 4;
+constexpr int AS_RUNS = 8;
 static size_t as_smem(int d, int k, bool wd) {
     const size_t parts = ((size_t)8 * (3 * (size_t)k * d + k) + 3) & ~(size_t)3;
     return parts * 4 + (size_t)8 * AS_STAGES * 32 * d * 4 + (wd ? (size_t)k * 32 : 0);
@@ -639,12 +645,10 @@ __global__ void __launch_bounds__(256) k_accum_small(const float* __restrict__ X
         __syncthreads();
     }
     const bool staged = ((uintptr_t)X & 15) == 0;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t c0 = w0 * chunk; c0 < n; c0 += nw * chunk) {
+    for (int64_t cb = (int64_t)blockIdx.x * 8 * chunk; cb < n; cb += (int64_t)gridDim.x * 8 * chunk) {
         for (int e = lane; e < 3 * kd + k; e += 32) a[e] = 0u;
         __syncwarp();
-        const int64_t c1 = min(n, c0 + chunk);
+        const int64_t c0 = min(n, cb + wib * chunk), c1 = min(n, c0 + chunk);  // the warp's rows
         auto fetch = [&](int64_t base, int slot) {
             if (staged && base < c1) {
                 const char* src = reinterpret_cast<const char*>(X + base * D);
@@ -735,32 +739,43 @@ __global__ void __launch_bounds__(256) k_accum_small(const float* __restrict__ X
             // true (unbiased) parts modulo 2^32
 #pragma unroll
             for (int t = 0; t < NP * D; t++) u[t] = u[t] - FixedScale::kBias;
-            // up to AS_FEW labels one after another, each summed over its lanes by a
-            // hardware reduction; what is left by the scan
-            unsigned rem = __ballot_sync(0xffffffffu, valid);
-            int left = j;
-            for (int it = 0; it < AS_FEW && rem; it++) {
-                const int lead = __ffs(rem) - 1, jl = __shfl_sync(0xffffffffu, left, lead);
-                const unsigned m = __ballot_sync(0xffffffffu, left == jl) & rem;
-                if ((m >> lane) & 1u) {
-                    unsigned* aj = a + 3 * jl * D;
+            const unsigned vm = __ballot_sync(0xffffffffu, valid);
+            const unsigned peers = __match_any_sync(0xffffffffu, j);
+            const bool lead = valid && lane == __ffs(peers) - 1;
+            unsigned rem = __ballot_sync(0xffffffffu, lead);  // each label's first lane
+            if (__popc(rem) <= AS_FEW) {
+                // one label after another, summed over its lanes by hardware reductions
+                for (; rem; rem &= rem - 1) {
+                    const int first = __ffs(rem) - 1;
+                    const unsigned m = __shfl_sync(0xffffffffu, peers, first);
+                    if ((m >> lane) & 1u) {
+                        unsigned* aj = a + 3 * j * D;
 #pragma unroll
-                    for (int t = 0; t < NP * D; t++) {
-                        const unsigned r = __reduce_add_sync(m, u[t]);
-                        if (lane == lead) aj[3 * (t / NP) + (3 - NP) + t % NP] += r;
+                        for (int t = 0; t < NP * D; t++) {
+                            const unsigned r = __reduce_add_sync(m, u[t]);
+                            if (lane == first) aj[3 * (t / NP) + (3 - NP) + t % NP] += r;
+                        }
+                        if (lane == first) cntw[j] += (unsigned)__popc(m);
                     }
-                    if (lane == lead) cntw[jl] += (unsigned)__popc(m);
-                    left = -1;
+                    __syncwarp();
+                }
+                continue;
+            }
+            const int jp = __shfl_up_sync(0xffffffffu, j, 1);
+            const bool head = lane == 0 || j != jp;
+            if (__popc(__ballot_sync(0xffffffffu, head) & vm) > AS_RUNS) {  // each row by itself
+                if (valid) {
+                    unsigned* aj = a + 3 * j * D;
+#pragma unroll
+                    for (int t = 0; t < NP * D; t++) atomicAdd(&aj[3 * (t / NP) + (3 - NP) + t % NP], u[t]);
+                    atomicAdd(&cntw[j], 1u);
                 }
                 __syncwarp();
-                rem &= ~m;
+                continue;
             }
-            if (!rem) continue;
-            unsigned cnt = left >= 0 ? 1u : 0u;
+            unsigned cnt = valid ? 1u : 0u;
 #pragma unroll
-            for (int t = 0; t < NP * D; t++) u[t] = left >= 0 ? u[t] : 0u;
-            const int jp = __shfl_up_sync(0xffffffffu, left, 1);
-            const bool head = lane == 0 || left != jp;
+            for (int t = 0; t < NP * D; t++) u[t] = valid ? u[t] : 0u;
             bool fl = head;  // segment flag of the scan
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
@@ -779,24 +794,32 @@ __global__ void __launch_bounds__(256) k_accum_small(const float* __restrict__ X
             }
             const bool next_head = __shfl_down_sync(0xffffffffu, head, 1);
             const bool tail = lane == 31 || next_head;
-            if (left >= 0 && tail) {
-                unsigned* aj = a + 3 * left * D;
+            if (valid && tail) {
+                unsigned* aj = a + 3 * j * D;
 #pragma unroll
                 for (int t = 0; t < NP * D; t++) atomicAdd(&aj[3 * (t / NP) + (3 - NP) + t % NP], u[t]);
-                atomicAdd(&cntw[left], cnt);
+                atomicAdd(&cntw[j], cnt);
             }
             __syncwarp();
         }
         flush();
         asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncwarp();
-        for (int e = lane; e < kd; e += 32) {
-            const long long s64 = FixedScale::combine(a[3 * e + 0], a[3 * e + 1], a[3 * e + 2], 0u);
+        __syncthreads();
+        // the eight warps' sums, one atomic each: the addresses are few
+        for (int e = threadIdx.x; e < kd; e += blockDim.x) {
+            long long s64 = 0;
+            for (int w = 0; w < 8; w++) {
+                const unsigned* aw = acc_sm + (size_t)w * (3 * kd + k) + 3 * e;
+                s64 += FixedScale::combine(aw[0], aw[1], aw[2], 0u);
+            }
             if (s64) atomicAdd(reinterpret_cast<unsigned long long*>(&sums[e]), (unsigned long long)s64);
         }
-        for (int jj = lane; jj < k; jj += 32)
-            if (cntw[jj]) atomicAdd(reinterpret_cast<unsigned long long*>(&counts[jj]), (unsigned long long)cntw[jj]);
-        __syncwarp();
+        for (int jj = threadIdx.x; jj < k; jj += blockDim.x) {
+            unsigned c = 0;
+            for (int w = 0; w < 8; w++) c += acc_sm[(size_t)w * (3 * kd + k) + 3 * kd + jj];
+            if (c) atomicAdd(reinterpret_cast<unsigned long long*>(&counts[jj]), (unsigned long long)c);
+        }
+        __syncthreads();
     }
 }
 
@@ -1292,8 +1315,9 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
     if (d <= 8 && (int64_t)k * d <= AS_MAX_KD && !sparse) {
         // small d: rows in order, per-warp shared accumulators (+ C for the distances)
         const size_t sm = as_smem(d, k, want_wd);
-        // about two chunks per resident warp, so that few rows still reach all SMs
-        const int chunk = (int)std::min<int64_t>(AS_CHUNK, std::max<int64_t>(32, n / ((int64_t)num_sms * 64) / 32 * 32));
+        // about two blocks per SM, so that few rows still reach all SMs while the folds,
+        // k d + k atomics each on the same addresses, stay few
+        const int chunk = (int)std::min<int64_t>(AS_CHUNK, std::max<int64_t>(32, (n / ((int64_t)num_sms * 16) + 31) / 32 * 32));
         const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * 8, (n + 8 * chunk - 1) / (8 * chunk)));
         typedef void (*SmallFn)(const float*, int64_t, int, int, const int32_t*, const unsigned*, int64_t, long long*,
                                 long long*, const float*, double*);
@@ -1331,12 +1355,12 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
                            const float*, double*);
     const bool v4 = vec && (!want_wd || ((uintptr_t)C_wd % 16) == 0);
     const int lpr = df_lpr(d), nv4 = df_nv4(d);
-    // few coordinates per row and not too few clusters: shared sums, folded once per
-    // block.  An update call of 100,000 x 10, k = 100 takes 32 us, 36 in the ordered
+    // few coordinates per row, not too few clusters and many rows of each: shared sums,
+    // folded once per block.  An update call of 100,000 x 10, k = 100 takes 32 us, 36 in the ordered
     // form below; 200,000 x 10, k = 200: 43 and 52.  With fewer clusters too many rows
     // share their addresses (131,072 x 16, k = 4: 46 and 34), with more the blocks'
     // folds weigh (131,072 x 16, k = 1000: 69 and 37).
-    if (d <= 16 && k >= 32 && k * d <= 2048 && n >= 16 * (int64_t)k && n * d <= (int64_t)1 << 21) {
+    if (d <= 16 && k >= 32 && k * d <= 2048 && n > 64 * (int64_t)k && n * d <= (int64_t)1 << 21) {
         const RowsFn fn = v4 ? (want_wd ? (RowsFn)k_accum_rows<1, 8, true, true> : (RowsFn)k_accum_rows<1, 8, true, false>)
                              : (want_wd ? (RowsFn)k_accum_rows<1, 8, false, true> : (RowsFn)k_accum_rows<1, 8, false, false>);
         e = allow_max_smem(fn);
@@ -1407,7 +1431,10 @@ cudaError_t launch_accumulate(const float* X, int64_t n, int d, const int32_t* l
             if (e != cudaSuccess) return e;
         }
         const int64_t resident_warps = (int64_t)num_sms * std::max(per_sm, 1) * 8;
-        const int seg = (int)std::min<int64_t>(SEG_MAX, std::max<int64_t>(32, n / (resident_warps * 4) / 32 * 32));
+        // (at least 64 rows where that still makes two items per warp: 500,000 x 12, k = 20
+        // 83 us a call with items of 32 rows, 72 of 64; 100,000 x 128, k = 500 47 and 49)
+        const int64_t least = n >= 128 * resident_warps ? 64 : 32;
+        const int seg = (int)std::min<int64_t>(SEG_MAX, std::max<int64_t>(least, n / (resident_warps * 4) / 32 * 32));
         const int big = seg < 64 ? (int)std::max<int64_t>(1, n / 4) : INT32_MAX;
         klaunch(k_bucket_scan, 1, 1024, 0, st, cnt32, k, seg, big, off, cursor, item_off, counts);
         e = allow_max_smem(k_bucket_scatter);

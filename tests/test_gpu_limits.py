@@ -306,3 +306,31 @@ def test_few_coordinates_time(ctx, d, k, than, most):
         C = X[:kk].clone()
         times.append(_time(lambda: ctx.assign_static(X, C, lab, md)))
     assert times[0] < most * times[1], times
+
+
+# small-d centre sums: chunks of 32 rows and more per warp, eight warps folded together, in the last
+# block too; steps of one label, a few, many in runs and in no order
+@pytest.mark.parametrize("kind", ["spread", "sorted", "one", "two", "most", "runs"])
+@pytest.mark.parametrize("n,d,k,offset", [(257, 1, 1, 0), (600, 8, 3, 0), (8191, 3, 7, 1), (77825, 5, 16, 0), (311301, 2, 256, 0),
+                                          (311299, 8, 64, 1), (2600000, 4, 100, 0)])
+def test_small_d_sums_of_any_labels(ctx, n, d, k, offset, kind):
+    r = np.random.default_rng(n + d + k)
+    X = torch.randn(n + offset, d, generator=torch.Generator(device="cuda").manual_seed(n), device="cuda").view(-1)[offset : offset + n * d].view(n, d)
+    lab = torch.from_numpy(_labels(kind, n, k, r)).cuda()
+    bits = ctx.absmax(X)
+    sums, counts = ctx.update_partial(X, lab, k, bits, n)
+    assert torch.equal(counts, torch.bincount(lab.long(), minlength=k))
+    assert torch.equal(sums, _sums(X, lab, k, bits, n))
+
+
+# and their time does not grow when no two neighbours share a label (folds of few rows each on the same
+# few addresses took four times as long as the rows)
+@pytest.mark.parametrize("n,d,k", [(409360, 5, 19), (1000000, 2, 256)])
+def test_small_d_sums_time(ctx, n, d, k):
+    import paper_2407_12208_gb300 as pkg
+    p, times = pkg.params("fp32", empty="keep"), []
+    X = torch.rand(n, d, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    for kind in ("spread", "sorted"):
+        lab = torch.from_numpy(_labels(kind, n, k, np.random.default_rng(3))).cuda()
+        times.append(_time(lambda: ctx.update_centroids(X, lab, X[:k], p, want_shift=False)))
+    assert times[0] < 1.8 * times[1], times
