@@ -260,6 +260,122 @@ __device__ __noinline__ bool resolve_row(const float* __restrict__ X, const floa
     return true;
 }
 
+// The same by one warp for a row whose smallest fp32 value is known: thr =
+// direct_upper of it.  Every centre whose interval reaches down to thr is evaluated
+// in binary64, up to four at a time (their products by all lanes, a lane each adds
+// one's in order).  scratch: the warp's `bytes` of shared memory, 16-byte aligned,
+// at least rw_bytes(d, 1).
+constexpr int RW_LIST = 32;  // candidates per evaluation
+__host__ __device__ constexpr size_t rw_bytes(int d, int batch) {
+    return (size_t)batch * d * sizeof(double) + ((size_t)d + RW_LIST) * sizeof(float);
+}
+__device__ __noinline__ void warp_resolve_row(const float* __restrict__ X, const float* __restrict__ C, int k, int d, int64_t i,
+                                              float thr, float gamma32, int32_t* __restrict__ labels,
+                                              double* __restrict__ min_dist, void* scratch, size_t bytes,
+                                              unsigned long long* ev64) {
+    const int lane = threadIdx.x & 31;
+    const int batch = bytes >= rw_bytes(d, 4) ? 4 : (bytes >= rw_bytes(d, 2) ? 2 : 1);
+    double* prod = reinterpret_cast<double*>(scratch);                  // batch x d products
+    float* xs = reinterpret_cast<float*>(prod + (size_t)batch * d);     // d
+    int* js = reinterpret_cast<int*>(xs + d);                           // RW_LIST
+    __syncwarp();
+    for (int l = lane; l < d; l += 32) xs[l] = X[i * d + l];
+    __syncwarp();
+    double best = INFINITY;
+    int arg = 0x7fffffff, cnt = 0;
+    auto evaluate = [&]() {
+        __syncwarp();
+        for (int b0 = 0; b0 < cnt; b0 += batch) {
+            const int nb = min(batch, cnt - b0);
+            for (int b = 0; b < nb; b++) {
+                const float* c = C + (int64_t)js[b0 + b] * d;
+                for (int l = lane; l < d; l += 32) {
+                    const double u = __dsub_rn((double)xs[l], (double)c[l]);
+                    prod[b * d + l] = __dmul_rn(u, u);
+                }
+            }
+            __syncwarp();
+            if (lane < nb) {
+                const int j = js[b0 + lane];
+                double t = 0.0;
+#pragma unroll 8
+                for (int l = 0; l < d; l++) t = __dadd_rn(t, prod[lane * d + l]);
+                if (t < best || (t == best && j < arg)) { best = t; arg = j; }
+                ++*ev64;
+            }
+            __syncwarp();
+        }
+        cnt = 0;
+    };
+    if (d < 32) {  // a centre per lane
+        const bool vec = d % 4 == 0 && ((uintptr_t)C & 15) == 0;
+        for (int j0 = 0; j0 < k; j0 += 32) {
+            const int j = j0 + lane;
+            float v = 0.0f;
+            if (j < k && vec) {
+                const float4* c4 = reinterpret_cast<const float4*>(C + (int64_t)j * d);
+                for (int l = 0; l < d; l += 4) {
+                    const float4 c = c4[l >> 2];
+                    const float t0 = xs[l] - c.x, t1 = xs[l + 1] - c.y, t2 = xs[l + 2] - c.z, t3 = xs[l + 3] - c.w;
+                    v = fmaf(t0, t0, v);
+                    v = fmaf(t1, t1, v);
+                    v = fmaf(t2, t2, v);
+                    v = fmaf(t3, t3, v);
+                }
+            } else if (j < k) {
+                for (int l = 0; l < d; l++) {
+                    const float t = xs[l] - C[(int64_t)j * d + l];
+                    v = fmaf(t, t, v);
+                }
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, j < k && direct_lower(v, gamma32) <= thr);
+            if (!m) continue;
+            if ((m >> lane) & 1u) js[__popc(m & ((1u << lane) - 1u))] = j;
+            cnt = __popc(m);
+            evaluate();
+        }
+    } else {
+        for (int j0 = 0; j0 < k; j0 += 4) {
+            float v[4];
+            warp_direct4(xs, C, k, d, j0, lane, v);
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (j0 + q < k && direct_lower(v[q], gamma32) <= thr) {
+                    if (lane == 0) js[cnt] = j0 + q;
+                    cnt++;
+                }
+            if (cnt > RW_LIST - 4) evaluate();
+        }
+        evaluate();
+    }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {  // (four lanes at most have evaluated)
+        const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+        const int oa = __shfl_xor_sync(0xffffffffu, arg, off);
+        if (ob < best || (ob == best && oa < arg)) { best = ob; arg = oa; }
+    }
+    if (lane == 0) {
+        labels[i] = arg < k ? arg : 0;  // (no value to compare, NaN: a valid label all the same)
+        min_dist[i] = best;
+    }
+}
+
+// A block's open rows: a warp each, eight at a time; the block, quicker on a row by
+// itself (its warps share the centres and the binary64 sums), takes a small rest in
+// turn (146,112 x 256, k = 9, an open row in most blocks: 170 us so, 193 by a warp).
+// scratch: resolve_bytes(d) at least, and 8 (rw_bytes(d, 1) + 16).
+__device__ __noinline__ void resolve_open(const float* __restrict__ X, const float* __restrict__ C, int k, int d,
+                                          const int* rows, const float* thr, int no, float gamma32,
+                                          int32_t* __restrict__ labels, double* __restrict__ min_dist, void* scratch,
+                                          size_t bytes, unsigned long long* ev64) {
+    const int wid = threadIdx.x >> 5;
+    const int byw = no % 8 > (k <= 64 ? 2 : 5) ? no : no & ~7;
+    const size_t per = bytes / 8 & ~(size_t)15;
+    for (int o = wid; o < byw; o += 8)
+        warp_resolve_row(X, C, k, d, rows[o], thr[o], gamma32, labels, min_dist, static_cast<char*>(scratch) + wid * per, per, ev64);
+    for (int o = byw; o < no; o++) resolve_row(X, C, k, d, rows[o], gamma32, labels, min_dist, scratch, bytes, ev64);
+}
+
 // Tiled fp32 direct distances, Eq. (dist-direct), any d (rows whose candidate
 // list overflowed, the fp32 direct path, km_assign_static): 32 RPT rows per
 // round resident in shared memory (zero-padded to a multiple of 4
@@ -315,6 +431,7 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
     const int ntile = (k + DT_C - 1) / DT_C, nck = (dp + DT_DK - 1) / DT_DK, nstep = ntile * nck;
     const float g = gamma32;
     __shared__ int open_rows[R], nopen;
+    __shared__ float open_thr[R];
     float amx = 0.0f;
     unsigned long long local_amb = 0, ev64 = 0;
     if (tid == 0) nopen = 0;
@@ -474,17 +591,19 @@ KM_DEV void direct_tiled(const float* __restrict__ X, int64_t n, const float* __
                     const int64_t gi = row_list ? (int64_t)row_list[base + r] : base + r;
                     labels[gi] = j1[i];
                     min_dist[gi] = (double)b1[i];
-                    if (!(direct_lower(b2[i], g) > direct_upper(b1[i], g, direct_tiny(d)))) {  // (Theorem 4.1)
-                        open_rows[atomicAdd(&nopen, 1)] = (int)gi;
+                    const float thr = direct_upper(b1[i], g, direct_tiny(d));
+                    if (!(direct_lower(b2[i], g) > thr)) {  // (Theorem 4.1)
+                        const int o = atomicAdd(&nopen, 1);
+                        open_rows[o] = (int)gi;
+                        open_thr[o] = thr;
                         local_amb++;
                     }
                 }
             }
         __syncthreads();
         if (const int no = nopen) {
-            // (the centre buffers are free: 512 ldc bytes, resolve_bytes(d) at most 68 d of them)
-            for (int o = 0; o < no; o++)
-                resolve_row(X, C, k, d, open_rows[o], g, labels, min_dist, Cs, (size_t)2 * DT_C * ldc * sizeof(float), &ev64);
+            // (the centre buffers are free)
+            resolve_open(X, C, k, d, open_rows, open_thr, no, g, labels, min_dist, Cs, (size_t)2 * DT_C * ldc * sizeof(float), &ev64);
             __syncthreads();
             if (tid == 0) {
                 nopen = 0;
@@ -636,8 +755,8 @@ KM_DEV unsigned ds_below(const float2 (&e)[4], float thr) {
 }
 
 // A lane's two rows u (row 0, row 1) against all centres: for each row the only
-// centre that can be the nearest, -1 when there are several.  DIRECT: squared
-// distances to the chunks at cs, those up to rel times the smallest (and W) count;
+// centre that can be the nearest, -1 when there are several; b1: their smallest
+// values.  DIRECT: squared distances to the chunks at cs, those up to rel times the smallest (and W) count;
 // else e, those within W of it.
 // Few centres (ds_few): the chunks that hold a row's smallest value so far, or one
 // near it, are looked at at once.  MANY: most chunks would be for one of the warp's
@@ -647,7 +766,7 @@ KM_DEV unsigned ds_below(const float2 (&e)[4], float thr) {
 // k = 100 60 -> 84).
 __host__ __device__ constexpr int ds_few(int d) { return d <= 2 ? 32 : 128; }
 template <int D, bool DIRECT, bool MANY>
-KM_DEV void ds_scan(const float* cs, int kp, const float2 (&u)[D], float2 W, float rel, int& ja, int& jb) {
+KM_DEV void ds_scan(const float* cs, int kp, const float2 (&u)[D], float2 W, float rel, int& ja, int& jb, float2& b1) {
     constexpr int L = DIRECT ? D : D + 1;
     float2 uu[2][D], e[2][4];
 #pragma unroll
@@ -658,7 +777,7 @@ KM_DEV void ds_scan(const float* cs, int kp, const float2 (&u)[D], float2 W, flo
     const float2 r2 = make_float2(rel, rel);
     auto upper = [&](float2 v) { return DIRECT ? __ffma2_rn(v, r2, W) : __fadd2_rn(v, W); };
     auto only = [](unsigned m) { return m != 0u && (m & (m - 1)) == 0u; };
-    float2 b1 = make_float2(INFINITY, INFINITY);
+    b1 = make_float2(INFINITY, INFINITY);
     ja = jb = -1;
     if constexpr (!MANY) {
         for (int j0 = 0; j0 < kp; j0 += 8) {
@@ -699,10 +818,11 @@ KM_DEV void ds_scan(const float* cs, int kp, const float2 (&u)[D], float2 W, flo
     }
 }
 
-// A row that is open still, by one thread; live: the lanes that call.
+// A row that the direct values leave open, by one thread: binary64 for every centre
+// whose interval reaches down to thr.  live: the lanes that call.
 template <int D>
 __device__ __noinline__ int small_open_row(unsigned live, const float* __restrict__ X, int64_t i, const float* __restrict__ C,
-                                           int k, float g, unsigned* amb, unsigned* ev64) {
+                                           int k, float g, float thr, unsigned* ev64) {
     float x[D];
 #pragma unroll
     for (int l = 0; l < D; l++) x[l] = X[i * D + l];
@@ -715,36 +835,31 @@ __device__ __noinline__ int small_open_row(unsigned live, const float* __restric
         }
         return acc;
     };
-    float b1 = INFINITY, b2 = INFINITY;
-    int j1 = 0;
-    for (int j = 0; j < k; j++) {
-        const float v = value(j);
-        if (v < b1) {
-            b2 = b1;
-            b1 = v;
-            j1 = j;
-        } else if (v < b2) {
-            b2 = v;
-        }
-    }
-    const float thr = direct_upper(b1, g, direct_tiny(D));
-    const bool open = !(direct_lower(b2, g) > thr);
-    *amb += open ? 1u : 0u;
-    // each lane goes on to its next candidate, then the lanes evaluate theirs together
-    // (each at its own index, where almost every index is some lane's, 1e6 rows x 5 on
-    // eight pairs of equal centres took 750 us, 115 so)
+    int j1 = 0;  // (no value to compare, NaN: a valid label all the same)
+    // the candidates are listed first, all lanes at the same centre, then the lanes
+    // evaluate theirs together (each when it comes to it, where almost every centre is
+    // some lane's, 1e6 rows x 5 on eight pairs of equal centres took 750 us, 116 so)
+    constexpr int LIST = 8;
+    int cj[LIST], cnt = 0;
     double best = INFINITY;
-    for (int j = open ? 0 : k;; j++) {
-        while (j < k && !(direct_lower(value(j), g) <= thr)) j++;
-        if (!__any_sync(live, j < k)) break;
-        if (j >= k) continue;
-        const double s = direct64(x, C + j * D, D);
-        ++*ev64;
-        if (s < best) {
-            best = s;
-            j1 = j;
+    auto evaluate = [&]() {
+        for (int t = 0; __any_sync(live, t < cnt); t++) {
+            if (t >= cnt) continue;
+            const int j = cj[t];
+            const double s = direct64(x, C + j * D, D);
+            ++*ev64;
+            if (s < best) {
+                best = s;
+                j1 = j;
+            }
         }
+        cnt = 0;
+    };
+    for (int j = 0; j < k; j++) {
+        if (direct_lower(value(j), g) <= thr) cj[cnt++] = j;
+        if (__any_sync(live, cnt == LIST)) evaluate();
     }
+    evaluate();
     return j1;
 }
 
@@ -889,6 +1004,7 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
         }
         slot = slot + 1 == DS_STAGES ? 0 : slot + 1;
         int ja = -1, jb = -1;
+        float2 b1;
         bool direct = !ds_window(D) || skip > 0;
         if constexpr (ds_window(D)) {
             if (!direct) {
@@ -900,7 +1016,7 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
                 }
                 const float2 W = __ffma2_rn(make_float2(wscale, wscale), __fadd2_rn(p, make_float2(qmax, qmax)),
                                             make_float2(0x1p-120f, 0x1p-120f));
-                ds_scan<D, false, MANY>(dsm, kp, y, W, 0.0f, ja, jb);
+                ds_scan<D, false, MANY>(dsm, kp, y, W, 0.0f, ja, jb, b1);
                 const unsigned o0 = __ballot_sync(0xffffffffu, valid0 && ja < 0), o1 = __ballot_sync(0xffffffffu, valid1 && jb < 0);
                 if (__popc(o0) + __popc(o1) > few) {
                     direct = true;
@@ -909,13 +1025,15 @@ __global__ void __launch_bounds__(256, 3) k_direct_small(const float* __restrict
             }
         }
         if (direct) {
-            ds_scan<D, true, MANY>(cdir, kp, x, make_float2(wdir, wdir), rel, ja, jb);
+            ds_scan<D, true, MANY>(cdir, kp, x, make_float2(wdir, wdir), rel, ja, jb, b1);
             skip -= skip > 0 ? 1 : 0;
         }
         unsigned o0 = __ballot_sync(0xffffffffu, valid0 && ja < 0), o1 = __ballot_sync(0xffffffffu, valid1 && jb < 0);
         if (__popc(o0) + __popc(o1) > few) {
-            if ((o0 >> lane) & 1u) ja = small_open_row<D>(o0, X, g0, C, k, gamma32, &local_amb, &ev64);
-            if ((o1 >> lane) & 1u) jb = small_open_row<D>(o1, X, g1, C, k, gamma32, &local_amb, &ev64);
+            // (only after the direct pass)
+            if ((o0 >> lane) & 1u) ja = small_open_row<D>(o0, X, g0, C, k, gamma32, direct_upper(b1.x, gamma32, direct_tiny(D)), &ev64);
+            if ((o1 >> lane) & 1u) jb = small_open_row<D>(o1, X, g1, C, k, gamma32, direct_upper(b1.y, gamma32, direct_tiny(D)), &ev64);
+            local_amb += ((o0 >> lane) & 1u) + ((o1 >> lane) & 1u);
         } else {
             for (; o0 | o1; o0 ? o0 &= o0 - 1 : o1 &= o1 - 1) {
                 const int b = __ffs(o0 ? o0 : o1) - 1;

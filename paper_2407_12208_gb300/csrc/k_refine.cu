@@ -361,6 +361,110 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
     if (lane == 0 && ev64) atomicAdd(&cnt->fp64_evals, ev64);
 }
 
+// One row by a warp: the candidates of its lists (cand: the row's column of them; n0,
+// n1, n2 entries) inside rlim, `total` of them, in fp32, and in binary64 where their
+// intervals overlap.  Returns the lane's binary64 evaluations, and 1 << 16 if any.
+KM_DEV unsigned refine_row_warp(const uint32_t* __restrict__ cand, int64_t n, int n0, int n1, int n2, float rlim,
+                                                 int total, int row, const float* __restrict__ X, const float* __restrict__ C,
+                                                 int d, uint32_t emask, float lscale, float g, int32_t* __restrict__ labels,
+                                                 int* js, float* vs, double* prod) {
+    constexpr int NE = TC_GROUPS * TC_LIST;
+    const int lane = threadIdx.x & 31, sl = lane & 7;
+    const float tiny = direct_tiny(d);
+    unsigned ev64 = 0;
+    uint32_t e[2];
+    unsigned m[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int t = lane + 32 * h, gr = t / TC_LIST, slot = t % TC_LIST;
+        const bool have = t < NE && slot < (gr == 0 ? n0 : (gr == 1 ? n1 : n2));
+        e[h] = have ? cand[(size_t)t * n] : 0u;
+        m[h] = have && cand_lower(e[h], emask, lscale) <= rlim ? entry_mask(e[h]) : 0u;
+    }
+    const int mine = __popc(m[0]) + __popc(m[1]);
+    int incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += o;
+    }
+    __syncwarp();
+    int w = incl - mine;
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+        for (unsigned bb = m[h]; bb; bb &= bb - 1) js[w++] = 4 * entry_quad(e[h], emask) + __ffs(bb) - 1;
+    __syncwarp();
+    const float* x = X + (int64_t)row * d;
+    for (int t0 = 0; t0 < total; t0 += 4) {
+        const int t = t0 + (lane >> 3);
+        float acc = t < total ? pair_value<0>(X, C, d, make_int2(row, js[t]), sl) : 0.0f;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (sl == 0 && t < total) vs[t] = acc;
+    }
+    __syncwarp();
+    float up = INFINITY;
+    for (int t = lane; t < total; t += 32) up = fminf(up, direct_upper(vs[t], g, tiny));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) up = fminf(up, __shfl_xor_sync(0xffffffffu, up, off));
+    int open = 0, bj = 0x7fffffff;
+    for (int t = lane; t < total; t += 32)
+        if (direct_lower(vs[t], g) <= up) {
+            open++;
+            bj = js[t];  // (the only one, when open is 1 over the warp)
+        }
+    const unsigned who = __ballot_sync(0xffffffffu, open != 0);
+    open = __reduce_add_sync(0xffffffffu, open);
+    if (open == 1) {
+        if (lane == __ffs(who) - 1) labels[row] = bj;
+        return 0u;
+    }
+    // binary64, two candidates at a time: products by all lanes, a lane each adds one's
+    double best = INFINITY;
+    bj = 0x7fffffff;
+    for (int t = 0; t < total;) {
+        int jc[2] = {0, 0}, nc = 0;
+        for (; t < total && nc < 2; t++)
+            if (direct_lower(vs[t], g) <= up) {
+                jc[1] = js[t];
+                if (nc++ == 0) jc[0] = jc[1];
+            }
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            if (c >= nc) break;
+            const float* cj = C + (int64_t)jc[c] * d;
+            for (int l = lane; l < d; l += 32) {
+                const double u = __dsub_rn((double)x[l], (double)cj[l]);
+                prod[c * d + l] = __dmul_rn(u, u);
+            }
+        }
+        __syncwarp();
+        if (lane < nc) {
+            const double* p = prod + lane * d;
+            const int j = lane ? jc[1] : jc[0];
+            double s = 0.0;
+#pragma unroll 8
+            for (int l = 0; l < d; l++) s = __dadd_rn(s, p[l]);
+            ev64++;
+            if (s < best || (s == best && j < bj)) { best = s; bj = j; }
+        }
+        __syncwarp();
+    }
+    const double ob = __shfl_xor_sync(0xffffffffu, best, 1);
+    const int oj = __shfl_xor_sync(0xffffffffu, bj, 1);
+    if (ob < best || (ob == best && oj < bj)) bj = oj;
+    if (lane == 0) labels[row] = bj != 0x7fffffff ? bj : js[0];  // (not a number: a valid label all the same)
+    return ev64 | 1u << 16;
+}
+// Out of line where the rows' coordinates are in registers (4e6 x 64: 220 -> 205 us),
+// in line where they are not (500,000 x 50: 187 us, 203 out of line).
+__device__ __noinline__ unsigned refine_row_warp_call(const uint32_t* __restrict__ cand, int64_t n, int n0, int n1, int n2,
+                                                      float rlim, int total, int row, const float* __restrict__ X,
+                                                      const float* __restrict__ C, int d, uint32_t emask, float lscale, float g,
+                                                      int32_t* __restrict__ labels, int* js, float* vs, double* prod) {
+    return refine_row_warp(cand, n, n0, n1, n2, rlim, total, row, X, C, d, emask, lscale, g, labels, js, vs, prod);
+}
+
 // 32 rows per warp and round.  A lane per row reads the entries of the row's
 // three lists (slot-major: 32 rows side by side) that lie inside the window of
 // the row's final d^ minimum, the smallest of the groups' minima.  Rows with 2
@@ -371,7 +475,7 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
 // or few centres: all of them in tiles take less than a row at a time; 89,201 x
 // 173, k = 28, all pairs open: 340 us one by one, 138 in tiles), else, like those whose intervals
 // overlap, they take the whole warp, which ends in binary64 (products in
-// parallel, one lane adds them in coordinate order).
+// parallel, two candidates' sums at a time, each added in coordinate order by a lane).
 // Labels only: every caller refines the winner's distance afterwards, to
 // binary64 accuracy.
 // LIST: the rows are list[0 .. *list_n) of X (r indexes the lists), else all n.
@@ -392,13 +496,13 @@ __global__ void __launch_bounds__(256, NV == 0 ? 4 : 0) k_refine(const int2* __r
     chain_enter();
     constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
     static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
-    extern __shared__ double rc_sm[];  // per warp: d products
+    extern __shared__ double rc_sm[];  // per warp: 2 d products
     __shared__ int js_sh[8][4 * NE];
     __shared__ float vs_sh[8][4 * NE];
     __shared__ int jl_sh[8][RF_FEW * 32], ord_sh[8][32];
     const int64_t nrows = LIST ? (int64_t)*list_n : n;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, sl = lane & 7;
-    double* prod = rc_sm + (size_t)wib * d;
+    double* prod = rc_sm + (size_t)wib * 2 * d;
     int* js = js_sh[wib];
     float* vs = vs_sh[wib];
     int *jl = jl_sh[wib], *ord = ord_sh[wib];
@@ -547,84 +651,26 @@ __global__ void __launch_bounds__(256, NV == 0 ? 4 : 0) k_refine(const int2* __r
             const int total = __shfl_sync(0xffffffffu, c, b);
             const int n0 = __shfl_sync(0xffffffffu, cnt_g[0], b), n1 = __shfl_sync(0xffffffffu, cnt_g[1], b);
             const int n2 = __shfl_sync(0xffffffffu, cnt_g[2], b);
-            uint32_t e[2];
-            unsigned m[2];
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const int t = lane + 32 * h, gr = t / TC_LIST, slot = t % TC_LIST;
-                const bool have = t < NE && slot < (gr == 0 ? n0 : (gr == 1 ? n1 : n2));
-                e[h] = have ? cand[(size_t)t * n + r0 + b] : 0u;
-                m[h] = have && cand_lower(e[h], emask, lscale) <= rlim ? entry_mask(e[h]) : 0u;
+            unsigned r;
+            if constexpr (NV > 0)
+                r = refine_row_warp_call(cand + r0 + b, n, n0, n1, n2, rlim, total, (int)row, X, C, d, emask, lscale, g, labels,
+                                         js, vs, prod);
+            else
+                r = refine_row_warp(cand + r0 + b, n, n0, n1, n2, rlim, total, (int)row, X, C, d, emask, lscale, g, labels, js,
+                                    vs, prod);
+            ev64 += r & 0xffffu;
+            if (lane == 0) {
+                amb += r >> 16;
+                if (total > RF_FEW) ev32 += total;
             }
-            const int mine = __popc(m[0]) + __popc(m[1]);
-            int incl = mine;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int o = __shfl_up_sync(0xffffffffu, incl, off);
-                if (lane >= off) incl += o;
-            }
-            __syncwarp();
-            int w = incl - mine;
-#pragma unroll
-            for (int h = 0; h < 2; h++)
-                for (unsigned bb = m[h]; bb; bb &= bb - 1) js[w++] = 4 * entry_quad(e[h], emask) + __ffs(bb) - 1;
-            __syncwarp();
-            const float* x = X + row * d;
-            for (int t0 = 0; t0 < total; t0 += 4) {
-                const int t = t0 + (lane >> 3);
-                float acc = t < total ? pair_value<0>(X, C, d, make_int2((int)row, js[t]), sl) : 0.0f;
-#pragma unroll
-                for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                if (sl == 0 && t < total) vs[t] = acc;
-            }
-            __syncwarp();
-            if (lane == 0 && total > RF_FEW) ev32 += total;
-            float up = INFINITY;
-            for (int t = lane; t < total; t += 32) up = fminf(up, direct_upper(vs[t], g, tiny));
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) up = fminf(up, __shfl_xor_sync(0xffffffffu, up, off));
-            int open = 0, bj = 0x7fffffff;
-            for (int t = lane; t < total; t += 32)
-                if (direct_lower(vs[t], g) <= up) {
-                    open++;
-                    bj = js[t];  // (the only one, when open is 1 over the warp)
-                }
-            const unsigned who = __ballot_sync(0xffffffffu, open != 0);
-            open = __reduce_add_sync(0xffffffffu, open);
-            if (open == 1) {
-                if (lane == __ffs(who) - 1) labels[row] = bj;
-                continue;
-            }
-            if (lane == 0) amb++;
-            double best = INFINITY;
-            bj = 0x7fffffff;
-            for (int t = 0; t < total; t++) {
-                if (!(direct_lower(vs[t], g) <= up)) continue;
-                const int j = js[t];
-                const float* cj = C + (int64_t)j * d;
-                for (int l = lane; l < d; l += 32) {
-                    const double u = __dsub_rn((double)x[l], (double)cj[l]);
-                    prod[l] = __dmul_rn(u, u);
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    double s = 0.0;
-#pragma unroll 8
-                    for (int l = 0; l < d; l++) s = __dadd_rn(s, prod[l]);
-                    ev64++;
-                    if (s < best || (s == best && j < bj)) { best = s; bj = j; }
-                }
-                __syncwarp();
-            }
-            if (lane == 0) labels[row] = bj != 0x7fffffff ? bj : js[0];  // (not a number: a valid label all the same)
         }
         __syncwarp();
     }
     ev32 = __reduce_add_sync(0xffffffffu, ev32);
+    if (ev64) atomicAdd(&cnt->fp64_evals, (unsigned long long)ev64);  // (lanes 0 and 1)
     ovf = __reduce_add_sync(0xffffffffu, ovf);
     if (lane == 0) {
         if (ev32) atomicAdd(&cnt->fp32_evals, (unsigned long long)ev32);
-        if (ev64) atomicAdd(&cnt->fp64_evals, (unsigned long long)ev64);
         if (amb) atomicAdd(&cnt->amb_rows, (unsigned long long)amb);
         if (ovf && !LIST) atomicAdd(&cnt->ovf_rows, (unsigned long long)ovf);
     }
@@ -689,7 +735,7 @@ static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs
     const int threads = LIST ? (a.n <= (int64_t)num_sms * 256 ? 32 : 256)
                              : 32 * (int)std::max<int64_t>(1, std::min<int64_t>(8, (warps + num_sms - 1) / num_sms));
     const int per_block = threads / 32 * rpw;
-    const size_t sm = (size_t)(threads / 32) * a.d * sizeof(double);
+    const size_t sm = (size_t)(threads / 32) * 2 * a.d * sizeof(double);
     cudaError_t e = allow_max_smem(fn);
     if (e != cudaSuccess) return e;
     int per_sm = 1;

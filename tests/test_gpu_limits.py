@@ -308,6 +308,31 @@ def test_few_coordinates_time(ctx, d, k, than, most):
     assert times[0] < most * times[1], times
 
 
+# ties: rows between equal centres, a few and all of a block's, by the warp (eight at a time; a centre
+# or a coordinate per lane, four, two or one binary64 sums together, more candidates than it lists at
+# once) and by the block
+@pytest.mark.parametrize("every", [1, 13, 40])
+@pytest.mark.parametrize("n,d,k,copies", [(365, 128, 20, 2), (200, 9, 17, 2), (333, 31, 70, 2), (333, 32, 70, 35), (300, 64, 66, 33),
+                                          (129, 217, 64, 2), (131, 218, 130, 3), (257, 256, 128, 64), (5000, 20, 300, 4),
+                                          (40000, 16, 65, 5), (300, 12, 200, 200)])
+def test_ties(ctx, n, d, k, copies, every):
+    import paper_2407_12208_gb300 as pkg
+    r = np.random.default_rng(n + d + k)
+    base = r.random(size=(k // copies, d)).astype(np.float32)
+    C = np.concatenate([np.tile(base, (copies, 1)), 9 + r.random(size=(k - k // copies * copies, d))]).astype(np.float32)
+    X = (9 + r.random(size=(n, d))).astype(np.float32)  # nearest to one of the last, or tied as well
+    X[::every] = r.random(size=X[::every].shape)
+    lab, md, _ = ctx.assign(_dev(X), _dev(C), pkg.params("fp32"))
+    lab, md = lab.cpu().numpy(), md.cpu().numpy()
+    olab, od1, _ = oracle.assign(X, C)
+    _, first, inverse = np.unique(C, axis=0, return_index=True, return_inverse=True)
+    assert np.array_equal(first[inverse.ravel()][lab], lab)
+    far = np.abs(lab - olab) > 0  # (ties between different rows of base: within rounding)
+    assert far.mean() < 0.01
+    np.testing.assert_allclose(md, oracle.dist_labelled(X, C, lab), rtol=RTOL_MD)
+    np.testing.assert_allclose(md, od1, rtol=1e-6)
+
+
 # small-d centre sums: chunks of 32 rows and more per warp, eight warps folded together, in the last
 # block too; steps of one label, a few, many in runs and in no order
 @pytest.mark.parametrize("kind", ["spread", "sorted", "one", "two", "most", "runs"])
@@ -334,3 +359,15 @@ def test_small_d_sums_time(ctx, n, d, k):
         lab = torch.from_numpy(_labels(kind, n, k, np.random.default_rng(3))).cuda()
         times.append(_time(lambda: ctx.update_centroids(X, lab, X[:k], p, want_shift=False)))
     assert times[0] < 1.8 * times[1], times
+
+
+# a block of tied rows takes its warps, not its turns
+def test_ties_time(ctx):
+    times = []
+    for copies in (1, 2):
+        X = torch.rand(365, 128, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+        C = X[: 20 // copies].repeat(copies, 1).contiguous()
+        lab = torch.empty(365, dtype=torch.int32, device="cuda")
+        md = torch.empty(365, dtype=torch.float64, device="cuda")
+        times.append(_time(lambda: ctx.assign_static(X, C, lab, md)))
+    assert times[1] < times[0] + 0.12, times
