@@ -361,17 +361,70 @@ __global__ void __launch_bounds__(256) k_amb_fp64(const int32_t* __restrict__ am
     if (lane == 0 && ev64) atomicAdd(&cnt->fp64_evals, ev64);
 }
 
+// The candidates of a row that the fp32 values vs[0 .. total) leave open (their interval
+// reaches up), in binary64 by a warp.  Returns the lane's evaluations.
+KM_DEV unsigned refine_row_exact(const float* __restrict__ x, const float* __restrict__ C, int d, int total, float g, float up,
+                                 int32_t* __restrict__ label, const int* js, const float* vs, double* prod) {
+    const int lane = threadIdx.x & 31;
+    unsigned ev64 = 0;
+    // two candidates at a time: products by all lanes, a lane each adds one's
+    double best = INFINITY;
+    int bj = 0x7fffffff;
+    for (int t = 0; t < total;) {
+        int jc[2] = {0, 0}, nc = 0;
+        for (; t < total && nc < 2; t++)
+            if (direct_lower(vs[t], g) <= up) {
+                jc[1] = js[t];
+                if (nc++ == 0) jc[0] = jc[1];
+            }
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            if (c >= nc) break;
+            const float* cj = C + (int64_t)jc[c] * d;
+            for (int l = lane; l < d; l += 32) {
+                const double u = __dsub_rn((double)x[l], (double)cj[l]);
+                prod[c * d + l] = __dmul_rn(u, u);
+            }
+        }
+        __syncwarp();
+        if (lane < nc) {
+            const double* p = prod + lane * d;
+            const int j = lane ? jc[1] : jc[0];
+            double s = 0.0;
+#pragma unroll 8
+            for (int l = 0; l < d; l++) s = __dadd_rn(s, p[l]);
+            ev64++;
+            if (s < best || (s == best && j < bj)) { best = s; bj = j; }
+        }
+        __syncwarp();
+    }
+    const double ob = __shfl_xor_sync(0xffffffffu, best, 1);
+    const int oj = __shfl_xor_sync(0xffffffffu, bj, 1);
+    if (ob < best || (ob == best && oj < bj)) bj = oj;
+    if (lane == 0) *label = bj != 0x7fffffff ? bj : js[0];  // (not a number: a valid label all the same)
+    return ev64;
+}
+
+// Out of line where the rows' coordinates are in registers, for few rows come this far
+// (4e6 x 64, k = 256, refinement with the winners' distances: bf16 497 us, 501 with the
+// fp32 part out of line as well, 510 with nothing; e4m3, where more rows take the
+// fp32 part, 908, 935 and 915), in line where they are not (500,000 x 50: 187 us, 203).
+__device__ __noinline__ unsigned refine_row_exact_call(const float* __restrict__ x, const float* __restrict__ C, int d, int total,
+                                                       float g, float up, int32_t* __restrict__ label, const int* js,
+                                                       const float* vs, double* prod) {
+    return refine_row_exact(x, C, d, total, g, up, label, js, vs, prod);
+}
+
 // One row by a warp: the candidates of its lists (cand: the row's column of them; n0,
 // n1, n2 entries) inside rlim, `total` of them, in fp32, and in binary64 where their
 // intervals overlap.  Returns the lane's binary64 evaluations, and 1 << 16 if any.
-KM_DEV unsigned refine_row_warp(const uint32_t* __restrict__ cand, int64_t n, int n0, int n1, int n2, float rlim,
-                                                 int total, int row, const float* __restrict__ X, const float* __restrict__ C,
-                                                 int d, uint32_t emask, float lscale, float g, int32_t* __restrict__ labels,
-                                                 int* js, float* vs, double* prod) {
+template <bool CALL>
+KM_DEV unsigned refine_row_warp(const uint32_t* __restrict__ cand, int64_t n, int n0, int n1, int n2, float rlim, int total,
+                                int row, const float* __restrict__ X, const float* __restrict__ C, int d, uint32_t emask,
+                                float lscale, float g, int32_t* __restrict__ labels, int* js, float* vs, double* prod) {
     constexpr int NE = TC_GROUPS * TC_LIST;
     const int lane = threadIdx.x & 31, sl = lane & 7;
     const float tiny = direct_tiny(d);
-    unsigned ev64 = 0;
     uint32_t e[2];
     unsigned m[2];
 #pragma unroll
@@ -419,50 +472,8 @@ KM_DEV unsigned refine_row_warp(const uint32_t* __restrict__ cand, int64_t n, in
         if (lane == __ffs(who) - 1) labels[row] = bj;
         return 0u;
     }
-    // binary64, two candidates at a time: products by all lanes, a lane each adds one's
-    double best = INFINITY;
-    bj = 0x7fffffff;
-    for (int t = 0; t < total;) {
-        int jc[2] = {0, 0}, nc = 0;
-        for (; t < total && nc < 2; t++)
-            if (direct_lower(vs[t], g) <= up) {
-                jc[1] = js[t];
-                if (nc++ == 0) jc[0] = jc[1];
-            }
-#pragma unroll
-        for (int c = 0; c < 2; c++) {
-            if (c >= nc) break;
-            const float* cj = C + (int64_t)jc[c] * d;
-            for (int l = lane; l < d; l += 32) {
-                const double u = __dsub_rn((double)x[l], (double)cj[l]);
-                prod[c * d + l] = __dmul_rn(u, u);
-            }
-        }
-        __syncwarp();
-        if (lane < nc) {
-            const double* p = prod + lane * d;
-            const int j = lane ? jc[1] : jc[0];
-            double s = 0.0;
-#pragma unroll 8
-            for (int l = 0; l < d; l++) s = __dadd_rn(s, p[l]);
-            ev64++;
-            if (s < best || (s == best && j < bj)) { best = s; bj = j; }
-        }
-        __syncwarp();
-    }
-    const double ob = __shfl_xor_sync(0xffffffffu, best, 1);
-    const int oj = __shfl_xor_sync(0xffffffffu, bj, 1);
-    if (ob < best || (ob == best && oj < bj)) bj = oj;
-    if (lane == 0) labels[row] = bj != 0x7fffffff ? bj : js[0];  // (not a number: a valid label all the same)
-    return ev64 | 1u << 16;
-}
-// Out of line where the rows' coordinates are in registers (4e6 x 64: 220 -> 205 us),
-// in line where they are not (500,000 x 50: 187 us, 203 out of line).
-__device__ __noinline__ unsigned refine_row_warp_call(const uint32_t* __restrict__ cand, int64_t n, int n0, int n1, int n2,
-                                                      float rlim, int total, int row, const float* __restrict__ X,
-                                                      const float* __restrict__ C, int d, uint32_t emask, float lscale, float g,
-                                                      int32_t* __restrict__ labels, int* js, float* vs, double* prod) {
-    return refine_row_warp(cand, n, n0, n1, n2, rlim, total, row, X, C, d, emask, lscale, g, labels, js, vs, prod);
+    if constexpr (CALL) return refine_row_exact_call(x, C, d, total, g, up, labels + row, js, vs, prod) | 1u << 16;
+    else return refine_row_exact(x, C, d, total, g, up, labels + row, js, vs, prod) | 1u << 16;
 }
 
 // 32 rows per warp and round.  A lane per row reads the entries of the row's
@@ -486,6 +497,7 @@ __device__ __noinline__ unsigned refine_row_warp_call(const uint32_t* __restrict
 // (NV = 0 keeps 64 registers: given its own way the compiler took 48 and spilled,
 // 300,000 x 77 134 us against 106.)
 constexpr int RF_FEW = 12;
+constexpr int RF_PROD_D = RF_FEW * 32 * (int)sizeof(int) / (2 * (int)sizeof(double));  // 2 d products in jl
 template <int NV, bool LIST>
 __global__ void __launch_bounds__(256, NV == 0 ? 4 : 0) k_refine(const int2* __restrict__ rowinfo, const float* __restrict__ roww, const uint32_t* __restrict__ cand,
                                                 int64_t n, int ng, int ebits, const int32_t* __restrict__ list,
@@ -496,16 +508,19 @@ __global__ void __launch_bounds__(256, NV == 0 ? 4 : 0) k_refine(const int2* __r
     chain_enter();
     constexpr int NE = TC_GROUPS * TC_LIST;  // entries of a row's lists
     static_assert(NE <= 64 && TC_GROUPS == 3, "two entries per lane of three lists");
-    extern __shared__ double rc_sm[];  // per warp: 2 d products
+    extern __shared__ double rc_sm[];  // per warp: 2 d products, where jl has no room for them
     __shared__ int js_sh[8][4 * NE];
     __shared__ float vs_sh[8][4 * NE];
-    __shared__ int jl_sh[8][RF_FEW * 32], ord_sh[8][32];
+    __shared__ __align__(8) int jl_sh[8][RF_FEW * 32];
+    __shared__ int ord_sh[8][32];
     const int64_t nrows = LIST ? (int64_t)*list_n : n;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, sl = lane & 7;
-    double* prod = rc_sm + (size_t)wib * 2 * d;
     int* js = js_sh[wib];
     float* vs = vs_sh[wib];
     int *jl = jl_sh[wib], *ord = ord_sh[wib];
+    // (a row that takes the whole warp comes after the round's last use of jl; 8 KB a
+    // block of their own, at d = 64, leave L1 that much less: 921 us for the 908 above)
+    double* prod = d <= RF_PROD_D ? reinterpret_cast<double*>(jl) : rc_sm + (size_t)wib * 2 * d;
     const uint32_t emask = (1u << ebits) - 1u;
     const float lscale = __uint_as_float((uint32_t)(127 + ebits - 23) << 23);  // 2^(ebits - 23)
     const float g = gamma32, tiny = direct_tiny(d);
@@ -651,13 +666,8 @@ __global__ void __launch_bounds__(256, NV == 0 ? 4 : 0) k_refine(const int2* __r
             const int total = __shfl_sync(0xffffffffu, c, b);
             const int n0 = __shfl_sync(0xffffffffu, cnt_g[0], b), n1 = __shfl_sync(0xffffffffu, cnt_g[1], b);
             const int n2 = __shfl_sync(0xffffffffu, cnt_g[2], b);
-            unsigned r;
-            if constexpr (NV > 0)
-                r = refine_row_warp_call(cand + r0 + b, n, n0, n1, n2, rlim, total, (int)row, X, C, d, emask, lscale, g, labels,
-                                         js, vs, prod);
-            else
-                r = refine_row_warp(cand + r0 + b, n, n0, n1, n2, rlim, total, (int)row, X, C, d, emask, lscale, g, labels, js,
-                                    vs, prod);
+            const unsigned r = refine_row_warp<(NV > 0)>(cand + r0 + b, n, n0, n1, n2, rlim, total, (int)row, X, C, d, emask,
+                                                         lscale, g, labels, js, vs, prod);
             ev64 += r & 0xffffu;
             if (lane == 0) {
                 amb += r >> 16;
@@ -735,7 +745,7 @@ static cudaError_t launch_refine_nv(const float* X, const float* C, const TcArgs
     const int threads = LIST ? (a.n <= (int64_t)num_sms * 256 ? 32 : 256)
                              : 32 * (int)std::max<int64_t>(1, std::min<int64_t>(8, (warps + num_sms - 1) / num_sms));
     const int per_block = threads / 32 * rpw;
-    const size_t sm = (size_t)(threads / 32) * 2 * a.d * sizeof(double);
+    const size_t sm = a.d <= RF_PROD_D ? 0 : (size_t)(threads / 32) * 2 * a.d * sizeof(double);
     cudaError_t e = allow_max_smem(fn);
     if (e != cudaSuccess) return e;
     int per_sm = 1;

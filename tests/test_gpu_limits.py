@@ -361,6 +361,23 @@ def test_small_d_sums_time(ctx, n, d, k):
     assert times[0] < 1.8 * times[1], times
 
 
+# ties in the refinement's one launch: the warp's binary64 products in the candidates' own shared memory
+# and past it, any width and alignment, odd and many candidates
+@pytest.mark.parametrize("low,n,d,k,copies", [("fp16", 500, 64, 30, 2), ("bf16", 300, 95, 60, 3), ("fp16", 300, 96, 60, 2),
+                                              ("bf16", 300, 97, 60, 3), ("fp16", 300, 100, 90, 18), ("bf16", 129, 256, 40, 20),
+                                              ("bf16", 5000, 33, 40, 3), ("e4m3", 5000, 64, 20, 4)])
+def test_ties_in_the_refinement(ctx, low, n, d, k, copies):
+    import paper_2407_12208_gb300 as pkg
+    r = np.random.default_rng(n + d + k)
+    base = 8 * r.integers(0, 2, size=(k // copies, d)) + r.random(size=(k // copies, d))
+    C = np.tile(base, (copies, 1)).astype(np.float32)
+    X = (C[r.integers(0, len(C), n)] + 0.1 * r.random(size=(n, d))).astype(np.float32)
+    lab, md, _ = ctx.assign(_dev(X), _dev(C), pkg.params(low))
+    lab, md = lab.cpu().numpy(), md.cpu().numpy()
+    assert np.array_equal(lab, oracle.assign(X, C)[0])
+    np.testing.assert_allclose(md, oracle.dist_labelled(X, C, lab), rtol=RTOL_MD)
+
+
 # a block of tied rows takes its warps, not its turns
 def test_ties_time(ctx):
     times = []
