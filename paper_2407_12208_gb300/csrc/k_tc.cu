@@ -26,7 +26,7 @@
 // us, with an epilogue that only releases its accumulators 262, and then 236 at
 // 4e6 x 64 x 256, whose tiles have half the MMAs: 1320 and 1190 cycles a tile of
 // the 411 per SM.  So that part is the tile's own (two bounded waits, a commit, an
-// accumulator's round trip), not the MMAs (117 us at the measured rate); the
+// accumulator's round trip), not the MMAs (135 us at the measured rate); the
 // walk over qualifying quads adds the rest, about 50 instructions an iteration
 // and a lane's worth of idle lanes.  Measured, with the row's numbers asked for
 // a block ahead (by the producer's L2 prefetch, then before the lists leave),
